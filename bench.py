@@ -891,7 +891,7 @@ def main():
         ss = std["stages_ms"]
         pix = d.num_views * d.width * d.height
         stages_roof["standard_composite"] = {
-            "kernel": "composite_full_binned_kernel (every pixel of every view into M_m)",
+            "kernel": "composite_views_warp_kernel (every pixel of every view into M_m)",
             **compositing_roofline(ss["composite"], ss["keys"], pix, ss["pairs_evaluated"],
                                    ss["pairs_blended"], hbm_gbs, hbm_source, alu_peaks)}
         stages_roof["standard_interweave"] = stage_roofline(

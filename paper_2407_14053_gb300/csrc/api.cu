@@ -125,6 +125,13 @@ constexpr int kRaysPerBlock = 128;
 // memory) falls back to the global radix sort.
 constexpr int kSmallCap = 1024;
 constexpr int kLargeCap = 16384;
+// Capacity of the block kernels' shared memory for lists of up to `keys` keys:
+// ten bytes a key, so in steps of 512 (a power of two would leave up to half
+// of it, and with it half of the resident blocks, unused).
+int list_capacity(int64_t keys) {
+    const int64_t c = (std::min<int64_t>(keys, int64_t(1) << 30) + 511) / 512 * 512;
+    return int(std::max<int64_t>(c, 2048));
+}
 
 size_t max_smem_optin(int device) {
     int v = 0;
@@ -1074,8 +1081,10 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
     const int64_t ngroups = int64_t(nv) * ntiles;
     if (ngroups >= (int64_t(1) << 31) - 1) return fail(ctx, DL_ERR_CAPACITY, "too many tiles");
     // DirectL: lists of up to warp_cap keys become warp items, longer ones go
-    // to the block kernel; standard: small / large block classes.
+    // to the block kernel; standard: the same split at 512 and 1024 keys
+    // (direct evaluation) or small / large block classes (transposed).
     const bool warp_path = mode != DL_STANDARD && ctx->warp_cap > 0;
+    const bool views_path = mode == DL_STANDARD && !ctx->eval_transposed[mode];
     // Sizing: the totals are read back (one host synchronisation) until a
     // frame of this signature has been sized; later frames run on the
     // signature's capacities and device counters, and are dropped on the
@@ -1179,6 +1188,12 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
                                     on_device ? d_nkeys : nullptr, key_cap,
                                     on_device ? d_status : nullptr, s),
               "partition");
+    } else if (views_path) {
+        GroupSlices sl;
+        sl.start = W.gstart.as<uint32_t>();
+        DL_CK(launch_partition_warp(nullptr, n_work, sl, 512u, 1024u, items, block_items, d_meta,
+                                    nullptr, 0u, nullptr, s),
+              "partition");
     } else {
         DL_CK(launch_partition(gwork, n_work, W.gstart.as<uint32_t>(), uint32_t(kSmallCap), small_list,
                                large_list, d_meta, s),
@@ -1186,7 +1201,7 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
     }
     DL_CK(mark(2), "event");
     int64_t nk = 0, n_visible = 0, n_small = 0, n_large = 0, n_mid = 0, max_len = 0;
-    int cap_large = warp_path ? 2048 : 1;
+    int cap_large = 2048;
     bool binned = true;
     if (on_device) {
         // upper bounds: the persistent kernels read the item counts on the device
@@ -1202,16 +1217,17 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
             reinterpret_cast<const uint32_t*>(reinterpret_cast<const char*>(W.h_total) + 128);
         n_small = h_meta[0];
         n_large = h_meta[1];
-        n_mid = warp_path ? int64_t(h_meta[4]) : 0;  // 1024-key warp class
+        n_mid = warp_path || views_path ? int64_t(h_meta[4]) : 0;  // 1024-key warp class
         max_len = h_meta[2];
         if (nkeys >= (1ull << 31) - 1)
             return fail(ctx, DL_ERR_CAPACITY, "frame needs %llu tile keys (limit 2^31-1)", nkeys);
         nk = int64_t(nkeys);
-        while (cap_large < max_len) cap_large <<= 1;
+        cap_large = list_capacity(max_len);
         const int binned_threads = mode == DL_STANDARD ? tw * th : kBinnedThreads;
-        const size_t class_smem = warp_path ? block_smem_bytes(cap_large)
-                                            : binned_smem_bytes(std::max(cap_large, kSmallCap),
-                                                                binned_threads);
+        const size_t class_smem = warp_path    ? block_smem_bytes(cap_large)
+                                  : views_path ? views_block_smem_bytes(cap_large)
+                                               : binned_smem_bytes(std::max(cap_large, kSmallCap),
+                                                                   binned_threads);
         binned = ctx->sort_mode != DL_SORT_RADIX && max_len <= kLargeCap &&
                  class_smem <= max_smem_optin(ctx->device);
         if (ctx->sort_mode == DL_SORT_BINNED && !binned)
@@ -1225,8 +1241,7 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
         if (warp_path && binned) {
             const int64_t laid = nk + nk / 8 + 16 * ngroups;
             const int64_t want = laid + laid / 4 + 65536;
-            int bc = 2048;
-            while (bc < kLargeCap && bc < max_len + max_len / 4) bc <<= 1;
+            const int bc = std::min(kLargeCap, list_capacity(max_len + max_len / 4));
             if (want < (int64_t(1) << 31) - 2 && block_smem_bytes(bc) <= max_smem_optin(ctx->device)) {
                 DL_CK(W.keys[0].reserve(8 * size_t(want)), "alloc keys");
                 hint.sized = true;
@@ -1300,14 +1315,20 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
         DL_CK(mark(5), "event");
         DL_CK(mark(6), "event");
         const unsigned long long* keys = W.keys[0].as<unsigned long long>();
-        if (mode == DL_STANDARD) {
+        if (views_path) {
+            const int64_t n[3] = {n_small, n_mid, n_large};
+            uint32_t* const cur[2] = {d_meta + 3, d_meta + 5};
+            DL_CK(launch_composite_views(cp, items, block_items, n_work, n, cap_large, cur, keys,
+                                         W.rec.as<float4>(), Mm, pairs, s),
+                  "composite views");
+        } else if (mode == DL_STANDARD) {
             DL_CK(launch_composite_full_binned(cp, small_list, n_small, kSmallCap,
                                                W.gstart.as<uint32_t>(), keys, W.rec.as<float4>(), Mm,
-                                               pairs, ctx->eval_transposed[mode], s),
+                                               pairs, s),
                   "composite full (small lists)");
             DL_CK(launch_composite_full_binned(cp, large_list, n_large, cap_large,
                                                W.gstart.as<uint32_t>(), keys, W.rec.as<float4>(), Mm,
-                                               pairs, ctx->eval_transposed[mode], s),
+                                               pairs, s),
                   "composite full (large lists)");
         } else if (warp_path) {
             // one frame through the frame-batched persistent kernels

@@ -15,6 +15,7 @@
 //    (Sec. 4 step (3): the channel reorder by precomputed indices).
 //  - composite_full_kernel (standard paradigm): one block per (view, tile),
 //    one thread per pixel, every pixel of every view into M_m.
+#include <algorithm>
 #include <climits>
 
 #include "dl_internal.cuh"
@@ -33,6 +34,12 @@ struct Acc {
 __device__ __forceinline__ float ex2_approx(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+__device__ __forceinline__ float rcp_approx(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
 
@@ -374,19 +381,30 @@ __global__ void composite_full_kernel(CompositeParams p, const uint2* __restrict
 }
 
 // ---------------------------------------------------------- binned path ---
-// Ascending bitonic sort of P (a power of two) unique keys in shared memory.
-__device__ void bitonic_sort(unsigned long long* s, int P) {
+// Ascending bitonic sort of n unique keys in shared memory, for any n: every
+// compared pair puts the larger key at the higher index, so positions past
+// the end act as larger than any key and are left out.
+__device__ void bitonic_sort(unsigned long long* s, int n) {
+    int P = 1;
+    while (P < n) P <<= 1;
+    auto order = [&](int lo, int hi) {
+        if (hi >= n) return;
+        const unsigned long long a = s[lo], b = s[hi];
+        if (a > b) {
+            s[lo] = b;
+            s[hi] = a;
+        }
+    };
     for (int k = 2; k <= P; k <<= 1) {
-        for (int j = k >> 1; j > 0; j >>= 1) {
+        for (int i = threadIdx.x; i < (P >> 1); i += blockDim.x) {  // mirrored pairs
+            const int off = i & ((k >> 1) - 1), base = (i - off) << 1;
+            order(base + off, base + k - 1 - off);
+        }
+        __syncthreads();
+        for (int j = k >> 2; j > 0; j >>= 1) {
             for (int i = threadIdx.x; i < (P >> 1); i += blockDim.x) {
                 const int lo = ((i & ~(j - 1)) << 1) | (i & (j - 1));
-                const int hi = lo + j;
-                const bool up = (lo & k) == 0;
-                const unsigned long long a = s[lo], b = s[hi];
-                if ((a > b) == up) {
-                    s[lo] = b;
-                    s[hi] = a;
-                }
+                order(lo, lo + j);
             }
             __syncthreads();
         }
@@ -430,29 +448,35 @@ __device__ void block_scan_counts(uint32_t* c, int n) {
     __syncthreads();
 }
 
-// largest bucket sorted inside its list (by one thread in the block sort, by
-// odd-even phases in the warp sort); a larger one sends the list to a bitonic sort
+// largest bucket whose keys the odd-even phases order; a larger one sends the
+// list to a bitonic sort
 constexpr int kBucketSortLimit = 64;
 
-// Sorts the group's keys (depth << 32 | Gaussian, all distinct) into sk:
-// a counting sort on the depth bucket floor((d - dmin) NB / (dmax - dmin + 1))
-// (monotone in d), then an insertion sort inside every bucket.  If a bucket
-// holds more than kBucketSortLimit keys (many equal depths), the whole list
-// is bitonic-sorted instead.  KPT > 0: the block holds the keys in registers
-// (len <= KPT * blockDim.x, one coalesced load); KPT == 0: the keys are read
-// from global memory once per pass.  sk holds next_pow2(len) keys; cnt holds
-// cap + 2 counters, cap >= len being the class capacity (a power of two).
-template <int KPT>
+// Sorts the group's keys (depth << 32 | Gaussian, all distinct) into sk: a
+// counting sort into depth buckets (monotone in the depth), then as many
+// odd-even transposition phases over the whole list as the most crowded
+// bucket holds keys (as in warp_sort below).  From 256 buckets on they are
+// equi-depth at a coarse grain: a first count over kBlockBins even bins gives
+// each bin a share of the buckets in proportion to its keys, since depths
+// cluster and crowded buckets set the number of phases.  If a bucket still
+// holds more than kBucketSortLimit keys (many equal depths), the whole list is
+// bitonic-sorted instead.  The keys are re-read (from L2) by every pass.  sk
+// holds cap keys and cnt cap / 2 counters, cap >= len being the class capacity
+// (a multiple of 512, at least 1024): ten bytes a key.  What bounds the block
+// classes is resident warps, which shared memory sets: 10 bytes a key of a
+// capacity in steps of 512, reused by the stream phase, against 12 of the next
+// power of two beside it, took 11,189 lists of up to 1862 keys (7.9-inch
+// panel) from 1.23 to 0.65 ms and 21,885 of up to 3072 (800 x 450 views) from
+// 3.4 to 2.5 ms.
+constexpr int kBlockBins = 128;
 __device__ void block_sort(const unsigned long long* __restrict__ keys, uint32_t start, int len,
                            int cap, unsigned long long* sk, uint32_t* cnt) {
-    __shared__ uint32_t s_lo, s_hi, s_big;
+    __shared__ uint32_t s_lo, s_hi, s_most;
     const int tid = threadIdx.x, nthr = blockDim.x;
-    constexpr int R = KPT > 0 ? KPT : 1;
-    unsigned long long kr[R];
     if (tid == 0) {
         s_lo = 0xFFFFFFFFu;
         s_hi = 0u;
-        s_big = 0u;
+        s_most = 0u;
     }
     __syncthreads();
     if (len <= 1) {
@@ -461,22 +485,10 @@ __device__ void block_sort(const unsigned long long* __restrict__ keys, uint32_t
         return;
     }
     uint32_t lo = 0xFFFFFFFFu, hi = 0u;
-    if (KPT > 0) {
-#pragma unroll
-        for (int j = 0; j < R; ++j) {
-            const int i = j * nthr + tid;
-            kr[j] = i < len ? keys[start + i] : ~0ull;
-            if (i < len) {
-                lo = min(lo, uint32_t(kr[j] >> 32));
-                hi = max(hi, uint32_t(kr[j] >> 32));
-            }
-        }
-    } else {
-        for (int i = tid; i < len; i += nthr) {
-            const uint32_t d = uint32_t(keys[start + i] >> 32);
-            lo = min(lo, d);
-            hi = max(hi, d);
-        }
+    for (int i = tid; i < len; i += nthr) {
+        const uint32_t d = uint32_t(keys[start + i] >> 32);
+        lo = min(lo, d);
+        hi = max(hi, d);
     }
     lo = __reduce_min_sync(0xffffffffu, lo);
     hi = __reduce_max_sync(0xffffffffu, hi);
@@ -484,71 +496,90 @@ __device__ void block_sort(const unsigned long long* __restrict__ keys, uint32_t
         atomicMin(&s_lo, lo);
         atomicMax(&s_hi, hi);
     }
+    // up to a bucket a key; the bins' table (kBlockBins + 1 words) ends the counters
+    constexpr int kTable = kBlockBins + 8;
     int NB = 1;
     while (NB < len) NB <<= 1;
-    NB = NB >> 1;
-    if (NB > cap / 2) NB = cap / 2;
-    if (NB < 1) NB = 1;
-    uint32_t* bstart = cnt;               // NB + 1
-    uint32_t* bfill = cnt + cap / 2 + 1;  // NB
-    for (int i = tid; i <= NB; i += nthr) bstart[i] = 0u;
-    for (int i = tid; i < NB; i += nthr) bfill[i] = 0u;
+    if (NB > cap / 2 - kTable) NB = cap / 2 - kTable;
+    const bool equi = NB >= 2 * kBlockBins;
+    uint32_t* const bstart = cnt;
+    uint32_t* const table = cnt + (cap / 2 - kTable);
+    for (int i = tid; i < NB; i += nthr) bstart[i] = 0u;
+    if (equi)
+        for (int i = tid; i <= kBlockBins; i += nthr) table[i] = 0u;
     __syncthreads();
     const uint32_t dmin = s_lo;
-    const float scale = float(NB) / (float(s_hi - s_lo) + 1.0f);
-    auto bucket = [&](unsigned long long k) {
-        return min(NB - 1, int(float(uint32_t(k >> 32) - dmin) * scale));
-    };
-    if (KPT > 0) {
-#pragma unroll
-        for (int j = 0; j < R; ++j)
-            if (j * nthr + tid < len) atomicAdd(&bstart[bucket(kr[j])], 1u);
-    } else {
-        for (int i = tid; i < len; i += nthr) atomicAdd(&bstart[bucket(keys[start + i])], 1u);
+    const float scale = float(equi ? kBlockBins : NB) / (float(s_hi - dmin) + 1.0f);
+    if (equi) {
+        for (int i = tid; i < len; i += nthr) {
+            const float t = float(uint32_t(keys[start + i] >> 32) - dmin) * scale;
+            atomicAdd(&table[min(kBlockBins - 1, int(t))], 1u);
+        }
+        __syncthreads();
+        for (int c = tid; c < kBlockBins; c += nthr) {
+            const uint32_t n = table[c];
+            table[c] = n ? uint32_t(uint64_t(n) * uint32_t(NB - kBlockBins) / uint32_t(len)) + 1u : 0u;
+        }
+        __syncthreads();
+        block_scan_counts(table, kBlockBins + 1);  // bin c: buckets [table[c], table[c + 1])
     }
+    auto bucket = [&](unsigned long long k) {
+        const float t = float(uint32_t(k >> 32) - dmin) * scale;
+        if (!equi) return min(NB - 1, int(t));
+        const int c = min(kBlockBins - 1, int(t));
+        const int first = int(table[c]), nb = int(table[c + 1]) - first;
+        return first + min(nb - 1, int((t - float(c)) * float(nb)));
+    };
+    for (int i = tid; i < len; i += nthr) atomicAdd(&bstart[bucket(keys[start + i])], 1u);
+    __syncthreads();
+    uint32_t most = 0u;
+    for (int b = tid; b < NB; b += nthr) most = max(most, bstart[b]);
+    most = __reduce_max_sync(0xffffffffu, most);
+    if ((tid & 31) == 0) atomicMax(&s_most, most);
     __syncthreads();
     block_scan_counts(bstart, NB);
-    if (tid == 0) bstart[NB] = uint32_t(len);
-    __syncthreads();
-    if (KPT > 0) {
-#pragma unroll
-        for (int j = 0; j < R; ++j)
-            if (j * nthr + tid < len) {
-                const int b = bucket(kr[j]);
-                sk[bstart[b] + atomicAdd(&bfill[b], 1u)] = kr[j];
-            }
-    } else {
-        for (int i = tid; i < len; i += nthr) {
-            const unsigned long long k = keys[start + i];
-            const int b = bucket(k);
-            sk[bstart[b] + atomicAdd(&bfill[b], 1u)] = k;
-        }
+    most = s_most;
+    for (int i = tid; i < len; i += nthr) {  // bstart[b]: the bucket's cursor
+        const unsigned long long k = keys[start + i];
+        sk[atomicAdd(&bstart[bucket(k)], 1u)] = k;
     }
     __syncthreads();
-    for (int b = tid; b < NB; b += nthr)
-        if (bstart[b + 1] - bstart[b] > uint32_t(kBucketSortLimit)) s_big = 1u;
-    __syncthreads();
-    if (s_big) {
-        int P = 1;
-        while (P < len) P <<= 1;
-        for (int i = len + tid; i < P; i += nthr) sk[i] = ~0ull;
-        __syncthreads();
-        bitonic_sort(sk, P);
+    if (most > uint32_t(kBucketSortLimit)) {
+        bitonic_sort(sk, len);
     } else {
-        for (int b = tid; b < NB; b += nthr) {
-            const int b0 = int(bstart[b]), b1 = int(bstart[b + 1]);
-            for (int i = b0 + 1; i < b1; ++i) {
-                const unsigned long long k = sk[i];
-                int j = i - 1;
-                while (j >= b0 && sk[j] > k) {
-                    sk[j + 1] = sk[j];
-                    --j;
+        ulonglong2* const two = reinterpret_cast<ulonglong2*>(sk);
+        for (uint32_t ph = 0; most > 1u && ph < most; ++ph) {
+            if ((ph & 1u) == 0u) {
+                for (int i = tid; 2 * i + 1 < len; i += nthr) {
+                    const ulonglong2 q = two[i];
+                    if (q.x > q.y) two[i] = make_ulonglong2(q.y, q.x);
                 }
-                sk[j + 1] = k;
+            } else {
+                for (int i = 2 * tid + 1; i + 1 < len; i += 2 * nthr) {
+                    const unsigned long long x = sk[i], y = sk[i + 1];
+                    if (x > y) {
+                        sk[i] = y;
+                        sk[i + 1] = x;
+                    }
+                }
             }
+            __syncthreads();
         }
+    }
+}
+
+// Keeps the low words of a block's sorted keys (Gaussian index << 4 | nibble)
+// in place of the keys, as narrow_keys below; returns them.
+__device__ __forceinline__ uint32_t* block_narrow(unsigned long long* sk, int len) {
+    uint32_t* const idx = reinterpret_cast<uint32_t*>(sk);
+    for (int base = 0; base < len; base += blockDim.x) {
+        const int i = base + int(threadIdx.x);
+        const uint32_t lo = i < len ? uint32_t(sk[i]) : 0u;
+        __syncthreads();
+        if (i < len) idx[i] = lo;
         __syncthreads();
     }
+    return idx;
 }
 
 // Streams the sorted list's records through two shared-memory batches of
@@ -579,7 +610,7 @@ __device__ __forceinline__ void stream_list(const CompositeParams& p, const unsi
     }
 }
 
-// Shared memory of a binned block: keys (cap), bucket counters (cap + 2),
+// Shared memory of a binned block: keys (cap), bucket counters (cap / 2),
 // a record batch (3 x nthr float4), compaction buffers (64 ints per warp).
 struct BinnedSmem {
     unsigned long long* sk;
@@ -588,23 +619,20 @@ struct BinnedSmem {
     int* wbuf;
 };
 
-// Bytes of the key array (cap keys) and the bucket counters (cap + 2) of
-// block_sort, rounded up to 16.
-__host__ __device__ __forceinline__ size_t block_sort_bytes(int cap) {
-    return (8 * size_t(cap) + 4 * size_t(cap + 2) + 15) & ~size_t(15);
-}
+// Bytes of the key array (cap keys) and the bucket counters (cap / 2) of
+// block_sort; a multiple of 16.
+__host__ __device__ __forceinline__ size_t block_sort_bytes(int cap) { return 10 * size_t(cap); }
 
 __device__ __forceinline__ BinnedSmem carve_binned(unsigned char* base, int cap, int nthr) {
     BinnedSmem m;
     m.sk = reinterpret_cast<unsigned long long*>(base);
     m.cnt = reinterpret_cast<uint32_t*>(base + 8 * size_t(cap));
-    const size_t off = (8 * size_t(cap) + 4 * size_t(cap + 2) + 15) & ~size_t(15);
-    m.buf = reinterpret_cast<float4*>(base + off);
+    m.buf = reinterpret_cast<float4*>(base + block_sort_bytes(cap));
     m.wbuf = reinterpret_cast<int*>(m.buf + 3 * nthr) + 64 * (threadIdx.x >> 5);
     return m;
 }
 
-template <bool TRANSPOSED, int KPT>
+template <bool TRANSPOSED>
 __global__ void __launch_bounds__(kBinnedThreads)
 composite_rays_binned_kernel(CompositeParams p, const int4* __restrict__ gwork,
                              const int32_t* __restrict__ list, int cap,
@@ -619,7 +647,7 @@ composite_rays_binned_kernel(CompositeParams p, const int4* __restrict__ gwork,
     const int v = wi.x / p.ntiles;
     const uint32_t start = gstart[wi.x];
     const int len = int(gstart[wi.x + 1] - start);
-    block_sort<KPT>(keys, start, len, cap, S.sk, S.cnt);
+    block_sort(keys, start, len, cap, S.sk, S.cnt);
     const int64_t vbase = int64_t(v) * p.n;
     uint32_t evals = 0, blended = 0;
     for (int r0 = wi.y; r0 < wi.z; r0 += nthr) {
@@ -645,11 +673,9 @@ composite_rays_binned_kernel(CompositeParams p, const int4* __restrict__ gwork,
     if (pairs) count_pairs(pairs, evals, blended);
 }
 
-// Direct evaluation at 32 registers a thread: the standard paradigm's blocks
-// (a thread per pixel, 256 for its 16 x 16 tiles) then run eight to an SM,
-// which its latency-bound per-pixel blend loop needs
-template <bool TRANSPOSED, int KPT>
-__global__ void __launch_bounds__(1024, TRANSPOSED ? 1 : 2)
+// The standard paradigm under DL_EVAL_TRANSPOSED: a block per (view, tile), a
+// thread per pixel.  (Direct evaluation, the default: composite_views_*.)
+__global__ void __launch_bounds__(1024, 1)
 composite_full_binned_kernel(CompositeParams p, const int32_t* __restrict__ list, int cap,
                              const uint32_t* __restrict__ gstart,
                              const unsigned long long* __restrict__ keys,
@@ -668,14 +694,14 @@ composite_full_binned_kernel(CompositeParams p, const int32_t* __restrict__ list
     const float px = float(col) - p.half_w, py = float(row) - p.half_h;
     const uint32_t start = gstart[group];
     const int len = int(gstart[group + 1] - start);
-    block_sort<KPT>(keys, start, len, cap, S.sk, S.cnt);
+    block_sort(keys, start, len, cap, S.sk, S.cnt);
     int bx0, bx1, by0, by1;
     warp_box(inside, col, row, bx0, bx1, by0, by1);
     const int64_t vbase = int64_t(v) * p.n;
     Acc a{1.f, 0.f, 0.f, 0.f, 0u};
     uint32_t evals = 0;
     bool done = !inside;
-    stream_list<TRANSPOSED>(p, S.sk, len, vbase, rec, S.buf, S.wbuf, a, done, evals, px, py, bx0,
+    stream_list<true>(p, S.sk, len, vbase, rec, S.buf, S.wbuf, a, done, evals, px, py, bx0,
                             bx1, by0, by1);
     if (pairs) count_pairs(pairs, evals, a.blended);
     if (inside) {
@@ -1099,7 +1125,7 @@ struct QuadPipe {
 // selected positions are compacted 32 at a time and their records fetched
 // with cp.async one batch ahead of the batch being evaluated (as in
 // warp_stream).
-__device__ void quadrant_stream(const unsigned long long* sk, int len, int q, int64_t vbase,
+__device__ void quadrant_stream(const uint32_t* idx, int len, int q, int64_t vbase,
                                 const float4* __restrict__ rec, QuadPipe& Q, Acc& a, bool& done,
                                 uint32_t& evals, float px, float py, int bx0, int bx1, int by0,
                                 int by1, float ox, float oy) {
@@ -1111,7 +1137,7 @@ __device__ void quadrant_stream(const unsigned long long* sk, int len, int q, in
     auto produce = [&](int slot) -> int {
         while (cnt < 32 && pos < len) {
             const int i = pos + lane;
-            const bool sel = i < len && ((uint32_t(sk[i]) >> q) & 1u);
+            const bool sel = i < len && ((idx[i] >> q) & 1u);
             const unsigned m = __ballot_sync(0xffffffffu, sel);
             if (sel) Q.stage[cnt + __popc(m & lt)] = i;
             cnt += __popc(m);
@@ -1126,7 +1152,7 @@ __device__ void quadrant_stream(const unsigned long long* sk, int len, int q, in
         Q.idx[slot][lane] = mine;
         cnt -= n;
         if (lane < n) {
-            const int64_t e = vbase + (uint32_t(sk[mine]) >> 4);
+            const int64_t e = vbase + (idx[mine] >> 4);
             cp_async16(&Q.buf[slot][0][lane], rec + kRecordFloat4 * e);
             cp_async16(&Q.buf[slot][1][lane], rec + kRecordFloat4 * e + 1);
         }
@@ -1259,7 +1285,7 @@ composite_rays_block_kernel(const FrameDesc* __restrict__ F, const int64_t* __re
     __shared__ int64_t s_item;
     unsigned long long* sk = reinterpret_cast<unsigned long long*>(smb);
     uint32_t* cnt = reinterpret_cast<uint32_t*>(smb + 8 * size_t(cap));
-    QuadPipe* pipes = reinterpret_cast<QuadPipe*>(smb + block_sort_bytes(cap));
+    QuadPipe* pipes = reinterpret_cast<QuadPipe*>(smb + 4 * size_t(cap));  // after the sort
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t n_items = __ldg(prefix + n_frames);
     uint32_t evals = 0, blended = 0;
@@ -1281,8 +1307,8 @@ composite_rays_block_kernel(const FrameDesc* __restrict__ F, const int64_t* __re
             const int qx = warp & 1, qy = warp >> 1;
             // the keys carry the quadrant bits (bit q: the record's pixel
             // box overlaps quadrant q, x half + 2 * y half, of the tile)
-            block_sort<0>(d.keys, start, len, cap, sk, cnt);
-            __syncthreads();
+            block_sort(d.keys, start, len, cap, sk, cnt);
+            const uint32_t* idx = block_narrow(sk, len);
             const int64_t vbase = int64_t(v) * d.cp.n;
             for (int r0 = wi.y; r0 < wi.z; r0 += 32) {
                 const int rid = r0 + lane;
@@ -1298,7 +1324,7 @@ composite_rays_block_kernel(const FrameDesc* __restrict__ F, const int64_t* __re
                           d.cp.half_h);
                 Acc a{1.f, 0.f, 0.f, 0.f, 0u};
                 bool done = !mine;
-                quadrant_stream(sk, len, warp, vbase, d.rec, pipes[warp], a, done, evals, px, py,
+                quadrant_stream(idx, len, warp, vbase, d.rec, pipes[warp], a, done, evals, px, py,
                                 bx0, bx1, by0, by1, ox, oy);
                 if (mine) {
                     float* o = d.raycol + 3 * int64_t(rid);  // grouped order
@@ -1315,6 +1341,359 @@ composite_rays_block_kernel(const FrameDesc* __restrict__ F, const int64_t* __re
         item = s_item;
     }
     if (pairs) count_pairs(pairs, evals, blended);
+}
+
+// ------------------------------------------------ standard paradigm ----
+// Every pixel of every view.  A warp owns one (view, tile) group, sorts its
+// keys in its own shared memory (warp_sort) and composites the tile one 8 x 8
+// patch after another, two horizontally adjacent pixels a lane.  The stage is
+// bound by issued instructions, so the work per (pixel, Gaussian) pair is
+// what counts:
+//  - a patch only walks the records whose alpha >= 1/255 ellipse reaches it:
+//    one pass over the list, a record a lane, makes the masks of four patches
+//    (a 16 x 16 quad) at once; a patch then gathers its records 32 at a time
+//    into a shared-memory batch that the loop reads by broadcast;
+//  - two pixels of a row share the row's terms of the quadratic (4 of its 7
+//    operations), the record's loads and the loop, and their transmittance
+//    and colour updates are packed FP32x2 operations (per component the
+//    rounding of the scalar ones);
+//  - a finished pixel is one whose alpha threshold is out of reach, so no
+//    select guards the blend; whether a pixel finishes is asked once every
+//    kBlendRun records, and the branch that finishes it is taken once.
+// A larger patch culls worse and a smaller one shares less.  A warp per tile
+// needs no block barrier for its sort.  Lists of more than 1024 keys:
+// composite_views_block_kernel.
+// Measured against a block per tile with one pixel a lane in 16 x 2 strips:
+// 1080p (200k Gaussians, 45 views) 11.25 -> 4.07 ms, 4K (1M) 47.3 -> 17.0 ms,
+// 4K panel with 800 x 450 views 9.17 -> 3.79 ms; of the 1080p stage the blend
+// loop is about 2.7 ms (35 instructions for 64 pairs, then 30 with the runs),
+// the sort 0.4 ms and the masks and batches the rest.
+constexpr int kPatch = 8;
+constexpr int kBlendRun = 4;  // records blended between two looks at the transmittance
+
+// A patch's records, as the blend loop reads them: (u, v, A, B), (-r, -r, -g,
+// -g), (-b, -b, C, L); the colours are negated and doubled for the packed
+// update below.  stage: list positions selected and not yet batched.
+struct PatchBatch {
+    float4 geo[32], rg[32], bcl[32];
+    uint32_t stage[64];
+};
+
+// Two pixels (x0, y), (x1, y) of a lane: transmittance and colour pairs, and
+// per pixel the negated alpha a record has to reach (-1/255; -inf once the
+// pixel is finished).
+struct Px2 {
+    float x0, x1, y, th0, th1;
+    float2 T, r, g, b;
+    uint32_t blended;
+};
+
+// Masks of the 32 records of a batch (lane i holds record i, `valid`) for the
+// four patches of the quad at (qx, qy): bit i of component k is set when the
+// record may reach alpha >= 1/255 at a pixel of patch k (x half + 2 * y
+// half).  That is the largest value of its quadratic over the patch (pixel
+// centres relative to the principal point) against the threshold: the
+// quadratic is concave, so with its centre outside the patch the maximum is
+// on one of the two edges that face the centre, at the best point of the
+// nearest vertical edge (dy = -B dx / 2C, clamped) or of the nearest
+// horizontal one.  The margin covers the rounding here and in log2_alpha:
+// every term is below q = |A| dx^2 + |C| dy^2 at the quad's far corner (so is
+// B dx dy, as B^2 <= 4 A C), and the two evaluations add less than 30
+// roundings of 2^-24 q each.  A record that is not a number is kept.
+__device__ __forceinline__ uint4 quad_masks(bool valid, float u, float v, float A, float B, float C,
+                                            float L, const float (&x0)[2], const float (&x1)[2],
+                                            const float (&y0)[2], const float (&y1)[2]) {
+    const float hb = -0.5f * B, rc = hb * rcp_approx(C), ra = hb * rcp_approx(A);
+    float lx[2], hx[2], ex[2], ly[2], hy[2], ey[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        lx[k] = x0[k] - u;
+        hx[k] = x1[k] - u;
+        ex[k] = fminf(fmaxf(0.f, lx[k]), hx[k]);
+        ly[k] = y0[k] - v;
+        hy[k] = y1[k] - v;
+        ey[k] = fminf(fmaxf(0.f, ly[k]), hy[k]);
+    }
+    const float fx = fmaxf(-lx[0], hx[1]), fy = fmaxf(-ly[0], hy[1]);
+    const float margin = fmaf(fmaf(-A * fx, fx, -C * fy * fy), 4e-6f, 0.01f);
+    const float need = kLog2MinAlpha - L - margin;
+    unsigned m[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int i = k & 1, j = k >> 1;
+        const float oy = fminf(fmaxf(ex[i] * rc, ly[j]), hy[j]);
+        const float ox = fminf(fmaxf(ey[j] * ra, lx[i]), hx[i]);
+        const float f1 = fmaf(ex[i], fmaf(A, ex[i], B * oy), C * oy * oy);
+        const float f2 = fmaf(ox, fmaf(A, ox, B * ey[j]), C * ey[j] * ey[j]);
+        m[k] = __ballot_sync(0xffffffffu, valid && !(fmaxf(f1, f2) < need));
+    }
+    return make_uint4(m[0], m[1], m[2], m[3]);
+}
+
+// blend() of kBlendRun records (from `k` of the batch) on a lane's two
+// pixels: the same operations in the same order per pixel (the signs of alpha
+// and of the colour are both flipped, which changes no rounding).  blend()'s
+// test of log2 alpha is implied by the one of alpha: one step below that
+// threshold 2^x is 2.9e-7 below FP32's 1/255, more than ex2's error of 2^-22.
+template <bool COUNT>
+__device__ __forceinline__ void blend_run(Px2& p, const PatchBatch& S, int k) {
+    float2 a[kBlendRun], w[kBlendRun];
+    float2 T = p.T;
+#pragma unroll
+    for (int j = 0; j < kBlendRun; ++j) {
+        const float4 geo = S.geo[k + j];
+        const float2 cl = reinterpret_cast<const float2*>(S.bcl + k + j)[1];
+        const float dy = p.y - geo.y, bdy = geo.w * dy, row = fmaf(cl.x * dy, dy, cl.y);
+        const float dx0 = p.x0 - geo.x, dx1 = p.x1 - geo.x;
+        const float l0 = fmaf(dx0, fmaf(geo.z, dx0, bdy), row);
+        const float l1 = fmaf(dx1, fmaf(geo.z, dx1, bdy), row);
+        const float a0 = fmaxf(-0.99f, -ex2_approx(l0)), a1 = fmaxf(-0.99f, -ex2_approx(l1));
+        a[j] = make_float2(a0 <= p.th0 ? a0 : 0.f, a1 <= p.th1 ? a1 : 0.f);
+        w[j] = __fmul2_rn(a[j], T);
+        T = __fadd2_rn(T, w[j]);
+    }
+    // the transmittance only falls, so the last one tells whether a pixel
+    // finishes inside the run; then the run is taken record by record
+    if (fminf(T.x, T.y) < 1e-4f) {
+        T = p.T;
+        bool d0 = false, d1 = false;
+#pragma unroll
+        for (int j = 0; j < kBlendRun; ++j) {
+            w[j] = __fmul2_rn(a[j], T);
+            const float2 Tn = __fadd2_rn(T, w[j]);
+            d0 = d0 || Tn.x < 1e-4f;
+            d1 = d1 || Tn.y < 1e-4f;
+            if (d0) { w[j].x = 0.f; a[j].x = 0.f; } else T.x = Tn.x;
+            if (d1) { w[j].y = 0.f; a[j].y = 0.f; } else T.y = Tn.y;
+        }
+        if (d0) p.th0 = -INFINITY;
+        if (d1) p.th1 = -INFINITY;
+    }
+    p.T = T;
+#pragma unroll
+    for (int j = 0; j < kBlendRun; ++j) {
+        const float4 rg = S.rg[k + j];
+        p.r = __ffma2_rn(w[j], make_float2(rg.x, rg.y), p.r);
+        p.g = __ffma2_rn(w[j], make_float2(rg.z, rg.w), p.g);
+        p.b = __ffma2_rn(w[j], reinterpret_cast<const float2*>(S.bcl + k + j)[0], p.b);
+        if (COUNT) p.blended += (a[j].x < 0.f) + (a[j].y < 0.f);
+    }
+}
+
+// Composites one patch for the warp (columns from col0, rows from row0 of
+// view v): the records index(0 .. len) that masks (component `comp` of a
+// batch's uint4) select, in list order, and writes its pixels.
+template <bool COUNT, class Index>
+__device__ __forceinline__ void composite_patch(const CompositeParams& p, int v, int col0, int row0,
+                                                const uint4* masks, int comp, Index index, int len,
+                                                const float4* __restrict__ base, PatchBatch& S,
+                                                float* __restrict__ Mm, uint32_t& evals,
+                                                uint32_t& blended) {
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    const int col = col0 + 2 * (lane & 3), row = row0 + (lane >> 2);
+    const bool in0 = col < p.width && row < p.height, in1 = col + 1 < p.width && row < p.height;
+    Px2 q;
+    q.x0 = float(col) - p.half_w;
+    q.x1 = float(col + 1) - p.half_w;
+    q.y = float(row) - p.half_h;
+    q.th0 = in0 ? -(1.0f / 255.0f) : -INFINITY;
+    q.th1 = in1 ? -(1.0f / 255.0f) : -INFINITY;
+    q.T = make_float2(1.f, 1.f);
+    q.r = q.g = q.b = make_float2(0.f, 0.f);
+    q.blended = 0u;
+    const int nbatch = (len + 31) >> 5;
+    int b = 0, cnt = 0;  // batches scanned, positions staged (uniform)
+    float4 n0, n1;
+    // the next up to 32 selected records, one a lane, requested; their number
+    auto produce = [&]() -> int {
+        for (; cnt < 32 && b < nbatch; ++b) {
+            const unsigned m = reinterpret_cast<const unsigned*>(masks + b)[comp];
+            if ((m >> lane) & 1u) S.stage[cnt + __popc(m & lt)] = index(32 * b + lane);
+            cnt += __popc(m);
+        }
+        __syncwarp();
+        const int n = cnt < 32 ? cnt : 32;
+        if (lane < n) {
+            const float4* r = base + kRecordFloat4 * int64_t(S.stage[lane]);
+            n0 = __ldg(r);
+            n1 = __ldg(r + 1);
+        }
+        const uint32_t rest = lane + 32 < cnt ? S.stage[lane + 32] : 0u;
+        __syncwarp();
+        if (lane + 32 < cnt) S.stage[lane] = rest;
+        cnt -= n;
+        return n;
+    };
+    int n = produce();
+    while (n > 0) {
+        if (lane < n) {
+            float r, g, bl;
+            unpack_rgb(n1.z, n1.w, r, g, bl);
+            S.geo[lane] = n0;
+            S.rg[lane] = make_float4(-r, -r, -g, -g);
+            S.bcl[lane] = make_float4(-bl, -bl, n1.x, n1.y);
+        } else {  // fills the last run: alpha 0
+            S.geo[lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+            S.rg[lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+            S.bcl[lane] = make_float4(0.f, 0.f, 0.f, -1e30f);
+        }
+        const int n_next = produce();
+        if (COUNT) evals += uint32_t(n) * ((q.th0 > -INFINITY) + (q.th1 > -INFINITY));
+        for (int k = 0; k < n; k += kBlendRun) blend_run<COUNT>(q, S, k);
+        if (__all_sync(0xffffffffu, q.th0 == -INFINITY && q.th1 == -INFINITY)) break;
+        __syncwarp();  // the batch is written again
+        n = n_next;
+    }
+    __syncwarp();
+    float* o = Mm + ((int64_t(v) * p.height + row) * p.width + col) * 3;
+    if (in0) {
+        o[0] = q.r.x;
+        o[1] = q.g.x;
+        o[2] = q.b.x;
+    }
+    if (in1) {
+        o[3] = q.r.y;
+        o[4] = q.g.y;
+        o[5] = q.b.y;
+    }
+    if (COUNT) blended += q.blended;
+}
+
+// A (view, tile) group's 16 x 16 quads, one after another: the masks of the
+// quad's batches first, then its patches (those inside the tile and the
+// view).  BLOCK: the warps of a block share the batches and then the patches
+// (barriers between); otherwise one warp does both.
+template <bool COUNT, bool BLOCK, class Index>
+__device__ __forceinline__ void composite_quads(const CompositeParams& p, int group, Index index,
+                                                int len, const float4* __restrict__ rec,
+                                                uint4* masks, PatchBatch& S,
+                                                float* __restrict__ Mm, uint32_t& evals,
+                                                uint32_t& blended) {
+    const int lane = threadIdx.x & 31, warp = BLOCK ? int(threadIdx.x >> 5) : 0;
+    const int nwarps = BLOCK ? int(blockDim.x >> 5) : 1;
+    const int v = group / p.ntiles;
+    const int tile = group - v * p.ntiles;
+    const int tx = (tile % p.ntx) * p.tile_w, ty = (tile / p.ntx) * p.tile_h;
+    const int xe = min(tx + p.tile_w, p.width), ye = min(ty + p.tile_h, p.height);
+    const float4* __restrict__ base = rec + kRecordFloat4 * (int64_t(v) * p.n);
+    for (int qy = ty; qy < ye; qy += 2 * kPatch) {
+        for (int qx = tx; qx < xe; qx += 2 * kPatch) {
+            float x0[2], x1[2], y0[2], y1[2];
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                x0[k] = float(qx + k * kPatch) - p.half_w;
+                x1[k] = fmaxf(x0[k], float(min(qx + k * kPatch + kPatch, xe) - 1) - p.half_w);
+                y0[k] = float(qy + k * kPatch) - p.half_h;
+                y1[k] = fmaxf(y0[k], float(min(qy + k * kPatch + kPatch, ye) - 1) - p.half_h);
+            }
+            float4 n0 = make_float4(0.f, 0.f, 0.f, 0.f);
+            float2 n1 = make_float2(0.f, 0.f);
+            auto fetch = [&](int i) {  // a batch ahead
+                if (i < len) {
+                    const float4* r = base + kRecordFloat4 * int64_t(index(i));
+                    n0 = __ldg(r);
+                    n1 = __ldg(reinterpret_cast<const float2*>(r + 1));
+                }
+            };
+            fetch(32 * warp + lane);
+            for (int b = 32 * warp; b < len; b += 32 * nwarps) {
+                const float4 c0 = n0;
+                const float2 c1 = n1;
+                fetch(b + 32 * nwarps + lane);
+                const uint4 m = quad_masks(b + lane < len, c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, x0, x1,
+                                           y0, y1);
+                if (lane == 0) masks[b >> 5] = m;
+            }
+            if (BLOCK) __syncthreads();
+            else __syncwarp();
+            for (int k = warp; k < 4; k += nwarps) {
+                const int col0 = qx + (k & 1) * kPatch, row0 = qy + (k >> 1) * kPatch;
+                if (col0 >= xe || row0 >= ye) continue;
+                composite_patch<COUNT>(p, v, col0, row0, masks, k, index, len, base, S, Mm, evals,
+                                       blended);
+            }
+            if (BLOCK) __syncthreads();  // the masks are written again
+        }
+    }
+}
+
+// The keys are sorted in the space that holds their indices, the masks and
+// the batch afterwards.
+template <int CAP>
+union ViewSmem {
+    WarpSort<CAP> s;
+    struct {
+        uint32_t idx[CAP];
+        uint4 masks[CAP / 32];
+        PatchBatch batch;
+    } c;
+};
+template <int CAP>
+constexpr int view_class_blocks() { return CAP <= 512 ? 8 : 5; }
+static_assert(view_class_blocks<512>() * (kWarpsPerBlock * sizeof(ViewSmem<512>) + 1024) <=
+                  228 * 1024, "512-key class: 8 blocks");
+static_assert(view_class_blocks<1024>() * (kWarpsPerBlock * sizeof(ViewSmem<1024>) + 1024) <=
+                  228 * 1024, "1024-key class: 5 blocks");
+
+// Persistent, a warp per (view, tile) list of up to CAP keys: item
+// {group, first key, -, keys} i of the class (BACK: from the end of `items`),
+// the first by warp id, the rest claimed from *cursor.
+template <int CAP, bool BACK, bool COUNT>
+__global__ void __launch_bounds__(kWarpsPerBlock * 32, view_class_blocks<CAP>())
+composite_views_warp_kernel(CompositeParams p, const int4* __restrict__ items, int64_t n_work,
+                            uint32_t n_items, uint32_t* __restrict__ cursor,
+                            const unsigned long long* __restrict__ keys,
+                            const float4* __restrict__ rec, float* __restrict__ Mm,
+                            unsigned long long* __restrict__ pairs) {
+    extern __shared__ __align__(16) unsigned char vsm_raw[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    ViewSmem<CAP>& W = reinterpret_cast<ViewSmem<CAP>*>(vsm_raw)[warp];
+    const uint32_t n_warps = gridDim.x * kWarpsPerBlock;
+    uint32_t item = blockIdx.x * kWarpsPerBlock + warp;
+    uint32_t evals = 0, blended = 0;
+    while (item < n_items) {
+        uint32_t c = 0;
+        if (lane == 0) c = atomicAdd(cursor, 1u);
+        const int4 it = __ldg(items + (BACK ? n_work - 1 - int64_t(item) : int64_t(item)));
+        const int len = it.w & 0xFFFF;
+        warp_sort<CAP>(keys, uint32_t(it.y), len, W.s);
+        for (int base = 0; base < len; base += 32) {  // as narrow_keys
+            const int i = base + lane;
+            const uint32_t lo = i < len ? uint32_t(W.s.sk[i]) >> 4 : 0u;
+            __syncwarp();
+            if (i < len) W.c.idx[i] = lo;
+            __syncwarp();
+        }
+        composite_quads<COUNT, false>(p, it.x, [&](int i) { return W.c.idx[i]; }, len, rec,
+                                      W.c.masks, W.c.batch, Mm, evals, blended);
+        item = n_warps + __shfl_sync(0xffffffffu, c, 0);
+    }
+    if (COUNT) count_pairs(pairs, evals, blended);
+}
+
+// Lists too long for a warp (up to `cap` keys): a block of
+// four warps sorts the list together, then its warps share the batches' tests
+// and the patches.
+template <bool COUNT>
+__global__ void __launch_bounds__(kBinnedThreads)
+composite_views_block_kernel(CompositeParams p, const int4* __restrict__ block_items, int cap,
+                             const unsigned long long* __restrict__ keys,
+                             const float4* __restrict__ rec, float* __restrict__ Mm,
+                             unsigned long long* __restrict__ pairs) {
+    extern __shared__ __align__(16) unsigned char smb[];
+    unsigned long long* sk = reinterpret_cast<unsigned long long*>(smb);
+    uint32_t* cnt = reinterpret_cast<uint32_t*>(smb + 8 * size_t(cap));
+    // after the sort: narrowed keys, batches, masks
+    PatchBatch* batches = reinterpret_cast<PatchBatch*>(smb + 4 * size_t(cap));
+    uint4* masks = reinterpret_cast<uint4*>(batches + kBinnedThreads / 32);
+    const int4 it = block_items[blockIdx.x];  // {group, first key, -, keys}
+    block_sort(keys, uint32_t(it.y), it.w, cap, sk, cnt);
+    const uint32_t* idx = block_narrow(sk, it.w);
+    uint32_t evals = 0, blended = 0;
+    composite_quads<COUNT, true>(p, it.x, [&](int i) { return idx[i] >> 4; }, it.w, rec, masks,
+                                 batches[threadIdx.x >> 5], Mm, evals, blended);
+    if (COUNT) count_pairs(pairs, evals, blended);
 }
 
 __global__ void batch_prefix_kernel(const FrameDesc* __restrict__ F, int n_frames,
@@ -1370,7 +1749,7 @@ __global__ void partition_warp_kernel(const int4* __restrict__ gwork, int64_t n_
     for (int64_t w = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; w < n_work;
          w += int64_t(gridDim.x) * blockDim.x) {
         const unsigned am = __activemask();
-        const int4 wi = gwork[w];
+        const int4 wi = gwork ? gwork[w] : make_int4(int(w), 0, 0, 0);
         const uint32_t st = first[wi.x];
         const uint32_t len = (S.cursor ? S.cursor[wi.x] : S.start[wi.x + 1]) - st;
         const uint32_t nr = uint32_t(wi.z - wi.y);
@@ -1519,12 +1898,12 @@ cudaError_t launch_composite_full(const CompositeParams& p, int32_t nv, const ui
 }
 
 size_t block_smem_bytes(int cap) {
-    return block_sort_bytes(cap) + (kBinnedThreads / 32) * sizeof(QuadPipe);
+    // the sort's keys and counters, then the narrowed keys and the pipes
+    return std::max(block_sort_bytes(cap), 4 * size_t(cap) + (kBinnedThreads / 32) * sizeof(QuadPipe));
 }
 
 size_t binned_smem_bytes(int cap, int nthr) {
-    const size_t off = (8 * size_t(cap) + 4 * size_t(cap + 2) + 15) & ~size_t(15);
-    return off + size_t(nthr) * 3 * sizeof(float4) + size_t(nthr / 32) * 64 * sizeof(int);
+    return block_sort_bytes(cap) + size_t(nthr) * 3 * sizeof(float4) + size_t(nthr / 32) * 64 * sizeof(int);
 }
 
 cudaError_t launch_composite_rays_binned(const CompositeParams& p, const int4* gwork,
@@ -1536,7 +1915,6 @@ cudaError_t launch_composite_rays_binned(const CompositeParams& p, const int4* g
     if (n_list <= 0) return cudaSuccess;
     const int nthr = kBinnedThreads;
     const size_t smem = binned_smem_bytes(cap, nthr);
-    const bool regs = false;
     auto go = [&](auto kernel) -> cudaError_t {
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              int(smem));
@@ -1545,30 +1923,83 @@ cudaError_t launch_composite_rays_binned(const CompositeParams& p, const int4* g
                                                     raycol, pairs);
         return cudaGetLastError();
     };
-    if (transposed) return regs ? go(composite_rays_binned_kernel<true, 8>)
-                                : go(composite_rays_binned_kernel<true, 0>);
-    return regs ? go(composite_rays_binned_kernel<false, 8>) : go(composite_rays_binned_kernel<false, 0>);
+    return transposed ? go(composite_rays_binned_kernel<true>) : go(composite_rays_binned_kernel<false>);
 }
 
 cudaError_t launch_composite_full_binned(const CompositeParams& p, const int32_t* list,
                                          int64_t n_list, int cap, const uint32_t* gstart,
                                          const unsigned long long* keys, const float4* rec,
-                                         float* Mm, unsigned long long* pairs, int transposed,
-                                         cudaStream_t s) {
+                                         float* Mm, unsigned long long* pairs, cudaStream_t s) {
     if (n_list <= 0) return cudaSuccess;
     const int nthr = p.tile_w * p.tile_h;
     const size_t smem = binned_smem_bytes(cap, nthr);
-    const bool regs = false;
-    auto go = [&](auto kernel) -> cudaError_t {
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             int(smem));
+    cudaError_t e = cudaFuncSetAttribute(composite_full_binned_kernel,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    if (e != cudaSuccess) return e;
+    composite_full_binned_kernel<<<unsigned(n_list), nthr, smem, s>>>(p, list, cap, gstart, keys, rec,
+                                                                      Mm, pairs);
+    return cudaGetLastError();
+}
+
+size_t views_block_smem_bytes(int cap) {
+    return std::max(block_sort_bytes(cap), 4 * size_t(cap) +
+                                               (kBinnedThreads / 32) * sizeof(PatchBatch) +
+                                               size_t(cap / 32) * sizeof(uint4));
+}
+
+namespace {
+template <int CAP, bool BACK, bool COUNT>
+cudaError_t launch_views_warp(const CompositeParams& p, const int4* items, int64_t n_work, int64_t n,
+                              uint32_t* cursor, const unsigned long long* keys, const float4* rec,
+                              float* Mm, unsigned long long* pairs, cudaStream_t s) {
+    if (n <= 0) return cudaSuccess;
+    const auto kernel = composite_views_warp_kernel<CAP, BACK, COUNT>;
+    const size_t smem = kWarpsPerBlock * sizeof(ViewSmem<CAP>);
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    if (e != cudaSuccess) return e;
+    int per_sm = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kWarpsPerBlock * 32, smem);
+    if (e != cudaSuccess) return e;
+    const int64_t need = (n + kWarpsPerBlock - 1) / kWarpsPerBlock;
+    const int64_t fit = int64_t(num_sms()) * (per_sm > 0 ? per_sm : 1);
+    kernel<<<unsigned(need < fit ? need : fit), kWarpsPerBlock * 32, smem, s>>>(
+        p, items, n_work, uint32_t(n), cursor, keys, rec, Mm, pairs);
+    return cudaGetLastError();
+}
+
+template <bool COUNT>
+cudaError_t launch_views(const CompositeParams& p, const int4* items, const int4* block_items,
+                         int64_t n_work, const int64_t n[3], int block_cap, uint32_t* const cursor[2],
+                         const unsigned long long* keys, const float4* rec, float* Mm,
+                         unsigned long long* pairs, cudaStream_t s) {
+    // the longest lists first: the short ones fill the tail
+    if (n[2] > 0) {
+        const size_t smem = views_block_smem_bytes(block_cap);
+        cudaError_t e = cudaFuncSetAttribute(composite_views_block_kernel<COUNT>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
         if (e != cudaSuccess) return e;
-        kernel<<<unsigned(n_list), nthr, smem, s>>>(p, list, cap, gstart, keys, rec, Mm, pairs);
-        return cudaGetLastError();
-    };
-    if (transposed) return regs ? go(composite_full_binned_kernel<true, 4>)
-                                : go(composite_full_binned_kernel<true, 0>);
-    return regs ? go(composite_full_binned_kernel<false, 4>) : go(composite_full_binned_kernel<false, 0>);
+        composite_views_block_kernel<COUNT><<<unsigned(n[2]), kBinnedThreads, smem, s>>>(
+            p, block_items, block_cap, keys, rec, Mm, pairs);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    const cudaError_t e = launch_views_warp<1024, true, COUNT>(p, items, n_work, n[1], cursor[1], keys,
+                                                               rec, Mm, pairs, s);
+    if (e != cudaSuccess) return e;
+    return launch_views_warp<512, false, COUNT>(p, items, n_work, n[0], cursor[0], keys, rec, Mm,
+                                                pairs, s);
+}
+}  // namespace
+
+cudaError_t launch_composite_views(const CompositeParams& p, const int4* items,
+                                   const int4* block_items, int64_t n_work, const int64_t n[3],
+                                   int block_cap, uint32_t* const cursor[2],
+                                   const unsigned long long* keys, const float4* rec, float* Mm,
+                                   unsigned long long* pairs, cudaStream_t s) {
+    return pairs ? launch_views<true>(p, items, block_items, n_work, n, block_cap, cursor, keys, rec,
+                                      Mm, pairs, s)
+                 : launch_views<false>(p, items, block_items, n_work, n, block_cap, cursor, keys, rec,
+                                       Mm, pairs, s);
 }
 
 namespace {

@@ -288,7 +288,7 @@ cudaError_t launch_composite_full(const CompositeParams& p, int32_t nv, const ui
                                   const uint32_t* vals, const float4* rec, float* Mm,
                                   unsigned long long* pairs, cudaStream_t s);
 // Binned paths: each block sorts its group's keys in shared memory (bucket
-// counting sort, up to `cap` keys, a power of two) and then composites in that
+// counting sort, up to `cap` keys, a multiple of 512) and then composites in that
 // order; `transposed` selects the evaluation strategy.
 // `list` selects the blocks' work entries (size class), gwork holds
 // {group, ray begin, ray end, -} per DirectL group with rays.
@@ -305,8 +305,18 @@ cudaError_t launch_composite_rays_binned(const CompositeParams& p, const int4* g
 cudaError_t launch_composite_full_binned(const CompositeParams& p, const int32_t* list,
                                          int64_t n_list, int cap_p, const uint32_t* gstart,
                                          const unsigned long long* keys, const float4* rec,
-                                         float* Mm, unsigned long long* pairs, int transposed,
-                                         cudaStream_t s);
+                                         float* Mm, unsigned long long* pairs, cudaStream_t s);
+// Standard paradigm with direct evaluation: n[0] lists of at most 512 keys
+// (items[0..]) and n[1] of at most 1024 (from items[n_work - 1] down), a warp
+// each, persistent, claimed from *cursor[0] and *cursor[1] (0 at launch); n[2]
+// longer ones (block_items, up to block_cap keys, a multiple of 512), a block
+// each.  The lists are launch_partition_warp's without gwork.
+size_t views_block_smem_bytes(int cap);
+cudaError_t launch_composite_views(const CompositeParams& p, const int4* items,
+                                   const int4* block_items, int64_t n_work, const int64_t n[3],
+                                   int block_cap, uint32_t* const cursor[2],
+                                   const unsigned long long* keys, const float4* rec, float* Mm,
+                                   unsigned long long* pairs, cudaStream_t s);
 // DirectL groups whose lists hold at most 512 or 1024 keys: one warp per
 // group (warp-level sort, cp.async batches of 32, transposed evaluation),
 // persistent over self-contained items {group, first key, first ray,
@@ -316,7 +326,8 @@ cudaError_t launch_composite_full_binned(const CompositeParams& p, const int32_t
 // key, gwork index, keys}; meta = {n_items1, n_block, max keys, -,
 // n_items2}.  When *total_keys (optional: the slices' end) exceeds key_cap
 // nothing is written and status |= 1; nothing is written either when status
-// bit 0 is already set (keys were dropped).
+// bit 0 is already set (keys were dropped).  gwork NULL: the entries are the
+// groups 0..n_work-1 themselves (standard paradigm).
 // Where each group's keys are: [start[g], start[g + 1]) when cursor is
 // null; else [s[g], cursor[g]) with s = start_alt when *use_alt != 0, else
 // start (the slices of a frame whose keys the projection emitted).
@@ -358,7 +369,7 @@ cudaError_t launch_composite_rays_warp(int cap, int cls, const FrameDesc* frames
                                        const int64_t* prefix, int32_t n_frames, int64_t max_items,
                                        uint32_t* cursor, unsigned long long* pairs, cudaStream_t s);
 // Block class (the block lists: lists too long for the warp classes, up to
-// block_cap keys, a power of two <= 16384; longer lists set status bit 1 and
+// block_cap keys, a multiple of 512 <= 16384; longer lists set status bit 1 and
 // are skipped), persistent: four warps sort a list together, then warp q
 // composites the rays in quadrant q of the tile over the records whose key
 // marks quadrant q.
