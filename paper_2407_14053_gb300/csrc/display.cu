@@ -16,10 +16,6 @@ __device__ __forceinline__ int64_t floor_div(int64_t a, int64_t b) {
     int64_t q = a / b;
     return (a % b != 0 && ((a < 0) != (b < 0))) ? q - 1 : q;
 }
-__device__ __forceinline__ int64_t ceil_div_pos(int64_t a, int64_t b) {  // b > 0
-    return -floor_div(-a, b);
-}
-
 // d_offset (Eq. (1)) of subpixel column s in row x, Q32.
 __device__ __forceinline__ int64_t d_offset(const DisplayQ& q, int64_t x, int64_t s) {
     return s * kQ32 + x * q.t3q - q.kq;
@@ -69,112 +65,160 @@ __global__ void view_map_kernel(DisplayQ q, uint16_t* __restrict__ V) {
 }
 
 // ------------------------------------------------------------------ a2 ---
-__device__ __forceinline__ int64_t area_of(const DisplayQ& q, int64_t x, int64_t s) {
-    return floor_div(floor_div(d_offset(q, x, s), q.lq), q.pw);
-}
-
 __device__ __forceinline__ uint32_t pack_px(int64_t x, int64_t y) {
     return (uint32_t(x) << 16) | uint32_t(y);
 }
 
-// Alg. 2, one warp per area (areas are independent, Sec. 5).  Inside an area
-// the subpixels are visited in row-major order; each chain samples a pixel
-// (Eq. (11)), parks its two other channels in B_rgb (Eq. (12)) and hands
-// them to the next subpixels of the same view found by the search
-// (Eqs. (13)-(14)).  The search is the first subpixel, in scan order (rows
-// ascending, columns from y outward, channels 0..2), that shows the chain's
-// view and whose channel has an idle subpixel parked; the chain ends when
-// that subpixel is outside the area or already filled.  Lane 0 owns all
-// reads and writes of M_i (src); the warp scans the search window in
-// parallel, 32 candidates per step, taking the first hit by ballot.
-__global__ void repurpose_kernel(DisplayQ q, const uint16_t* __restrict__ V,
-                                 uint32_t* __restrict__ src) {
-    const int lane = threadIdx.x & 31;
-    const int64_t warp = (blockIdx.x * int64_t(blockDim.x) + threadIdx.x) >> 5;
-    if (warp >= q.n_areas) return;
-    const int64_t a = q.area_min + warp;
-    const int64_t S = 3 * int64_t(q.w);
-    const int64_t lo_d = a * q.pw * q.lq;       // area covers d in [lo_d, hi_d)
-    const int64_t hi_d = (a + 1) * q.pw * q.lq;
-    for (int64_t x = 0; x < q.h; ++x) {
-        const int64_t base = x * q.t3q - q.kq;
-        int64_t s_lo = ceil_div_pos(lo_d - base, kQ32);
-        int64_t s_hi = ceil_div_pos(hi_d - base, kQ32) - 1;
-        if (s_lo < 0) s_lo = 0;
-        if (s_hi > S - 1) s_hi = S - 1;
-        for (int64_t s = s_lo; s <= s_hi; ++s) {
-            int64_t ci = x * S + s;
-            uint32_t cur = 0;
-            if (lane == 0) cur = src[ci];
-            cur = __shfl_sync(0xffffffffu, cur, 0);
-            if (cur != kEmpty) continue;
-            const uint16_t vi = V[ci];
-            uint32_t B0 = kEmpty, B1 = kEmpty, B2 = kEmpty;  // B_rgb(v_i, .)
-            int64_t cx = x, cy = s / 3;
-            int ck = int(s % 3);
-            while (true) {
-                const uint32_t Bk = ck == 0 ? B0 : (ck == 1 ? B1 : B2);
-                if (Bk != kEmpty) {  // Eq. (13)
-                    if (lane == 0) src[ci] = Bk;
-                    if (ck == 0) B0 = kEmpty;
-                    else if (ck == 1) B1 = kEmpty;
-                    else B2 = kEmpty;
-                } else {  // Eqs. (11), (12)
-                    const uint32_t p = pack_px(cx, cy);
-                    if (lane == 0) src[ci] = p;
-                    if (ck == 0) { B1 = p; B2 = p; }
-                    else if (ck == 1) { B0 = p; B2 = p; }
-                    else { B0 = p; B1 = p; }
+// ceil(x / 2^32)
+__device__ __forceinline__ int64_t ceil_q32(int64_t x) { return (x + (kQ32 - 1)) >> 32; }
+
+// Alg. 2, four lanes per (area, view).  Areas are independent (Sec. 5), and
+// inside an area so are the views: a chain (Eqs. (11)-(14)) starts at an
+// empty subpixel of view v_i, parks and looks up idle channels in
+// B_rgb(v_i, .) only, which is cleared when it ends, and fills only subpixels
+// that show v_i.  So each view's chains run alone, in row-major order of
+// their starts, and nothing they read is written by another group of lanes.
+//
+// Which subpixels of a row show view v follows from the map itself: those of
+// grating unit u lie at d in [u L_x + vlo, u L_x + vhi) with vlo = ceil(v L_x
+// / N_v), vhi = ceil((v + 1) L_x / N_v) in Q32 (v = floor(N_v x_offset / L_x)
+// exactly then), i.e. at s from ceil((u L_x + vlo - base) / 2^32) on, base =
+// x 3 tan - K.  Neither the walk nor the search reads V.
+//
+// A chain ends when the subpixel that the search finds (the first one in scan
+// order: rows ascending, columns from y outward, channels 0..2, that shows v
+// and whose channel has an idle subpixel parked) is outside the area or
+// already filled.
+//
+// Bound by the latency of a chain's dependent steps, so the groups are many
+// (35 thousand at 4K: 783 areas x 45 views, about 780 subpixels each) and take
+// four rows at a time, of the walk as of the search.  The warp's eight groups
+// advance together, one such look each an iteration, whatever the others do:
+// as nested loops a thread per (area, view) took 30.8 ms at 4K, every lane
+// waiting for each lane's chains, and a warp per area that took the views'
+// chains in turn and searched V 32 candidates at a time 48.6 ms.
+constexpr int kChainLanes = 4;
+
+__global__ void __launch_bounds__(32)
+repurpose_kernel(DisplayQ q, uint32_t* src) {
+    const int64_t lq = q.lq;
+    // moves the unit bound to the unit that holds d
+    auto follow = [lq](int64_t& unit, int64_t d) {
+        const int64_t t = d - unit;
+        if (t < -8 * lq || t >= 8 * lq) unit += floor_div(t, lq) * lq;
+        while (unit > d) unit -= lq;
+        while (unit + lq <= d) unit += lq;
+    };
+    const int lane = threadIdx.x, sub = lane % kChainLanes;
+    const unsigned group = ((1u << kChainLanes) - 1u) << (lane - sub);
+    const int32_t S = 3 * q.w, h = q.h;
+    const int64_t last_d = int64_t(S - 1) * kQ32;
+    const int64_t most_u = (int64_t(1) << 53) / lq + 2;  // past every panel's units
+    const int64_t total = int64_t(q.n_areas) * q.nv;
+    constexpr int kGroups = 32 / kChainLanes;
+    for (int64_t id0 = int64_t(blockIdx.x) * kGroups; id0 < total; id0 += int64_t(gridDim.x) * kGroups) {
+        const int64_t id = id0 + lane / kChainLanes;
+        bool done = id >= total;
+        const int64_t a = q.area_min + (done ? 0 : id / q.nv), v = done ? 0 : id % q.nv;
+        const int64_t vlo = (v * lq + q.nv - 1) / q.nv, vhi = ((v + 1) * lq + q.nv - 1) / q.nv;
+        // the area's d range
+        const int64_t u_lo = max(a * q.pw, -most_u) * lq, u_hi = min((a + 1) * q.pw, most_u) * lq;
+        int64_t ru = u_lo;            // unit of the lane's row of the walk, at s = 0
+        int64_t wu = u_lo;            // unit of the lane's row of the search, at its first column
+        int32_t x = 0;                // the walk's first row
+        bool chain = false, fresh = false;  // a chain is running; it stands at a new subpixel
+        int32_t cx = 0, cs = 0;       // the chain's subpixel
+        uint32_t B0 = kEmpty, B1 = kEmpty, B2 = kEmpty;  // B_rgb(v_i, .)
+        int32_t r_cur = 0, r_hi = 0, w0 = 0, w1 = 0;     // rows and subpixel columns left to search
+        while (!__all_sync(0xffffffffu, done)) {
+            // the walk: the first empty subpixel of view v of each lane's row
+            int32_t at = -1;
+            if (!done && !chain && x + sub < h) {
+                const int64_t base = int64_t(x + sub) * q.t3q - q.kq;
+                follow(ru, base);
+                const int64_t u_end = min(u_hi, base + last_d + 1);
+                for (int64_t u = max(ru, u_lo); u < u_end && at < 0; u += lq) {
+                    const int64_t s0 = max(ceil_q32(u + vlo - base), int64_t(0));
+                    const int64_t s1 = min(ceil_q32(u + vhi - base), int64_t(S));
+                    for (int64_t s = s0; s < s1; ++s)
+                        if (src[int64_t(x + sub) * S + s] == kEmpty) {
+                            at = int32_t(s);
+                            break;
+                        }
                 }
-                // Eq. (14)
-                const int64_t x_low = cx + 2 < q.h - 1 ? cx + 2 : q.h - 1;
-                const int64_t x_high = cx + q.win_dx < q.h - 1 ? cx + q.win_dx : q.h - 1;
-                int64_t y_last, step;
-                if (!q.slant_neg) {
-                    y_last = cy - q.win_dy > 0 ? cy - q.win_dy : 0;
-                    step = -1;
-                } else {
-                    y_last = cy + q.win_dy < q.w - 1 ? cy + q.win_dy : q.w - 1;
-                    step = 1;
-                }
-                const int64_t ncols = (y_last - cy) * step + 1;
-                const int64_t nrows = x_high - x_low + 1;
-                const int64_t ncand = nrows > 0 ? nrows * ncols * 3 : 0;
-                int64_t found = -1;
-                for (int64_t b = 0; b < ncand; b += 32) {
-                    const int64_t j = b + lane;
-                    bool match = false;
-                    if (j < ncand) {
-                        const int64_t r = x_low + j / (ncols * 3);
-                        const int64_t rem = j % (ncols * 3);
-                        const int64_t c = cy + step * (rem / 3);
-                        const int ch = int(rem % 3);
-                        const uint32_t Bc = ch == 0 ? B0 : (ch == 1 ? B1 : B2);
-                        match = (Bc != kEmpty) && (V[r * S + 3 * c + ch] == vi);
-                    }
-                    const unsigned bal = __ballot_sync(0xffffffffu, match);
-                    if (bal) {
-                        found = b + (__ffs(bal) - 1);
-                        break;
-                    }
-                }
-                if (found < 0) break;  // no position left for view v_i
-                const int64_t r = x_low + found / (ncols * 3);
-                const int64_t rem = found % (ncols * 3);
-                const int64_t c = cy + step * (rem / 3);
-                const int ch = int(rem % 3);
-                // while condition of Alg. 2: inside the area and still empty
-                if (area_of(q, r, 3 * c + ch) != a) break;
-                const int64_t ni = r * S + 3 * c + ch;
-                uint32_t nsrc = 0;
-                if (lane == 0) nsrc = src[ni];
-                nsrc = __shfl_sync(0xffffffffu, nsrc, 0);
-                if (nsrc != kEmpty) break;
-                cx = r;
-                cy = c;
-                ck = ch;
-                ci = ni;
             }
+            const unsigned hit = __ballot_sync(0xffffffffu, at >= 0) & group;
+            const int32_t start = __shfl_sync(0xffffffffu, at, hit ? __ffs(hit) - 1 : lane);
+            if (!done && !chain) {
+                if (hit) {
+                    x += (__ffs(hit) - 1) % kChainLanes;
+                    cx = x;
+                    cs = start;
+                    B0 = B1 = B2 = kEmpty;
+                    chain = fresh = true;
+                } else {
+                    x += kChainLanes;
+                    done = x >= h;
+                }
+            }
+            if (fresh) {
+                fresh = false;
+                const int32_t cy = cs / 3, ck = cs - 3 * cy;
+                const uint32_t Bk = ck == 0 ? B0 : (ck == 1 ? B1 : B2);
+                const bool idle = Bk != kEmpty;
+                const uint32_t own = pack_px(cx, cy);
+                if (sub == 0) src[int64_t(cx) * S + cs] = idle ? Bk : own;  // Eq. (13) / (11)
+                // Eq. (12); used channels are cleared
+                B0 = ck == 0 ? kEmpty : (idle ? B0 : own);
+                B1 = ck == 1 ? kEmpty : (idle ? B1 : own);
+                B2 = ck == 2 ? kEmpty : (idle ? B2 : own);
+                // Eq. (14): rows [x + 2, x + win_dx], columns from y outward
+                r_cur = min(cx + 2, h - 1);
+                r_hi = min(cx + q.win_dx, h - 1);
+                w0 = 3 * (q.slant_neg ? cy : max(cy - q.win_dy, 0));
+                w1 = 3 * (q.slant_neg ? min(cy + q.win_dy, q.w - 1) : cy) + 2;
+            }
+            // the search: the first candidate of each lane's row
+            int32_t found = -1;
+            bool inside = false;  // in the chain's area
+            if (chain && r_cur + sub <= r_hi) {
+                const int64_t rb = int64_t(r_cur + sub) * q.t3q - q.kq;
+                const int64_t d0 = int64_t(w0) * kQ32 + rb, d1 = int64_t(w1) * kQ32 + rb;
+                follow(wu, d0);
+                int32_t fcol = -1;
+                for (int64_t t = wu; t + vlo <= d1; t += lq) {
+                    const int64_t a0 = max(ceil_q32(t + vlo - rb), int64_t(w0));
+                    const int64_t a1 = min(ceil_q32(t + vhi - rb) - 1, int64_t(w1));
+                    for (int32_t j = int32_t(a0); j <= a1; ++j) {
+                        const int32_t c = j / 3, ch = j - 3 * c;
+                        if ((ch == 0 ? B0 : (ch == 1 ? B1 : B2)) == kEmpty) continue;
+                        // the nearest column first, then the lowest channel
+                        if (found < 0 || (!q.slant_neg && c > fcol)) {
+                            found = j;
+                            fcol = c;
+                            inside = t >= u_lo && t < u_hi;
+                        }
+                    }
+                    if (q.slant_neg && found >= 0) break;
+                }
+            }
+            const unsigned fb = __ballot_sync(0xffffffffu, found >= 0) & group;
+            const unsigned ib = __ballot_sync(0xffffffffu, inside) & group;
+            const int32_t next = __shfl_sync(0xffffffffu, found, fb ? __ffs(fb) - 1 : lane);
+            if (chain) {
+                if (fb) {
+                    // while condition of Alg. 2: inside the area and still empty
+                    const int32_t fr = r_cur + (__ffs(fb) - 1) % kChainLanes;
+                    chain = ((ib >> (__ffs(fb) - 1)) & 1u) && src[int64_t(fr) * S + next] == kEmpty;
+                    fresh = chain;
+                    cx = fr;
+                    cs = next;
+                } else {
+                    r_cur += kChainLanes;
+                    chain = r_cur <= r_hi;  // no position left for view v_i
+                }
+            }
+            __syncwarp();  // the group's lanes read what its first lane wrote
         }
     }
 }
@@ -388,17 +432,16 @@ cudaError_t launch_view_map(const DisplayQ& q, uint16_t* V, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_repurpose(const DisplayQ& q, const uint16_t* V, uint32_t* src, int identity,
-                             cudaStream_t s) {
+cudaError_t launch_repurpose(const DisplayQ& q, uint32_t* src, int identity, cudaStream_t s) {
     if (identity) {
         identity_src_kernel<<<grid_for(3 * int64_t(q.w) * q.h, 256), 256, 0, s>>>(q.w, q.h, src);
         return cudaGetLastError();
     }
     cudaError_t e = cudaMemsetAsync(src, 0xFF, sizeof(uint32_t) * 3 * size_t(q.w) * q.h, s);
     if (e != cudaSuccess) return e;
-    const int warps_per_block = 4;
-    const int blocks = (q.n_areas + warps_per_block - 1) / warps_per_block;
-    repurpose_kernel<<<blocks, 32 * warps_per_block, 0, s>>>(q, V, src);
+    // a warp a block: the warps' lengths differ with the areas on the panel
+    const int64_t blocks = (int64_t(q.n_areas) * q.nv * kChainLanes + 31) / 32;
+    repurpose_kernel<<<unsigned(blocks < 0x7FFFFFFF ? blocks : 0x7FFFFFFF), 32, 0, s>>>(q, src);
     return cudaGetLastError();
 }
 
