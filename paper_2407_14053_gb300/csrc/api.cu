@@ -159,69 +159,62 @@ dl_status get_groups(dl_ctx* ctx, Display& D, RaySet& R, int32_t tw, int32_t th,
     G->ntiles = G->ntx * G->nty;
     const int64_t ngroups = int64_t(D.q.nv) * G->ntiles;
     const int64_t nr = R.n_rays;
-    DevBuf k0, k1, v0, v1, rtmp, ranges;
+    DevBuf k0, k1, v0, v1, rtmp, ranges, counts;
     DL_CK(k0.reserve(8 * size_t(nr)), "alloc");
     DL_CK(k1.reserve(8 * size_t(nr)), "alloc");
     DL_CK(v0.reserve(4 * size_t(nr)), "alloc");
     DL_CK(v1.reserve(4 * size_t(nr)), "alloc");
     DL_CK(rtmp.reserve(radix_tmp_bytes(nr)), "alloc");
     DL_CK(ranges.reserve(8 * size_t(ngroups)), "alloc");
+    const int shift = 2 * bits_for(std::max(tw, th));  // Morton bits (powers of two)
     DL_CK(launch_ray_group_keys(R.ray_view.as<uint32_t>(), R.ray_pix.as<uint32_t>(), nr, tw, th,
-                                G->ntx, D.q.nv, k0.as<unsigned long long>(), v0.as<uint32_t>(), s),
+                                G->ntx, D.q.nv, shift, k0.as<unsigned long long>(),
+                                v0.as<uint32_t>(), s),
           "group keys");
     int alt = 0;
     DL_CK(radix_sort_pairs(k0.as<unsigned long long>(), v0.as<uint32_t>(),
-                           k1.as<unsigned long long>(), v1.as<uint32_t>(), nr, bits_for(ngroups) + 16,
-                           rtmp.p, &alt, s),
+                           k1.as<unsigned long long>(), v1.as<uint32_t>(), nr,
+                           bits_for(ngroups) + shift, rtmp.p, &alt, s),
           "group sort");
     unsigned long long* ks = alt ? k1.as<unsigned long long>() : k0.as<unsigned long long>();
     uint32_t* vs = alt ? v1.as<uint32_t>() : v0.as<uint32_t>();
     DL_CK(cudaMemsetAsync(ranges.p, 0, 8 * size_t(ngroups), s), "memset");
-    DL_CK(launch_key_ranges(ks, nr, 16, ranges.as<uint2>(), ngroups, s), "group ranges");
+    DL_CK(launch_key_ranges(ks, nr, shift, ranges.as<uint2>(), ngroups, s), "group ranges");
     DL_CK(G->grouped.reserve(8 * size_t(nr)), "alloc");
     DL_CK(launch_ray_group_gather(vs, R.ray_pix.as<uint32_t>(), nr, G->grouped.as<int2>(), s),
           "group gather");
+    // the work lists, made on the device from the ranges: the compositing
+    // items in view-major order (consecutive items are neighbouring tiles of
+    // one view, which share records in L2; tile-major items measured 1.6 x
+    // the DRAM reads).  The loops over the groups took the host 3 ms at 4K.
+    const size_t ng1 = size_t(ngroups + 1);
+    const size_t scan_bytes = scan_tmp_bytes(ngroups + 1);
+    DL_CK(counts.reserve(16 * ng1 + scan_bytes + 512), "alloc");
+    uint32_t* chunks = counts.as<uint32_t>();
+    uint32_t *used = chunks + ng1, *chunk_at = used + ng1, *used_at = chunk_at + ng1;
+    uint32_t* totals = used_at + ng1;
+    void* scan_tmp = counts.as<char>() + (16 * ng1 + 8 + 255) / 256 * 256;
+    DL_CK(launch_list_counts(ranges.as<uint2>(), ngroups, G->ntiles, D.q.nv, kRaysPerBlock, chunks,
+                             used, s),
+          "list counts");
+    DL_CK(launch_exclusive_scan(chunks, chunk_at, ngroups + 1, totals, scan_tmp, s), "list scan");
+    DL_CK(launch_exclusive_scan(used, used_at, ngroups + 1, totals + 1, scan_tmp, s), "list scan");
+    uint32_t h_totals[2] = {0u, 0u};
+    DL_CK(cudaMemcpyAsync(h_totals, totals, 8, cudaMemcpyDeviceToHost, s), "copy");
     const int64_t nsub = 3 * int64_t(D.q.w) * D.q.h;
     DL_CK(G->slot_of.reserve(4 * size_t(nsub)), "alloc");
     DL_CK(launch_group_slots(G->grouped.as<int2>(), nr, R.ray_of.as<uint32_t>(), nsub,
                              alt ? v0.as<uint32_t>() : v1.as<uint32_t>(), G->slot_of.as<uint32_t>(),
                              s),
           "group slots");
-    std::vector<uint2> h_ranges(static_cast<size_t>(ngroups));
-    DL_CK(cudaMemcpyAsync(h_ranges.data(), ranges.p, 8 * size_t(ngroups), cudaMemcpyDeviceToHost, s),
-          "copy");
     DL_CK(cudaStreamSynchronize(s), "sync");
-    // h_ranges[tile * nv + v]: the rays of group g = v * ntiles + tile, in
-    // the grouping's (tile-major) order
-    const int64_t nv = D.q.nv;
-    auto group_of = [&](int64_t k) { return (k % nv) * G->ntiles + k / nv; };
-    std::vector<int4> work;
-    work.reserve(size_t(nr / kRaysPerBlock + ngroups / 4 + 16));
-    for (int64_t k = 0; k < ngroups; ++k) {
-        const uint2 r = h_ranges[size_t(k)];
-        const int64_t g = group_of(k);
-        for (uint32_t b = r.x; b < r.y; b += kRaysPerBlock)
-            work.push_back(make_int4(int(g), int(b), int(std::min<uint32_t>(b + kRaysPerBlock, r.y)), 0));
-    }
-    G->n_work = int64_t(work.size());
-    DL_CK(G->work.reserve(16 * std::max<size_t>(work.size(), 1)), "alloc");
-    if (!work.empty())
-        DL_CK(cudaMemcpyAsync(G->work.p, work.data(), 16 * work.size(), cudaMemcpyHostToDevice, s),
-              "copy");
-    // the compositing items in view-major order: consecutive items are
-    // neighbouring tiles of one view, which share records in L2 (tile-major
-    // items measured 1.6 x the DRAM reads)
-    std::vector<int4> gwork;
-    for (int64_t g = 0; g < ngroups; ++g) {
-        const int64_t k = (g % G->ntiles) * nv + g / G->ntiles;
-        const uint2 r = h_ranges[size_t(k)];
-        if (r.y > r.x) gwork.push_back(make_int4(int(g), int(r.x), int(r.y), 0));
-    }
-    G->n_gwork = int64_t(gwork.size());
-    DL_CK(G->gwork.reserve(16 * std::max<size_t>(gwork.size(), 1)), "alloc");
-    if (!gwork.empty())
-        DL_CK(cudaMemcpyAsync(G->gwork.p, gwork.data(), 16 * gwork.size(), cudaMemcpyHostToDevice, s),
-              "copy");
+    G->n_work = int64_t(h_totals[0]);
+    G->n_gwork = int64_t(h_totals[1]);
+    DL_CK(G->work.reserve(16 * size_t(std::max<int64_t>(G->n_work, 1))), "alloc");
+    DL_CK(G->gwork.reserve(16 * size_t(std::max<int64_t>(G->n_gwork, 1))), "alloc");
+    DL_CK(launch_list_fill(ranges.as<uint2>(), ngroups, G->ntiles, D.q.nv, kRaysPerBlock, chunk_at,
+                           used_at, G->work.as<int4>(), G->gwork.as<int4>(), s),
+          "list fill");
     DL_CK(cudaStreamSynchronize(s), "sync");
     *out = G.get();
     R.groups[key] = std::move(G);
@@ -1412,7 +1405,7 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
                                         s),
                   "composite rays");
         }
-        launches += 3 + 1 + 3 * ((nk > 1) ? (sort_bits + 7) / 8 : 0) + (nk > 0 ? 1 : 0) +
+        launches += 3 + 1 + radix_sort_launches(nk, sort_bits) + (nk > 0 ? 1 : 0) +
                     (mode == DL_STANDARD ? 1 : (G->n_work > 0 ? 1 : 0));
     }
     DL_CK(mark(7), "event");

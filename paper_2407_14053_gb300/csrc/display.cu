@@ -23,8 +23,13 @@ __device__ __forceinline__ int64_t d_offset(const DisplayQ& q, int64_t x, int64_
 
 // ------------------------------------------------------------------ a1 ---
 // v = floor(N_v (d mod L_x) / L_x), Eqs. (2)-(3), mod taken into [0, L_x).
-// One thread writes 8 consecutive views (one 16-byte store).
-__global__ void view_map_kernel(DisplayQ q, uint16_t* __restrict__ V) {
+// One thread writes 8 consecutive views (one 16-byte store).  N_v x_offset =
+// v L_x + rem is kept as (v, rem): one subpixel on, N_v 2^32 = step_v L_x +
+// step_rem is added, and a view past N_v wraps by N_v (x_offset by L_x), so
+// only a thread's first subpixel and a row's first are divided out (with a
+// division a subpixel the kernel was bound by it: 0.171 ms at 4K).
+__global__ void view_map_kernel(DisplayQ q, int64_t step_v, int64_t step_rem,
+                                uint16_t* __restrict__ V) {
     const int64_t S = 3 * int64_t(q.w);
     const int64_t total = S * q.h;
     const int64_t n8 = (total + 7) / 8;
@@ -32,23 +37,31 @@ __global__ void view_map_kernel(DisplayQ q, uint16_t* __restrict__ V) {
          t += int64_t(gridDim.x) * blockDim.x) {
         const int64_t i0 = t * 8;
         int64_t x = i0 / S, s = i0 - x * S;
-        int64_t d = d_offset(q, x, s);
-        int64_t xo = d % q.lq;
-        if (xo < 0) xo += q.lq;
+        int64_t v = 0, rem = 0;
+        auto divide = [&]() {
+            int64_t xo = d_offset(q, x, s) % q.lq;
+            if (xo < 0) xo += q.lq;
+            const int64_t n = int64_t(q.nv) * xo;
+            v = n / q.lq;
+            rem = n - v * q.lq;
+        };
+        divide();
         uint16_t out[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-            out[j] = (uint16_t)((int64_t(q.nv) * xo) / q.lq);
-            // next subpixel: same row adds 2^32, a new row restarts at s = 0
-            if (++s == S) {
+            out[j] = uint16_t(v);
+            if (++s == S) {  // a new row restarts at s = 0
                 s = 0;
                 ++x;
-                d = d_offset(q, x, 0);
-                xo = d % q.lq;
-                if (xo < 0) xo += q.lq;
+                divide();
             } else {
-                xo += kQ32;
-                if (xo >= q.lq) xo %= q.lq;
+                v += step_v;
+                rem += step_rem;
+                if (rem >= q.lq) {
+                    rem -= q.lq;
+                    ++v;
+                }
+                if (v >= q.nv) v -= q.nv;  // step_v < N_v: at most one wrap
             }
         }
         if (i0 + 8 <= total && ((reinterpret_cast<uintptr_t>(V + i0) & 15) == 0)) {
@@ -69,8 +82,8 @@ __device__ __forceinline__ uint32_t pack_px(int64_t x, int64_t y) {
     return (uint32_t(x) << 16) | uint32_t(y);
 }
 
-// ceil(x / 2^32)
-__device__ __forceinline__ int64_t ceil_q32(int64_t x) { return (x + (kQ32 - 1)) >> 32; }
+// ceil(x / 2^32); |x| < 2^54 here (panels end near 2^53), so it fits 32 bits
+__device__ __forceinline__ int32_t ceil_q32(int64_t x) { return int32_t((x + (kQ32 - 1)) >> 32); }
 
 // Alg. 2, four lanes per (area, view).  Areas are independent (Sec. 5), and
 // inside an area so are the views: a chain (Eqs. (11)-(14)) starts at an
@@ -93,26 +106,20 @@ __device__ __forceinline__ int64_t ceil_q32(int64_t x) { return (x + (kQ32 - 1))
 // Bound by the latency of a chain's dependent steps, so the groups are many
 // (35 thousand at 4K: 783 areas x 45 views, about 780 subpixels each) and take
 // four rows at a time, of the walk as of the search.  The warp's eight groups
-// advance together, one such look each an iteration, whatever the others do:
-// as nested loops a thread per (area, view) took 30.8 ms at 4K, every lane
-// waiting for each lane's chains, and a warp per area that took the views'
-// chains in turn and searched V 32 candidates at a time 48.6 ms.
+// advance together, one such look each an iteration, whatever the others do.
+// 4.0 ms at 4K (6.1 with two lanes a group, 4.7 with eight).  As nested loops
+// a thread per (area, view) took 30.8 ms, every lane waiting for each lane's
+// chains, and a warp per area that took the views' chains in turn and
+// searched V 32 candidates at a time 48.6 ms.
 constexpr int kChainLanes = 4;
 
 __global__ void __launch_bounds__(32)
 repurpose_kernel(DisplayQ q, uint32_t* src) {
     const int64_t lq = q.lq;
-    // moves the unit bound to the unit that holds d
-    auto follow = [lq](int64_t& unit, int64_t d) {
-        const int64_t t = d - unit;
-        if (t < -8 * lq || t >= 8 * lq) unit += floor_div(t, lq) * lq;
-        while (unit > d) unit -= lq;
-        while (unit + lq <= d) unit += lq;
-    };
+    const int64_t far = 8 * lq;  // from here on a division is cheaper than steps
     const int lane = threadIdx.x, sub = lane % kChainLanes;
     const unsigned group = ((1u << kChainLanes) - 1u) << (lane - sub);
     const int32_t S = 3 * q.w, h = q.h;
-    const int64_t last_d = int64_t(S - 1) * kQ32;
     const int64_t most_u = (int64_t(1) << 53) / lq + 2;  // past every panel's units
     const int64_t total = int64_t(q.n_areas) * q.nv;
     constexpr int kGroups = 32 / kChainLanes;
@@ -123,7 +130,7 @@ repurpose_kernel(DisplayQ q, uint32_t* src) {
         const int64_t vlo = (v * lq + q.nv - 1) / q.nv, vhi = ((v + 1) * lq + q.nv - 1) / q.nv;
         // the area's d range
         const int64_t u_lo = max(a * q.pw, -most_u) * lq, u_hi = min((a + 1) * q.pw, most_u) * lq;
-        int64_t ru = u_lo;            // unit of the lane's row of the walk, at s = 0
+        const int64_t span = vhi - vlo;
         int64_t wu = u_lo;            // unit of the lane's row of the search, at its first column
         int32_t x = 0;                // the walk's first row
         bool chain = false, fresh = false;  // a chain is running; it stands at a new subpixel
@@ -134,15 +141,15 @@ repurpose_kernel(DisplayQ q, uint32_t* src) {
             // the walk: the first empty subpixel of view v of each lane's row
             int32_t at = -1;
             if (!done && !chain && x + sub < h) {
-                const int64_t base = int64_t(x + sub) * q.t3q - q.kq;
-                follow(ru, base);
-                const int64_t u_end = min(u_hi, base + last_d + 1);
-                for (int64_t u = max(ru, u_lo); u < u_end && at < 0; u += lq) {
-                    const int64_t s0 = max(ceil_q32(u + vlo - base), int64_t(0));
-                    const int64_t s1 = min(ceil_q32(u + vhi - base), int64_t(S));
-                    for (int64_t s = s0; s < s1; ++s)
+                const int64_t base = int64_t(x + sub) * q.t3q - q.kq, off = vlo - base;
+                int64_t u = u_lo;  // or, in wide areas, the row's first unit
+                if (base - u >= far) u += floor_div(base - u, lq) * lq;
+                for (; u < u_hi && at < 0; u += lq) {
+                    const int32_t s0 = ceil_q32(u + off), s1 = min(ceil_q32(u + off + span), S);
+                    if (s0 >= S) break;
+                    for (int32_t s = max(s0, 0); s < s1; ++s)
                         if (src[int64_t(x + sub) * S + s] == kEmpty) {
-                            at = int32_t(s);
+                            at = s;
                             break;
                         }
                 }
@@ -182,14 +189,19 @@ repurpose_kernel(DisplayQ q, uint32_t* src) {
             int32_t found = -1;
             bool inside = false;  // in the chain's area
             if (chain && r_cur + sub <= r_hi) {
-                const int64_t rb = int64_t(r_cur + sub) * q.t3q - q.kq;
-                const int64_t d0 = int64_t(w0) * kQ32 + rb, d1 = int64_t(w1) * kQ32 + rb;
-                follow(wu, d0);
+                const int64_t rb = int64_t(r_cur + sub) * q.t3q - q.kq, off = vlo - rb;
+                // the first unit whose subpixels of view v end past column w0
+                const int64_t t0 = int64_t(w0) * kQ32 + rb - wu;
+                if (t0 < -far || t0 >= far) wu += floor_div(t0, lq) * lq;
+                while (ceil_q32(wu + off + span) > w0) wu -= lq;
+                do wu += lq;
+                while (ceil_q32(wu + off + span) <= w0);
                 int32_t fcol = -1;
-                for (int64_t t = wu; t + vlo <= d1; t += lq) {
-                    const int64_t a0 = max(ceil_q32(t + vlo - rb), int64_t(w0));
-                    const int64_t a1 = min(ceil_q32(t + vhi - rb) - 1, int64_t(w1));
-                    for (int32_t j = int32_t(a0); j <= a1; ++j) {
+                for (int64_t t = wu;; t += lq) {
+                    const int32_t a0 = ceil_q32(t + off);
+                    if (a0 > w1) break;
+                    const int32_t a1 = min(ceil_q32(t + off + span) - 1, w1);
+                    for (int32_t j = max(a0, w0); j <= a1; ++j) {
                         const int32_t c = j / 3, ch = j - 3 * c;
                         if ((ch == 0 ? B0 : (ch == 1 ? B1 : B2)) == kEmpty) continue;
                         // the nearest column first, then the lowest channel
@@ -237,17 +249,13 @@ __global__ void identity_src_kernel(int32_t w, int32_t h, uint32_t* __restrict__
 // the source pixel with the lowest channel k0 showing view v.  Rays are
 // numbered in order of first use by the R subpixels (row-major), then G,
 // then B (Sec. 5: R~_rays follows the R subpixels): an owner's order key is
-// the first R pixel using it, else wh + the first G pixel, else 2wh + the
-// first B pixel, and its ray id is the rank of that key.
+// the lowest of its subpixels' keys k wh + pixel, and its ray id is the rank
+// of that key.
 struct RayTmp {
-    uint32_t* owner;        // 3wh: owner subpixel of each subpixel's ray
-    uint32_t* ray_of_owner; // 3wh: ray id per owner (kEmpty when not an owner)
-    uint32_t* first_r;      // 3wh: first R pixel index using the owner
-    uint32_t* first_g;      // 3wh
-    uint32_t* first_b;      // 3wh
-    uint32_t* key_of;       // 3wh: order key of each owner
-    uint32_t* flag;         // 3wh: 1 at every used order key
-    uint32_t* rank;         // 3wh + 1
+    uint32_t* owner;  // 3wh: owner subpixel of each subpixel's ray
+    uint32_t* id_of;  // 3wh: order key, then ray id, per owner (kEmpty when not an owner)
+    uint32_t* flag;   // 3wh: 1 at every used order key
+    uint32_t* rank;   // 3wh
     void* scan_tmp;
 };
 
@@ -261,73 +269,53 @@ __host__ RayTmp carve(const DisplayQ& q, void* tmp) {
         return r;
     };
     t.owner = reinterpret_cast<uint32_t*>(take(4 * n));
-    t.ray_of_owner = reinterpret_cast<uint32_t*>(take(4 * n));
-    t.first_r = reinterpret_cast<uint32_t*>(take(4 * n));
-    t.first_g = reinterpret_cast<uint32_t*>(take(4 * n));
-    t.first_b = reinterpret_cast<uint32_t*>(take(4 * n));
-    t.key_of = reinterpret_cast<uint32_t*>(take(4 * n));
+    t.id_of = reinterpret_cast<uint32_t*>(take(4 * n));
     t.flag = reinterpret_cast<uint32_t*>(take(4 * n));
-    t.rank = reinterpret_cast<uint32_t*>(take(4 * n + 4));
+    t.rank = reinterpret_cast<uint32_t*>(take(4 * n));
     t.scan_tmp = take(0);
     return t;
 }
 
+// id_of holds kEmpty everywhere at the launch
 __global__ void owner_kernel(int32_t w, int32_t h, int64_t n, const uint16_t* __restrict__ V,
                              const uint32_t* __restrict__ src, RayTmp t) {
+    const uint32_t wh = uint32_t(n / 3);
     for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n;
          i += int64_t(gridDim.x) * blockDim.x) {
-        const uint32_t s = src[i];
+        const uint32_t s = src[i], p = uint32_t(i) / 3u;
         // a source outside the panel (never produced by the repurposing) is
         // read as the subpixel's own pixel rather than followed
         const bool ok = (s >> 16) < uint32_t(h) && (s & 0xFFFF) < uint32_t(w);
-        const int64_t sp = ok ? int64_t(s >> 16) * w + (s & 0xFFFF) : i / 3;
+        const int64_t sp = ok ? int64_t(s >> 16) * w + (s & 0xFFFF) : int64_t(p);
         const uint16_t v = V[i];
         int k0 = 0;
         while (k0 < 2 && V[3 * sp + k0] != v) ++k0;
-        t.owner[i] = uint32_t(3 * sp + k0);
-        t.ray_of_owner[i] = kEmpty;
-        t.first_r[i] = kEmpty;
-        t.first_g[i] = kEmpty;
-        t.first_b[i] = kEmpty;
-        t.key_of[i] = kEmpty;
+        const uint32_t o = uint32_t(3 * sp + k0);
+        t.owner[i] = o;
+        atomicMin(&t.id_of[o], (uint32_t(i) - 3u * p) * wh + p);
     }
 }
 
-__global__ void first_use_kernel(int64_t wh, RayTmp t) {
-    for (int64_t p = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; p < wh;
-         p += int64_t(gridDim.x) * blockDim.x) {
-        atomicMin(&t.first_r[t.owner[3 * p]], uint32_t(p));
-        atomicMin(&t.first_g[t.owner[3 * p + 1]], uint32_t(p));
-        atomicMin(&t.first_b[t.owner[3 * p + 2]], uint32_t(p));
-    }
-}
-
-__global__ void mark_keys_kernel(int64_t n, int64_t wh, RayTmp t) {
+__global__ void mark_keys_kernel(int64_t n, RayTmp t) {
     for (int64_t o = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; o < n;
          o += int64_t(gridDim.x) * blockDim.x) {
-        uint32_t key = kEmpty;
-        if (t.first_r[o] != kEmpty) key = t.first_r[o];
-        else if (t.first_g[o] != kEmpty) key = uint32_t(wh) + t.first_g[o];
-        else if (t.first_b[o] != kEmpty) key = uint32_t(2 * wh) + t.first_b[o];
-        if (key != kEmpty) {
-            t.key_of[o] = key;
-            t.flag[key] = 1;
-        }
+        const uint32_t key = t.id_of[o];
+        if (key != kEmpty) t.flag[key] = 1;
     }
 }
 
 __global__ void assign_kernel(int64_t n, RayTmp t) {
     for (int64_t o = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; o < n;
          o += int64_t(gridDim.x) * blockDim.x) {
-        const uint32_t key = t.key_of[o];
-        if (key != kEmpty) t.ray_of_owner[o] = t.rank[key];
+        const uint32_t key = t.id_of[o];
+        if (key != kEmpty) t.id_of[o] = t.rank[key];
     }
 }
 
 __global__ void ray_of_kernel(int64_t n, const RayTmp t, uint32_t* __restrict__ ray_of) {
     for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n;
          i += int64_t(gridDim.x) * blockDim.x)
-        ray_of[i] = t.ray_of_owner[t.owner[i]];
+        ray_of[i] = t.id_of[t.owner[i]];
 }
 
 __global__ void ray_attr_kernel(int32_t w, int64_t n, const uint16_t* __restrict__ V,
@@ -335,18 +323,18 @@ __global__ void ray_attr_kernel(int32_t w, int64_t n, const uint16_t* __restrict
                                 uint32_t* __restrict__ ray_pix) {
     for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n;
          i += int64_t(gridDim.x) * blockDim.x) {
-        const uint32_t r = t.ray_of_owner[i];
+        const uint32_t r = t.id_of[i];
         if (r != kEmpty) {  // i is an owner subpixel
-            const int64_t p = i / 3;
+            const uint32_t p = uint32_t(i) / 3u, x = p / uint32_t(w);
             ray_view[r] = V[i];
-            ray_pix[r] = pack_px(p / w, p % w);
+            ray_pix[r] = pack_px(x, p - x * uint32_t(w));
         }
     }
 }
 
 __global__ void group_keys_kernel(const uint32_t* __restrict__ ray_view,
                                   const uint32_t* __restrict__ ray_pix, int64_t n, int32_t tw,
-                                  int32_t th, int32_t ntx, int32_t nv,
+                                  int32_t th, int32_t ntx, int32_t nv, int shift,
                                   unsigned long long* __restrict__ keys,
                                   uint32_t* __restrict__ vals) {
     for (int64_t r = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; r < n;
@@ -359,7 +347,7 @@ __global__ void group_keys_kernel(const uint32_t* __restrict__ ray_view,
         // rays cover a compact patch
         uint32_t x = col % tw, y = row % th, m = 0;
         for (int b = 0; b < 8; ++b) m |= (((x >> b) & 1u) << (2 * b)) | (((y >> b) & 1u) << (2 * b + 1));
-        keys[r] = (g << 16) | m;
+        keys[r] = (g << shift) | m;
         vals[r] = uint32_t(r);
     }
 }
@@ -390,6 +378,39 @@ __global__ void group_slot_kernel(const uint32_t* __restrict__ ray_of, int64_t n
         slot_of[i] = pos[ray_of[i]];
 }
 
+// Work lists of a grouping: ranges[k], k = tile * nv + view, are the rays of
+// group g = view * ntiles + tile.  chunks[k]: pieces of at most `piece` rays;
+// used[g]: 1 when the group holds rays.  Entry n_groups of both is 0.
+__global__ void list_counts_kernel(const uint2* __restrict__ ranges, int64_t n_groups, int64_t ntiles,
+                                   int64_t nv, uint32_t piece, uint32_t* __restrict__ chunks,
+                                   uint32_t* __restrict__ used) {
+    for (int64_t k = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; k <= n_groups;
+         k += int64_t(gridDim.x) * blockDim.x) {
+        const uint2 r = k < n_groups ? ranges[k] : make_uint2(0u, 0u);
+        const int64_t tile = k / nv;
+        chunks[k] = (r.y - r.x + piece - 1) / piece;
+        used[k < n_groups ? (k - tile * nv) * ntiles + tile : k] = r.y > r.x ? 1u : 0u;
+    }
+}
+
+// work: every piece {group, first ray, end ray, -} in k order; gwork: every
+// group with rays {group, first ray, end ray, -} in g (view-major) order.
+__global__ void list_fill_kernel(const uint2* __restrict__ ranges, int64_t n_groups, int64_t ntiles,
+                                 int64_t nv, uint32_t piece, const uint32_t* __restrict__ chunk_at,
+                                 const uint32_t* __restrict__ used_at, int4* __restrict__ work,
+                                 int4* __restrict__ gwork) {
+    for (int64_t k = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; k < n_groups;
+         k += int64_t(gridDim.x) * blockDim.x) {
+        const uint2 r = ranges[k];
+        if (r.y <= r.x) continue;
+        const int64_t tile = k / nv, g = (k - tile * nv) * ntiles + tile;
+        gwork[used_at[g]] = make_int4(int(g), int(r.x), int(r.y), 0);
+        uint32_t w = chunk_at[k];
+        for (uint32_t b = r.x; b < r.y; b += piece)
+            work[w++] = make_int4(int(g), int(b), int(min(b + piece, r.y)), 0);
+    }
+}
+
 __global__ void rays_export_kernel(const uint32_t* __restrict__ ray_view,
                                    const uint32_t* __restrict__ ray_pix, int64_t n,
                                    int32_t* __restrict__ out) {
@@ -407,7 +428,7 @@ __global__ void ray_triplets_kernel(int32_t w, int64_t n, const uint16_t* __rest
                                     const RayTmp t, int32_t* __restrict__ out) {
     for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n;
          i += int64_t(gridDim.x) * blockDim.x) {
-        const uint32_t r = t.ray_of_owner[i];
+        const uint32_t r = t.id_of[i];
         if (r != kEmpty) {
             const int64_t p = i / 3;
             out[3 * int64_t(r)] = int32_t(V[i]);
@@ -428,7 +449,9 @@ int grid_for(int64_t n, int block) {
 
 cudaError_t launch_view_map(const DisplayQ& q, uint16_t* V, cudaStream_t s) {
     const int64_t n8 = (3 * int64_t(q.w) * q.h + 7) / 8;
-    view_map_kernel<<<grid_for(n8, 256), 256, 0, s>>>(q, V);
+    // 2^32 mod L_x: whole lens lines (a pitch below a subpixel) do not count
+    const int64_t n = int64_t(q.nv) * (kQ32 % q.lq);
+    view_map_kernel<<<grid_for(n8, 256), 256, 0, s>>>(q, n / q.lq, n % q.lq, V);
     return cudaGetLastError();
 }
 
@@ -447,19 +470,18 @@ cudaError_t launch_repurpose(const DisplayQ& q, uint32_t* src, int identity, cud
 
 size_t ray_table_tmp_bytes(const DisplayQ& q) {
     const size_t n = 3 * size_t(q.w) * q.h;
-    return 7 * ((4 * n + 255) & ~size_t(255)) + ((4 * n + 4 + 255) & ~size_t(255)) +
-           scan_tmp_bytes(int64_t(n)) + 256;
+    return 4 * ((4 * n + 255) & ~size_t(255)) + scan_tmp_bytes(int64_t(n)) + 256;
 }
 
 cudaError_t launch_ray_table(const DisplayQ& q, const uint16_t* V, const uint32_t* src,
                              uint32_t* ray_of, void* tmp, uint32_t* d_n_rays, cudaStream_t s) {
-    const int64_t wh = int64_t(q.w) * q.h, n = 3 * wh;
+    const int64_t n = 3 * int64_t(q.w) * q.h;
     RayTmp t = carve(q, tmp);
     cudaError_t e = cudaMemsetAsync(t.flag, 0, sizeof(uint32_t) * size_t(n), s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(t.id_of, 0xFF, sizeof(uint32_t) * size_t(n), s);
     if (e != cudaSuccess) return e;
     owner_kernel<<<grid_for(n, 256), 256, 0, s>>>(q.w, q.h, n, V, src, t);
-    first_use_kernel<<<grid_for(wh, 256), 256, 0, s>>>(wh, t);
-    mark_keys_kernel<<<grid_for(n, 256), 256, 0, s>>>(n, wh, t);
+    mark_keys_kernel<<<grid_for(n, 256), 256, 0, s>>>(n, t);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     e = launch_exclusive_scan(t.flag, t.rank, n, d_n_rays, t.scan_tmp, s);
@@ -478,10 +500,26 @@ cudaError_t launch_ray_attributes(const DisplayQ& q, const uint16_t* V, const vo
 }
 
 cudaError_t launch_ray_group_keys(const uint32_t* ray_view, const uint32_t* ray_pix, int64_t n_rays,
-                                  int32_t tile_w, int32_t tile_h, int32_t ntx, int32_t nv,
+                                  int32_t tile_w, int32_t tile_h, int32_t ntx, int32_t nv, int shift,
                                   unsigned long long* keys, uint32_t* vals, cudaStream_t s) {
     group_keys_kernel<<<grid_for(n_rays, 256), 256, 0, s>>>(ray_view, ray_pix, n_rays, tile_w,
-                                                             tile_h, ntx, nv, keys, vals);
+                                                             tile_h, ntx, nv, shift, keys, vals);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_list_counts(const uint2* ranges, int64_t n_groups, int32_t ntiles, int32_t nv,
+                               int32_t piece, uint32_t* chunks, uint32_t* used, cudaStream_t s) {
+    list_counts_kernel<<<grid_for(n_groups + 1, 256), 256, 0, s>>>(ranges, n_groups, ntiles, nv,
+                                                                   uint32_t(piece), chunks, used);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_list_fill(const uint2* ranges, int64_t n_groups, int32_t ntiles, int32_t nv,
+                             int32_t piece, const uint32_t* chunk_at, const uint32_t* used_at,
+                             int4* work, int4* gwork, cudaStream_t s) {
+    list_fill_kernel<<<grid_for(n_groups, 256), 256, 0, s>>>(ranges, n_groups, ntiles, nv,
+                                                             uint32_t(piece), chunk_at, used_at, work,
+                                                             gwork);
     return cudaGetLastError();
 }
 

@@ -142,14 +142,24 @@ cudaError_t launch_ray_table(const DisplayQ& q, const uint16_t* V, const uint32_
                              uint32_t* ray_of, void* tmp, uint32_t* d_n_rays, cudaStream_t s);
 cudaError_t launch_ray_attributes(const DisplayQ& q, const uint16_t* V, const void* tmp,
                                   uint32_t* ray_view, uint32_t* ray_pix, cudaStream_t s);
-// Group keys of rays for a compositing tile shape: key = (tile*nv + v) << 16
-// | Morton code of the pixel inside the tile; value = ray id.  Sorted, the
-// rays are grouped tile-major (every view of a tile, then the next tile), so
-// a tile's ray colours are one run and the reorder's gathers for a patch of
-// the panel stay in a few kilobytes.
+// Group keys of rays for a compositing tile shape: key = (tile*nv + v) <<
+// shift | Morton code of the pixel inside the tile (2 log2 of the tile's
+// longer side bits, the least shift); value = ray id.  Sorted, the rays are
+// grouped tile-major (every view of a tile, then the next tile), so a tile's
+// ray colours are one run and the reorder's gathers for a patch of the panel
+// stay in a few kilobytes.
 cudaError_t launch_ray_group_keys(const uint32_t* ray_view, const uint32_t* ray_pix, int64_t n_rays,
-                                  int32_t tile_w, int32_t tile_h, int32_t ntx, int32_t nv,
+                                  int32_t tile_w, int32_t tile_h, int32_t ntx, int32_t nv, int shift,
                                   unsigned long long* keys, uint32_t* vals, cudaStream_t s);
+// The grouping's work lists from its ranges (uint2 per tile * nv + view):
+// per range its pieces of at most `piece` rays (chunks) and per group (view *
+// ntiles + tile) whether it holds rays (used), n_groups + 1 entries each, the
+// last one 0; then, with both scanned, the lists of pieces and of groups.
+cudaError_t launch_list_counts(const uint2* ranges, int64_t n_groups, int32_t ntiles, int32_t nv,
+                               int32_t piece, uint32_t* chunks, uint32_t* used, cudaStream_t s);
+cudaError_t launch_list_fill(const uint2* ranges, int64_t n_groups, int32_t ntiles, int32_t nv,
+                             int32_t piece, const uint32_t* chunk_at, const uint32_t* used_at,
+                             int4* work, int4* gwork, cudaStream_t s);
 // (view, row, col) int32 triplets of every ray.
 cudaError_t launch_rays_export(const uint32_t* ray_view, const uint32_t* ray_pix, int64_t n_rays,
                                int32_t* out, cudaStream_t s);
@@ -253,6 +263,8 @@ size_t radix_tmp_bytes(int64_t n);
 cudaError_t radix_sort_pairs(unsigned long long* keys, uint32_t* vals, unsigned long long* keys_alt,
                              uint32_t* vals_alt, int64_t n, int bits, void* tmp,
                              int* result_in_alt, cudaStream_t s);
+// kernels radix_sort_pairs launches for these arguments
+int radix_sort_launches(int64_t n, int bits);
 // ranges[g] = [first, last) index of keys whose key >> shift == g < n_groups.
 // ranges must be zeroed first.
 cudaError_t launch_key_ranges(const unsigned long long* keys, int64_t n, int shift, uint2* ranges,

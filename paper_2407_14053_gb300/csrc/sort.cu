@@ -121,6 +121,7 @@ constexpr int kRadixWarps = kRadixThreads / 32;
 constexpr int kRadixItems = 12;
 constexpr int kRadixTile = kRadixThreads * kRadixItems;
 constexpr int kBins = 256;
+constexpr int64_t kRadixScanMax = 16384;  // largest histogram radix_scan_kernel scans
 
 __global__ void __launch_bounds__(kRadixThreads)
 radix_upsweep_kernel(const unsigned long long* __restrict__ keys, int64_t n, int64_t chunk,
@@ -286,8 +287,14 @@ cudaError_t launch_exclusive_scan(const uint32_t* in, uint32_t* out, int64_t n, 
 
 size_t radix_tmp_bytes(int64_t n) {
     int64_t chunk;
-    const int G = radix_grid(n > 0 ? n : 1, &chunk);
-    return size_t(kBins) * G * sizeof(uint32_t) + 256;
+    const int64_t hist = int64_t(kBins) * radix_grid(n > 0 ? n : 1, &chunk);
+    return 2 * size_t(hist) * sizeof(uint32_t) + scan_tmp_bytes(hist) + 256;
+}
+
+int radix_sort_launches(int64_t n, int bits) {
+    if (n <= 1 || bits <= 0) return 0;
+    int64_t chunk;
+    return (bits + 7) / 8 * (int64_t(kBins) * radix_grid(n, &chunk) > kRadixScanMax ? 5 : 3);
 }
 
 cudaError_t radix_sort_pairs(unsigned long long* keys, uint32_t* vals, unsigned long long* keys_alt,
@@ -305,7 +312,12 @@ cudaError_t radix_sort_pairs(unsigned long long* keys, uint32_t* vals, unsigned 
     }
     int64_t chunk;
     const int G = radix_grid(n, &chunk);
-    uint32_t* hist = static_cast<uint32_t*>(tmp);
+    const int64_t nh = int64_t(kBins) * G;
+    uint32_t* const hist = static_cast<uint32_t*>(tmp);
+    // one block scans a small histogram in one launch; a large one (155 k
+    // counters for a 4K panel's rays) took it 146 us a pass, the device-wide
+    // scan's three launches 12
+    uint32_t* const offsets = nh > kRadixScanMax ? hist + nh : hist;
     unsigned long long *ki = keys, *ko = keys_alt;
     uint32_t *vi = vals, *vo = vals_alt;
     int flips = 0;
@@ -313,10 +325,15 @@ cudaError_t radix_sort_pairs(unsigned long long* keys, uint32_t* vals, unsigned 
         const int nb = bits - shift < 8 ? bits - shift : 8;
         const uint32_t mask = (1u << nb) - 1u;
         radix_upsweep_kernel<<<G, kRadixThreads, 0, s>>>(ki, n, chunk, shift, mask, hist);
-        radix_scan_kernel<<<1, 1024, 0, s>>>(hist, int64_t(kBins) * G);
+        cudaError_t e = cudaSuccess;
+        if (nh > kRadixScanMax)
+            e = launch_exclusive_scan(hist, offsets, nh, nullptr, offsets + nh, s);
+        else
+            radix_scan_kernel<<<1, 1024, 0, s>>>(hist, nh);
+        if (e != cudaSuccess) return e;
         radix_downsweep_kernel<<<G, kRadixThreads, smem, s>>>(ki, vi, ko, vo, n, chunk, shift, mask,
-                                                               hist);
-        cudaError_t e = cudaGetLastError();
+                                                               offsets);
+        e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         unsigned long long* tk = ki; ki = ko; ko = tk;
         uint32_t* tv = vi; vi = vo; vo = tv;
