@@ -858,9 +858,8 @@ def main():
 
     # ---- rooflines of the other stages (HBM-bound; per frame) ----
     ne = d.num_views * wl.scene.n
-    # the library's default emits the keys from the projection for scenes of
-    # 131,072 Gaussians or more
-    if args.two_pass_emission or wl.scene.n < 131072:
+    # the library's default emits the keys from the projection
+    if args.two_pass_emission:
         stages_roof = {
             "project": stage_roofline(
                 "project_kernel (with the camera upload and counter resets before it)",

@@ -285,10 +285,8 @@ enum { DL_OPT_SORT_MODE = 1, DL_OPT_EVAL_DIRECTL = 2, DL_OPT_EVAL_STANDARD = 3,
  * into slices sized from its own counts, on the device, before compositing.
  * 0: the projection writes per-(view, Gaussian) tile metadata and a second
  * kernel emits the keys into slices sized from this frame's counts (Sec. 4
- * step (2) as two passes).  2 (default): 1 for scenes of at least 131,072
- * Gaussians, else 0 (a small scene has too few warps in flight to hide the
- * projection's waits on its cursor atomics).  All give the same keys, so
- * the same image. */
+ * step (2) as two passes).  2 (default): the library's choice, at present 1
+ * for every scene.  All give the same keys, so the same image. */
 /* DL_OPT_HEAP_CAPACITY: c_h of DL_RAYCAST, the number of nearest
  * intersections each ray keeps and blends (1..256, default 128).
  *

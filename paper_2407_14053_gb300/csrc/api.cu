@@ -1085,10 +1085,7 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
     const bool on_device = warp_path && hint.sized && ctx->sort_mode != DL_SORT_RADIX;
     // keys emitted by the projection, into the slices the signature's last
     // frame laid out
-    // (by default only for scenes of 131,072 Gaussians or more: a warp's
-    // views run one after another, each waiting on its cursor atomics, which
-    // only enough warps in flight hide)
-    const bool in_projection = emit_in_projection(ctx->key_emission, S.n);
+    const bool in_projection = emit_in_projection(ctx->key_emission);
     const bool direct = on_device && in_projection && hint.slices_ready;
     DL_CK(W.rec.reserve(16 * kRecordFloat4 * size_t(ne)), "alloc records");
     if (!direct) DL_CK(W.meta.reserve(16 * size_t(ne)), "alloc tile metadata");

@@ -437,7 +437,7 @@ dl_status dl_batch_assign(dl_batch* b, int32_t slot, int32_t scene_id, int32_t d
     z.out = out_dev;
     z.pp = make_project_params(*S, *D, tw, th);
     z.ngroups = ng;
-    z.direct = emit_in_projection(ctx->key_emission, S->n);
+    z.direct = emit_in_projection(ctx->key_emission);
     if (z.direct) {  // empty slices: the first launch emits into slices of its own counts
         DL_CK(cudaMemsetAsync(b->at<uint32_t>(z.o_slices), 0, 4 * size_t(ng + 1), nullptr),
               "memset");

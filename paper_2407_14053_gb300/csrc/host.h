@@ -111,13 +111,12 @@ struct PendingFrame {
 // slices of the key buffer its next frame emits into: every group gets its
 // key count in the last frame plus an eighth and 16 (slices[cur]); a frame
 // writes the next layout into slices[cur ^ 1] and flips cur.
-// DL_OPT_KEY_EMISSION 2: the projection emits the keys for scenes of at
-// least this many Gaussians (with fewer, too few warps are in flight to hide
-// its waits on the cursor atomics)
-constexpr int64_t kEmitInProjectionMin = 131072;
-inline bool emit_in_projection(int32_t option, int64_t n_gaussians) {
-    return option == 1 || (option == 2 && n_gaussians >= kEmitInProjectionMin);
-}
+// DL_OPT_KEY_EMISSION: 0 is the two-pass emission; 1 and 2 (the library's
+// choice) have the projection emit the keys.  With the views split into ranges
+// for small scenes that is the faster one at every size measured: 107 against
+// 115 us a frame at 2,000 Gaussians, 365 against 388 at 41,003, 607 against
+// 675 at 120,000 (frames of 240x135 and 955x541).
+inline bool emit_in_projection(int32_t option) { return option != 0; }
 
 struct FrameHint {
     bool sized = false;

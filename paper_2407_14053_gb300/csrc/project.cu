@@ -6,6 +6,8 @@
 // Sigma' = J W Sigma W^T J^T + 0.3 I, conic, SH colour for the view's
 // direction, and the tile rectangle that holds every pixel where alpha can
 // reach 1/255.  All arithmetic is FP32.
+#include <algorithm>
+
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -53,8 +55,9 @@ __device__ __forceinline__ GaussState load_gauss(const GaussiansView<T>& G, int6
     s.mx = G.mean[3 * g];
     s.my = G.mean[3 * g + 1];
     s.mz = G.mean[3 * g + 2];
-    float qw = to_f(G.rot[4 * g]), qx = to_f(G.rot[4 * g + 1]);
-    float qy = to_f(G.rot[4 * g + 2]), qz = to_f(G.rot[4 * g + 3]);
+    struct alignas(4 * sizeof(T)) Quat { T w, x, y, z; };  // one load
+    const Quat rot = *reinterpret_cast<const Quat*>(G.rot + 4 * g);
+    float qw = to_f(rot.w), qx = to_f(rot.x), qy = to_f(rot.y), qz = to_f(rot.z);
     const float qn = rsqrtf(qw * qw + qx * qx + qy * qy + qz * qz);
     qw *= qn; qx *= qn; qy *= qn; qz *= qn;
     const float R00 = 1.f - 2.f * (qy * qy + qz * qz), R01 = 2.f * (qx * qy - qw * qz),
@@ -80,16 +83,51 @@ __device__ __forceinline__ GaussState load_gauss(const GaussiansView<T>& G, int6
     return s;
 }
 
+// Where coefficients 4 q .. 4 q + 3 of the block's Gaussian t are staged: a
+// warp's reads of one q, and the block's writes of consecutive q, are both
+// (nearly) free of bank conflicts.
+__device__ __forceinline__ int sh_slot(int q, int t) { return q * kProjectThreads + (t ^ (q & 7)); }
+template <int DEG>
+constexpr size_t sh_smem_bytes() { return sizeof(float4) * kProjectThreads * size_t(sh_float4<DEG>()); }
+
+// Stages the SH coefficients of the block's Gaussians [g0, g0 + count).  They
+// are one run of memory, so the block reads it in 16-byte pieces, thread after
+// thread (g0 is a multiple of 256 and the array 256-byte aligned, so every
+// piece is aligned).  A thread reading its own Gaussian's coefficients one by
+// one made every load touch 32 lines: at 41,003 Gaussians (FP16, SH degree 2)
+// a second copy of that cost the projection 20 us.  Ends with a barrier.
 template <typename T, int DEG>
-__device__ __forceinline__ void stage_sh(const GaussiansView<T>& G, int64_t g, float4* s_sh) {
-    constexpr int NF = 3 * (DEG + 1) * (DEG + 1), NF4 = sh_float4<DEG>();
+__device__ __forceinline__ void stage_sh(const T* __restrict__ sh, int64_t g0, int count,
+                                         float4* s_sh) {
+    constexpr int NF = 3 * (DEG + 1) * (DEG + 1), VE = 16 / int(sizeof(T));
+    const T* __restrict__ run = sh + g0 * NF;
+    float* const dst = reinterpret_cast<float*>(s_sh);
+    const int total = count * NF;
+    for (int e0 = int(threadIdx.x) * VE; e0 < total; e0 += kProjectThreads * VE) {
+        alignas(16) T v[VE];
+        if (e0 + VE <= total) {
+            *reinterpret_cast<uint4*>(v) = __ldg(reinterpret_cast<const uint4*>(run + e0));
+        } else {
 #pragma unroll
-    for (int q = 0; q < NF4; ++q) {
-        float v[4];
+            for (int k = 0; k < VE; ++k) v[k] = e0 + k < total ? run[e0 + k] : T(0.f);
+        }
+        if (NF % 4 == 0) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) v[k] = 4 * q + k < NF ? to_f(G.sh[g * NF + 4 * q + k]) : 0.f;
-        s_sh[q * kProjectThreads + threadIdx.x] = make_float4(v[0], v[1], v[2], v[3]);
+            for (int k = 0; k < VE; k += 4) {  // four coefficients of one Gaussian
+                const int t = (e0 + k) / NF, q = ((e0 + k) - t * NF) / 4;
+                if (e0 + k < total)
+                    s_sh[sh_slot(q, t)] =
+                        make_float4(to_f(v[k]), to_f(v[k + 1]), to_f(v[k + 2]), to_f(v[k + 3]));
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < VE; ++k) {
+                const int t = (e0 + k) / NF, f = (e0 + k) - t * NF;
+                if (e0 + k < total) dst[4 * sh_slot(f >> 2, t) + (f & 3)] = to_f(v[k]);
+            }
+        }
     }
+    __syncthreads();
 }
 
 // A Gaussian in one view: the EWA 2D covariance (Eq. (9)), its projected
@@ -177,7 +215,7 @@ __device__ __forceinline__ void write_record(const GaussState& s, const Cam& cam
     float acc[3] = {0.f, 0.f, 0.f};
 #pragma unroll
     for (int q = 0; q < NF4; ++q) {
-        const float4 w4 = s_sh[q * kProjectThreads + threadIdx.x];
+        const float4 w4 = s_sh[sh_slot(q, threadIdx.x)];
         const float w[4] = {w4.x, w4.y, w4.z, w4.w};
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
@@ -194,21 +232,53 @@ __device__ __forceinline__ void write_record(const GaussState& s, const Cam& cam
     rec[1] = make_float4(-0.5f * kLog2e * o.cxx * id, s.log2o, clo, chi);
 }
 
+// The views [view_begin, view_end) of a block: grid.y equal ranges.
+__device__ __forceinline__ int32_t view_begin(int32_t nv) {
+    return int32_t(int64_t(nv) * blockIdx.y / gridDim.y);
+}
+__device__ __forceinline__ int32_t view_end(int32_t nv) {
+    return int32_t(int64_t(nv) * (blockIdx.y + 1) / gridDim.y);
+}
+
+// Ranges the views are split into (grid.y) for a scene of `blocks` blocks.  A
+// thread projects its Gaussian into its range's views one after another, so
+// with one range a scene of few blocks takes as long as a large one, and one
+// of a few blocks more than are resident (four an SM) twice as long.  The
+// number taken makes the waves of resident blocks, times a block's views and
+// one more for loading its Gaussians, least: at 45 views 45 ranges for 2,000
+// Gaussians (57 -> 6 us), three for 200,000 (782 blocks on 608 resident ones:
+// 210 -> 160 us), one for a million.
+int view_ranges(int64_t blocks, int32_t nv) {
+    const int64_t slots = int64_t(num_sms()) * 4;
+    int best = 1;
+    int64_t least = INT64_MAX;
+    const int most = int(std::min<int64_t>(nv, 8 * slots / std::max<int64_t>(blocks, 1) + 1));
+    for (int r = 1; r <= most; ++r) {
+        const int64_t cost = (blocks * r + slots - 1) / slots * ((nv + r - 1) / r + 1);
+        if (cost < least) {
+            least = cost;
+            best = r;
+        }
+    }
+    return best;
+}
+
 template <typename T, int DEG>
 __global__ void __launch_bounds__(kProjectThreads, 4) project_kernel(GaussiansView<T> G, ProjectParams p,
                                                       const Cam* __restrict__ cams, int32_t nv,
                                                       ProjectOut out) {
-    extern __shared__ float4 s_sh[];  // [NF4][kProjectThreads]
-    const int64_t g = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+    extern __shared__ float4 s_sh[];  // [NF4][kProjectThreads], sh_slot
+    const int64_t g0 = blockIdx.x * int64_t(blockDim.x), g = g0 + threadIdx.x;
     unsigned long long my_total = 0;
     uint32_t my_visible = 0;
+    stage_sh<T, DEG>(G.sh, g0, int(min(p.n - g0, int64_t(kProjectThreads))), s_sh);
     if (g < p.n) {
         const GaussState gs = load_gauss(G, g);
-        stage_sh<T, DEG>(G, g, s_sh);
-        // warps start at different views (and wrap around), so warps in
-        // flight add to the counters of different views' tiles
-        int32_t v = int32_t((g >> 5) % nv);
-        for (int32_t k = 0; k < nv; ++k, v = v + 1 == nv ? 0 : v + 1) {
+        // warps start at different views of their range (and wrap around), so
+        // warps in flight add to the counters of different views' tiles
+        const int32_t va = view_begin(nv), vb = view_end(nv);
+        int32_t v = va + int32_t((g >> 5) % max(vb - va, 1));
+        for (int32_t k = va; k < vb; ++k, v = v + 1 == vb ? va : v + 1) {
             const Cam cam = load_cam(cams + v);
             const int64_t e = int64_t(v) * p.n + g;
             uint32_t cnt = 0;
@@ -217,8 +287,8 @@ __global__ void __launch_bounds__(kProjectThreads, 4) project_kernel(GaussiansVi
             if (project_splat(gs, cam, p, sp)) {
                 cnt = uint32_t(sp.tx1 - sp.tx0 + 1) * uint32_t(sp.ty1 - sp.ty0 + 1);
                 if (out.gcount) {  // keys per (view, tile) group
-                    const uint32_t vb = uint32_t(v) * uint32_t(p.ntx * p.nty);
-                    const uint32_t g0 = vb + uint32_t(sp.ty0 * p.ntx + sp.tx0);
+                    const uint32_t gb = uint32_t(v) * uint32_t(p.ntx * p.nty);
+                    const uint32_t g0 = gb + uint32_t(sp.ty0 * p.ntx + sp.tx0);
                     // the warp's Gaussians are neighbours in space: when
                     // every active lane covers the same single tile, one
                     // lane adds for all of them
@@ -231,7 +301,7 @@ __global__ void __launch_bounds__(kProjectThreads, 4) project_kernel(GaussiansVi
                     } else {
                         for (int ty = sp.ty0; ty <= sp.ty1; ++ty)
                             for (int tx = sp.tx0; tx <= sp.tx1; ++tx)
-                                atomicAdd(out.gcount + vb + uint32_t(ty * p.ntx + tx), 1u);
+                                atomicAdd(out.gcount + gb + uint32_t(ty * p.ntx + tx), 1u);
                     }
                 }
                 write_record<DEG>(gs, cam, sp, s_sh, out.rec + kRecordFloat4 * e);
@@ -465,24 +535,23 @@ __global__ void __launch_bounds__(kProjectThreads, 4)
 project_direct_kernel(GaussiansView<T> G, ProjectParams p, const Cam* __restrict__ cams, int32_t nv,
                       ProjectOut out) {
     if (KEYS_ONLY && *out.gate == 0u) return;
-    extern __shared__ float4 s_sh[];  // [NF4][kProjectThreads]
-    const int64_t g = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+    extern __shared__ float4 s_sh[];  // [NF4][kProjectThreads], sh_slot
+    const int64_t g0 = blockIdx.x * int64_t(blockDim.x), g = g0 + threadIdx.x;
     unsigned long long my_total = 0;
     uint32_t my_visible = 0;
     GaussState gs{};
     gs.vis = false;
-    if (g < p.n) {
-        gs = load_gauss(G, g);
-        if (!KEYS_ONLY) stage_sh<T, DEG>(G, g, s_sh);
-    }
+    if (!KEYS_ONLY)
+        stage_sh<T, DEG>(G.sh, g0, int(min(p.n - g0, int64_t(kProjectThreads))), s_sh);
+    if (g < p.n) gs = load_gauss(G, g);
     const uint32_t ntiles = uint32_t(p.ntx * p.nty);
     bool over = false;
     // every warp walks the views in the same order, so the keys in flight
     // go to one or two views' slices, whose open ends stay in L2 (warps
     // that start at different views spread them over every view's slices:
     // 4 % slower at 4K, 4 % at 8K with 100 views)
-    int32_t v = 0;
-    for (int32_t k = 0; k < nv; ++k, v = v + 1 == nv ? 0 : v + 1) {
+    const int32_t ve = view_end(nv);
+    for (int32_t v = view_begin(nv); v < ve; ++v) {
         const Cam cam = load_cam(cams + v);
         uint32_t cnt = 0;
         Splat sp;
@@ -559,13 +628,13 @@ static cudaError_t launch_project_t(const void* const* attrs, const ProjectParam
     G.opacity_logit = static_cast<const T*>(attrs[3]);
     G.sh = static_cast<const T*>(attrs[4]);
     const int block = kProjectThreads;
-    const int64_t grid = (p.n + block - 1) / block;
-    auto smem = [](int deg) { return size_t(16) * kProjectThreads * size_t((3 * (deg + 1) * (deg + 1) + 3) / 4); };
+    const int64_t blocks = (p.n + block - 1) / block;
+    const dim3 grid(unsigned(blocks), unsigned(view_ranges(blocks, nv)));
     switch (p.sh_degree) {
-        case 0: project_kernel<T, 0><<<unsigned(grid), block, smem(0), s>>>(G, p, cams, nv, out); break;
-        case 1: project_kernel<T, 1><<<unsigned(grid), block, smem(1), s>>>(G, p, cams, nv, out); break;
-        case 2: project_kernel<T, 2><<<unsigned(grid), block, smem(2), s>>>(G, p, cams, nv, out); break;
-        default: project_kernel<T, 3><<<unsigned(grid), block, smem(3), s>>>(G, p, cams, nv, out); break;
+        case 0: project_kernel<T, 0><<<grid, block, sh_smem_bytes<0>(), s>>>(G, p, cams, nv, out); break;
+        case 1: project_kernel<T, 1><<<grid, block, sh_smem_bytes<1>(), s>>>(G, p, cams, nv, out); break;
+        case 2: project_kernel<T, 2><<<grid, block, sh_smem_bytes<2>(), s>>>(G, p, cams, nv, out); break;
+        default: project_kernel<T, 3><<<grid, block, sh_smem_bytes<3>(), s>>>(G, p, cams, nv, out); break;
     }
     return cudaGetLastError();
 }
@@ -588,18 +657,18 @@ static cudaError_t launch_project_direct_t(const void* const* attrs, const Proje
     G.opacity_logit = static_cast<const T*>(attrs[3]);
     G.sh = static_cast<const T*>(attrs[4]);
     const int block = kProjectThreads;
-    const int64_t grid = (p.n + block - 1) / block;
-    if (grid <= 0) return cudaSuccess;
-    auto smem = [](int deg) { return size_t(16) * kProjectThreads * size_t((3 * (deg + 1) * (deg + 1) + 3) / 4); };
+    const int64_t blocks = (p.n + block - 1) / block;
+    if (blocks <= 0) return cudaSuccess;
+    const dim3 grid(unsigned(blocks), unsigned(view_ranges(blocks, nv)));
     if (keys_only) {  // no colour: the SH degree does not matter
-        project_direct_kernel<T, 0, true><<<unsigned(grid), block, 0, s>>>(G, p, cams, nv, out);
+        project_direct_kernel<T, 0, true><<<grid, block, 0, s>>>(G, p, cams, nv, out);
         return cudaGetLastError();
     }
     switch (p.sh_degree) {
-        case 0: project_direct_kernel<T, 0, false><<<unsigned(grid), block, smem(0), s>>>(G, p, cams, nv, out); break;
-        case 1: project_direct_kernel<T, 1, false><<<unsigned(grid), block, smem(1), s>>>(G, p, cams, nv, out); break;
-        case 2: project_direct_kernel<T, 2, false><<<unsigned(grid), block, smem(2), s>>>(G, p, cams, nv, out); break;
-        default: project_direct_kernel<T, 3, false><<<unsigned(grid), block, smem(3), s>>>(G, p, cams, nv, out); break;
+        case 0: project_direct_kernel<T, 0, false><<<grid, block, sh_smem_bytes<0>(), s>>>(G, p, cams, nv, out); break;
+        case 1: project_direct_kernel<T, 1, false><<<grid, block, sh_smem_bytes<1>(), s>>>(G, p, cams, nv, out); break;
+        case 2: project_direct_kernel<T, 2, false><<<grid, block, sh_smem_bytes<2>(), s>>>(G, p, cams, nv, out); break;
+        default: project_direct_kernel<T, 3, false><<<grid, block, sh_smem_bytes<3>(), s>>>(G, p, cams, nv, out); break;
     }
     return cudaGetLastError();
 }

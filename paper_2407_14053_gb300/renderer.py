@@ -176,8 +176,8 @@ class Renderer:
         """Binned DirectL frames: "projection" (or True) has the projection
         kernel emit the tile keys into slices laid out from the previous
         frame; "two_pass" (or False) uses tile metadata and a separate
-        emission kernel; "auto" (default) picks the projection for scenes of
-        at least 131,072 Gaussians."""
+        emission kernel; "auto" (default) is the library's choice, at present
+        the projection."""
         value = {True: 1, False: 0, "projection": 1, "two_pass": 0, "auto": 2}[where]
         B.dl_set_option(self.ctx, B.DL_OPT_KEY_EMISSION, value)
 
