@@ -508,7 +508,7 @@ dl_status render_raycast(dl_ctx* ctx, Scene& S, Display& D, const double L0_c2w[
     float* dst = nullptr;
     st = out_target(ctx, out, kind, out_bytes, s, &dst);
     if (st) return st;
-    DL_CK(launch_reorder(G->slot_of.as<uint32_t>(), W.raycol.as<float>(), 3 * int64_t(w) * h, dst,
+    DL_CK(launch_reorder(G->slot_of.as<uint32_t>(), W.raycol.as<float>(), w, h, dst,
                          nullptr, s),
           "reorder");
     DL_CK(mark(8), "event");
@@ -805,7 +805,7 @@ dl_status dl_encode_rays(dl_ctx* ctx, int32_t display_id, const float* ray_rgb, 
     auto it = ctx->displays.find(display_id);
     if (it == ctx->displays.end()) return fail(ctx, DL_ERR_NOT_FOUND, "display %d", display_id);
     const Display& D = *it->second;
-    DL_CK(launch_reorder(D.rep.ray_of.as<uint32_t>(), ray_rgb, 3 * int64_t(D.q.w) * D.q.h, out,
+    DL_CK(launch_reorder(D.rep.ray_of.as<uint32_t>(), ray_rgb, D.q.w, D.q.h, out,
                          nullptr, static_cast<cudaStream_t>(stream)),
           "encode rays");
     return DL_OK;
@@ -1413,10 +1413,10 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
         DL_CK(launch_repurposed_interweave(w, h, D.V.as<uint16_t>(), D.rep.src.as<uint32_t>(), Mm, dst, s),
               "repurposed interweave");
     } else if (mode == DL_STANDARD) {
-        DL_CK(launch_interweave(w, h, nv, D.V.as<uint16_t>(), Mm, dst, s), "interweave");
+        DL_CK(launch_interweave(w, h, D.V.as<uint16_t>(), Mm, dst, s), "interweave");
     } else {
         // a dropped frame (status set) leaves the output untouched
-        DL_CK(launch_reorder(G->slot_of.as<uint32_t>(), raycol, 3 * int64_t(w) * h, dst,
+        DL_CK(launch_reorder(G->slot_of.as<uint32_t>(), raycol, w, h, dst,
                              on_device ? d_status : nullptr, s),
               "reorder");
     }
@@ -1434,9 +1434,7 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
         rbk->hint = &hint;
         W.rb_next = (W.rb_next + 1) % kReadbacks;
     }
-    launches += (mode == DL_STANDARD || lowres || sr)
-                    ? 1
-                    : reorder_launches(G->slot_of.as<uint32_t>(), 3 * int64_t(w) * h, dst);
+    launches += 1;
     DL_CK(mark(8), "event");
     st = out_finish(ctx, out, kind, dst, out_bytes, s, cs);
     if (st) return st;

@@ -248,7 +248,7 @@ dl_status enqueue(dl_batch* b, cudaStream_t s) {
         Slot& z = b->slots[size_t(i)];
         if (!z.active) continue;
         DL_CK(launch_reorder(z.G->slot_of.as<uint32_t>(), b->at<float>(z.o_raycol),
-                             3 * int64_t(z.D->q.w) * z.D->q.h, z.out, b->status_d() + i, s),
+                             z.D->q.w, z.D->q.h, z.out, b->status_d() + i, s),
               "reorder");
     }
     DL_CK(cudaMemcpyAsync(b->status_h, b->status_d(), 4 * size_t(n_slots), cudaMemcpyDeviceToHost, s),

@@ -290,10 +290,8 @@ cudaError_t launch_composite_rays(const CompositeParams& p, const int4* work, in
 // with ray_of either the ray ids (colours in ray-id order) or a tile
 // grouping's slot_of (colours in grouped order).
 // Nothing is written when skip (optional, device) holds a nonzero word.
-cudaError_t launch_reorder(const uint32_t* ray_of, const float* raycol, int64_t n_subpixels,
+cudaError_t launch_reorder(const uint32_t* ray_of, const float* raycol, int32_t w, int32_t h,
                            float* out, const uint32_t* skip, cudaStream_t s);
-// kernels launch_reorder launches for these arguments (1 or 2)
-int reorder_launches(const uint32_t* ray_of, int64_t n_subpixels, const float* out);
 // Standard paradigm: every pixel of every view into Mm (nv x h x w x 3).
 cudaError_t launch_composite_full(const CompositeParams& p, int32_t nv, const uint2* ranges,
                                   const uint32_t* vals, const float4* rec, float* Mm,
@@ -403,8 +401,8 @@ cudaError_t launch_resize_interweave(int32_t w, int32_t h, int32_t rw, int32_t r
 // "HR w SR": out[i] = channel k of view V[i] at the repurposed source pixel src[i].
 cudaError_t launch_repurposed_interweave(int32_t w, int32_t h, const uint16_t* V, const uint32_t* src,
                                         const float* Mm, float* out, cudaStream_t s);
-cudaError_t launch_interweave(int32_t w, int32_t h, int32_t nv, const uint16_t* V, const float* Mm,
-                              float* out, cudaStream_t s);
+cudaError_t launch_interweave(int32_t w, int32_t h, const uint16_t* V, const float* Mm, float* out,
+                              cudaStream_t s);
 
 int num_sms();
 
