@@ -344,6 +344,33 @@ __device__ __forceinline__ float rc_alpha(const float4* __restrict__ gauss, int6
     return fminf(0.99f, a.w * __expf(-0.5f * q));
 }
 
+// SH colour of a Gaussian (coefficient index outer, RGB inner) in the
+// direction whose basis values are Y.  Every lane of a warp reads another
+// Gaussian, so a load touches a line per lane whatever its width: the
+// coefficients are read in pieces of 16 bytes where their size allows (the
+// array is 256-byte aligned), the last ones one by one.
+template <typename T, int DEG>
+__device__ __forceinline__ void sh_colour(const T* __restrict__ sh, const float* Y, float* col) {
+    constexpr int NF = 3 * (DEG + 1) * (DEG + 1), VE = 16 / int(sizeof(T));
+    constexpr int NV = NF % VE == 0 ? NF / VE : 0;  // pieces (degrees 1 and 3; FP32 and, for 3, 16-bit)
+    float acc[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+    for (int p = 0; p < NV; ++p) {
+        const uint4 raw = __ldg(reinterpret_cast<const uint4*>(sh) + p);
+        T v[VE];
+        memcpy(v, &raw, 16);
+#pragma unroll
+        for (int k = 0; k < VE; ++k) {
+            const int f = p * VE + k;
+            acc[f % 3] = fmaf(Y[f / 3], to_f(v[k]), acc[f % 3]);
+        }
+    }
+#pragma unroll
+    for (int f = NV * VE; f < NF; ++f) acc[f % 3] = fmaf(Y[f / 3], to_f(sh[f]), acc[f % 3]);
+#pragma unroll
+    for (int ch = 0; ch < 3; ++ch) col[ch] = fmaxf(acc[ch] + 0.5f, 0.f);
+}
+
 constexpr int kTraceThreads = 128;
 constexpr int kTraceWarps = kTraceThreads / 32;
 constexpr int kListHead = 16;  // list slots 0..15 (the 16 nearest) in shared memory
@@ -563,13 +590,7 @@ rc_trace_kernel(const float4* __restrict__ gauss, const RayNode* __restrict__ no
             const float tn = tr * (1.f - a);
             if (tn < 1e-4f) break;
             float col[3];
-#pragma unroll
-            for (int ch = 0; ch < 3; ++ch) {
-                float acc = 0.f;
-#pragma unroll
-                for (int j = 0; j < NC; ++j) acc = fmaf(Y[j], to_f(sh[(g * NC + j) * 3 + ch]), acc);
-                col[ch] = fmaxf(acc + 0.5f, 0.f);
-            }
+            sh_colour<T, DEG>(sh + g * (3 * NC), Y, col);
             const float w = a * tr;
             c0 = fmaf(w, col[0], c0);
             c1 = fmaf(w, col[1], c1);
