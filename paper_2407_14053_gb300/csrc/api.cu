@@ -417,6 +417,24 @@ dl_status harvest_readbacks(dl_ctx* ctx, bool wait) {
     return DL_OK;
 }
 
+// Copies a frame's counter block to the next pinned slot of the ring (a slot
+// still in use is waited for and read first).
+static dl_status enqueue_readback(dl_ctx* ctx, FrameHint& hint, int64_t frame, cudaStream_t s) {
+    Workspace& W = ctx->ws;
+    Readback& r = W.rb[W.rb_next];
+    if (r.busy) {
+        DL_CK(cudaEventSynchronize(r.done), "wait for frame counters");
+        apply_readback(ctx, r);
+    }
+    DL_CK(cudaMemcpyAsync(r.h, W.small.p, 256, cudaMemcpyDeviceToHost, s), "copy counters");
+    DL_CK(cudaEventRecord(r.done, s), "event");
+    r.busy = true;
+    r.frame = frame;
+    r.hint = &hint;
+    W.rb_next = (W.rb_next + 1) % kReadbacks;
+    return DL_OK;
+}
+
 // Where a frame's last kernel writes it, by output kind: the caller's device
 // buffer; the workspace frame, copied to the host on `s` (the call waits for
 // it); or one of two device frames used in turn, copied to the host on the
@@ -472,11 +490,103 @@ dl_status out_finish(dl_ctx* ctx, float* out, int32_t kind, const float* dst, si
     return DL_OK;
 }
 
+// The tile lists of a DL_RAYCAST frame: per (view, Gaussian) the outline of its
+// alpha >= 1/255 ellipsoid, and a key in every tile that it reaches, emitted
+// into slices laid out from the signature's previous frame (and again, on the
+// device, into slices of the frame's own counts when one is outgrown).  The
+// first frame of a signature starts from empty slices and reads its key total
+// back once to size the key buffer.  *over (device) is set when the keys do
+// not fit after all; *ready is false, and nothing is left to use, when the
+// signature's lists cannot be held (memory, or 2^31 entries).
+dl_status build_cast_lists(dl_ctx* ctx, Scene& S, Display& D, TileGroups& G, FrameHint& hint,
+                           int64_t chunk, cudaStream_t s, GroupSlices* sl, uint32_t** over,
+                           int32_t* launches, bool* ready) {
+    Workspace& W = ctx->ws;
+    *ready = false;
+    const int32_t nv = D.q.nv;
+    const ProjectParams pp = make_project_params(S, D, G.tw, G.th);
+    const int64_t ne = int64_t(nv) * S.n, ngroups = int64_t(nv) * G.ntiles;
+    if (hint.no_lists || ne >= (int64_t(1) << 31) || ngroups >= (int64_t(1) << 31) - 1) return DL_OK;
+    const size_t words = 4 * size_t(ngroups + 1);
+    // memory that the tree would not need: without it the tree renders
+    auto reserve = [&](DevBuf& b, size_t bytes) {
+        const size_t had = b.bytes;
+        if (b.reserve(bytes) == cudaSuccess) return true;
+        // the buffer was given up for the larger one: other signatures' sizing
+        // counts on it
+        if (had == 0 || b.reserve(had - had / 8) != cudaSuccess)
+            for (auto& h : ctx->hints) h.second.sized = false;
+        return false;
+    };
+    const bool sizing = !hint.sized || !hint.slices_ready;
+    if (!reserve(W.rec, 16 * kRecordFloat4 * size_t(ne)) || !reserve(W.gcount, words) ||
+        !reserve(W.gfill, words) || !reserve(W.gscan_tmp, scan_tmp_bytes(ngroups + 1)) ||
+        !reserve(hint.slices[0], words) || !reserve(hint.slices[1], words) ||
+        !reserve(W.cast, cast_tmp_bytes(chunk, ctx->heap_cap))) {
+        hint.no_lists = true;
+        return DL_OK;
+    }
+    unsigned long long* d_total64 = W.small.as<unsigned long long>();
+    uint32_t* d_total32 = reinterpret_cast<uint32_t*>(W.small.as<char>() + 64);
+    uint32_t* d_redo = d_total32 + 1;
+    *over = reinterpret_cast<uint32_t*>(W.small.as<char>() + 160);
+    uint32_t* const slice = hint.slices[hint.cur].as<uint32_t>();
+    uint32_t* const next = hint.slices[hint.cur ^ 1].as<uint32_t>();
+    uint32_t* const cursor = W.gfill.as<uint32_t>();
+    if (sizing) DL_CK(cudaMemsetAsync(slice, 0, words, s), "empty slices");
+    DL_CK(cudaMemcpyAsync(cursor, slice, 4 * size_t(ngroups), cudaMemcpyDeviceToDevice, s), "cursors");
+    const void* attrs[5] = {S.mean.p, S.log_scale.p, S.rot.p, S.opacity.p, S.sh.p};
+    ProjectOut po{W.rec.as<float4>(), nullptr, d_total64, nullptr};
+    po.keys = W.keys[0].as<unsigned long long>();
+    po.cursor = cursor;
+    po.slice = slice;
+    po.key_cap =
+        sizing ? 0u : uint32_t(std::min<size_t>(W.keys[0].bytes / 8, size_t((1u << 31) - 2)));
+    po.overflow = d_redo;
+    DL_CK(launch_project_outline(S.dtype, attrs, pp, W.cams.as<Cam>(), nv, po, false, s), "outlines");
+    DL_CK(launch_pad_counts(cursor, slice, ngroups, W.gcount.as<uint32_t>(), s), "pad counts");
+    DL_CK(launch_exclusive_scan(W.gcount.as<uint32_t>(), next, ngroups + 1, d_total32, W.gscan_tmp.p, s),
+          "slice scan");
+    if (sizing) {
+        DL_CK(cudaMemcpyAsync(W.h_total, d_total64, 8, cudaMemcpyDeviceToHost, s), "copy totals");
+        DL_CK(cudaStreamSynchronize(s), "sync");
+        const unsigned long long nk = W.h_total[0];
+        const int64_t laid = nk < (1ull << 31) ? int64_t(nk + nk / 8) + 16 * ngroups : int64_t(1) << 31;
+        const int64_t want = laid + laid / 4 + 65536;
+        if (want >= (int64_t(1) << 31) - 2 || !reserve(W.keys[0], 8 * size_t(want))) {
+            hint.no_lists = true;
+            return DL_OK;
+        }
+        hint.sized = true;
+        hint.slices_ready = true;
+        hint.key_cap = want;
+        po.keys = W.keys[0].as<unsigned long long>();
+        po.key_cap = uint32_t(std::min<size_t>(W.keys[0].bytes / 8, size_t((1u << 31) - 2)));
+    }
+    DL_CK(launch_reset_cursor(d_redo, next, ngroups, cursor, s), "cursors");
+    po.slice = next;
+    po.gate = d_redo;
+    po.overflow = *over;
+    DL_CK(launch_project_outline(S.dtype, attrs, pp, W.cams.as<Cam>(), nv, po, true, s), "re-emit keys");
+    sl->start = slice;
+    sl->start_alt = next;
+    sl->use_alt = d_redo;
+    sl->cursor = cursor;
+    hint.cur ^= 1;
+    *launches += 7;
+    *ready = true;
+    return DL_OK;
+}
+
 // DL_RAYCAST frame: the DirectL rays cast through the scene (Alg. 3), then
-// the ray colours gathered into the encoded image.  E: stage events (when
-// stage timing is on), the unused stages recorded empty.
-dl_status render_raycast(dl_ctx* ctx, Scene& S, Display& D, const double L0_c2w[16], float* out,
-                         int32_t kind, cudaStream_t s, cudaStream_t cs, StageEvents* E) {
+// the ray colours gathered into the encoded image.  The rays meet the
+// Gaussians of their tile's list; a frame whose lists do not fit walks the
+// scene's tree instead (decided on the device once the signature has been
+// sized).  E: stage events (when stage timing is on), the unused stages
+// recorded empty.
+dl_status render_raycast(dl_ctx* ctx, int32_t scene_id, int32_t display_id, Scene& S, Display& D,
+                         const double L0_c2w[16], float* out, int32_t kind, cudaStream_t s,
+                         cudaStream_t cs, StageEvents* E, int64_t frame) {
     Workspace& W = ctx->ws;
     auto mark = [&](int i) -> cudaError_t { return E ? cudaEventRecord(E->e[i], s) : cudaSuccess; };
     RaySet& R = D.rep;
@@ -494,23 +604,65 @@ dl_status render_raycast(dl_ctx* ctx, Scene& S, Display& D, const double L0_c2w[
     TileGroups* G = nullptr;
     st = get_groups(ctx, D, R, ctx->tile[DL_DIRECTL][0], ctx->tile[DL_DIRECTL][1], s, &G);
     if (st) return st;
+    DL_CK(W.small.reserve(256), "alloc");
+    DL_CK(cudaMemsetAsync(W.small.p, 0, 256, s), "memset");
+    FrameHint& hint = ctx->hints[FrameSig{scene_id, display_id, DL_RAYCAST, G->tw, G->th, w, h}];
+    GroupSlices sl;
+    uint32_t* over = nullptr;
+    int32_t launches = int32_t((D.q.nv + kCamBatch - 1) / kCamBatch);
+    bool lists = false;
+    // rays a chunk: 2 GB of lists, evenly
+    const int64_t most = std::max<int64_t>((int64_t(1) << 31) / (8 * ctx->heap_cap), 1);
+    const int64_t chunks = (R.n_rays + most - 1) / most;
+    const int64_t chunk = chunks > 0 ? (R.n_rays + chunks - 1) / chunks : 1;
+    st = build_cast_lists(ctx, S, D, *G, hint, chunk, s, &sl, &over, &launches, &lists);
+    if (st) return st;
     for (int i = 1; i <= 6; ++i) DL_CK(mark(i), "event");
     DL_CK(W.raycol.reserve(12 * size_t(R.n_rays > 0 ? R.n_rays : 1)), "alloc ray colours");
     const double pi = 3.14159265358979323846;
     const double focal = 0.5 * w / std::tan(0.5 * D.prm.fov_x_deg * pi / 180.0);
+    if (lists) {
+        CastParams cp{};
+        cp.gauss = S.rc_gauss.as<float4>();
+        cp.rec = W.rec.as<float4>();
+        cp.keys = W.keys[0].as<unsigned long long>();
+        cp.work = G->work.as<int4>();
+        cp.grouped = G->grouped.as<int2>();
+        cp.ray_view = R.ray_view.as<uint32_t>();
+        cp.cams = W.cams.as<Cam>();
+        cp.slices = sl;
+        cp.n = S.n;
+        cp.n_work = G->n_work;
+        cp.chunk = chunk;
+        cp.ntiles = G->ntiles;
+        cp.heap_cap = ctx->heap_cap;
+        cp.focal = float(focal);
+        cp.half_w = 0.5f * float(w);
+        cp.half_h = 0.5f * float(h);
+        cp.skip = over;
+        cp.raycol = W.raycol.as<float>();
+        DL_CK(launch_raycast_lists(S.dtype, S.sh_degree, cp, R.n_rays, W.cast.p, S.sh.p, s),
+              "ray-order rendering (lists)");
+        launches += int32_t(2 * chunks);
+    }
+    // without lists, or (on the device) when their keys did not fit
     DL_CK(launch_raycast(S.dtype, S.sh_degree, S.rc_gauss.as<float4>(), S.rc_nodes.as<RayNode>(),
                          S.n, S.sh.p, R.ray_view.as<uint32_t>(),
                          R.ray_pix.as<uint32_t>(), G->grouped.as<int2>(), R.n_rays, W.cams.as<Cam>(), float(focal),
-                         0.5f * float(w), 0.5f * float(h), ctx->heap_cap, W.raycol.as<float>(), s),
+                         0.5f * float(w), 0.5f * float(h), ctx->heap_cap, W.raycol.as<float>(),
+                         lists ? over : nullptr, s),
           "ray-order rendering");
     DL_CK(mark(7), "event");
     const size_t out_bytes = 12 * size_t(w) * size_t(h);
     float* dst = nullptr;
     st = out_target(ctx, out, kind, out_bytes, s, &dst);
     if (st) return st;
-    DL_CK(launch_reorder(G->slot_of.as<uint32_t>(), W.raycol.as<float>(), w, h, dst,
-                         nullptr, s),
+    DL_CK(launch_reorder(G->slot_of.as<uint32_t>(), W.raycol.as<float>(), w, h, dst, nullptr, s),
           "reorder");
+    if (lists) {
+        st = enqueue_readback(ctx, hint, frame, s);
+        if (st) return st;
+    }
     DL_CK(mark(8), "event");
     st = out_finish(ctx, out, kind, dst, out_bytes, s, cs);
     if (st) return st;
@@ -518,7 +670,7 @@ dl_status render_raycast(dl_ctx* ctx, Scene& S, Display& D, const double L0_c2w[
     fs = dl_frame_stats{};
     W.last_async = -1;
     fs.n_rays = R.n_rays;
-    fs.n_launches = int32_t((D.q.nv + kCamBatch - 1) / kCamBatch) + 2;
+    fs.n_launches = launches + 2;
     if (E) {
         PendingFrame& pf = W.pending.back();
         pf.n_rays = fs.n_rays;
@@ -1025,7 +1177,8 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
         return timing ? cudaEventRecord(E->e[i], s) : cudaSuccess;
     };
     DL_CK(mark(0), "event");
-    if (mode == DL_RAYCAST) return render_raycast(ctx, S, D, L0_c2w, out, kind, s, cs, E);
+    if (mode == DL_RAYCAST)
+        return render_raycast(ctx, scene_id, display_id, S, D, L0_c2w, out, kind, s, cs, E, frame);
     // "HR w SR" renders as DL_STANDARD (views at panel resolution) and
     // gathers each subpixel from its repurposed source pixel at the end
     const bool sr = mode == DL_STANDARD_SR;
@@ -1423,16 +1576,8 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
     Readback* rbk = nullptr;
     if (on_device) {  // the frame's counter block, read when it has arrived
         rbk = &W.rb[W.rb_next];
-        if (rbk->busy) {
-            DL_CK(cudaEventSynchronize(rbk->done), "wait for frame counters");
-            apply_readback(ctx, *rbk);
-        }
-        DL_CK(cudaMemcpyAsync(rbk->h, W.small.p, 256, cudaMemcpyDeviceToHost, s), "copy counters");
-        DL_CK(cudaEventRecord(rbk->done, s), "event");
-        rbk->busy = true;
-        rbk->frame = frame;
-        rbk->hint = &hint;
-        W.rb_next = (W.rb_next + 1) % kReadbacks;
+        st = enqueue_readback(ctx, hint, frame, s);
+        if (st) return st;
     }
     launches += 1;
     DL_CK(mark(8), "event");

@@ -187,6 +187,12 @@ cudaError_t launch_project(int dtype, const void* const* attrs, const ProjectPar
 cudaError_t launch_project_direct(int dtype, const void* const* attrs, const ProjectParams& p,
                                   const Cam* cams, int32_t nv, ProjectOut out, bool keys_only,
                                   cudaStream_t s);
+// The same for the ray-order renderer: per (view, Gaussian) the outline of its
+// alpha >= 1/255 ellipsoid (records as described there) and its tiles' keys,
+// whose upper word is the bits of a lower bound of its hits' camera depth.
+cudaError_t launch_project_outline(int dtype, const void* const* attrs, const ProjectParams& p,
+                                   const Cam* cams, int32_t nv, ProjectOut out, bool keys_only,
+                                   cudaStream_t s);
 // padded[g] = count + count / 8 + 16 with count = cursor[g] - slice[g]
 // (slice == nullptr: count = cursor[g]); padded[n_groups] = 0.
 cudaError_t launch_pad_counts(const uint32_t* cursor, const uint32_t* slice, int64_t n_groups,
@@ -240,6 +246,7 @@ cudaError_t raycast_build_binary(const float4* gbox, int64_t n, void* tmp, int64
 // nodes, *depth the deepest wide level (0: the root alone).
 cudaError_t raycast_collapse(const float4* gbox, int64_t n, void* tmp, int64_t n_bin,
                              RayNode* nodes, int64_t* n_wide, int* depth, cudaStream_t s);
+// gate (optional, device): nothing runs unless it holds a nonzero word.
 // One thread per ray (view ray_view, pixel ray_pix): ray colours into raycol
 // (3 floats per thread, in thread order).  Thread i casts ray order[i].y
 // (order: a permutation of the rays as {pixel, ray id}, e.g. a tile
@@ -249,7 +256,7 @@ cudaError_t launch_raycast(int dtype, int sh_degree, const float4* gauss, const 
                            int64_t n, const void* sh, const uint32_t* ray_view,
                            const uint32_t* ray_pix, const int2* order, int64_t n_rays,
                            const Cam* cams, float focal, float half_w, float half_h, int heap_cap,
-                           float* raycol, cudaStream_t s);
+                           float* raycol, const uint32_t* gate, cudaStream_t s);
 
 // ---- scan / radix sort / ranges (sort.cu) ---------------------------------
 size_t scan_tmp_bytes(int64_t n);
@@ -346,6 +353,38 @@ struct GroupSlices {
     const uint32_t* use_alt = nullptr;
     const uint32_t* cursor = nullptr;
 };
+// Ray-order rendering from tile lists (raycast.cu): a warp per entry of `work`
+// ({group, ray begin, ray end, -}, at most kCastSpill rays each, in ascending
+// ray order) casts its rays through the Gaussians of its group's list
+// (launch_project_outline's keys and records), persistent; then a thread a
+// ray blends what was found; ray colours into raycol in grouped order.  The
+// rays are taken `chunk` at a time, whose lists (heap_cap entries a ray) are in
+// tmp (cast_tmp_bytes).  Nothing runs when *skip holds a nonzero word.
+constexpr int kCastSpill = 128;  // rays that an entry may reach past its chunk
+struct CastParams {
+    const float4* gauss;
+    const float4* rec;
+    const unsigned long long* keys;
+    const int4* work;
+    const int2* grouped;
+    const uint32_t* ray_view;
+    const Cam* cams;
+    GroupSlices slices;
+    int64_t n, n_work, chunk;
+    int32_t ntiles, heap_cap;
+    float focal, half_w, half_h;
+    const uint32_t* skip;
+    float* raycol;
+    // set by the launch
+    int64_t ray0;
+    unsigned long long* hits;
+    int32_t* count;
+    uint32_t* claimed;
+};
+size_t cast_tmp_bytes(int64_t chunk, int heap_cap);
+cudaError_t launch_raycast_lists(int dtype, int sh_degree, const CastParams& p, int64_t n_rays,
+                                 void* tmp, const void* sh, cudaStream_t s);
+
 cudaError_t launch_partition_warp(const int4* gwork, int64_t n_work, const GroupSlices& slices,
                                   uint32_t cap1, uint32_t cap2, int4* items, int4* block_items,
                                   uint32_t* meta, const uint32_t* total_keys, uint32_t key_cap,

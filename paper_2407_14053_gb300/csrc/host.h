@@ -123,6 +123,7 @@ struct FrameHint {
     int32_t block_cap = 2048;
     int64_t key_cap = 0;
     bool slices_ready = false;
+    bool no_lists = false;  // DL_RAYCAST: the tile lists do not fit; walk the tree
     int cur = 0;
     DevBuf slices[2];  // n_groups + 1 slot offsets each
 };
@@ -143,7 +144,7 @@ struct Readback {
 
 struct Workspace {
     DevBuf cams, rec, meta, count, offset, scan_tmp, keys[2], vals[2], ranges, radix_tmp, Mm, out, small,
-        pairs, gcount, gstart, gfill, lists, gscan_tmp, raycol, fdesc;
+        pairs, gcount, gstart, gfill, lists, gscan_tmp, raycol, fdesc, cast;
     unsigned long long* h_total = nullptr;  // pinned, 256 bytes (copy of `small`)
     Readback rb[kReadbacks];
     int rb_next = 0;
@@ -181,7 +182,7 @@ struct Workspace {
         size_t b = cams.bytes + rec.bytes + meta.bytes + count.bytes + offset.bytes + scan_tmp.bytes +
                    ranges.bytes +
                    radix_tmp.bytes + Mm.bytes + out.bytes + small.bytes + gcount.bytes + gstart.bytes +
-                   gfill.bytes + lists.bytes + gscan_tmp.bytes + raycol.bytes;
+                   gfill.bytes + lists.bytes + gscan_tmp.bytes + raycol.bytes + cast.bytes;
         for (int i = 0; i < 2; ++i) b += keys[i].bytes + vals[i].bytes + aout[i].bytes;
         return b;
     }

@@ -595,6 +595,126 @@ project_direct_kernel(GaussiansView<T> G, ProjectParams p, const Cam* __restrict
     }
 }
 
+// The outline of a Gaussian's alpha >= 1/255 ellipsoid in one view, for the
+// ray-order renderer's tile lists (exact for a pinhole camera, where the
+// splat above is its linearisation).  With Q = K Sigma in the camera's axes
+// and m the mean, the rays that meet the ellipsoid fill the ellipse with
+// centre c = (m_xy m_z - Q_xy,z) / D and shape matrix E = (Q_xy + (m_xy m_xy^T
+// Q_zz - m_z (m_xy Q_z,xy^T + Q_xy,z m_xy^T) + Q_xy,z Q_z,xy^T) / D) / D,
+// D = m_z^2 - Q_zz (the dual of its outline conic C* = Q - m m^T), in units of
+// the focal length.  Q is widened by 0.2 % and by 1e-6 of the distance (the
+// rounding of a hit's position), E by half a pixel (squared) and 2e-5 of its
+// trace (its own rounding), so every ray that the exact test finds is inside:
+// q0 = (u, v, A, B), q1 = (C, depth, 0, 0) with A dx^2 + B dx dy + C dy^2 >= -1
+// there; depth bounds the camera depth of every hit from below.  An ellipsoid
+// that reaches the camera's plane has no such outline: it gets the whole view.
+__device__ __forceinline__ bool project_outline(const GaussState& s, const Cam& cam,
+                                                const ProjectParams& p, Splat& o, float4& q0,
+                                                float4& q1) {
+    if (!s.vis) return false;
+    const float tx = cam.r[0] * s.mx + cam.r[1] * s.my + cam.r[2] * s.mz + cam.t[0];
+    const float ty = cam.r[3] * s.mx + cam.r[4] * s.my + cam.r[5] * s.mz + cam.t[1];
+    const float tz = cam.r[6] * s.mx + cam.r[7] * s.my + cam.r[8] * s.mz + cam.t[2];
+    float w[3][3];  // W Sigma
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const float r0 = cam.r[3 * i], r1 = cam.r[3 * i + 1], r2 = cam.r[3 * i + 2];
+        w[i][0] = r0 * s.S00 + r1 * s.S01 + r2 * s.S02;
+        w[i][1] = r0 * s.S01 + r1 * s.S11 + r2 * s.S12;
+        w[i][2] = r0 * s.S02 + r1 * s.S12 + r2 * s.S22;
+    }
+    const float k = 1.002f * s.K, far2 = 5e-10f * (tx * tx + ty * ty + tz * tz);
+    auto q = [&](int i, int j) {
+        return k * (w[i][0] * cam.r[3 * j] + w[i][1] * cam.r[3 * j + 1] + w[i][2] * cam.r[3 * j + 2]);
+    };
+    const float qxx = q(0, 0) + far2, qyy = q(1, 1) + far2, qzz = q(2, 2) + far2;
+    const float qxy = q(0, 1), qxz = q(0, 2), qyz = q(1, 2);
+    const float hz = sqrtf(qzz), near_z = tz - hz;
+    if (!(tz + hz > 0.f)) return false;  // behind the camera
+    o.dk = __float_as_uint(fmaxf(near_z * 0.9999f, 0.f));
+    int ic0 = 0, ic1 = p.width - 1, ir0 = 0, ir1 = p.height - 1;
+    q0 = make_float4(0.f, 0.f, 0.f, 0.f);
+    q1 = make_float4(0.f, fmaxf(near_z * 0.9999f, 0.f), 0.f, 0.f);
+    if (near_z > 0.02f) {
+        const float iD = 1.f / (near_z * (tz + hz));
+        float exx = (qxx + (tx * tx * qzz - 2.f * tx * tz * qxz + qxz * qxz) * iD) * iD;
+        float eyy = (qyy + (ty * ty * qzz - 2.f * ty * tz * qyz + qyz * qyz) * iD) * iD;
+        float exy = (qxy + (tx * ty * qzz - tz * (tx * qyz + ty * qxz) + qxz * qyz) * iD) * iD;
+        const float f2 = p.focal * p.focal, add = 0.5f + 2e-5f * f2 * (exx + eyy);
+        exx = f2 * exx + add;
+        eyy = f2 * eyy + add;
+        exy *= f2;
+        const float det = exx * eyy - exy * exy;
+        const float u = p.focal * (tx * tz - qxz) * iD + cam.shift;
+        const float v = p.focal * (ty * tz - qyz) * iD;
+        const float rx = sqrtf(exx) * 1.0001f + 1e-2f, ry = sqrtf(eyy) * 1.0001f + 1e-2f;
+        if (det > 0.f && det < INFINITY && fabsf(u) < 1e9f && fabsf(v) < 1e9f) {
+            const float c_lo = ceilf(u + p.half_w - rx), c_hi = floorf(u + p.half_w + rx);
+            const float r_lo = ceilf(v + p.half_h - ry), r_hi = floorf(v + p.half_h + ry);
+            if (!(c_hi >= 0.f && r_hi >= 0.f && c_lo <= float(p.width - 1) &&
+                  r_lo <= float(p.height - 1) && c_lo <= c_hi && r_lo <= r_hi))
+                return false;
+            ic0 = int(fmaxf(c_lo, 0.f));
+            ic1 = int(fminf(c_hi, float(p.width - 1)));
+            ir0 = int(fmaxf(r_lo, 0.f));
+            ir1 = int(fminf(r_hi, float(p.height - 1)));
+            const float id = 1.f / det;
+            q0 = make_float4(u, v, -eyy * id, 2.f * exy * id);
+            q1.x = -exx * id;
+        }
+    }
+    o.tx0 = ic0 >> p.tile_sx;
+    o.tx1 = ic1 >> p.tile_sx;
+    o.ty0 = ir0 >> p.tile_sy;
+    o.ty1 = ir1 >> p.tile_sy;
+    o.rect_c = uint32_t(ic0) | (uint32_t(ic1) << 16);
+    o.rect_r = uint32_t(ir0) | (uint32_t(ir1) << 16);
+    return true;
+}
+
+// project_direct_kernel for outlines: records and keys (depth << 32 |
+// Gaussian << 4 | nibble) into the laid-out slices; KEYS_ONLY: the gated pass
+// that emits again.
+template <typename T, bool KEYS_ONLY>
+__global__ void __launch_bounds__(kProjectThreads, 4)
+project_outline_kernel(GaussiansView<T> G, ProjectParams p, const Cam* __restrict__ cams, int32_t nv,
+                       int32_t ranges, ProjectOut out) {
+    if (KEYS_ONLY && *out.gate == 0u) return;
+    const BlockWork bw = block_work<false>(nv, ranges);
+    const int64_t g = bw.gblock * int64_t(kProjectThreads) + threadIdx.x;
+    GaussState gs{};
+    gs.vis = false;
+    if (g < p.n) gs = load_gauss(G, g);
+    const uint32_t ntiles = uint32_t(p.ntx * p.nty);
+    unsigned long long my_total = 0;
+    bool over = false;
+    for (int32_t v = bw.v0; v < bw.v1; ++v) {
+        const Cam cam = load_cam(cams + v);
+        uint32_t cnt = 0;
+        Splat sp;
+        sp.tx0 = sp.ty0 = sp.tx1 = sp.ty1 = 0;
+        sp.rect_c = sp.rect_r = sp.dk = 0u;
+        float4 q0, q1;
+        if (gs.vis && project_outline(gs, cam, p, sp, q0, q1)) {
+            cnt = uint32_t(sp.tx1 - sp.tx0 + 1) * uint32_t(sp.ty1 - sp.ty0 + 1);
+            if (!KEYS_ONLY) {
+                float4* r = out.rec + kRecordFloat4 * (int64_t(v) * p.n + g);
+                r[0] = q0;
+                r[1] = q1;
+            }
+        }
+        my_total += cnt;
+        warp_emit<true>(p, cnt, sp.tx0, sp.ty0, sp.tx1 - sp.tx0 + 1, uint32_t(v) * ntiles, sp.dk,
+                        uint32_t(g) << 4, sp.rect_c, sp.rect_r, out.cursor, out.slice, out.keys,
+                        out.key_cap, over);
+    }
+    if (__any_sync(0xffffffffu, over) && (threadIdx.x & 31) == 0) atomicOr(out.overflow, 1u);
+    if (!KEYS_ONLY) {
+        my_total = warp_sum(my_total);
+        if ((threadIdx.x & 31) == 0 && my_total) atomicAdd(out.total, my_total);
+    }
+}
+
 // Slices for the next layout: group g gets its key count (cursor[g] -
 // slice[g], or cursor[g] alone without a slice array) plus an eighth and
 // 16 slots; entry n_groups is 0, so an exclusive scan of n_groups + 1
@@ -698,6 +818,35 @@ cudaError_t launch_project_direct(int dtype, const void* const* attrs, const Pro
     if (dtype == 1) return launch_project_direct_t<__nv_bfloat16>(attrs, p, cams, nv, out, keys_only, s);
     if (dtype == 2) return launch_project_direct_t<__half>(attrs, p, cams, nv, out, keys_only, s);
     return launch_project_direct_t<float>(attrs, p, cams, nv, out, keys_only, s);
+}
+
+template <typename T>
+static cudaError_t launch_project_outline_t(const void* const* attrs, const ProjectParams& p,
+                                            const Cam* cams, int32_t nv, ProjectOut out,
+                                            bool keys_only, cudaStream_t s) {
+    GaussiansView<T> G;
+    G.mean = static_cast<const float*>(attrs[0]);
+    G.log_scale = static_cast<const T*>(attrs[1]);
+    G.rot = static_cast<const T*>(attrs[2]);
+    G.opacity_logit = static_cast<const T*>(attrs[3]);
+    G.sh = nullptr;
+    const int64_t blocks = (p.n + kProjectThreads - 1) / kProjectThreads;
+    if (blocks <= 0) return cudaSuccess;
+    const int32_t ranges = view_ranges(blocks, nv);
+    const unsigned grid = unsigned(blocks * ranges);
+    if (keys_only)
+        project_outline_kernel<T, true><<<grid, kProjectThreads, 0, s>>>(G, p, cams, nv, ranges, out);
+    else
+        project_outline_kernel<T, false><<<grid, kProjectThreads, 0, s>>>(G, p, cams, nv, ranges, out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_project_outline(int dtype, const void* const* attrs, const ProjectParams& p,
+                                   const Cam* cams, int32_t nv, ProjectOut out, bool keys_only,
+                                   cudaStream_t s) {
+    if (dtype == 1) return launch_project_outline_t<__nv_bfloat16>(attrs, p, cams, nv, out, keys_only, s);
+    if (dtype == 2) return launch_project_outline_t<__half>(attrs, p, cams, nv, out, keys_only, s);
+    return launch_project_outline_t<float>(attrs, p, cams, nv, out, keys_only, s);
 }
 
 cudaError_t launch_pad_counts(const uint32_t* cursor, const uint32_t* slice, int64_t n_groups,

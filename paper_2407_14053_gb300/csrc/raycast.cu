@@ -9,7 +9,13 @@
 // list orders by (t, index), so the image does not depend on the traversal
 // order.
 //
-// Acceleration (Sec. 7: a compact 8-wide bounding-volume hierarchy built with
+// Two ways to the Gaussians a ray meets.  Rays normally go through the list of
+// their (view, tile), which holds every Gaussian whose alpha >= 1/255 outline
+// reaches the tile (rc_cast_kernel).  When the lists of a frame do not fit
+// their memory, the rays walk the scene's tree (rc_trace_kernel).  Both test
+// with rc_alpha and keep the same list, so the image is the same.
+//
+// The tree (Sec. 7: a compact 8-wide bounding-volume hierarchy built with
 // the surface area heuristic): every Gaussian is bounded by the box of its
 // alpha >= 1/255 ellipsoid.  A binary tree is built top down over the
 // scene's stored order (a 3D Morton curve of the means), so every node holds
@@ -27,6 +33,7 @@
 
 #include "dl_internal.cuh"
 #include "sh.cuh"
+#include "warp_sort.cuh"
 
 namespace dl {
 namespace {
@@ -327,10 +334,14 @@ __global__ void leaf_root_kernel(const float4* __restrict__ gbox, uint32_t n, Ra
     wide[0] = nd;
 }
 
-// Highest-density point and alpha of Gaussian g along the ray.
-__device__ __forceinline__ float rc_alpha(const float4* __restrict__ gauss, int64_t g, float ox,
-                                          float oy, float oz, float dx, float dy, float dz, float& t) {
-    const float4 a = gauss[3 * g], b = gauss[3 * g + 1], c = gauss[3 * g + 2];
+// Highest-density point and alpha along the ray of the Gaussian whose three
+// float4 are at pa, pb, pc (global or shared memory).  They are read into
+// locals first: taking them by reference changed the compiler's choice of
+// fused multiply-adds, and a few pixels in a million with it.
+__device__ __forceinline__ float rc_alpha(const float4* pa, const float4* pb, const float4* pc,
+                                          float ox, float oy, float oz, float dx, float dy, float dz,
+                                          float& t) {
+    const float4 a = *pa, b = *pb, c = *pc;
     // S d and d^T S d, S = [[b.x b.y b.z] [b.y b.w c.x] [b.z c.x c.y]]
     const float sx = b.x * dx + b.y * dy + b.z * dz;
     const float sy = b.y * dx + b.w * dy + c.x * dz;
@@ -343,37 +354,51 @@ __device__ __forceinline__ float rc_alpha(const float4* __restrict__ gauss, int6
                     2.f * (b.y * px * py + b.z * px * pz + c.x * py * pz);
     return fminf(0.99f, a.w * __expf(-0.5f * q));
 }
+__device__ __forceinline__ float rc_alpha(const float4* __restrict__ gauss, int64_t g, float ox,
+                                          float oy, float oz, float dx, float dy, float dz, float& t) {
+    return rc_alpha(gauss + 3 * g, gauss + 3 * g + 1, gauss + 3 * g + 2, ox, oy, oz, dx, dy, dz, t);
+}
 
-// SH colour of a Gaussian (coefficient index outer, RGB inner) in the
-// direction whose basis values are Y.  Every lane of a warp reads another
-// Gaussian, so a load touches a line per lane whatever its width: the
-// coefficients are read in pieces of 16 bytes where their size allows (the
-// array is 256-byte aligned), the last ones one by one.
+// Whole 16-byte pieces of a Gaussian's SH coefficients, 0 when their size is no
+// multiple of that (degree 3, and degree 1 in FP32, is).
+template <typename T, int DEG>
+constexpr int sh_pieces() {
+    constexpr int bytes = 3 * (DEG + 1) * (DEG + 1) * int(sizeof(T));
+    return bytes % 16 == 0 ? bytes / 16 : 0;
+}
+
+// Adds the coefficients of piece p to the colour sums acc[0..2], Y being the
+// basis values of the direction (coefficient index outer, RGB inner).
+template <typename T>
+__device__ __forceinline__ void sh_piece(const uint4& raw, int p, const float* Y, float* acc) {
+    constexpr int VE = 16 / int(sizeof(T));
+    T v[VE];
+    memcpy(v, &raw, 16);
+#pragma unroll
+    for (int k = 0; k < VE; ++k) {
+        const int f = p * VE + k;
+        acc[f % 3] = fmaf(Y[f / 3], to_f(v[k]), acc[f % 3]);
+    }
+}
+
+// SH colour of a Gaussian.  Every lane of a warp reads another Gaussian, so a
+// load touches a line per lane whatever its width: the coefficients are read
+// in pieces of 16 bytes where their size allows (the array is 256-byte
+// aligned), else one by one.
 template <typename T, int DEG>
 __device__ __forceinline__ void sh_colour(const T* __restrict__ sh, const float* Y, float* col) {
-    constexpr int NF = 3 * (DEG + 1) * (DEG + 1), VE = 16 / int(sizeof(T));
-    constexpr int NV = NF % VE == 0 ? NF / VE : 0;  // pieces (degrees 1 and 3; FP32 and, for 3, 16-bit)
+    constexpr int NF = 3 * (DEG + 1) * (DEG + 1), NP = sh_pieces<T, DEG>();
     float acc[3] = {0.f, 0.f, 0.f};
 #pragma unroll
-    for (int p = 0; p < NV; ++p) {
-        const uint4 raw = __ldg(reinterpret_cast<const uint4*>(sh) + p);
-        T v[VE];
-        memcpy(v, &raw, 16);
+    for (int p = 0; p < NP; ++p) sh_piece<T>(__ldg(reinterpret_cast<const uint4*>(sh) + p), p, Y, acc);
 #pragma unroll
-        for (int k = 0; k < VE; ++k) {
-            const int f = p * VE + k;
-            acc[f % 3] = fmaf(Y[f / 3], to_f(v[k]), acc[f % 3]);
-        }
-    }
-#pragma unroll
-    for (int f = NV * VE; f < NF; ++f) acc[f % 3] = fmaf(Y[f / 3], to_f(sh[f]), acc[f % 3]);
+    for (int f = NP ? NF : 0; f < NF; ++f) acc[f % 3] = fmaf(Y[f / 3], to_f(sh[f]), acc[f % 3]);
 #pragma unroll
     for (int ch = 0; ch < 3; ++ch) col[ch] = fmaxf(acc[ch] + 0.5f, 0.f);
 }
 
 constexpr int kTraceThreads = 128;
 constexpr int kTraceWarps = kTraceThreads / 32;
-constexpr int kListHead = 16;  // list slots 0..15 (the 16 nearest) in shared memory
 
 // A ray's entry into a box (+inf when it misses the box or the box lies
 // behind the near plane).
@@ -387,11 +412,36 @@ __device__ __forceinline__ float slab_enter(const float4& lo, const float4& hi, 
     return (tn <= tf && tf > kNearT) ? tn : INFINITY;
 }
 
-// A ray's ascending list of its c_h nearest intersections: slots below
-// kListHead in shared memory, the rest in the thread's local memory.
-struct RayList {
-    unsigned long long* head;  // slot k < kListHead at head[32 k]
-    unsigned long long* rest;  // slot k >= kListHead at rest[k - kListHead]
+// A ray: camera centre, unit direction through its pixel (camera ray ((c -
+// w/2 - shift)/f, (r - h/2)/f, 1) to world).
+struct Ray {
+    float ox, oy, oz, dx, dy, dz;
+};
+__device__ __forceinline__ Ray make_ray(const Cam& cam, uint32_t pixel, float focal, float half_w,
+                                        float half_h) {
+    Ray r;
+    const float cx = (float(pixel & 0xFFFFu) - half_w - cam.shift) / focal;
+    const float cy = (float(pixel >> 16) - half_h) / focal;
+    r.dx = cam.r[0] * cx + cam.r[3] * cy + cam.r[6];
+    r.dy = cam.r[1] * cx + cam.r[4] * cy + cam.r[7];
+    r.dz = cam.r[2] * cx + cam.r[5] * cy + cam.r[8];
+    const float dn = rsqrtf(r.dx * r.dx + r.dy * r.dy + r.dz * r.dz);
+    r.dx *= dn; r.dy *= dn; r.dz *= dn;
+    r.ox = cam.c[0];
+    r.oy = cam.c[1];
+    r.oz = cam.c[2];
+    return r;
+}
+
+// A ray's ascending list of its c_h nearest intersections, packed as t's FP32
+// bits << 32 | Gaussian index: t > 0, so the integer order of the packed key
+// is the (t, index) order.  The tree walk keeps slots below kListHead in
+// shared memory (slot k at head[32 k]) and the rest in the thread's local
+// memory; the cast keeps slot k of every ray of a chunk together.
+constexpr int kListHead = 16;
+struct WalkList {
+    unsigned long long* head;
+    unsigned long long* rest;
     __device__ __forceinline__ unsigned long long get(int k) const {
         return k < kListHead ? head[32 * k] : rest[k - kListHead];
     }
@@ -400,6 +450,91 @@ struct RayList {
         else rest[k - kListHead] = v;
     }
 };
+struct CastList {
+    unsigned long long* slot0;
+    int64_t stride;
+    __device__ __forceinline__ unsigned long long get(int k) const { return slot0[k * stride]; }
+    __device__ __forceinline__ void set(int k, unsigned long long v) const { slot0[k * stride] = v; }
+};
+
+// What a ray has found: its list and the transmittance bound.  tb is set once
+// the intersections found so far (every one at t <= tmax) multiply T below
+// 5e-5.  Sorted, they alone take T below 1e-4 by t = tmax, so blending stops
+// at or before tmax and nothing beyond tb can be blended.  (5e-5, not 1e-4:
+// the product is formed in another order than the blend's.)
+// LAST: the list's largest key is kept in a register, so a hit that comes in
+// order is stored without a read (the cast; the tree walk has no register to
+// spare).
+template <class List, bool LAST>
+struct RayHits {
+    List list;
+    int n = 0, cap;
+    float prodT = 1.f, tmax = 0.f, tb = INFINITY;
+    unsigned long long top = 0ull;
+    __device__ __forceinline__ unsigned long long largest() const { return LAST ? top : list.get(n - 1); }
+    // no intersection beyond this is kept
+    __device__ __forceinline__ float bound() const {
+        return fminf(tb, n == cap ? __uint_as_float(uint32_t(largest() >> 32)) : INFINITY);
+    }
+    __device__ __forceinline__ void add(float a, float t, uint32_t g) {
+        if (!(a >= kMinAlpha) || !(t > kNearT) || t > tb) return;
+        if (tb == INFINITY) {
+            prodT *= 1.f - a;
+            tmax = fmaxf(tmax, t);
+            if (prodT < 5e-5f) tb = tmax;
+        }
+        const unsigned long long key = (static_cast<unsigned long long>(__float_as_uint(t)) << 32) | g;
+        if (LAST && key > top) {
+            if (n == cap) return;  // full and farther than all
+            list.set(n++, key);
+            top = key;
+            return;
+        }
+        if (n == cap) {  // full: drop the farthest if this one is nearer
+            if (!LAST && !(key < list.get(n - 1))) return;
+            --n;
+        }
+        // insert into the ascending list: rays find their intersections
+        // nearly in order, so few entries move
+        int k = n++;
+        while (k > 0) {
+            const unsigned long long vp = list.get(k - 1);
+            if (!(key < vp)) break;
+            list.set(k, vp);
+            --k;
+        }
+        list.set(k, key);
+        if (LAST && n == cap) top = list.get(n - 1);
+    }
+};
+
+// Blends a ray's list of n front to back, colour from the SH at the ray direction,
+// into o[0..2].
+template <typename T, int DEG, class List>
+__device__ __forceinline__ void blend_hits(const List& list, int n, const float4* __restrict__ gauss,
+                                           const T* __restrict__ sh, const Ray& r, float* o) {
+    constexpr int NC = (DEG + 1) * (DEG + 1);
+    float Y[16];
+    sh_basis<DEG>(r.dx, r.dy, r.dz, Y);
+    float tr = 1.f, c0 = 0.f, c1 = 0.f, c2 = 0.f;  // transmittance, colour
+    for (int k = 0; k < n; ++k) {
+        float t;
+        const int64_t g = int64_t(uint32_t(list.get(k)));
+        const float a = rc_alpha(gauss, g, r.ox, r.oy, r.oz, r.dx, r.dy, r.dz, t);
+        const float tn = tr * (1.f - a);
+        if (tn < 1e-4f) break;
+        float col[3];
+        sh_colour<T, DEG>(sh + g * (3 * NC), Y, col);
+        const float w = a * tr;
+        c0 = fmaf(w, col[0], c0);
+        c1 = fmaf(w, col[1], c1);
+        c2 = fmaf(w, col[2], c2);
+        tr = tn;
+    }
+    o[0] = c0;
+    o[1] = c1;
+    o[2] = c2;
+}
 
 // Traversal of the 8-wide tree is by the whole warp: its rays share a camera
 // centre and nearly a direction, so they need nearly the same nodes.  A
@@ -419,8 +554,9 @@ rc_trace_kernel(const float4* __restrict__ gauss, const RayNode* __restrict__ no
                 int64_t n, const T* __restrict__ sh, const uint32_t* __restrict__ ray_view,
                 const uint32_t* __restrict__ ray_pix, const int2* __restrict__ order,
                 int64_t n_rays, const Cam* __restrict__ cams, float focal, float half_w,
-                float half_h, int heap_cap, float* __restrict__ raycol) {
-    constexpr int NC = (DEG + 1) * (DEG + 1);
+                float half_h, int heap_cap, float* __restrict__ raycol,
+                const uint32_t* __restrict__ gate) {
+    if (gate && *gate == 0u) return;
     __shared__ uint32_t s_ref[kTraceWarps][kRayStack];
     __shared__ uint32_t s_lanes[kTraceWarps][kRayStack];
     __shared__ unsigned long long s_head[kTraceWarps][kListHead][32];  // [slot][lane]
@@ -431,29 +567,14 @@ rc_trace_kernel(const float4* __restrict__ gauss, const RayNode* __restrict__ no
     // thread i casts ray order[i].y: the rays grouped by (view, tile) and
     // Morton-ordered inside a tile
     const int64_t r = order ? int64_t(order[i].y) : i;
-    const uint32_t px = ray_pix[r];
-    const Cam& cam = cams[ray_view[r]];
-    // direction: camera ray ((c - w/2 - shift)/f, (r - h/2)/f, 1) to world
-    const float cx = (float(px & 0xFFFFu) - half_w - cam.shift) / focal;
-    const float cy = (float(px >> 16) - half_h) / focal;
-    float dx = cam.r[0] * cx + cam.r[3] * cy + cam.r[6];
-    float dy = cam.r[1] * cx + cam.r[4] * cy + cam.r[7];
-    float dz = cam.r[2] * cx + cam.r[5] * cy + cam.r[8];
-    const float dn = rsqrtf(dx * dx + dy * dy + dz * dz);
-    dx *= dn; dy *= dn; dz *= dn;
-    const float ox = cam.c[0], oy = cam.c[1], oz = cam.c[2];
+    const Ray ray = make_ray(cams[ray_view[r]], ray_pix[r], focal, half_w, half_h);
+    const float dx = ray.dx, dy = ray.dy, dz = ray.dz;
+    const float ox = ray.ox, oy = ray.oy, oz = ray.oz;
     const float ix = 1.f / dx, iy = 1.f / dy, iz = 1.f / dz;
-    // list entries packed as t's FP32 bits << 32 | Gaussian index: t > 0, so
-    // the integer order of the packed key is the (t, index) order
     unsigned long long rest[kMaxHeap - kListHead];
-    const RayList hl{&s_head[warp][0][lane], rest};
-    int hn = 0;
-    // Transmittance bound: tb is set once the intersections found so far
-    // (every one at t <= tmax) multiply T below 5e-5.  Sorted, they alone
-    // take T below 1e-4 by t = tmax, so blending stops at or before tmax and
-    // nothing beyond tb can be blended; the walk skips it.  (5e-5, not
-    // 1e-4: the product is formed in another order than the blend's.)
-    float prodT = 1.f, tmax = 0.f, tb = INFINITY;
+    RayHits<WalkList, false> hits;
+    hits.list = {&s_head[warp][0][lane], rest};
+    hits.cap = heap_cap;
     uint32_t* const st_ref = s_ref[warp];
     uint32_t* const st_lanes = s_lanes[warp];
     const unsigned all = __ballot_sync(0xffffffffu, valid);
@@ -468,8 +589,7 @@ rc_trace_kernel(const float4* __restrict__ gauss, const RayNode* __restrict__ no
         const uint32_t e = st_ref[sp];
         const bool mine = (st_lanes[sp] >> lane) & 1u;
         __syncwarp();
-        const float bound = fminf(
-            tb, hn == heap_cap ? __uint_as_float(uint32_t(hl.get(hn - 1) >> 32)) : INFINITY);
+        const float bound = hits.bound();
         if (e & kRayLeafBit) {  // leaf: Gaussians first .. first + count - 1
             if (mine) {
                 const uint32_t first = (e & ~kRayLeafBit) >> 3, cnt = (e & 7u) + 1u;
@@ -487,30 +607,7 @@ rc_trace_kernel(const float4* __restrict__ gauss, const RayNode* __restrict__ no
 #pragma unroll
                     for (int q = 0; q < kLeafMax; ++q) {
                         if (base + q >= cnt) break;
-                        const uint32_t g = first + base + q;
-                        const float a = al[q], t = tl[q];
-                        if (!(a >= kMinAlpha) || !(t > kNearT) || t > tb) continue;
-                        if (tb == INFINITY) {
-                            prodT *= 1.f - a;
-                            tmax = fmaxf(tmax, t);
-                            if (prodT < 5e-5f) tb = tmax;
-                        }
-                        const unsigned long long key =
-                            (static_cast<unsigned long long>(__float_as_uint(t)) << 32) | g;
-                        if (hn == heap_cap) {  // full: drop the farthest if this one is nearer
-                            if (!(key < hl.get(hn - 1))) continue;
-                            --hn;
-                        }
-                        // insert into the ascending list: rays find their
-                        // intersections nearly in order, so few entries move
-                        int k = hn++;
-                        while (k > 0) {
-                            const unsigned long long vp = hl.get(k - 1);
-                            if (!(key < vp)) break;
-                            hl.set(k, vp);
-                            --k;
-                        }
-                        hl.set(k, key);
+                        hits.add(al[q], tl[q], first + base + q);
                     }
                 }
             }
@@ -578,30 +675,218 @@ rc_trace_kernel(const float4* __restrict__ gauss, const RayNode* __restrict__ no
             __syncwarp();
         }
     }
-    if (valid) {
-        // blend front to back, colour from the SH at the ray direction
-        float Y[16];
-        sh_basis<DEG>(dx, dy, dz, Y);
-        float tr = 1.f, c0 = 0.f, c1 = 0.f, c2 = 0.f;  // transmittance, colour
-        for (int k = 0; k < hn; ++k) {
-            float t;
-            const int64_t g = int64_t(uint32_t(hl.get(k)));
-            const float a = rc_alpha(gauss, g, ox, oy, oz, dx, dy, dz, t);
-            const float tn = tr * (1.f - a);
-            if (tn < 1e-4f) break;
-            float col[3];
-            sh_colour<T, DEG>(sh + g * (3 * NC), Y, col);
-            const float w = a * tr;
-            c0 = fmaf(w, col[0], c0);
-            c1 = fmaf(w, col[1], c1);
-            c2 = fmaf(w, col[2], c2);
-            tr = tn;
-        }
-        // colours in thread order: the grouped order when `order` is given
-        raycol[3 * i] = c0;
-        raycol[3 * i + 1] = c1;
-        raycol[3 * i + 2] = c2;
+    // colours in thread order: the grouped order when `order` is given
+    if (valid) blend_hits<T, DEG>(hits.list, hits.n, gauss, sh, ray, raycol + 3 * i);
+}
+
+// ---- rays cast through tile lists ------------------------------------------
+// The rays of a (view, tile) group against the Gaussians whose alpha >= 1/255
+// outline reaches the tile (launch_project_outline), which is the set the
+// tree's walk would find, without the walk.  A warp owns a group: it sorts
+// the list by the hits' least depth, up to kCastCap keys at a time, streams
+// the records 32 at a time (cp.async, one batch ahead), tests each record's
+// outline against all of the warp's rays (a lane a record, as in the
+// compositing kernels: packed FMAs and ballots), and each lane takes its own
+// candidates through the exact rc_alpha into its list.  In depth order a ray
+// finds its hits nearly sorted, and a list ends for the warp once every ray's
+// bound lies before the next record's least depth.  The lists only say which
+// Gaussians are tested and in which order, so the image is the tree walk's bit
+// for bit.
+//
+// Bound by the latency of the candidates' evaluation and insertion at half the
+// lanes (rays have different numbers of candidates in a batch).  1080p frame,
+// 200k Gaussians, c_h 128: 4.38 ms, of which outlines and keys 0.28, cast 2.5,
+// blend 1.6; the tree walk takes 10.0 ms.
+constexpr int kCastCap = 512;
+constexpr int kCastWarps = 4;
+constexpr int kCastBlocks = 4;  // resident blocks an SM
+constexpr int kCastSlots = 2;  // record batches: one evaluated, the next in flight
+
+__device__ __forceinline__ void cast_copy16(void* smem, const void* gmem) {
+    const unsigned s = static_cast<unsigned>(__cvta_generic_to_shared(smem));
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gmem) : "memory");
+}
+
+union CastSmem {
+    WarpSort<kCastCap> s;
+    struct {
+        uint32_t idx[kCastCap];
+        float4 rec[kCastSlots][2][32];    // outlines
+        float4 gauss[kCastSlots][3][32];  // rc_prepare_kernel's data
+        float4 rx[8], ry[8];              // the rays' pixels about their box centre
+        uint4 mask[8];                    // per ray, its candidates in the batch
+    } c;
+};
+
+// First entry of work ({group, ray begin, ray end, -}, ascending rays) whose
+// rays begin at or after ray r.
+__device__ __forceinline__ int64_t first_work(const int4* __restrict__ work, int64_t n, int64_t r) {
+    int64_t lo = 0, hi = n;
+    while (lo < hi) {
+        const int64_t mid = (lo + hi) >> 1;
+        if (int64_t(__ldg(&work[mid].y)) < r) lo = mid + 1;
+        else hi = mid;
     }
+    return lo;
+}
+
+__global__ void __launch_bounds__(kCastWarps * 32, 5) rc_cast_kernel(CastParams P) {
+    if (P.skip && *P.skip) return;
+    extern __shared__ __align__(16) unsigned char cast_smem[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    CastSmem& W = reinterpret_cast<CastSmem*>(cast_smem)[warp];
+    const uint32_t* __restrict__ first =
+        P.slices.use_alt && *P.slices.use_alt ? P.slices.start_alt : P.slices.start;
+    const int64_t n_warps = int64_t(gridDim.x) * kCastWarps;
+    const int64_t w_end = first_work(P.work, P.n_work, P.ray0 + P.chunk);
+    int64_t item = first_work(P.work, P.n_work, P.ray0) + int64_t(blockIdx.x) * kCastWarps + warp;
+    const int64_t claim0 = item - (int64_t(blockIdx.x) * kCastWarps + warp) + n_warps;
+    while (item < w_end) {
+        uint32_t claim = 0;
+        if (lane == 0) claim = atomicAdd(P.claimed, 1u) + 1u;  // from -1 on
+        const int4 wi = __ldg(P.work + item);
+        const uint32_t start = first[wi.x], end = P.slices.cursor[wi.x];
+        const int view = wi.x / P.ntiles;
+        const Cam& cam = P.cams[view];
+        const int64_t vbase = int64_t(view) * P.n;
+        for (int r0 = wi.y; r0 < wi.z; r0 += 32) {
+            const int rid = r0 + lane;
+            const bool active = rid < wi.z;
+            const uint32_t pixel = uint32_t(P.grouped[active ? rid : wi.z - 1].x);
+            const Ray ray = make_ray(cam, pixel, P.focal, P.half_w, P.half_h);
+            const int col = int(pixel & 0xFFFFu), row = int(pixel >> 16);
+            const float ox = 0.5f * float(__reduce_min_sync(0xffffffffu, col) +
+                                          __reduce_max_sync(0xffffffffu, col));
+            const float oy = 0.5f * float(__reduce_min_sync(0xffffffffu, row) +
+                                          __reduce_max_sync(0xffffffffu, row));
+            // lanes past the group's rays add nothing (their rays are not open)
+            RayHits<CastList, true> hits;
+            hits.list = {P.hits + (rid - P.ray0), P.chunk + kCastSpill};
+            hits.cap = P.heap_cap;
+            for (uint32_t c0 = start; c0 < end; c0 += kCastCap) {
+                const int len = int(min(end - c0, uint32_t(kCastCap)));
+                warp_sort<kCastCap>(P.keys, c0, len, W.s);
+                for (int base = 0; base < len; base += 32) {  // low words in place of the keys
+                    const int i = base + lane;
+                    const uint32_t lo = i < len ? uint32_t(W.s.sk[i]) >> 4 : 0u;
+                    __syncwarp();
+                    if (i < len) W.c.idx[i] = lo;
+                    __syncwarp();
+                }
+                reinterpret_cast<float*>(W.c.rx)[lane] = active ? float(col) - ox : 1e18f;
+                reinterpret_cast<float*>(W.c.ry)[lane] = active ? float(row) - oy : 1e18f;
+                const int nbatch = (len + 31) / 32;
+                auto issue = [&](int b) {
+                    const int i = b * 32 + lane, slot = b % kCastSlots;
+                    if (i < len) {
+                        const int64_t g = W.c.idx[i];
+                        const float4* r = P.rec + kRecordFloat4 * (vbase + g);
+                        cast_copy16(&W.c.rec[slot][0][lane], r);
+                        cast_copy16(&W.c.rec[slot][1][lane], r + 1);
+#pragma unroll
+                        for (int k = 0; k < 3; ++k)
+                            cast_copy16(&W.c.gauss[slot][k][lane], P.gauss + 3 * g + k);
+                    }
+                    asm volatile("cp.async.commit_group;\n" ::: "memory");
+                };
+                issue(0);
+                for (int b = 0; b < nbatch; ++b) {
+                    issue(b + 1);  // an empty group past the end
+                    asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+                    __syncwarp();
+                    const int slot = b % kCastSlots, n = min(32, len - b * 32);
+                    // the batch's least depth against what the rays still keep
+                    const bool open = active && !(hits.bound() < W.c.rec[slot][1][0].y);
+                    const unsigned act = __ballot_sync(0xffffffffu, open);
+                    if (act == 0u) break;
+                    float A = 0.f, B = 0.f, C = 0.f, D = 0.f, E = 0.f, F = -1e30f;
+                    if (lane < n) {
+                        // 1 + the outline's quadratic, expanded about (ox, oy),
+                        // and a margin of 0.02 for its rounding: a ray inside is
+                        // at most sqrt(e) + 45 pixels from the centre, e the
+                        // largest of E, and the terms at most that squared over
+                        // E's floor 0.5 + 2e-5 e, i.e. below 5e4
+                        const float4 q0 = W.c.rec[slot][0][lane];
+                        const float du = q0.x - (ox - P.half_w), dv = q0.y - (oy - P.half_h);
+                        A = q0.z;
+                        B = q0.w;
+                        C = W.c.rec[slot][1][lane].x;
+                        D = -fmaf(2.f * A, du, B * dv);
+                        E = -fmaf(2.f * C, dv, B * du);
+                        F = fmaf(du, fmaf(A, du, B * dv), C * dv * dv) + 1.02f;
+                    }
+                    const float2 A2 = make_float2(A, A), B2 = make_float2(B, B), C2 = make_float2(C, C);
+                    const float2 D2 = make_float2(D, D), E2 = make_float2(E, E), F2 = make_float2(F, F);
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) {
+                        if (!((act >> (4 * q)) & 0xFu)) continue;
+                        const float4 qx = W.c.rx[q], qy = W.c.ry[q];
+                        unsigned m[4];
+#pragma unroll
+                        for (int k = 0; k < 2; ++k) {
+                            const float2 x = k ? make_float2(qx.z, qx.w) : make_float2(qx.x, qx.y);
+                            const float2 y = k ? make_float2(qy.z, qy.w) : make_float2(qy.x, qy.y);
+                            const float2 t1 = __ffma2_rn(A2, x, __ffma2_rn(B2, y, D2));
+                            const float2 v =
+                                __ffma2_rn(x, t1, __ffma2_rn(y, __ffma2_rn(C2, y, E2), F2));
+                            m[2 * k] = __ballot_sync(0xffffffffu, v.x >= 0.f);
+                            m[2 * k + 1] = __ballot_sync(0xffffffffu, v.y >= 0.f);
+                        }
+                        if (lane == 0) W.c.mask[q] = make_uint4(m[0], m[1], m[2], m[3]);
+                    }
+                    __syncwarp();
+                    unsigned mine = open ? reinterpret_cast<const unsigned*>(W.c.mask)[lane] : 0u;
+                    while (mine) {
+                        // two candidates evaluated together, taken in order
+                        const int s1 = __ffs(mine) - 1;
+                        mine &= mine - 1u;
+                        const bool two = mine != 0u;
+                        const int s2 = two ? __ffs(mine) - 1 : s1;
+                        mine &= mine - 1u;
+                        float t1, t2;
+                        const float a1 = rc_alpha(&W.c.gauss[slot][0][s1], &W.c.gauss[slot][1][s1],
+                                                  &W.c.gauss[slot][2][s1], ray.ox, ray.oy, ray.oz,
+                                                  ray.dx, ray.dy, ray.dz, t1);
+                        const float a2 = rc_alpha(&W.c.gauss[slot][0][s2], &W.c.gauss[slot][1][s2],
+                                                  &W.c.gauss[slot][2][s2], ray.ox, ray.oy, ray.oz,
+                                                  ray.dx, ray.dy, ray.dz, t2);
+                        hits.add(a1, t1, W.c.idx[b * 32 + s1]);
+                        if (two) hits.add(a2, t2, W.c.idx[b * 32 + s2]);
+                    }
+                    __syncwarp();  // the slot and the masks are written again
+                }
+                asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+                __syncwarp();  // the next chunk's keys take the space
+            }
+            if (active) P.count[rid - P.ray0] = hits.n;
+        }
+        item = claim0 + int64_t(__shfl_sync(0xffffffffu, claim, 0));
+    }
+}
+
+constexpr int kBlendThreads = 256;
+
+// Blends the lists that rc_cast_kernel found for a chunk's rays (count >= 0: a
+// ray of this chunk), a thread a ray.  A kernel of its own: what it needs is
+// the first-level cache (neighbouring rays, and the views of a tile, blend
+// nearly the same Gaussians) and many warps in flight, where the cast needs
+// shared memory.  Bound by the lines its gathers look up in that cache (15
+// loads of up to 32 lines a step); at the end of the cast's own loop, with
+// little of it left, the blending took 3.4 of 5.7 ms at 1080p.  Copying the
+// step's Gaussians to shared memory row by row instead was no faster there
+// (5.2 ms: it gave up the cache altogether).
+template <typename T, int DEG>
+__global__ void __launch_bounds__(kBlendThreads) rc_blend_kernel(CastParams P, const T* __restrict__ sh) {
+    if (P.skip && *P.skip) return;
+    const int64_t j = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+    if (j >= P.chunk + kCastSpill) return;
+    const int n = P.count[j];
+    if (n < 0) return;
+    const int64_t i = P.ray0 + j;
+    const int2 order = P.grouped[i];
+    const Ray ray = make_ray(P.cams[P.ray_view[order.y]], uint32_t(order.x), P.focal, P.half_w, P.half_h);
+    blend_hits<T, DEG>(CastList{P.hits + j, P.chunk + kCastSpill}, n, P.gauss, sh, ray,
+                       P.raycol + 3 * i);
 }
 
 int grid_of(int64_t n, int block) {
@@ -734,13 +1019,13 @@ cudaError_t launch_raycast(int dtype, int sh_degree, const float4* gauss, const 
                            int64_t n, const void* sh, const uint32_t* ray_view,
                            const uint32_t* ray_pix, const int2* order, int64_t n_rays,
                            const Cam* cams, float focal, float half_w, float half_h, int heap_cap,
-                           float* raycol, cudaStream_t s) {
+                           float* raycol, const uint32_t* gate, cudaStream_t s) {
     if (n_rays <= 0) return cudaSuccess;
     const unsigned grid = unsigned((n_rays + kTraceThreads - 1) / kTraceThreads);
 #define DL_RC(T, D)                                                                          \
     rc_trace_kernel<T, D><<<grid, kTraceThreads, 0, s>>>(gauss, nodes, n, static_cast<const T*>(sh),   \
                                                ray_view, ray_pix, order, n_rays, cams, focal,  \
-                                               half_w, half_h, heap_cap, raycol)
+                                               half_w, half_h, heap_cap, raycol, gate)
 #define DL_RC_DEG(T)                  \
     switch (sh_degree) {              \
         case 0: DL_RC(T, 0); break;   \
@@ -755,9 +1040,64 @@ cudaError_t launch_raycast(int dtype, int sh_degree, const float4* gauss, const 
     } else {
         DL_RC_DEG(float)
     }
-#undef DL_RC_DEG
 #undef DL_RC
     return cudaGetLastError();
+}
+
+size_t cast_tmp_bytes(int64_t chunk, int heap_cap) {
+    const size_t rays = size_t(chunk + kCastSpill);
+    return 8 * rays * size_t(heap_cap) + 4 * rays + 256;
+}
+
+namespace {
+template <typename T, int DEG>
+cudaError_t launch_cast(CastParams p, int64_t n_rays, void* tmp, const void* sh, cudaStream_t s) {
+    const size_t smem = kCastWarps * sizeof(CastSmem);
+    cudaError_t e = cudaFuncSetAttribute(rc_cast_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         int(smem));
+    if (e != cudaSuccess) return e;
+    int per_sm = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rc_cast_kernel, kCastWarps * 32, smem);
+    if (e != cudaSuccess) return e;
+    // kCastBlocks an SM (fewer than fit): the rays' lists and the keys need the
+    // rest as first-level cache (six blocks 4.43, five 4.42, four 4.30 ms)
+    if (per_sm > kCastBlocks) per_sm = kCastBlocks;
+    e = cudaFuncSetAttribute(rc_cast_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                             int(100 * kCastBlocks * (smem + 1024) / (228 * 1024)) + 1);
+    if (e != cudaSuccess) return e;
+    const int64_t need = (p.n_work + kCastWarps - 1) / kCastWarps;
+    const int64_t fit = int64_t(num_sms()) * (per_sm > 0 ? per_sm : 1);
+    const int64_t rays = p.chunk + kCastSpill;
+    p.hits = static_cast<unsigned long long*>(tmp);
+    p.count = reinterpret_cast<int32_t*>(p.hits + rays * p.heap_cap);
+    p.claimed = reinterpret_cast<uint32_t*>(p.count + rays);
+    for (p.ray0 = 0; p.ray0 < n_rays; p.ray0 += p.chunk) {
+        // counts and the claim counter start at -1
+        e = cudaMemsetAsync(p.count, 0xFF, 4 * size_t(rays + 1), s);
+        if (e != cudaSuccess) return e;
+        rc_cast_kernel<<<unsigned(need < fit ? need : fit), kCastWarps * 32, smem, s>>>(p);
+        rc_blend_kernel<T, DEG><<<unsigned((rays + kBlendThreads - 1) / kBlendThreads), kBlendThreads, 0, s>>>(p, static_cast<const T*>(sh));
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+}  // namespace
+
+cudaError_t launch_raycast_lists(int dtype, int sh_degree, const CastParams& p, int64_t n_rays,
+                                 void* tmp, const void* sh, cudaStream_t s) {
+    if (p.n_work <= 0 || n_rays <= 0) return cudaSuccess;
+#define DL_RC(T, D) return launch_cast<T, D>(p, n_rays, tmp, sh, s)
+    if (dtype == 1) {
+        DL_RC_DEG(__nv_bfloat16)
+    } else if (dtype == 2) {
+        DL_RC_DEG(__half)
+    } else {
+        DL_RC_DEG(float)
+    }
+#undef DL_RC
+#undef DL_RC_DEG
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace dl
