@@ -270,14 +270,22 @@ bool make_cams(const dl_display_params& p, const double L0[16], std::vector<Cam>
     return true;
 }
 
-dl_status upload_cams(dl_ctx* ctx, const std::vector<Cam>& cams, cudaStream_t s) {
-    DL_CK(ctx->ws.cams.reserve(sizeof(Cam) * cams.size()), "alloc cams");
-    Cam* dst = ctx->ws.cams.as<Cam>();
+// Starts a frame on the device: cameras, the 256-byte counter block at zero
+// and, with a layout, the groups' cursors; one launch for up to kCamBatch views.
+dl_status begin_frame(dl_ctx* ctx, const std::vector<Cam>& cams, const uint32_t* layout,
+                      int64_t n_groups, uint32_t* cursor, cudaStream_t s, int32_t* launches) {
+    Workspace& W = ctx->ws;
+    DL_CK(W.cams.reserve(sizeof(Cam) * cams.size()), "alloc cams");
+    DL_CK(W.small.reserve(256), "alloc");
+    Cam* dst = W.cams.as<Cam>();
     for (size_t v0 = 0; v0 < cams.size(); v0 += kCamBatch) {
         CamBatch b;
         const int32_t n = int32_t(std::min<size_t>(kCamBatch, cams.size() - v0));
         std::memcpy(b.cam, cams.data() + v0, sizeof(Cam) * size_t(n));
-        DL_CK(launch_store_cams(b, n, dst + v0, s), "store cams");
+        DL_CK(launch_begin_frame(b, n, dst + v0, W.small.as<uint32_t>(), v0 == 0 ? 64 : 0,
+                                 v0 == 0 ? layout : nullptr, n_groups, cursor, s),
+              "begin frame");
+        ++*launches;
     }
     return DL_OK;
 }
@@ -499,8 +507,8 @@ dl_status out_finish(dl_ctx* ctx, float* out, int32_t kind, const float* dst, si
 // not fit after all; *ready is false, and nothing is left to use, when the
 // signature's lists cannot be held (memory, or 2^31 entries).
 dl_status build_cast_lists(dl_ctx* ctx, Scene& S, Display& D, TileGroups& G, FrameHint& hint,
-                           int64_t chunk, cudaStream_t s, GroupSlices* sl, uint32_t** over,
-                           int32_t* launches, bool* ready) {
+                           const std::vector<Cam>& cams, int64_t chunk, cudaStream_t s,
+                           GroupSlices* sl, uint32_t** over, int32_t* launches, bool* ready) {
     Workspace& W = ctx->ws;
     *ready = false;
     const int32_t nv = D.q.nv;
@@ -519,13 +527,14 @@ dl_status build_cast_lists(dl_ctx* ctx, Scene& S, Display& D, TileGroups& G, Fra
         return false;
     };
     const bool sizing = !hint.sized || !hint.slices_ready;
-    if (!reserve(W.rec, 16 * kRecordFloat4 * size_t(ne)) || !reserve(W.gcount, words) ||
-        !reserve(W.gfill, words) || !reserve(W.gscan_tmp, scan_tmp_bytes(ngroups + 1)) ||
+    if (!reserve(W.rec, 16 * kRecordFloat4 * size_t(ne)) || !reserve(W.gfill, words) ||
+        !reserve(W.gscan_tmp, slice_tmp_bytes(ngroups)) ||
         !reserve(hint.slices[0], words) || !reserve(hint.slices[1], words) ||
         !reserve(W.cast, cast_tmp_bytes(chunk, ctx->heap_cap))) {
         hint.no_lists = true;
         return DL_OK;
     }
+    DL_CK(W.small.reserve(256), "alloc");
     unsigned long long* d_total64 = W.small.as<unsigned long long>();
     uint32_t* d_total32 = reinterpret_cast<uint32_t*>(W.small.as<char>() + 64);
     uint32_t* d_redo = d_total32 + 1;
@@ -534,7 +543,8 @@ dl_status build_cast_lists(dl_ctx* ctx, Scene& S, Display& D, TileGroups& G, Fra
     uint32_t* const next = hint.slices[hint.cur ^ 1].as<uint32_t>();
     uint32_t* const cursor = W.gfill.as<uint32_t>();
     if (sizing) DL_CK(cudaMemsetAsync(slice, 0, words, s), "empty slices");
-    DL_CK(cudaMemcpyAsync(cursor, slice, 4 * size_t(ngroups), cudaMemcpyDeviceToDevice, s), "cursors");
+    const dl_status st = begin_frame(ctx, cams, slice, ngroups, cursor, s, launches);
+    if (st) return st;
     const void* attrs[5] = {S.mean.p, S.log_scale.p, S.rot.p, S.opacity.p, S.sh.p};
     ProjectOut po{W.rec.as<float4>(), nullptr, d_total64, nullptr};
     po.keys = W.keys[0].as<unsigned long long>();
@@ -544,9 +554,9 @@ dl_status build_cast_lists(dl_ctx* ctx, Scene& S, Display& D, TileGroups& G, Fra
         sizing ? 0u : uint32_t(std::min<size_t>(W.keys[0].bytes / 8, size_t((1u << 31) - 2)));
     po.overflow = d_redo;
     DL_CK(launch_project_outline(S.dtype, attrs, pp, W.cams.as<Cam>(), nv, po, false, s), "outlines");
-    DL_CK(launch_pad_counts(cursor, slice, ngroups, W.gcount.as<uint32_t>(), s), "pad counts");
-    DL_CK(launch_exclusive_scan(W.gcount.as<uint32_t>(), next, ngroups + 1, d_total32, W.gscan_tmp.p, s),
-          "slice scan");
+    // (sizing: every key found its empty slice full, so the cursors move too)
+    DL_CK(launch_slice_layout(cursor, slice, ngroups, W.gscan_tmp.p, next, d_total32, d_redo, s),
+          "slice layout");
     if (sizing) {
         DL_CK(cudaMemcpyAsync(W.h_total, d_total64, 8, cudaMemcpyDeviceToHost, s), "copy totals");
         DL_CK(cudaStreamSynchronize(s), "sync");
@@ -563,7 +573,6 @@ dl_status build_cast_lists(dl_ctx* ctx, Scene& S, Display& D, TileGroups& G, Fra
         po.keys = W.keys[0].as<unsigned long long>();
         po.key_cap = uint32_t(std::min<size_t>(W.keys[0].bytes / 8, size_t((1u << 31) - 2)));
     }
-    DL_CK(launch_reset_cursor(d_redo, next, ngroups, cursor, s), "cursors");
     po.slice = next;
     po.gate = d_redo;
     po.overflow = *over;
@@ -573,7 +582,7 @@ dl_status build_cast_lists(dl_ctx* ctx, Scene& S, Display& D, TileGroups& G, Fra
     sl->use_alt = d_redo;
     sl->cursor = cursor;
     hint.cur ^= 1;
-    *launches += 7;
+    *launches += 4;
     *ready = true;
     return DL_OK;
 }
@@ -594,8 +603,7 @@ dl_status render_raycast(dl_ctx* ctx, int32_t scene_id, int32_t display_id, Scen
     std::vector<Cam> cams;
     if (!make_cams(D.prm, L0_c2w, cams))
         return fail(ctx, DL_ERR_INVALID_ARG, "off-axis rig: the world origin is not in front of L0");
-    dl_status st = upload_cams(ctx, cams, s);
-    if (st) return st;
+    dl_status st = DL_OK;
     if (!S.rc_built) {
         st = build_raycast(ctx, S, s);
         if (st) return st;
@@ -604,19 +612,21 @@ dl_status render_raycast(dl_ctx* ctx, int32_t scene_id, int32_t display_id, Scen
     TileGroups* G = nullptr;
     st = get_groups(ctx, D, R, ctx->tile[DL_DIRECTL][0], ctx->tile[DL_DIRECTL][1], s, &G);
     if (st) return st;
-    DL_CK(W.small.reserve(256), "alloc");
-    DL_CK(cudaMemsetAsync(W.small.p, 0, 256, s), "memset");
     FrameHint& hint = ctx->hints[FrameSig{scene_id, display_id, DL_RAYCAST, G->tw, G->th, w, h}];
     GroupSlices sl;
     uint32_t* over = nullptr;
-    int32_t launches = int32_t((D.q.nv + kCamBatch - 1) / kCamBatch);
+    int32_t launches = 0;
     bool lists = false;
     // rays a chunk: 2 GB of lists, evenly
     const int64_t most = std::max<int64_t>((int64_t(1) << 31) / (8 * ctx->heap_cap), 1);
     const int64_t chunks = (R.n_rays + most - 1) / most;
     const int64_t chunk = chunks > 0 ? (R.n_rays + chunks - 1) / chunks : 1;
-    st = build_cast_lists(ctx, S, D, *G, hint, chunk, s, &sl, &over, &launches, &lists);
+    st = build_cast_lists(ctx, S, D, *G, hint, cams, chunk, s, &sl, &over, &launches, &lists);
     if (st) return st;
+    if (!lists) {
+        st = begin_frame(ctx, cams, nullptr, 0, nullptr, s, &launches);
+        if (st) return st;
+    }
     for (int i = 1; i <= 6; ++i) DL_CK(mark(i), "event");
     DL_CK(W.raycol.reserve(12 * size_t(R.n_rays > 0 ? R.n_rays : 1)), "alloc ray colours");
     const double pi = 3.14159265358979323846;
@@ -1217,8 +1227,6 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
     view_prm.height = rh;
     if (!make_cams(view_prm, L0_c2w, cams))
         return fail(ctx, DL_ERR_INVALID_ARG, "off-axis rig: the world origin is not in front of L0");
-    st = upload_cams(ctx, cams, s);
-    if (st) return st;
     const ProjectParams pp = make_project_params(S, D, tw, th, rw, rh);
     const int64_t ntiles = int64_t(pp.ntx) * pp.nty;
     const int64_t ne = int64_t(nv) * S.n;
@@ -1245,14 +1253,14 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
     DL_CK(W.gcount.reserve(4 * size_t(ngroups + 1)), "alloc group counts");
     DL_CK(W.gstart.reserve(4 * size_t(ngroups + 1)), "alloc group starts");
     DL_CK(W.gfill.reserve(4 * size_t(ngroups)), "alloc cursors");
-    DL_CK(W.gscan_tmp.reserve(scan_tmp_bytes(ngroups + 1)), "alloc scan");
+    DL_CK(W.gscan_tmp.reserve(std::max(scan_tmp_bytes(ngroups + 1), slice_tmp_bytes(ngroups))),
+          "alloc scan");
     DL_CK(W.small.reserve(256), "alloc");
     unsigned long long* d_total64 = W.small.as<unsigned long long>();
     uint32_t* d_total32 = reinterpret_cast<uint32_t*>(W.small.as<char>() + 64);
     uint32_t* d_redo = d_total32 + 1;  // a key found its slice full (direct emission)
     uint32_t* d_meta = reinterpret_cast<uint32_t*>(W.small.as<char>() + 128);
     uint32_t* d_status = d_meta + 7;
-    DL_CK(cudaMemsetAsync(W.small.p, 0, 256, s), "memset");
     // the key buffer only grows, so its capacity covers every earlier sizing
     const uint32_t key_cap =
         on_device ? uint32_t(std::min<size_t>(W.keys[0].bytes / 8, size_t((1u << 31) - 2))) : 0u;
@@ -1267,12 +1275,45 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
     int32_t* small_list = W.lists.as<int32_t>();
     int32_t* large_list = small_list + nw1;
     uint32_t* cursor = W.gfill.as<uint32_t>();
+    if (mode != DL_STANDARD)
+        DL_CK(W.raycol.reserve(12 * size_t(R->n_rays > 0 ? R->n_rays : 1)), "alloc ray colours");
+    CompositeParams cp{};
+    cp.n = S.n;
+    cp.width = rw;
+    cp.height = rh;
+    cp.half_w = pp.half_w;
+    cp.half_h = pp.half_h;
+    cp.tile_w = tw;
+    cp.tile_h = th;
+    cp.ntx = pp.ntx;
+    cp.ntiles = int32_t(ntiles);
+    cp.meta = W.meta.as<uint4>();
+    // one frame through the frame-batched persistent kernels
+    SingleFrame single;
+    if (warp_path) {
+        DL_CK(W.fdesc.reserve(sizeof(FrameDesc)), "alloc frame table");
+        FrameDesc& fd = single.fd;
+        fd.cp = cp;
+        fd.grouped = G->grouped.as<int2>();
+        fd.keys = W.keys[0].as<unsigned long long>();
+        fd.rec = W.rec.as<float4>();
+        fd.raycol = W.raycol.as<float>();
+        fd.items = items;
+        fd.gwork = G->gwork.as<int4>();
+        fd.block_items = block_items;
+        fd.meta = d_meta;
+        fd.status = d_status;
+        fd.n_work = n_work;
+    }
+    int64_t* const prefix = reinterpret_cast<int64_t*>(W.small.as<char>() + 192);
+    int launches = 0;
+    st = begin_frame(ctx, cams, direct ? hint.slices[hint.cur].as<uint32_t>() : nullptr, ngroups,
+                     cursor, s, &launches);
+    if (st) return st;
     if (direct) {
         DL_CK(hint.slices[hint.cur ^ 1].reserve(4 * size_t(ngroups + 1)), "alloc slices");
         const uint32_t* slice = hint.slices[hint.cur].as<uint32_t>();
         uint32_t* next = hint.slices[hint.cur ^ 1].as<uint32_t>();
-        DL_CK(cudaMemcpyAsync(cursor, slice, 4 * size_t(ngroups), cudaMemcpyDeviceToDevice, s),
-              "cursors");
         ProjectOut po{W.rec.as<float4>(), nullptr, d_total64, nullptr, d_total64 + 1};
         po.keys = W.keys[0].as<unsigned long long>();
         po.cursor = cursor;
@@ -1282,15 +1323,12 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
         DL_CK(launch_project_direct(S.dtype, attrs, pp, W.cams.as<Cam>(), nv, po, false, s),
               "project");
         DL_CK(mark(1), "event");
-        // the next frame's slices, from this frame's counts (the scan's
-        // total, at d_total32, is read back with the frame's counters)
-        DL_CK(launch_pad_counts(cursor, slice, ngroups, W.gcount.as<uint32_t>(), s), "pad counts");
-        DL_CK(launch_exclusive_scan(W.gcount.as<uint32_t>(), next, ngroups + 1, d_total32,
-                                    W.gscan_tmp.p, s),
-              "slice scan");
-        // a frame that outgrew a slice emits its keys again, into those
-        // slices (no key past key_cap: the frame is dropped, status bit 0)
-        DL_CK(launch_reset_cursor(d_redo, next, ngroups, cursor, s), "cursors");
+        // the next frame's slices, from this frame's counts (their end, at
+        // d_total32, is read back with the frame's counters); a frame that
+        // outgrew a slice emits its keys again, into those slices (no key
+        // past key_cap: the frame is dropped, status bit 0)
+        DL_CK(launch_slice_layout(cursor, slice, ngroups, W.gscan_tmp.p, next, d_total32, d_redo, s),
+              "slice layout");
         ProjectOut po2 = po;
         po2.slice = next;
         po2.gate = d_redo;
@@ -1302,9 +1340,13 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
         sl.start_alt = next;
         sl.use_alt = d_redo;
         sl.cursor = cursor;
+        // (the key buffer is final: the partition can store the frame's table)
+        single.dst = W.fdesc.as<FrameDesc>();
+        single.prefix = prefix;
+        single.done = d_meta + 8;
         DL_CK(launch_partition_warp(gwork, n_work, sl, uint32_t(ctx->warp_cap),
                                     ctx->warp_cap < 1024 ? 1024u : 0u, items, block_items, d_meta,
-                                    nullptr, key_cap, d_status, s),
+                                    nullptr, key_cap, d_status, single, s),
               "partition");
         hint.cur ^= 1;
     } else {
@@ -1328,13 +1370,13 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
         DL_CK(launch_partition_warp(gwork, n_work, sl, uint32_t(ctx->warp_cap),
                                     ctx->warp_cap < 1024 ? 1024u : 0u, items, block_items, d_meta,
                                     on_device ? d_nkeys : nullptr, key_cap,
-                                    on_device ? d_status : nullptr, s),
+                                    on_device ? d_status : nullptr, single, s),
               "partition");
     } else if (views_path) {
         GroupSlices sl;
         sl.start = W.gstart.as<uint32_t>();
         DL_CK(launch_partition_warp(nullptr, n_work, sl, 512u, 1024u, items, block_items, d_meta,
-                                    nullptr, 0u, nullptr, s),
+                                    nullptr, 0u, nullptr, single, s),
               "partition");
     } else {
         DL_CK(launch_partition(gwork, n_work, W.gstart.as<uint32_t>(), uint32_t(kSmallCap), small_list,
@@ -1395,17 +1437,6 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
     unsigned long long* pairs =
         timing && ctx->count_pairs ? W.pairs.as<unsigned long long>() : nullptr;
 
-    CompositeParams cp{};
-    cp.n = S.n;
-    cp.width = rw;
-    cp.height = rh;
-    cp.half_w = pp.half_w;
-    cp.half_h = pp.half_h;
-    cp.tile_w = tw;
-    cp.tile_h = th;
-    cp.ntx = pp.ntx;
-    cp.ntiles = int32_t(ntiles);
-    cp.meta = W.meta.as<uint4>();
     const size_t out_bytes = 12 * size_t(w) * size_t(h);
     float* dst = nullptr;
     st = out_target(ctx, out, kind, out_bytes, s, &dst);
@@ -1416,14 +1447,12 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
         DL_CK(W.Mm.reserve(12 * size_t(nv) * size_t(rw) * size_t(rh)), "alloc M_m");
         Mm = W.Mm.as<float>();
     } else {
-        DL_CK(W.raycol.reserve(12 * size_t(R->n_rays > 0 ? R->n_rays : 1)), "alloc ray colours");
         raycol = W.raycol.as<float>();
     }
     int sort_bits = 0;
-    // cameras, projection, scan, partition (direct emission: and the counts'
-    // padding, the cursor reset and the gated re-emission)
-    int launches = int32_t((nv + kCamBatch - 1) / kCamBatch) + 1 + 3 + (n_work > 0 ? 1 : 0) +
-                   (direct ? 3 : 0);
+    // projection, scan (direct emission: the layout's two and the gated
+    // re-emission), partition
+    launches += 1 + 3 + (n_work > 0 ? 1 : 0);
     DL_CK(W.keys[0].reserve(8 * size_t(nk > 0 ? nk : 1)), "alloc keys");
     if (binned) {
         // ---- binned keys, sorted per tile in shared memory while compositing ----
@@ -1442,15 +1471,11 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
                 // projection, from this frame's counts
                 for (DevBuf& b : hint.slices)
                     DL_CK(b.reserve(4 * size_t(ngroups + 1)), "alloc slices");
-                DL_CK(launch_pad_counts(W.gcount.as<uint32_t>(), nullptr, ngroups,
-                                        hint.slices[hint.cur ^ 1].as<uint32_t>(), s),
-                      "pad counts");
-                DL_CK(launch_exclusive_scan(hint.slices[hint.cur ^ 1].as<uint32_t>(),
-                                            hint.slices[hint.cur].as<uint32_t>(), ngroups + 1,
-                                            d_total32, W.gscan_tmp.p, s),
-                      "slice scan");
+                DL_CK(launch_slice_layout(W.gcount.as<uint32_t>(), nullptr, ngroups, W.gscan_tmp.p,
+                                          hint.slices[hint.cur].as<uint32_t>(), d_total32, nullptr, s),
+                      "slice layout");
                 hint.slices_ready = true;
-                launches += 4;
+                launches += 2;
             }
         }
         DL_CK(mark(4), "event");
@@ -1473,34 +1498,29 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
                                                pairs, s),
                   "composite full (large lists)");
         } else if (warp_path) {
-            // one frame through the frame-batched persistent kernels
-            FrameDesc fd{};
-            fd.cp = cp;
-            fd.grouped = G->grouped.as<int2>();
-            fd.keys = keys;
-            fd.rec = W.rec.as<float4>();
-            fd.raycol = raycol;
-            fd.items = items;
-            fd.gwork = G->gwork.as<int4>();
-            fd.block_items = block_items;
-            fd.meta = d_meta;
-            fd.status = d_meta + 7;
-            fd.n_work = n_work;
-            DL_CK(W.fdesc.reserve(sizeof(FrameDesc)), "alloc frame table");
-            // pageable source: staged by the call, so fd may go out of scope
-            DL_CK(cudaMemcpyAsync(W.fdesc.p, &fd, sizeof(FrameDesc), cudaMemcpyHostToDevice, s),
-                  "copy frame table");
             const FrameDesc* dF = W.fdesc.as<FrameDesc>();
-            int64_t* prefix = reinterpret_cast<int64_t*>(W.small.as<char>() + 192);
-            DL_CK(launch_batch_prefix(dF, 1, prefix, s), "prefix");
+            if (!direct) {  // (direct: stored by the partition)
+                single.fd.keys = keys;
+                // pageable source: staged by the call, so it may go out of scope
+                DL_CK(cudaMemcpyAsync(W.fdesc.p, &single.fd, sizeof(FrameDesc), cudaMemcpyHostToDevice,
+                                      s),
+                      "copy frame table");
+                DL_CK(launch_batch_prefix(dF, 1, prefix, s), "prefix");
+                launches += 1;
+            }
+            // the classes beside one another, the longest lists first
+            DL_CK(W.side.create(2), "streams");
+            DL_CK(W.side.fork(s, 2), "fork");
+            DL_CK(launch_composite_rays_block(cap_large, dF, prefix, 1, n_large, d_meta + 6, pairs,
+                                              W.side.st[0]),
+                  "composite rays (block per group)");
+            DL_CK(launch_composite_rays_warp(1024, 1, dF, prefix, 1, n_mid, d_meta + 5, pairs,
+                                             W.side.st[1]),
+                  "composite rays (warp per group, 1024 keys)");
             DL_CK(launch_composite_rays_warp(ctx->warp_cap, 0, dF, prefix, 1, n_small, d_meta + 3,
                                              pairs, s),
                   "composite rays (warp per group)");
-            DL_CK(launch_composite_rays_warp(1024, 1, dF, prefix, 1, n_mid, d_meta + 5, pairs, s),
-                  "composite rays (warp per group, 1024 keys)");
-            DL_CK(launch_composite_rays_block(cap_large, dF, prefix, 1, n_large, d_meta + 6, pairs, s),
-                  "composite rays (block per group)");
-            launches += 1;
+            DL_CK(W.side.join(s, 2), "join");
         } else {
             DL_CK(launch_composite_rays_binned(cp, G->gwork.as<int4>(), small_list, n_small, kSmallCap,
                                                G->grouped.as<int2>(), W.gstart.as<uint32_t>(), keys,

@@ -19,6 +19,7 @@ namespace {
 // lists of <= 512 and <= 1024 keys: one warp each (two shared-memory sizes);
 // longer lists: the four-warp quadrant blocks
 constexpr int kWarpCap1 = 512, kWarpCap2 = 1024;
+constexpr int kMaxSide = 8;     // streams beside the caller's
 constexpr int kMetaWords = 16;  // per slot: partition counters, key total (u64 at word 8)
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -31,7 +32,7 @@ struct Slot {
     size_t o_rec = 0, o_meta = 0, o_zero = 0, o_gstart = 0, o_keys = 0, o_lists = 0, o_raycol = 0;
     // keys emitted by the projection: the slices this launch emits into
     // (A) and the ones its counts lay out for the next launch (B, copied to
-    // A at the end), ng_cap + 1 words each
+    // A when that starts), ng_cap + 1 words each
     size_t o_slices = 0;
     bool direct = false;
     size_t zero_bytes = 0;  // gcount | gfill | meta, zeroed by every launch
@@ -65,6 +66,10 @@ struct dl_batch {
     size_t o_prefix = 0, o_globals = 0, globals_bytes = 0;  // arena offsets
     int32_t block_cap = 2048;
     cudaEvent_t done = nullptr;
+    // the slots' own steps, and the compositing classes, run beside one
+    // another: alone, a small frame's kernels leave most of the GPU idle
+    SideStreams side;
+    size_t scan_stride = 0;  // scan scratch of one stream
     bool launched = false;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -117,7 +122,7 @@ void release_slot(Slot& z) {
 }
 
 // Everything one launch enqueues (also what a capture records).
-dl_status enqueue(dl_batch* b, cudaStream_t s) {
+dl_status enqueue(dl_batch* b, cudaStream_t main) {
     dl_ctx* ctx = b->ctx;
     const int32_t n_slots = int32_t(b->slots.size());
     // frame table of the assigned slots, in slot order
@@ -150,30 +155,35 @@ dl_status enqueue(dl_batch* b, cudaStream_t s) {
         fd.n_work = z.G->n_gwork;
         max_items += z.G->n_gwork;
     }
-    DL_CK(cudaMemcpyAsync(b->stage_d.p, b->stage_h, b->stage_bytes, cudaMemcpyHostToDevice, s),
+    DL_CK(cudaMemcpyAsync(b->stage_d.p, b->stage_h, b->stage_bytes, cudaMemcpyHostToDevice, main),
           "upload frame table and cameras");
-    DL_CK(cudaMemsetAsync(b->at<char>(b->o_globals), 0, b->globals_bytes, s), "memset");
+    DL_CK(cudaMemsetAsync(b->at<char>(b->o_globals), 0, b->globals_bytes, main), "memset");
+    // slot f of a launch runs on stream f of the side streams, in turn (one
+    // slot: on the caller's)
+    const int n_side = n_act > 1 ? std::min<int>(n_act, int(b->side.st.size())) : 0;
+    auto stream_of = [&](int32_t f) { return n_side ? b->side.st[size_t(f % n_side)] : main; };
+    DL_CK(b->side.fork(main, n_side), "fork");
     int32_t f = 0;
     for (int32_t i = 0; i < n_slots; ++i) {
         Slot& z = b->slots[size_t(i)];
         if (!z.active) continue;
+        const cudaStream_t s = stream_of(f);
+        void* const scan_tmp = b->scan_tmp.as<char>() + (n_side ? size_t(f % n_side) : 0) * b->scan_stride;
         const FrameDesc& fd = b->frames_h()[f++];
         uint32_t* gcount = b->at<uint32_t>(z.o_zero);
         uint32_t* gfill = gcount + (z.ng_cap + 1);
         uint32_t* meta = const_cast<uint32_t*>(fd.meta);
-        DL_CK(cudaMemsetAsync(gcount, 0, z.zero_bytes, s), "memset");
         const Scene& S = *z.S;
         const int32_t nv = z.D->q.nv;
         const void* attrs[5] = {S.mean.p, S.log_scale.p, S.rot.p, S.opacity.p, S.sh.p};
         if (z.direct) {
-            // the projection emits the keys into slices A (laid out by the
-            // slot's previous launch); B from this launch's counts; a slot
+            // the projection emits the keys into slices A, the layout B of the
+            // slot's previous launch; B anew from this launch's counts; a slot
             // that outgrew A emits again into B (meta word 12: the flag)
             uint32_t* sa = b->at<uint32_t>(z.o_slices);
             uint32_t* sb = sa + (z.ng_cap + 1);
             uint32_t* redo = meta + 12;
-            DL_CK(cudaMemcpyAsync(gfill, sa, 4 * size_t(z.ngroups), cudaMemcpyDeviceToDevice, s),
-                  "cursors");
+            DL_CK(launch_begin_slot(meta, kMetaWords, sb, z.ngroups, gfill, sa, s), "begin slot");
             ProjectOut po{b->at<float4>(z.o_rec), nullptr,
                           reinterpret_cast<unsigned long long*>(meta + 8), nullptr};
             po.keys = b->at<unsigned long long>(z.o_keys);
@@ -184,10 +194,8 @@ dl_status enqueue(dl_batch* b, cudaStream_t s) {
             DL_CK(launch_project_direct(S.dtype, attrs, z.pp, b->cams_d() + z.cam_first, nv, po,
                                         false, s),
                   "project");
-            DL_CK(launch_pad_counts(gfill, sa, z.ngroups, gcount, s), "pad counts");
-            DL_CK(launch_exclusive_scan(gcount, sb, z.ngroups + 1, nullptr, b->scan_tmp.p, s),
-                  "slice scan");
-            DL_CK(launch_reset_cursor(redo, sb, z.ngroups, gfill, s), "cursors");
+            DL_CK(launch_slice_layout(gfill, sa, z.ngroups, scan_tmp, sb, nullptr, redo, s),
+                  "slice layout");
             ProjectOut po2 = po;
             po2.slice = sb;
             po2.gate = redo;
@@ -203,18 +211,16 @@ dl_status enqueue(dl_batch* b, cudaStream_t s) {
             DL_CK(launch_partition_warp(z.G->gwork.as<int4>(), z.G->n_gwork, sl, kWarpCap1,
                                         kWarpCap2, const_cast<int4*>(fd.items),
                                         const_cast<int4*>(fd.block_items), meta, nullptr,
-                                        uint32_t(z.key_cap), fd.status, s),
+                                        uint32_t(z.key_cap), fd.status, SingleFrame{}, s),
                   "partition");
-            // the next launch's slices (the items hold this launch's offsets)
-            DL_CK(cudaMemcpyAsync(sa, sb, 4 * size_t(z.ngroups + 1), cudaMemcpyDeviceToDevice, s),
-                  "next slices");
             continue;
         }
+        DL_CK(cudaMemsetAsync(gcount, 0, z.zero_bytes, s), "memset");
         ProjectOut po{b->at<float4>(z.o_rec), b->at<uint4>(z.o_meta),
                       reinterpret_cast<unsigned long long*>(meta + 8), gcount};
         DL_CK(launch_project(S.dtype, attrs, z.pp, b->cams_d() + z.cam_first, nv, po, s), "project");
         uint32_t* gstart = b->at<uint32_t>(z.o_gstart);
-        DL_CK(launch_exclusive_scan(gcount, gstart, z.ngroups + 1, nullptr, b->scan_tmp.p, s),
+        DL_CK(launch_exclusive_scan(gcount, gstart, z.ngroups + 1, nullptr, scan_tmp, s),
               "group scan");
         DL_CK(cudaMemcpyAsync(gfill, gstart, 4 * size_t(z.ngroups), cudaMemcpyDeviceToDevice, s),
               "cursors");
@@ -226,32 +232,39 @@ dl_status enqueue(dl_batch* b, cudaStream_t s) {
         sl.start = gstart;
         DL_CK(launch_partition_warp(z.G->gwork.as<int4>(), z.G->n_gwork, sl, kWarpCap1, kWarpCap2,
                                     const_cast<int4*>(fd.items), const_cast<int4*>(fd.block_items),
-                                    meta, gstart + z.ngroups, uint32_t(z.key_cap), fd.status, s),
+                                    meta, gstart + z.ngroups, uint32_t(z.key_cap), fd.status,
+                                    SingleFrame{}, s),
               "partition");
     }
+    DL_CK(b->side.join(main, n_side), "join");
     if (n_act > 0) {
         int64_t* prefix = b->at<int64_t>(b->o_prefix);
         uint32_t* cur = b->cursors_d();
-        DL_CK(launch_batch_prefix(b->frames_d(), n_act, prefix, s), "prefix");
-        DL_CK(launch_composite_rays_warp(kWarpCap1, 0, b->frames_d(), prefix, n_act, max_items, cur,
-                                         nullptr, s),
-              "composite rays (warp class 512)");
-        if (kWarpCap2 > 0)
-            DL_CK(launch_composite_rays_warp(kWarpCap2, 1, b->frames_d(), prefix, n_act, max_items,
-                                             cur + 1, nullptr, s),
-                  "composite rays (warp class 1024)");
+        DL_CK(launch_batch_prefix(b->frames_d(), n_act, prefix, main), "prefix");
+        // the classes beside one another, the longest lists first
+        DL_CK(b->side.fork(main, 2), "fork");
         DL_CK(launch_composite_rays_block(b->block_cap, b->frames_d(), prefix, n_act, max_items,
-                                          cur + 2, nullptr, s),
+                                          cur + 2, nullptr, b->side.st[0]),
               "composite rays (block class)");
+        DL_CK(launch_composite_rays_warp(kWarpCap2, 1, b->frames_d(), prefix, n_act, max_items,
+                                         cur + 1, nullptr, b->side.st[1]),
+              "composite rays (warp class 1024)");
+        DL_CK(launch_composite_rays_warp(kWarpCap1, 0, b->frames_d(), prefix, n_act, max_items, cur,
+                                         nullptr, main),
+              "composite rays (warp class 512)");
+        DL_CK(b->side.join(main, 2), "join");
     }
+    DL_CK(b->side.fork(main, n_side), "fork");
+    f = 0;
     for (int32_t i = 0; i < n_slots; ++i) {
         Slot& z = b->slots[size_t(i)];
         if (!z.active) continue;
         DL_CK(launch_reorder(z.G->slot_of.as<uint32_t>(), b->at<float>(z.o_raycol),
-                             z.D->q.w, z.D->q.h, z.out, b->status_d() + i, s),
+                             z.D->q.w, z.D->q.h, z.out, b->status_d() + i, stream_of(f++)),
               "reorder");
     }
-    DL_CK(cudaMemcpyAsync(b->status_h, b->status_d(), 4 * size_t(n_slots), cudaMemcpyDeviceToHost, s),
+    DL_CK(b->side.join(main, n_side), "join");
+    DL_CK(cudaMemcpyAsync(b->status_h, b->status_d(), 4 * size_t(n_slots), cudaMemcpyDeviceToHost, main),
           "copy status");
     return DL_OK;
 }
@@ -335,7 +348,7 @@ dl_status dl_batch_create(dl_ctx* ctx, int32_t n_slots, const dl_slot_plan* plan
         z.key_cap = std::min<int64_t>(int64_t(std::ceil(double(laid) * margin)) + 4096,
                                       (int64_t(1) << 31) - 2);
         longest = std::max<int64_t>(longest, int64_t(std::ceil(double(ctx->stats.max_list) * margin)));
-        scan_bytes = std::max(scan_bytes, scan_tmp_bytes(z.ng_cap + 1));
+        scan_bytes = std::max({scan_bytes, scan_tmp_bytes(z.ng_cap + 1), slice_tmp_bytes(z.ng_cap)});
     }
     ctx->tile[DL_DIRECTL][0] = saved_tile[0];
     ctx->tile[DL_DIRECTL][1] = saved_tile[1];
@@ -369,7 +382,10 @@ dl_status dl_batch_create(dl_ctx* ctx, int32_t n_slots, const dl_slot_plan* plan
     b->globals_bytes = 4 * (8 + size_t(n_slots));
     b->o_globals = take(b->globals_bytes);
     DL_CK(b->arena.reserve(off), "alloc batch arena");
-    DL_CK(b->scan_tmp.reserve(std::max<size_t>(scan_bytes, 256)), "alloc scan scratch");
+    const int n_side = std::max(2, std::min<int>(n_slots, kMaxSide));
+    DL_CK(b->side.create(n_side), "streams");
+    b->scan_stride = align_up(std::max<size_t>(scan_bytes, 256), 256);
+    DL_CK(b->scan_tmp.reserve(b->scan_stride * size_t(n_side)), "alloc scan scratch");
     b->cams_offset = align_up(sizeof(FrameDesc) * size_t(n_slots), 256);
     b->stage_bytes = b->cams_offset + sizeof(Cam) * size_t(b->total_views);
     DL_CK(b->stage_d.reserve(b->stage_bytes), "alloc staging");
@@ -438,8 +454,9 @@ dl_status dl_batch_assign(dl_batch* b, int32_t slot, int32_t scene_id, int32_t d
     z.pp = make_project_params(*S, *D, tw, th);
     z.ngroups = ng;
     z.direct = emit_in_projection(ctx->key_emission);
-    if (z.direct) {  // empty slices: the first launch emits into slices of its own counts
-        DL_CK(cudaMemsetAsync(b->at<uint32_t>(z.o_slices), 0, 4 * size_t(ng + 1), nullptr),
+    if (z.direct) {  // an empty layout: the first launch emits into slices of its own counts
+        DL_CK(cudaMemsetAsync(b->at<uint32_t>(z.o_slices) + (z.ng_cap + 1), 0, 4 * size_t(ng + 1),
+                              nullptr),
               "memset");
         DL_CK(cudaStreamSynchronize(nullptr), "sync");
     }

@@ -1533,7 +1533,7 @@ __global__ void partition_warp_kernel(const int4* __restrict__ gwork, int64_t n_
                                       int4* __restrict__ items, int4* __restrict__ block_items,
                                       uint32_t* __restrict__ meta,
                                       const uint32_t* __restrict__ total_keys, uint32_t key_cap,
-                                      uint32_t* __restrict__ status) {
+                                      uint32_t* __restrict__ status, SingleFrame single) {
     if (total_keys && *total_keys > key_cap) {  // keys were not emitted
         if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(status, 1u);
         return;
@@ -1573,6 +1573,21 @@ __global__ void partition_warp_kernel(const int4* __restrict__ gwork, int64_t n_
             block_items[s2] = make_int4(wi.x, int(st), int(w), int(len));
         const uint32_t longest = __reduce_max_sync(am, len);
         if (int(threadIdx.x & 31) == __ffs(am) - 1) atomicMax(meta + 2, longest);
+    }
+    if (!single.dst) return;
+    // the last block to finish sees every block's counts
+    __shared__ bool s_last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(single.done, 1u) == gridDim.x - 1u;
+    __syncthreads();
+    if (s_last && threadIdx.x == 0) {
+        *single.dst = single.fd;
+        // one frame: {0, items} per class
+        single.prefix[0] = single.prefix[2] = single.prefix[4] = 0;
+        single.prefix[1] = int64_t(atomicAdd(meta, 0u));
+        single.prefix[3] = int64_t(atomicAdd(meta + 4, 0u));
+        single.prefix[5] = int64_t(atomicAdd(meta + 1, 0u));
     }
 }
 
@@ -1894,14 +1909,14 @@ cudaError_t launch_composite_rays_block(int block_cap, const FrameDesc* frames,
 cudaError_t launch_partition_warp(const int4* gwork, int64_t n_work, const GroupSlices& slices,
                                   uint32_t cap1, uint32_t cap2, int4* items, int4* block_items,
                                   uint32_t* meta, const uint32_t* total_keys, uint32_t key_cap,
-                                  uint32_t* status, cudaStream_t s) {
+                                  uint32_t* status, const SingleFrame& single, cudaStream_t s) {
     if (n_work <= 0) return cudaSuccess;
     int64_t grid = (n_work + 255) / 256;
     const int64_t lim = int64_t(num_sms()) * 16;
     if (grid > lim) grid = lim;
     partition_warp_kernel<<<unsigned(grid), 256, 0, s>>>(gwork, n_work, slices, cap1, cap2, items,
                                                          block_items, meta, total_keys, key_cap,
-                                                         status);
+                                                         status, single);
     return cudaGetLastError();
 }
 

@@ -175,8 +175,16 @@ cudaError_t launch_group_slots(const int2* grouped, int64_t n_rays, const uint32
 
 // ---- a5/a6: projection, key emission (project.cu) ------------------------
 // dtype: 0 f32, 1 bf16, 2 f16
-// Copies up to kCamBatch cameras from a kernel parameter into device memory.
-cudaError_t launch_store_cams(const CamBatch& b, int32_t n, Cam* dst, cudaStream_t s);
+// Start of a frame: up to kCamBatch cameras from a kernel parameter into device
+// memory, n_zero counter words set to 0 and (with a layout) every group's
+// cursor at its slice's start, layout[g].
+cudaError_t launch_begin_frame(const CamBatch& b, int32_t n_cams, Cam* dst, uint32_t* zero,
+                               int32_t n_zero, const uint32_t* layout, int64_t n_groups,
+                               uint32_t* cursor, cudaStream_t s);
+// The same for a batch slot (its cameras are in the staging block); the layout
+// (n_groups + 1 entries) is also copied to `copy`.
+cudaError_t launch_begin_slot(uint32_t* zero, int32_t n_zero, const uint32_t* layout, int64_t n_groups,
+                              uint32_t* cursor, uint32_t* copy, cudaStream_t s);
 cudaError_t launch_project(int dtype, const void* const* attrs, const ProjectParams& p,
                            const Cam* cams, int32_t nv, ProjectOut out, cudaStream_t s);
 // Projection that emits the binned keys itself (no tile metadata, no
@@ -193,13 +201,14 @@ cudaError_t launch_project_direct(int dtype, const void* const* attrs, const Pro
 cudaError_t launch_project_outline(int dtype, const void* const* attrs, const ProjectParams& p,
                                    const Cam* cams, int32_t nv, ProjectOut out, bool keys_only,
                                    cudaStream_t s);
-// padded[g] = count + count / 8 + 16 with count = cursor[g] - slice[g]
-// (slice == nullptr: count = cursor[g]); padded[n_groups] = 0.
-cudaError_t launch_pad_counts(const uint32_t* cursor, const uint32_t* slice, int64_t n_groups,
-                              uint32_t* padded, cudaStream_t s);
-// cursor[g] = start[g] for every group when *flag != 0 (else nothing).
-cudaError_t launch_reset_cursor(const uint32_t* flag, const uint32_t* start, int64_t n_groups,
-                                uint32_t* cursor, cudaStream_t s);
+// Slices for the next layout from the groups' key counts (cursor[g] - slice[g];
+// cursor[g] without a slice array): count + count / 8 + 16 slots each, next[g]
+// the start of group g's, next[n_groups] = *d_total (optional) the end.  redo
+// (optional, device): when *redo != 0 the cursors are set to the new starts.
+size_t slice_tmp_bytes(int64_t n_groups);
+cudaError_t launch_slice_layout(uint32_t* cursor, const uint32_t* slice, int64_t n_groups, void* tmp,
+                                uint32_t* next, uint32_t* d_total, const uint32_t* redo,
+                                cudaStream_t s);
 // Keys depth << 32 | Gaussian << 4 | quadrant bits (Gaussians < 2^28; bit q
 // of the nibble: the pixel box overlaps quadrant q, x half + 2 * y half, of
 // the tile) into their group's slice
@@ -333,6 +342,30 @@ cudaError_t launch_composite_views(const CompositeParams& p, const int4* items,
                                    int block_cap, uint32_t* const cursor[2],
                                    const unsigned long long* keys, const float4* rec, float* Mm,
                                    unsigned long long* pairs, cudaStream_t s);
+// One DirectL frame's compositing inputs, as read by the frame-batched
+// persistent kernels (device memory, one entry per frame).
+struct FrameDesc {
+    CompositeParams cp;
+    const int2* grouped;              // {pixel, ray id} per grouped ray
+    const unsigned long long* keys;   // binned keys (the items give each group's slice)
+    const float4* rec;                // records, view-major
+    float* raycol;                    // 3 floats per ray id
+    const int4* items;                // launch_partition_warp output
+    const int4* gwork;                // {group, ray begin, ray end, -}
+    const int4* block_items;          // {group, first key, gwork index, keys}
+    const uint32_t* meta;             // {n_items1, n_block, max, -, n_items2}
+    uint32_t* status;                 // bit 0 keys overflow, bit 1 list longer than the block cap
+    int64_t n_work;
+};
+// A frame that is alone in its launches: the partition stores its table entry
+// and, once every group is placed, its class prefixes (so neither a copy nor
+// a launch_batch_prefix is needed).  done: a word, 0 at the launch.
+struct SingleFrame {
+    FrameDesc fd;
+    FrameDesc* dst = nullptr;
+    int64_t* prefix = nullptr;
+    uint32_t* done = nullptr;
+};
 // DirectL groups whose lists hold at most 512 or 1024 keys: one warp per
 // group (warp-level sort, cp.async batches of 32, transposed evaluation),
 // persistent over self-contained items {group, first key, first ray,
@@ -388,23 +421,8 @@ cudaError_t launch_raycast_lists(int dtype, int sh_degree, const CastParams& p, 
 cudaError_t launch_partition_warp(const int4* gwork, int64_t n_work, const GroupSlices& slices,
                                   uint32_t cap1, uint32_t cap2, int4* items, int4* block_items,
                                   uint32_t* meta, const uint32_t* total_keys, uint32_t key_cap,
-                                  uint32_t* status, cudaStream_t s);
+                                  uint32_t* status, const SingleFrame& single, cudaStream_t s);
 
-// One DirectL frame's compositing inputs, as read by the frame-batched
-// persistent kernels (device memory, one entry per frame).
-struct FrameDesc {
-    CompositeParams cp;
-    const int2* grouped;              // {pixel, ray id} per grouped ray
-    const unsigned long long* keys;   // binned keys (the items give each group's slice)
-    const float4* rec;                // records, view-major
-    float* raycol;                    // 3 floats per ray id
-    const int4* items;                // launch_partition_warp output
-    const int4* gwork;                // {group, ray begin, ray end, -}
-    const int4* block_items;          // {group, first key, gwork index, keys}
-    const uint32_t* meta;             // {n_items1, n_block, max, -, n_items2}
-    uint32_t* status;                 // bit 0 keys overflow, bit 1 list longer than the block cap
-    int64_t n_work;
-};
 // prefix[c * (n_frames + 1) + f] = items of class c (0: <= 512 keys,
 // 1: <= 1024 keys, 2: block list) in frames before f; one block.
 cudaError_t launch_batch_prefix(const FrameDesc* frames, int32_t n_frames, int64_t* prefix,

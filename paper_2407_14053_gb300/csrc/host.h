@@ -118,6 +118,51 @@ struct PendingFrame {
 // 675 at 120,000 (frames of 240x135 and 955x541).
 inline bool emit_in_projection(int32_t option) { return option != 0; }
 
+// Streams beside the caller's for work of one launch sequence that is
+// independent of itself.  fork() makes them wait for the caller's stream,
+// join() the caller's stream for the first `used` of them, so everything is
+// ordered on the caller's stream before and after, and a capture of that
+// stream includes them.
+struct SideStreams {
+    std::vector<cudaStream_t> st;
+    std::vector<cudaEvent_t> ev;  // one per stream, and the fork's at the end
+    cudaError_t create(int n) {
+        for (int i = int(st.size()); i < n; ++i) {
+            cudaStream_t x = nullptr;
+            const cudaError_t e = cudaStreamCreateWithFlags(&x, cudaStreamNonBlocking);
+            if (e != cudaSuccess) return e;
+            st.push_back(x);
+        }
+        while (ev.size() < st.size() + 1) {
+            cudaEvent_t x = nullptr;
+            const cudaError_t e = cudaEventCreateWithFlags(&x, cudaEventDisableTiming);
+            if (e != cudaSuccess) return e;
+            ev.push_back(x);
+        }
+        return cudaSuccess;
+    }
+    cudaError_t fork(cudaStream_t s, int used) {
+        cudaError_t e = cudaEventRecord(ev.back(), s);
+        for (int i = 0; i < used && e == cudaSuccess; ++i) e = cudaStreamWaitEvent(st[size_t(i)], ev.back(), 0);
+        return e;
+    }
+    cudaError_t join(cudaStream_t s, int used) {
+        cudaError_t e = cudaSuccess;
+        for (int i = 0; i < used && e == cudaSuccess; ++i) {
+            e = cudaEventRecord(ev[size_t(i)], st[size_t(i)]);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(s, ev[size_t(i)], 0);
+        }
+        return e;
+    }
+    ~SideStreams() {
+        for (cudaEvent_t x : ev) cudaEventDestroy(x);
+        for (cudaStream_t x : st) cudaStreamDestroy(x);
+    }
+    SideStreams() = default;
+    SideStreams(const SideStreams&) = delete;
+    SideStreams& operator=(const SideStreams&) = delete;
+};
+
 struct FrameHint {
     bool sized = false;
     int32_t block_cap = 2048;
@@ -161,6 +206,7 @@ struct Workspace {
     cudaEvent_t ev_frame[2] = {nullptr, nullptr}, ev_copied[2] = {nullptr, nullptr};
     bool copy_pending[2] = {false, false};
     int aslot = 0;
+    SideStreams side;  // compositing classes of a frame beside one another
     ~Workspace() {
         if (h_total) cudaFreeHost(h_total);
         for (Readback& r : rb) {

@@ -715,43 +715,145 @@ project_outline_kernel(GaussiansView<T> G, ProjectParams p, const Cam* __restric
     }
 }
 
-// Slices for the next layout: group g gets its key count (cursor[g] -
-// slice[g], or cursor[g] alone without a slice array) plus an eighth and
-// 16 slots; entry n_groups is 0, so an exclusive scan of n_groups + 1
-// entries ends with the total.
-__global__ void pad_counts_kernel(const uint32_t* __restrict__ cursor,
-                                  const uint32_t* __restrict__ slice, int64_t n_groups,
-                                  uint32_t* __restrict__ padded) {
-    for (int64_t g = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; g <= n_groups;
-         g += int64_t(gridDim.x) * blockDim.x) {
-        if (g == n_groups) {
-            padded[g] = 0u;
-        } else {
-            const uint32_t c = cursor[g] - (slice ? slice[g] : 0u);
-            padded[g] = c + (c >> 3) + 16u;
-        }
+// The next layout: group g gets its key count (cursor[g] - slice[g], or
+// cursor[g] alone without a slice array) plus an eighth and 16 slots; next[g]
+// is where its slots start, next[n_groups] the end.  Two launches: the sums of
+// kSliceTile groups, then the layout, each block adding up the sums before its
+// own.  When *redo is set (a key found its slice full) the cursors go to the
+// new starts, for the pass that emits again.
+constexpr int kSliceThreads = 256, kSliceItems = 16, kSliceTile = kSliceThreads * kSliceItems;
+
+__device__ __forceinline__ uint32_t padded_count(const uint32_t* cursor, const uint32_t* slice,
+                                                 int64_t g, int64_t n_groups) {
+    if (g >= n_groups) return 0u;
+    const uint32_t c = cursor[g] - (slice ? slice[g] : 0u);
+    return c + (c >> 3) + 16u;
+}
+
+// Sum of v over the block (every thread gets it).
+__device__ __forceinline__ uint32_t block_sum(uint32_t v) {
+    __shared__ uint32_t s_w[kSliceThreads / 32];
+    v = __reduce_add_sync(0xffffffffu, v);
+    if ((threadIdx.x & 31) == 0) s_w[threadIdx.x >> 5] = v;
+    __syncthreads();
+    uint32_t t = 0;
+#pragma unroll
+    for (int w = 0; w < kSliceThreads / 32; ++w) t += s_w[w];
+    __syncthreads();
+    return t;
+}
+
+__global__ void __launch_bounds__(kSliceThreads)
+slice_sums_kernel(const uint32_t* __restrict__ cursor, const uint32_t* __restrict__ slice,
+                  int64_t n_groups, uint32_t* __restrict__ sums) {
+    const int64_t base = int64_t(blockIdx.x) * kSliceTile + threadIdx.x;
+    uint32_t v = 0;
+#pragma unroll 4
+    for (int j = 0; j < kSliceItems; ++j)
+        v += padded_count(cursor, slice, base + j * kSliceThreads, n_groups);
+    v = block_sum(v);
+    if (threadIdx.x == 0) sums[blockIdx.x] = v;
+}
+
+__global__ void __launch_bounds__(kSliceThreads)
+slice_layout_kernel(uint32_t* cursor, const uint32_t* __restrict__ slice, int64_t n_groups,
+                    const uint32_t* __restrict__ sums, uint32_t* __restrict__ next,
+                    uint32_t* __restrict__ d_total, const uint32_t* __restrict__ redo) {
+    uint32_t before = 0;
+    for (int b = threadIdx.x; b < int(blockIdx.x); b += kSliceThreads) before += sums[b];
+    before = block_sum(before);
+    const int64_t base = int64_t(blockIdx.x) * kSliceTile + int64_t(threadIdx.x) * kSliceItems;
+    uint32_t v[kSliceItems], mine = 0;
+#pragma unroll
+    for (int j = 0; j < kSliceItems; ++j) {
+        v[j] = padded_count(cursor, slice, base + j, n_groups);
+        mine += v[j];
+    }
+    __shared__ uint32_t s_w[kSliceThreads / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t inc = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += t;
+    }
+    if (lane == 31) s_w[warp] = inc;
+    __syncthreads();
+    uint32_t run = before + inc - mine;
+    for (int w = 0; w < warp; ++w) run += s_w[w];
+    const bool again = redo && *redo != 0u;
+#pragma unroll
+    for (int j = 0; j < kSliceItems; ++j) {
+        const int64_t g = base + j;
+        if (g <= n_groups) next[g] = run;
+        if (again && g < n_groups) cursor[g] = run;
+        if (g == n_groups && d_total) *d_total = run;
+        run += v[j];
     }
 }
 
-// cursor = start, only when *flag is set
-__global__ void reset_cursor_kernel(const uint32_t* __restrict__ flag,
-                                    const uint32_t* __restrict__ start, int64_t n_groups,
-                                    uint32_t* __restrict__ cursor) {
-    if (*flag == 0u) return;
-    for (int64_t g = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; g < n_groups;
-         g += int64_t(gridDim.x) * blockDim.x)
-        cursor[g] = start[g];
+// What a frame needs before its projection: its cameras, its counters at zero,
+// every group's cursor at its slice's start (and a copy of the layout).
+__device__ __forceinline__ void begin_groups(const uint32_t* __restrict__ layout, int64_t n_groups,
+                                             uint32_t* __restrict__ cursor, uint32_t* __restrict__ copy) {
+    for (int64_t g = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; g <= n_groups;
+         g += int64_t(gridDim.x) * blockDim.x) {
+        const uint32_t v = layout[g];
+        if (g < n_groups) cursor[g] = v;
+        if (copy) copy[g] = v;
+    }
 }
 
-__global__ void store_cams_kernel(CamBatch b, int32_t n, Cam* __restrict__ dst) {
-    const int i = threadIdx.x;
-    if (i < n) dst[i] = b.cam[i];
+__global__ void begin_frame_kernel(CamBatch b, int32_t n_cams, Cam* __restrict__ dst,
+                                   uint32_t* __restrict__ zero, int32_t n_zero,
+                                   const uint32_t* __restrict__ layout, int64_t n_groups,
+                                   uint32_t* __restrict__ cursor) {
+    if (blockIdx.x == 0) {
+        if (int(threadIdx.x) < n_cams) dst[threadIdx.x] = b.cam[threadIdx.x];
+        for (int i = threadIdx.x; i < n_zero; i += blockDim.x) zero[i] = 0u;
+    }
+    if (layout) begin_groups(layout, n_groups, cursor, nullptr);
+}
+
+__global__ void begin_slot_kernel(uint32_t* __restrict__ zero, int32_t n_zero,
+                                  const uint32_t* __restrict__ layout, int64_t n_groups,
+                                  uint32_t* __restrict__ cursor, uint32_t* __restrict__ copy) {
+    if (blockIdx.x == 0)
+        for (int i = threadIdx.x; i < n_zero; i += blockDim.x) zero[i] = 0u;
+    begin_groups(layout, n_groups, cursor, copy);
+}
+
+unsigned group_grid(int64_t n_groups) {
+    return unsigned(std::min<int64_t>((n_groups + 256) / 256, int64_t(num_sms()) * 8));
 }
 
 }  // namespace
 
-cudaError_t launch_store_cams(const CamBatch& b, int32_t n, Cam* dst, cudaStream_t s) {
-    store_cams_kernel<<<1, kCamBatch, 0, s>>>(b, n, dst);
+cudaError_t launch_begin_frame(const CamBatch& b, int32_t n_cams, Cam* dst, uint32_t* zero,
+                               int32_t n_zero, const uint32_t* layout, int64_t n_groups,
+                               uint32_t* cursor, cudaStream_t s) {
+    begin_frame_kernel<<<layout ? group_grid(n_groups) : 1u, 256, 0, s>>>(b, n_cams, dst, zero, n_zero,
+                                                                         layout, n_groups, cursor);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_begin_slot(uint32_t* zero, int32_t n_zero, const uint32_t* layout, int64_t n_groups,
+                              uint32_t* cursor, uint32_t* copy, cudaStream_t s) {
+    begin_slot_kernel<<<group_grid(n_groups), 256, 0, s>>>(zero, n_zero, layout, n_groups, cursor, copy);
+    return cudaGetLastError();
+}
+
+size_t slice_tmp_bytes(int64_t n_groups) {
+    return 4 * size_t((n_groups + kSliceTile) / kSliceTile) + 256;
+}
+
+cudaError_t launch_slice_layout(uint32_t* cursor, const uint32_t* slice, int64_t n_groups, void* tmp,
+                                uint32_t* next, uint32_t* d_total, const uint32_t* redo,
+                                cudaStream_t s) {
+    const unsigned grid = unsigned((n_groups + kSliceTile) / kSliceTile);  // of n_groups + 1 entries
+    uint32_t* const sums = static_cast<uint32_t*>(tmp);
+    slice_sums_kernel<<<grid, kSliceThreads, 0, s>>>(cursor, slice, n_groups, sums);
+    slice_layout_kernel<<<grid, kSliceThreads, 0, s>>>(cursor, slice, n_groups, sums, next, d_total, redo);
     return cudaGetLastError();
 }
 
@@ -847,24 +949,6 @@ cudaError_t launch_project_outline(int dtype, const void* const* attrs, const Pr
     if (dtype == 1) return launch_project_outline_t<__nv_bfloat16>(attrs, p, cams, nv, out, keys_only, s);
     if (dtype == 2) return launch_project_outline_t<__half>(attrs, p, cams, nv, out, keys_only, s);
     return launch_project_outline_t<float>(attrs, p, cams, nv, out, keys_only, s);
-}
-
-cudaError_t launch_pad_counts(const uint32_t* cursor, const uint32_t* slice, int64_t n_groups,
-                              uint32_t* padded, cudaStream_t s) {
-    int64_t grid = (n_groups + 256) / 256;
-    const int64_t cap = int64_t(num_sms()) * 16;
-    if (grid > cap) grid = cap;
-    pad_counts_kernel<<<unsigned(grid), 256, 0, s>>>(cursor, slice, n_groups, padded);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_reset_cursor(const uint32_t* flag, const uint32_t* start, int64_t n_groups,
-                                uint32_t* cursor, cudaStream_t s) {
-    int64_t grid = (n_groups + 255) / 256;
-    const int64_t cap = int64_t(num_sms()) * 16;
-    if (grid > cap) grid = cap;
-    reset_cursor_kernel<<<unsigned(grid > 0 ? grid : 1), 256, 0, s>>>(flag, start, n_groups, cursor);
-    return cudaGetLastError();
 }
 
 cudaError_t launch_emit_binned(const ProjectParams& p, int32_t nv, const uint4* meta,
