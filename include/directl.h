@@ -276,8 +276,9 @@ dl_status dl_ray_table_static(int32_t width, int32_t height, const uint16_t* V,
 enum { DL_OPT_SORT_MODE = 1, DL_OPT_EVAL_DIRECTL = 2, DL_OPT_EVAL_STANDARD = 3,
        DL_OPT_WARP_LIST_CAP = 4, DL_OPT_STANDARD_VIEW_SIZE = 5, DL_OPT_HEAP_CAPACITY = 6,
        DL_OPT_KEY_EMISSION = 7 };
-/* DL_OPT_KEY_EMISSION: where the binned path of DL_DIRECTL / DL_REQUIRED_ONLY
- * writes its tile keys, once a frame of the same signature has been sized.
+/* DL_OPT_KEY_EMISSION: where the binned path of DL_DIRECTL, DL_REQUIRED_ONLY
+ * and (with direct evaluation) the standard modes writes its tile keys, once a
+ * frame of the same signature has been sized.
  * 1: the projection kernel emits every (view, tile, Gaussian) key itself,
  * into per-(view, tile) slices of the key buffer laid out from the
  * signature's previous frame (its key count per group plus an eighth and

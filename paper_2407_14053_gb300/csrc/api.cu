@@ -1191,6 +1191,7 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
         return render_raycast(ctx, scene_id, display_id, S, D, L0_c2w, out, kind, s, cs, E, frame);
     // "HR w SR" renders as DL_STANDARD (views at panel resolution) and
     // gathers each subpixel from its repurposed source pixel at the end
+    const int32_t asked = mode;
     const bool sr = mode == DL_STANDARD_SR;
     if (sr) mode = DL_STANDARD;
 
@@ -1247,7 +1248,12 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
     // keys emitted by the projection, into the slices the signature's last
     // frame laid out
     const bool in_projection = emit_in_projection(ctx->key_emission);
-    const bool direct = on_device && in_projection && hint.slices_ready;
+    // (the standard paradigm too, though it reads its totals back every frame:
+    // a frame that did not fit is then rendered again by the two passes).  Its
+    // 93 million rays at 1080p: projection and emission 0.50 against 0.69 ms;
+    // at 4K 2.19 against 2.72 + the metadata's scan, frame 19.7 against 20.3
+    const bool laid_out = on_device || (views_path && hint.sized && ctx->sort_mode != DL_SORT_RADIX);
+    const bool direct = laid_out && in_projection && hint.slices_ready;
     DL_CK(W.rec.reserve(16 * kRecordFloat4 * size_t(ne)), "alloc records");
     if (!direct) DL_CK(W.meta.reserve(16 * size_t(ne)), "alloc tile metadata");
     DL_CK(W.gcount.reserve(4 * size_t(ngroups + 1)), "alloc group counts");
@@ -1263,7 +1269,7 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
     uint32_t* d_status = d_meta + 7;
     // the key buffer only grows, so its capacity covers every earlier sizing
     const uint32_t key_cap =
-        on_device ? uint32_t(std::min<size_t>(W.keys[0].bytes / 8, size_t((1u << 31) - 2))) : 0u;
+        laid_out ? uint32_t(std::min<size_t>(W.keys[0].bytes / 8, size_t((1u << 31) - 2))) : 0u;
     const void* attrs[5] = {S.mean.p, S.log_scale.p, S.rot.p, S.opacity.p, S.sh.p};
     const int4* gwork = mode == DL_STANDARD ? nullptr : G->gwork.as<int4>();
     const int64_t n_work = mode == DL_STANDARD ? ngroups : G->n_gwork;
@@ -1340,13 +1346,14 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
         sl.start_alt = next;
         sl.use_alt = d_redo;
         sl.cursor = cursor;
-        // (the key buffer is final: the partition can store the frame's table)
-        single.dst = W.fdesc.as<FrameDesc>();
-        single.prefix = prefix;
-        single.done = d_meta + 8;
-        DL_CK(launch_partition_warp(gwork, n_work, sl, uint32_t(ctx->warp_cap),
-                                    ctx->warp_cap < 1024 ? 1024u : 0u, items, block_items, d_meta,
-                                    nullptr, key_cap, d_status, single, s),
+        if (warp_path) {  // the key buffer is final: the partition stores the frame's table
+            single.dst = W.fdesc.as<FrameDesc>();
+            single.prefix = prefix;
+            single.done = d_meta + 8;
+        }
+        const uint32_t cap1 = warp_path ? uint32_t(ctx->warp_cap) : 512u;
+        DL_CK(launch_partition_warp(gwork, n_work, sl, cap1, cap1 < 1024u ? 1024u : 0u, items,
+                                    block_items, d_meta, nullptr, key_cap, d_status, single, s),
               "partition");
         hint.cur ^= 1;
     } else {
@@ -1414,21 +1421,42 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
                                                                    binned_threads);
         binned = ctx->sort_mode != DL_SORT_RADIX && max_len <= kLargeCap &&
                  class_smem <= max_smem_optin(ctx->device);
+        if (direct) {
+            // the standard paradigm's keys are in their slices, unless they (or
+            // a list) outgrew what this signature was sized for
+            const int64_t end = reinterpret_cast<const uint32_t*>(
+                reinterpret_cast<const char*>(W.h_total) + 64)[0];
+            if (end * 100 > hint.key_cap * 85) hint.sized = false;  // sized again next time
+            if (h_meta[7] != 0u || !binned) {
+                hint.sized = false;
+                if (timing) {
+                    W.pending.pop_back();
+                    W.ev_free.push_back(E);
+                }
+                return render_frame(ctx, scene_id, display_id, L0_c2w, asked, out, kind, s, cs);
+            }
+        }
         if (ctx->sort_mode == DL_SORT_BINNED && !binned)
             return fail(ctx, DL_ERR_CAPACITY, "a tile list holds %lld keys (binned limit %d)",
                         (long long)max_len, kLargeCap);
         // capacities for the signature's later frames: a quarter more keys
         // (and 65,536) than the slices this frame's counts lay out (its keys,
         // an eighth more and 16 a group), lists up to 1.25 times its longest
-        hint.sized = false;
-        hint.slices_ready = false;
-        if (warp_path && binned) {
+        if (!direct) {
+            hint.sized = false;
+            hint.slices_ready = false;
+        }
+        if ((warp_path || views_path) && binned && !direct) {
             const int64_t laid = nk + nk / 8 + 16 * ngroups;
             const int64_t want = laid + laid / 4 + 65536;
             const int bc = std::min(kLargeCap, list_capacity(max_len + max_len / 4));
-            if (want < (int64_t(1) << 31) - 2 && block_smem_bytes(bc) <= max_smem_optin(ctx->device)) {
-                DL_CK(W.keys[0].reserve(8 * size_t(want)), "alloc keys");
-                hint.sized = true;
+            if (want < (int64_t(1) << 31) - 2 &&
+                (views_path || block_smem_bytes(bc) <= max_smem_optin(ctx->device))) {
+                const cudaError_t room = W.keys[0].reserve(8 * size_t(want));
+                // (the standard paradigm's views may leave no room for the
+                // larger buffer: its frames then keep to the two passes)
+                if (warp_path) DL_CK(room, "alloc keys");
+                hint.sized = room == cudaSuccess;
                 hint.key_cap = want;
                 hint.block_cap = bc;
             }
@@ -1466,7 +1494,7 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
                                      on_device ? d_nkeys : nullptr, key_cap,
                                      on_device ? d_status : nullptr, s),
                   "emit binned");
-            if (warp_path && hint.sized && in_projection) {
+            if ((warp_path || views_path) && hint.sized && in_projection) {
                 // the signature's first slices for keys emitted by the
                 // projection, from this frame's counts
                 for (DevBuf& b : hint.slices)
@@ -1615,6 +1643,8 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
     fs.n_launches = launches;
     if (!on_device) {
         fs.n_keys = nk;
+        fs.reemitted = direct && reinterpret_cast<const uint32_t*>(
+                                     reinterpret_cast<const char*>(W.h_total) + 64)[1] != 0u;
         fs.n_visible = n_visible;
         fs.lists_small = n_small + n_mid;
         fs.lists_large = n_large;
@@ -1630,6 +1660,7 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
         pf.lists_small = fs.lists_small;
         pf.lists_large = fs.lists_large;
         pf.max_list = fs.max_list;
+        pf.reemitted = fs.reemitted;
     }
     W.last_bytes = W.footprint();
     if (kind == kOutHost) {

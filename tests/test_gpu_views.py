@@ -94,3 +94,24 @@ def test_views_saturating_pixels_stop(renderer):
     assert ((got >= ref["lo"] - 2e-3) & (got <= ref["hi"] + 2e-3)).all()
     r.free_display(did)
     r.free_scene(sid)
+
+
+def test_views_keys_outgrow_their_slices(renderer):
+    """The projection emits a frame's keys into slices laid out from the frame
+    before: a small move fits, a larger one emits again, and one that needs
+    many times the keys is rendered again from the start.  Every frame is the
+    radix path's."""
+    r = renderer
+    scene = W.make_scene(W.SceneSpec(3000, 1, "uniform", "f32", seed=8))
+    scene["mean"] *= np.float32(0.3)
+    d = W.Display(200, 120, 4, 5.3, 1 / 6, view_span_deg=10.0)
+    sid, did = r.load_gaussians(scene, "f32"), r.set_display(d)
+    poses = [(30.0, 0.0), (30.0, 0.2), (24.0, 1.0), (0.8, 0.0), (0.8, 0.1), (30.0, 0.0)]
+    L0s = [W.light_field_centre(distance, yaw) for distance, yaw in poses]
+    frames = [_render(r, sid, did, L0) for L0 in L0s]
+    for L0, (img, st) in zip(L0s, frames):
+        radix, _ = _render(r, sid, did, L0, sort="radix")
+        assert np.array_equal(img, radix)
+    assert any(st["reemitted"] for _, st in frames)
+    r.free_display(did)
+    r.free_scene(sid)
