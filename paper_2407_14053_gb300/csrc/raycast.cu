@@ -695,8 +695,8 @@ rc_trace_kernel(const float4* __restrict__ gauss, const RayNode* __restrict__ no
 //
 // Bound by the latency of the candidates' evaluation and insertion at half the
 // lanes (rays have different numbers of candidates in a batch).  1080p frame,
-// 200k Gaussians, c_h 128: 4.38 ms, of which outlines and keys 0.28, cast 2.5,
-// blend 1.6; the tree walk takes 10.0 ms.
+// 200k Gaussians, c_h 128: 3.8 ms, of which outlines and keys 0.28, cast 2.4,
+// blend 1.2; the tree walk takes 10.0 ms.
 constexpr int kCastCap = 512;
 constexpr int kCastWarps = 4;
 constexpr int kCastBlocks = 4;  // resident blocks an SM
@@ -866,28 +866,138 @@ __global__ void __launch_bounds__(kCastWarps * 32, 5) rc_cast_kernel(CastParams 
 
 constexpr int kBlendThreads = 256;
 
+// Four lanes of a warp blend a ray's list four intersections at a time.  Lane q
+// evaluates intersection k + q; the lanes step the transmittance through the
+// four together, in order.  Each intersection's SH coefficients are then read
+// by all four lanes, 64 contiguous bytes a load (lane q takes the 16-byte
+// pieces q, q + 4, ...), and the four lanes' partial sums are reduced so that
+// lane q ends with the colour of its own intersection.  Float f of a row
+// belongs to channel f mod 3: lane q's sum s holds channel (s + q V) mod 3, V the
+// floats of a piece, and the exchanges pick the matching sum of the partner.
+template <typename T, int DEG>
+__device__ __forceinline__ void blend_quads(const CastList& list, int n, const float4* __restrict__ gauss,
+                                            const T* __restrict__ sh, const Ray& r, float* o) {
+    constexpr int NC = (DEG + 1) * (DEG + 1), NP = sh_pieces<T, DEG>(), V = 16 / int(sizeof(T));
+    constexpr int R = (NP + 3) / 4;  // pieces a lane
+    const int lane = threadIdx.x & 31, q = lane & 3, quad = lane & ~3;
+    float Y[16];
+    sh_basis<DEG>(r.dx, r.dy, r.dz, Y);
+    float y[R][V];  // the basis values of the lane's floats
+#pragma unroll
+    for (int i = 0; i < R; ++i)
+#pragma unroll
+        for (int e = 0; e < V; ++e) {
+            y[i][e] = 0.f;
+#pragma unroll
+            for (int l = 0; l < 4; ++l)
+                if (l + 4 * i < NP && q == l) y[i][e] = Y[((l + 4 * i) * V + e) / 3];
+        }
+    float tr = 1.f, c[3] = {0.f, 0.f, 0.f};
+    bool live = n > 0;
+    uint32_t g = q < n ? uint32_t(list.get(q)) : 0u;
+    for (int k = 0; __any_sync(0xffffffffu, live); k += 4) {
+        const uint32_t next = live && k + 4 + q < n ? uint32_t(list.get(k + 4 + q)) : 0u;
+        float a = 0.f, t;
+        if (live && k + q < n) a = rc_alpha(gauss, g, r.ox, r.oy, r.oz, r.dx, r.dy, r.dz, t);
+        float w = 0.f;
+        uint32_t used = 0u;  // the intersections that are blended
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+            const float ah = __shfl_sync(0xffffffffu, a, quad + h);
+            const float tn = tr * (1.f - ah);
+            live = live && k + h < n && !(tn < 1e-4f);
+            if (live) {
+                if (q == h) w = ah * tr;
+                tr = tn;
+                used |= 1u << h;
+            }
+        }
+        float acc[4][3];
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+            const int64_t gh = __shfl_sync(0xffffffffu, g, quad + h);
+            acc[h][0] = acc[h][1] = acc[h][2] = 0.f;
+            if ((used >> h) & 1u) {
+                const uint4* row = reinterpret_cast<const uint4*>(sh + gh * (3 * NC)) + q;
+                uint4 raw[R];
+#pragma unroll
+                for (int i = 0; i < R; ++i)
+                    raw[i] = q + 4 * i < NP ? __ldg(row + 4 * i) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+                for (int i = 0; i < R; ++i) {
+                    T v[V];
+                    memcpy(v, &raw[i], 16);
+#pragma unroll
+                    for (int e = 0; e < V; ++e)
+                        acc[h][(4 * i * V + e) % 3] = fmaf(y[i][e], to_f(v[e]), acc[h][(4 * i * V + e) % 3]);
+                }
+            }
+        }
+        // lanes 0 and 1 keep intersections k and k + 1, lanes 2 and 3 the others;
+        // then an even lane the first of its two
+        constexpr int D2 = 2 * V % 3, D1 = V % 3;
+        const bool hi = q & 2, odd = q & 1;
+        float two[2][3], col[3];
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int s = 0; s < 3; ++s) {
+                const float send = hi ? acc[h][(s + 3 - D2) % 3] : acc[h + 2][(s + D2) % 3];
+                two[h][s] = (hi ? acc[h + 2][s] : acc[h][s]) + __shfl_xor_sync(0xffffffffu, send, 2);
+            }
+#pragma unroll
+        for (int s = 0; s < 3; ++s) {
+            const float send = odd ? two[0][(s + 3 - D1) % 3] : two[1][(s + D1) % 3];
+            col[s] = (odd ? two[1][s] : two[0][s]) + __shfl_xor_sync(0xffffffffu, send, 1);
+            c[s] = fmaf(w, fmaxf(col[s] + 0.5f, 0.f), c[s]);
+        }
+        g = next;
+    }
+    // the lanes' colours, by channel, added up; lane q < 3 writes channel q
+    const int turn = q * V % 3;  // sum s is channel (s + turn) mod 3
+    float out = 0.f;
+#pragma unroll
+    for (int ch = 0; ch < 3; ++ch) {
+        const float mine = turn == 0 ? c[ch] : turn == 1 ? c[(ch + 2) % 3] : c[(ch + 1) % 3];
+        float sum = mine + __shfl_xor_sync(0xffffffffu, mine, 2);
+        sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+        if (q == ch) out = sum;
+    }
+    if (n >= 0 && q < 3) o[q] = out;
+}
+
 // Blends the lists that rc_cast_kernel found for a chunk's rays (count >= 0: a
-// ray of this chunk), a thread a ray.  A kernel of its own: what it needs is
-// the first-level cache (neighbouring rays, and the views of a tile, blend
-// nearly the same Gaussians) and many warps in flight, where the cast needs
-// shared memory.  Bound by the lines its gathers look up in that cache (15
-// loads of up to 32 lines a step); at the end of the cast's own loop, with
-// little of it left, the blending took 3.4 of 5.7 ms at 1080p.  Copying the
-// step's Gaussians to shared memory row by row instead was no faster there
-// (5.2 ms: it gave up the cache altogether).
+// ray of this chunk).  A kernel of its own: what it needs is the first-level
+// cache (neighbouring rays, and the views of a tile, blend nearly the same
+// Gaussians) and many warps in flight, where the cast needs shared memory; at
+// the end of the cast's own loop, with little of that cache left, the blending
+// took 3.4 of 5.7 ms at 1080p.  It is bound by the cache lines its gathers look
+// up: a thread a ray looks up to 32 lines for each of 15 loads a step, four
+// lanes a ray (blend_quads, where the coefficients come in whole 16-byte pieces)
+// 32 for three of them and 8 for the twelve others.  1080p, 200k Gaussians, FP32
+// SH3, c_h 128: 1.66 -> 1.16 ms.
 template <typename T, int DEG>
 __global__ void __launch_bounds__(kBlendThreads) rc_blend_kernel(CastParams P, const T* __restrict__ sh) {
     if (P.skip && *P.skip) return;
-    const int64_t j = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-    if (j >= P.chunk + kCastSpill) return;
-    const int n = P.count[j];
-    if (n < 0) return;
-    const int64_t i = P.ray0 + j;
+    constexpr bool kQuads = sh_pieces<T, DEG>() > 0;
+    const int64_t tid = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+    const int64_t j = kQuads ? tid >> 2 : tid;
+    const bool in = j < P.chunk + kCastSpill;
+    const int n = in ? P.count[j] : -1;
+    if (kQuads ? __all_sync(0xffffffffu, n < 0) : n < 0) return;
+    const int64_t jj = n < 0 ? 0 : j;  // (a lane without a ray blends nothing)
+    const int64_t i = P.ray0 + (n < 0 ? 0 : j);
     const int2 order = P.grouped[i];
     const Ray ray = make_ray(P.cams[P.ray_view[order.y]], uint32_t(order.x), P.focal, P.half_w, P.half_h);
-    blend_hits<T, DEG>(CastList{P.hits + j, P.chunk + kCastSpill}, n, P.gauss, sh, ray,
-                       P.raycol + 3 * i);
+    const CastList list{P.hits + jj, P.chunk + kCastSpill};
+    if constexpr (kQuads)
+        blend_quads<T, DEG>(list, n, P.gauss, sh, ray, P.raycol + 3 * i);
+    else
+        blend_hits<T, DEG>(list, n, P.gauss, sh, ray, P.raycol + 3 * i);
 }
+// lanes a ray
+template <typename T, int DEG>
+constexpr int blend_lanes() { return sh_pieces<T, DEG>() > 0 ? 4 : 1; }
 
 int grid_of(int64_t n, int block) {
     int64_t g = (n + block - 1) / block;
@@ -1076,7 +1186,8 @@ cudaError_t launch_cast(CastParams p, int64_t n_rays, void* tmp, const void* sh,
         e = cudaMemsetAsync(p.count, 0xFF, 4 * size_t(rays + 1), s);
         if (e != cudaSuccess) return e;
         rc_cast_kernel<<<unsigned(need < fit ? need : fit), kCastWarps * 32, smem, s>>>(p);
-        rc_blend_kernel<T, DEG><<<unsigned((rays + kBlendThreads - 1) / kBlendThreads), kBlendThreads, 0, s>>>(p, static_cast<const T*>(sh));
+        rc_blend_kernel<T, DEG><<<unsigned((rays * blend_lanes<T, DEG>() + kBlendThreads - 1) / kBlendThreads),
+                                  kBlendThreads, 0, s>>>(p, static_cast<const T*>(sh));
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }

@@ -72,3 +72,26 @@ def test_a_frame_that_outgrows_its_lists_is_complete(renderer):
         _check(img, scene, d, L0, sub)
     r.free_display(did)
     r.free_scene(sid)
+
+
+# four lanes blend a ray where the SH coefficients are whole 16-byte pieces (3,
+# 6 or 12 of them), one lane where they are not; lists shorter than four, not a
+# multiple of four, and cut by the transmittance
+@pytest.mark.parametrize("dtype,degree", [("f32", 0), ("f32", 1), ("f32", 3), ("bf16", 1),
+                                          ("bf16", 3), ("f16", 3)])
+@pytest.mark.parametrize("cap", [1, 6, 128])
+def test_blending_by_pieces(renderer, dtype, degree, cap):
+    r = renderer
+    scene = W.make_scene(W.SceneSpec(900, degree, "uniform", dtype, seed=degree + cap))
+    d = W.Display(37, 29, 5, 5.3, 1 / 6, view_span_deg=15.0)
+    sid, did = r.load_gaussians(scene, dtype), r.set_display(d)
+    r.set_heap_capacity(cap)
+    try:
+        L0 = W.light_field_centre(3.0, 1.0)
+        img = r.render(sid, did, L0, "raycast").cpu().numpy()
+        stored = scene if dtype == "f32" else W.quantise_storage(scene, dtype)
+        _check(img, stored, d, L0, np.arange(img.size), cap)
+    finally:
+        r.set_heap_capacity(128)
+        r.free_display(did)
+        r.free_scene(sid)
