@@ -380,7 +380,8 @@ static void apply_readback(dl_ctx* ctx, Readback& r) {
     const int32_t status = int32_t(m[7]);
     if (r.hint && (status != 0 || nkeys * 100 > r.hint->key_cap * 85 ||
                    slice_end * 100 > r.hint->key_cap * 85 ||
-                   longest * 100 > int64_t(r.hint->block_cap) * 85))
+                   longest * 100 > int64_t(r.hint->block_cap) * 85 ||
+                   longest > int64_t(r.hint->block_keys)))
         r.hint->sized = false;
     if (status != 0) ++W.dropped;
     for (PendingFrame& f : W.pending)
@@ -1397,7 +1398,7 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
     if (on_device) {
         // upper bounds: the persistent kernels read the item counts on the device
         n_small = n_mid = n_large = n_work;
-        cap_large = hint.block_cap;
+        cap_large = hint.block_keys;
         nk = int64_t(key_cap);
     } else {
         DL_CK(cudaMemcpyAsync(W.h_total, W.small.p, 256, cudaMemcpyDeviceToHost, s), "copy totals");
@@ -1441,24 +1442,34 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
                         (long long)max_len, kLargeCap);
         // capacities for the signature's later frames: a quarter more keys
         // (and 65,536) than the slices this frame's counts lay out (its keys,
-        // an eighth more and 16 a group), lists up to 1.25 times its longest
+        // an eighth more and 16 a group), lists up to the power of two above
+        // 1.25 times its longest, of which shared memory takes 1.25 times
         if (!direct) {
             hint.sized = false;
             hint.slices_ready = false;
         }
         if ((warp_path || views_path) && binned && !direct) {
-            const int64_t laid = nk + nk / 8 + 16 * ngroups;
-            const int64_t want = laid + laid / 4 + 65536;
-            const int bc = std::min(kLargeCap, list_capacity(max_len + max_len / 4));
+            const int64_t laid = slice_entries(nk, ngroups);
+            int64_t want = laid + laid / 4 + 65536;
+            int bc = 2048;
+            while (bc < kLargeCap && bc < max_len + max_len / 4) bc <<= 1;
             if (want < (int64_t(1) << 31) - 2 &&
                 (views_path || block_smem_bytes(bc) <= max_smem_optin(ctx->device))) {
-                const cudaError_t room = W.keys[0].reserve(8 * size_t(want));
+                cudaError_t room = cudaErrorMemoryAllocation;
+                if (in_projection) {  // as many keys again in slices
+                    const int64_t most =
+                        std::min(slice_entries(want, ngroups), (int64_t(1) << 31) - 2);
+                    room = W.keys[0].reserve(8 * size_t(most));
+                    if (room == cudaSuccess) want = most;
+                }
+                if (room != cudaSuccess) room = W.keys[0].reserve(8 * size_t(want));
                 // (the standard paradigm's views may leave no room for the
                 // larger buffer: its frames then keep to the two passes)
                 if (warp_path) DL_CK(room, "alloc keys");
                 hint.sized = room == cudaSuccess;
                 hint.key_cap = want;
                 hint.block_cap = bc;
+                hint.block_keys = std::min(bc, list_capacity(max_len + max_len / 4));
             }
         }
     }
@@ -1539,9 +1550,13 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
             // the classes beside one another, the longest lists first
             DL_CK(W.side.create(2), "streams");
             DL_CK(W.side.fork(s, 2), "fork");
-            DL_CK(launch_composite_rays_block(cap_large, dF, prefix, 1, n_large, d_meta + 6, pairs,
-                                              W.side.st[0]),
+            const int longest = on_device ? hint.block_cap : cap_large;
+            DL_CK(launch_composite_rays_block(cap_large, longest, dF, prefix, 1, n_large, d_meta + 6,
+                                              pairs, W.side.st[0]),
                   "composite rays (block per group)");
+            DL_CK(launch_composite_rays_long(cap_large, longest, dF, prefix, pairs, W.side.st[0]),
+                  "composite rays (longer lists)");
+            launches += longest > cap_large ? 1 : 0;
             DL_CK(launch_composite_rays_warp(1024, 1, dF, prefix, 1, n_mid, d_meta + 5, pairs,
                                              W.side.st[1]),
                   "composite rays (warp per group, 1024 keys)");

@@ -243,7 +243,7 @@ dl_status enqueue(dl_batch* b, cudaStream_t main) {
         DL_CK(launch_batch_prefix(b->frames_d(), n_act, prefix, main), "prefix");
         // the classes beside one another, the longest lists first
         DL_CK(b->side.fork(main, 2), "fork");
-        DL_CK(launch_composite_rays_block(b->block_cap, b->frames_d(), prefix, n_act, max_items,
+        DL_CK(launch_composite_rays_block(b->block_cap, b->block_cap, b->frames_d(), prefix, n_act, max_items,
                                           cur + 2, nullptr, b->side.st[0]),
               "composite rays (block class)");
         DL_CK(launch_composite_rays_warp(kWarpCap2, 1, b->frames_d(), prefix, n_act, max_items,
@@ -341,12 +341,12 @@ dl_status dl_batch_create(dl_ctx* ctx, int32_t n_slots, const dl_slot_plan* plan
         z.ng_cap = int64_t(D->q.nv) * G->ntiles;
         z.nrays_cap = D->rep.n_rays;
         z.nwork_cap = G->n_gwork;
-        // room for the slices the keys are emitted into (count + count/8 +
-        // 16 a group) when the projection emits them
-        const int64_t nk = ctx->stats.n_keys;
-        const int64_t laid = nk + nk / 8 + 16 * z.ng_cap;
-        z.key_cap = std::min<int64_t>(int64_t(std::ceil(double(laid) * margin)) + 4096,
-                                      (int64_t(1) << 31) - 2);
+        // room for `margin` times the slices that this frame's keys take, and
+        // for the slices of that many keys
+        const int64_t laid = slice_entries(ctx->stats.n_keys, z.ng_cap);
+        z.key_cap = std::min<int64_t>(
+            slice_entries(int64_t(std::ceil(double(laid) * margin)) + 4096, z.ng_cap),
+            (int64_t(1) << 31) - 2);
         longest = std::max<int64_t>(longest, int64_t(std::ceil(double(ctx->stats.max_list) * margin)));
         scan_bytes = std::max({scan_bytes, scan_tmp_bytes(z.ng_cap + 1), slice_tmp_bytes(z.ng_cap)});
     }

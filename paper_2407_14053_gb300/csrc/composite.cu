@@ -1078,6 +1078,43 @@ composite_rays_warp_kernel(const FrameDesc* __restrict__ F, const int64_t* __res
     if (COUNT) count_pairs(pairs, evals, blended);
 }
 
+// Warp q's part of a group whose list a block has sorted: the rays in quadrant q
+// of the tile, over the records marked for it.
+__device__ __forceinline__ void composite_quadrant(const FrameDesc& d, const int4& wi, const uint32_t* idx,
+                                                   int len, QuadPipe& pipe, uint32_t& evals,
+                                                   uint32_t& blended) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int v = wi.x / d.cp.ntiles;
+    const int tile = wi.x - v * d.cp.ntiles;
+    const int xm = (tile % d.cp.ntx) * d.cp.tile_w + (d.cp.tile_w >> 1);
+    const int ym = (tile / d.cp.ntx) * d.cp.tile_h + (d.cp.tile_h >> 1);
+    const int qx = warp & 1, qy = warp >> 1;
+    const int64_t vbase = int64_t(v) * d.cp.n;
+    for (int r0 = wi.y; r0 < wi.z; r0 += 32) {
+        const int rid = r0 + lane;
+        const int2 ray = rid < wi.z ? d.grouped[rid] : make_int2(0, -1);
+        const int col = int(uint32_t(ray.x) & 0xFFFFu), row = int(uint32_t(ray.x) >> 16);
+        const bool mine = rid < wi.z && int(col >= xm) == qx && int(row >= ym) == qy;
+        if (!__any_sync(0xffffffffu, mine)) continue;
+        const float px = float(col) - d.cp.half_w, py = float(row) - d.cp.half_h;
+        int bx0, bx1, by0, by1;
+        warp_box(mine, col, row, bx0, bx1, by0, by1);
+        float ox, oy;
+        ray_table(pipe.rays, mine, px, py, ox, oy, bx0, bx1, by0, by1, d.cp.half_w, d.cp.half_h);
+        Acc a{1.f, 0.f, 0.f, 0.f, 0u};
+        bool done = !mine;
+        quadrant_stream(idx, len, warp, vbase, d.rec, pipe, a, done, evals, px, py, bx0, bx1, by0, by1,
+                        ox, oy);
+        if (mine) {
+            float* o = d.raycol + 3 * int64_t(rid);  // grouped order
+            o[0] = a.c0;
+            o[1] = a.c1;
+            o[2] = a.c2;
+        }
+        blended += a.blended;
+    }
+}
+
 // Block class across frames: one block of four warps per group list too long
 // for a warp (sorted together in shared memory up to `cap` keys); warp q then
 // composites the group's rays in quadrant q of the tile (x half + 2 * y half)
@@ -1086,14 +1123,15 @@ composite_rays_warp_kernel(const FrameDesc* __restrict__ F, const int64_t* __res
 // classes.
 __global__ void __launch_bounds__(kBinnedThreads)
 composite_rays_block_kernel(const FrameDesc* __restrict__ F, const int64_t* __restrict__ prefix,
-                            int n_frames, int cap, uint32_t* __restrict__ cursor,
+                            int n_frames, int2 caps, uint32_t* __restrict__ cursor,
                             unsigned long long* __restrict__ pairs) {
     extern __shared__ __align__(16) unsigned char smb[];
     __shared__ int64_t s_item;
+    const int cap = caps.x;  // keys in shared memory; caps.y: the longest list
     unsigned long long* sk = reinterpret_cast<unsigned long long*>(smb);
     uint32_t* cnt = reinterpret_cast<uint32_t*>(smb + 8 * size_t(cap));
     QuadPipe* pipes = reinterpret_cast<QuadPipe*>(smb + 4 * size_t(cap));  // after the sort
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = threadIdx.x >> 5;
     const int64_t n_items = __ldg(prefix + n_frames);
     uint32_t evals = 0, blended = 0;
     int64_t item = blockIdx.x;
@@ -1104,48 +1142,55 @@ composite_rays_block_kernel(const FrameDesc* __restrict__ F, const int64_t* __re
         const int4 wi = d.gwork[bi.z];
         const uint32_t start = uint32_t(bi.y);
         const int len = bi.w;
-        if (len > cap) {
+        if (len > caps.y) {
             if (threadIdx.x == 0) atomicOr(d.status, 2u);
-        } else {
-            const int v = wi.x / d.cp.ntiles;
-            const int tile = wi.x - v * d.cp.ntiles;
-            const int xm = (tile % d.cp.ntx) * d.cp.tile_w + (d.cp.tile_w >> 1);
-            const int ym = (tile / d.cp.ntx) * d.cp.tile_h + (d.cp.tile_h >> 1);
-            const int qx = warp & 1, qy = warp >> 1;
+        } else if (len <= cap) {  // (the ones between: composite_rays_long_kernel)
             // the keys carry the quadrant bits (bit q: the record's pixel
             // box overlaps quadrant q, x half + 2 * y half, of the tile)
             block_sort(d.keys, start, len, cap, sk, cnt);
-            const uint32_t* idx = block_narrow(sk, len);
-            const int64_t vbase = int64_t(v) * d.cp.n;
-            for (int r0 = wi.y; r0 < wi.z; r0 += 32) {
-                const int rid = r0 + lane;
-                const int2 ray = rid < wi.z ? d.grouped[rid] : make_int2(0, -1);
-                const int col = int(uint32_t(ray.x) & 0xFFFFu), row = int(uint32_t(ray.x) >> 16);
-                const bool mine = rid < wi.z && int(col >= xm) == qx && int(row >= ym) == qy;
-                if (!__any_sync(0xffffffffu, mine)) continue;
-                const float px = float(col) - d.cp.half_w, py = float(row) - d.cp.half_h;
-                int bx0, bx1, by0, by1;
-                warp_box(mine, col, row, bx0, bx1, by0, by1);
-                float ox, oy;
-                ray_table(pipes[warp].rays, mine, px, py, ox, oy, bx0, bx1, by0, by1, d.cp.half_w,
-                          d.cp.half_h);
-                Acc a{1.f, 0.f, 0.f, 0.f, 0u};
-                bool done = !mine;
-                quadrant_stream(idx, len, warp, vbase, d.rec, pipes[warp], a, done, evals, px, py,
-                                bx0, bx1, by0, by1, ox, oy);
-                if (mine) {
-                    float* o = d.raycol + 3 * int64_t(rid);  // grouped order
-                    o[0] = a.c0;
-                    o[1] = a.c1;
-                    o[2] = a.c2;
-                }
-                blended += a.blended;
-            }
+            composite_quadrant(d, wi, block_narrow(sk, len), len, pipes[warp], evals, blended);
         }
         __syncthreads();  // shared memory reused by the next item
         if (threadIdx.x == 0) s_item = int64_t(gridDim.x) + int64_t(atomicAdd(cursor, 1u));
         __syncthreads();
         item = s_item;
+    }
+    if (pairs) count_pairs(pairs, evals, blended);
+}
+
+// One frame's block lists of more than caps.x and at most caps.y keys: lists
+// that outgrew the shared memory their signature was sized for, sorted where
+// they lie (a slice of the key buffer is its group's own).  Few frames hold any
+// (the next one is sized again), so a block looks through its share of the items
+// a thread each.  Within the block class's kernel it cost that 3 % (7.9-inch
+// panel, whole frame 2.07 -> 2.11 ms).
+__global__ void __launch_bounds__(kBinnedThreads)
+composite_rays_long_kernel(const FrameDesc* __restrict__ F, const int64_t* __restrict__ prefix, int2 caps,
+                           unsigned long long* __restrict__ pairs) {
+    __shared__ QuadPipe pipes[kBinnedThreads / 32];
+    __shared__ uint32_t s_long[kBinnedThreads / 32];
+    const FrameDesc& d = *F;
+    const int64_t n_items = prefix[1];
+    const int warp = threadIdx.x >> 5;
+    uint32_t evals = 0, blended = 0;
+    for (int64_t i0 = 0; i0 * gridDim.x + blockIdx.x < n_items; i0 += kBinnedThreads) {
+        const int64_t mine = (i0 + threadIdx.x) * gridDim.x + blockIdx.x;
+        const int len = mine < n_items ? d.block_items[mine].w : 0;
+        const uint32_t m = __ballot_sync(0xffffffffu, len > caps.x && len <= caps.y);
+        if ((threadIdx.x & 31) == 0) s_long[warp] = m;
+        __syncthreads();
+        for (int w = 0; w < kBinnedThreads / 32; ++w) {
+            for (uint32_t left = s_long[w]; left; left &= left - 1u) {
+                const int t = 32 * w + __ffs(left) - 1;
+                const int4 bi = d.block_items[(i0 + t) * gridDim.x + blockIdx.x];
+                unsigned long long* const own =
+                    const_cast<unsigned long long*>(d.keys) + uint32_t(bi.y);
+                bitonic_sort(own, bi.w);
+                composite_quadrant(d, d.gwork[bi.z], block_narrow(own, bi.w), bi.w, pipes[warp], evals,
+                                   blended);
+            }
+        }
+        __syncthreads();  // s_long is written again
     }
     if (pairs) count_pairs(pairs, evals, blended);
 }
@@ -1856,10 +1901,10 @@ cudaError_t launch_composite_views(const CompositeParams& p, const int4* items,
 }
 
 namespace {
-template <class K>
+template <class K, class Extra>
 cudaError_t launch_persistent(K kernel, int threads, size_t smem, int64_t max_blocks,
                               const FrameDesc* frames, const int64_t* prefix, int32_t n_frames,
-                              int extra, uint32_t* cursor, unsigned long long* pairs, cudaStream_t s) {
+                              Extra extra, uint32_t* cursor, unsigned long long* pairs, cudaStream_t s) {
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     if (e != cudaSuccess) return e;
     int per_sm = 0;
@@ -1897,13 +1942,22 @@ cudaError_t launch_composite_rays_warp(int cap, int cls, const FrameDesc* frames
                                      n_frames, cls, cursor, pairs, s);
 }
 
-cudaError_t launch_composite_rays_block(int block_cap, const FrameDesc* frames,
+cudaError_t launch_composite_rays_block(int block_cap, int longest, const FrameDesc* frames,
                                         const int64_t* prefix, int32_t n_frames, int64_t max_items,
                                         uint32_t* cursor, unsigned long long* pairs, cudaStream_t s) {
     if (max_items <= 0 || n_frames <= 0) return cudaSuccess;
     const size_t smem = block_smem_bytes(block_cap);
     return launch_persistent(composite_rays_block_kernel, kBinnedThreads, smem, max_items, frames,
-                             prefix + 2 * (n_frames + 1), n_frames, block_cap, cursor, pairs, s);
+                             prefix + 2 * (n_frames + 1), n_frames,
+                             make_int2(block_cap, std::max(block_cap, longest)), cursor, pairs, s);
+}
+
+cudaError_t launch_composite_rays_long(int block_cap, int longest, const FrameDesc* frame,
+                                       const int64_t* prefix, unsigned long long* pairs, cudaStream_t s) {
+    if (longest <= block_cap) return cudaSuccess;
+    composite_rays_long_kernel<<<unsigned(num_sms() * 4), kBinnedThreads, 0, s>>>(
+        frame, prefix + 4, make_int2(block_cap, longest), pairs);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_partition_warp(const int4* gwork, int64_t n_work, const GroupSlices& slices,

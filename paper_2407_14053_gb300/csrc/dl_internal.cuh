@@ -435,13 +435,17 @@ cudaError_t launch_composite_rays_warp(int cap, int cls, const FrameDesc* frames
                                        const int64_t* prefix, int32_t n_frames, int64_t max_items,
                                        uint32_t* cursor, unsigned long long* pairs, cudaStream_t s);
 // Block class (the block lists: lists too long for the warp classes, up to
-// block_cap keys, a multiple of 512 <= 16384; longer lists set status bit 1 and
-// are skipped), persistent: four warps sort a list together, then warp q
-// composites the rays in quadrant q of the tile over the records whose key
-// marks quadrant q.
-cudaError_t launch_composite_rays_block(int block_cap, const FrameDesc* frames,
+// block_cap keys, a multiple of 512 <= 16384; lists of more than `longest` set
+// status bit 1, those between are left to launch_composite_rays_long),
+// persistent: four warps sort a list together, then warp q composites the rays
+// in quadrant q of the tile over the records whose key marks quadrant q.
+cudaError_t launch_composite_rays_block(int block_cap, int longest, const FrameDesc* frames,
                                         const int64_t* prefix, int32_t n_frames, int64_t max_items,
                                         uint32_t* cursor, unsigned long long* pairs, cudaStream_t s);
+// One frame's block lists of more than block_cap and at most `longest` keys, sorted
+// in the key buffer; nothing is launched when longest <= block_cap.
+cudaError_t launch_composite_rays_long(int block_cap, int longest, const FrameDesc* frame,
+                                       const int64_t* prefix, unsigned long long* pairs, cudaStream_t s);
 // Splits work entries by their group's key count: <= small_cap -> small
 // list, else large list; meta = {n_small, n_large, max count}.  gwork NULL:
 // the entries are the groups 0..n_work-1 themselves.

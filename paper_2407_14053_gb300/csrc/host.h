@@ -106,7 +106,8 @@ struct PendingFrame {
 // capacities, with no host synchronisation; a frame that exceeds them is
 // dropped on the device (its output left untouched, its status word set),
 // and the next frame of the signature is sized on the host again, as is one
-// after a frame that used more than 85 % of either capacity.
+// after a frame that used more than 85 % of either capacity or had a list that
+// its block class could not sort in shared memory.
 // With the keys emitted by the projection, the signature also keeps the
 // slices of the key buffer its next frame emits into: every group gets its
 // key count in the last frame plus an eighth and 16 (slices[cur]); a frame
@@ -117,6 +118,10 @@ struct PendingFrame {
 // 115 us a frame at 2,000 Gaussians, 365 against 388 at 41,003, 607 against
 // 675 at 120,000 (frames of 240x135 and 955x541).
 inline bool emit_in_projection(int32_t option) { return option != 0; }
+// Key buffer entries that the slices of `keys` keys in `groups` groups take at
+// most (slice_layout_kernel): a capacity meant for `keys` keys holds this many,
+// so that no frame of so many is dropped for its slices' padding.
+inline int64_t slice_entries(int64_t keys, int64_t groups) { return keys + keys / 8 + 16 * groups; }
 
 // Streams beside the caller's for work of one launch sequence that is
 // independent of itself.  fork() makes them wait for the caller's stream,
@@ -165,7 +170,8 @@ struct SideStreams {
 
 struct FrameHint {
     bool sized = false;
-    int32_t block_cap = 2048;
+    int32_t block_cap = 2048;   // longest list of a later frame, a power of two
+    int32_t block_keys = 2048;  // keys the block class sorts in shared memory
     int64_t key_cap = 0;
     bool slices_ready = false;
     bool no_lists = false;  // DL_RAYCAST: the tile lists do not fit; walk the tree

@@ -32,3 +32,33 @@ def test_projection_edges(n, deg, dtype, views):
             assert r.stats()["status"] == 0
             assert ((img >= ref["lo"] - 2e-3) & (img <= ref["hi"] + 2e-3)).all()
     r.close()
+
+
+@pytest.mark.parametrize("mode", ["directl", "raycast"])
+@pytest.mark.parametrize("n,w,h,views", [(60, 24, 16, 3), (2000, 240, 135, 45), (40000, 320, 200, 9)])
+def test_frames_back_to_back(mode, n, w, h, views):
+    """A frame's kernels start while the ones before them drain: frames enqueued
+    one behind the other, moving nearer and farther so that some emit their keys
+    again, equal the same frames rendered with a wait after each."""
+    from paper_2407_14053_gb300 import Renderer
+    import torch
+    scene = W.make_scene(W.SceneSpec(n, 1, "uniform", "f32", seed=n))
+    d = W.Display(w, h, views, 5.3, 1 / 6, view_span_deg=12.0)
+    poses = [W.light_field_centre(4.0 + 0.4 * (i % 5), 0.3 * i) for i in range(12)]
+    frames = []
+    for wait in (True, False):
+        r = Renderer(0)
+        sid, did = r.load_gaussians(scene, "f32"), r.set_display(d)
+        for distance in (4.0, 4.0):
+            r.render(sid, did, W.light_field_centre(distance, 0.0), mode)
+        got = []
+        for L0 in poses:
+            got.append(r.render(sid, did, L0, mode).clone())
+            if wait:
+                torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        frames.append([g.cpu().numpy() for g in got])
+        r.close()
+    for a, b in zip(*frames):
+        assert np.array_equal(a, b)
+    assert max(f.max() for f in frames[0]) > 0.05
