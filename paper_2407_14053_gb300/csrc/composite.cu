@@ -1579,6 +1579,7 @@ __global__ void partition_warp_kernel(const int4* __restrict__ gwork, int64_t n_
                                       uint32_t* __restrict__ meta,
                                       const uint32_t* __restrict__ total_keys, uint32_t key_cap,
                                       uint32_t* __restrict__ status, SingleFrame single) {
+    after_previous(gwork, S.start, S.start_alt, S.use_alt, S.cursor, total_keys, status);
     if (total_keys && *total_keys > key_cap) {  // keys were not emitted
         if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(status, 1u);
         return;
@@ -1968,10 +1969,8 @@ cudaError_t launch_partition_warp(const int4* gwork, int64_t n_work, const Group
     int64_t grid = (n_work + 255) / 256;
     const int64_t lim = int64_t(num_sms()) * 16;
     if (grid > lim) grid = lim;
-    partition_warp_kernel<<<unsigned(grid), 256, 0, s>>>(gwork, n_work, slices, cap1, cap2, items,
-                                                         block_items, meta, total_keys, key_cap,
-                                                         status, single);
-    return cudaGetLastError();
+    return launch_after(partition_warp_kernel, unsigned(grid), 256, 0, s, gwork, n_work, slices, cap1, cap2,
+                        items, block_items, meta, total_keys, key_cap, status, single);
 }
 
 cudaError_t launch_partition(const int4* gwork, int64_t n_work, const uint32_t* gstart,

@@ -8,6 +8,40 @@
 
 namespace dl {
 
+// Launch of a kernel that begins with after_previous(): its blocks may become
+// resident while the kernel before it on the stream drains, so a chain of short
+// kernels does not pay a launch between any two of them.  The chain begin frame,
+// projection, slice sums, slice layout, gated projection, partition runs so: the
+// 240 x 135 frame of 2,000 Gaussians takes 69.8 us instead of 81.8.
+template <class... K, class... A>
+inline cudaError_t launch_after(void (*kernel)(K...), unsigned grid, unsigned block, size_t smem,
+                                cudaStream_t s, A... args) {
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, K(args)...);
+}
+
+// Waits for the kernel before this one to complete, then lets the next one's
+// blocks become resident (so at most two kernels of a chain overlap).  What
+// earlier kernels write is read only after it, through the pointers given: they
+// are made opaque here, so that no load through them, read-only ones included,
+// can be moved above the wait.
+template <class... P>
+__device__ __forceinline__ void after_previous(P&... pointers) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    auto opaque = [](auto& p) { asm volatile("" : "+l"(p)::"memory"); };
+    (opaque(pointers), ...);
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 constexpr uint32_t kEmpty = 0xFFFFFFFFu;
 
 // Display constants as the kernels see them.  t3q, lq, kq are the Q32

@@ -551,7 +551,10 @@ template <typename T, int DEG, bool KEYS_ONLY>
 __global__ void __launch_bounds__(kProjectThreads, 4)
 project_direct_kernel(GaussiansView<T> G, ProjectParams p, const Cam* __restrict__ cams, int32_t nv,
                       int32_t ranges, ProjectOut out) {
-    if (KEYS_ONLY && *out.gate == 0u) return;
+    if (KEYS_ONLY) {
+        after_previous(cams, out.gate, out.slice);
+        if (*out.gate == 0u) return;
+    }
     extern __shared__ float4 s_sh[];  // [NF4][kProjectThreads], sh_slot
     const BlockWork bw = block_work<false>(nv, ranges);
     const int64_t g0 = bw.gblock * int64_t(kProjectThreads), g = g0 + threadIdx.x;
@@ -562,6 +565,8 @@ project_direct_kernel(GaussiansView<T> G, ProjectParams p, const Cam* __restrict
     if (!KEYS_ONLY)
         stage_sh<T, DEG>(G.sh, g0, int(min(p.n - g0, int64_t(kProjectThreads))), s_sh);
     if (g < p.n) gs = load_gauss(G, g);
+    // (the scene was there before the frame began)
+    if (!KEYS_ONLY) after_previous(cams, out.slice);
     const uint32_t ntiles = uint32_t(p.ntx * p.nty);
     bool over = false;
     // every warp walks the views in the same order, so the keys in flight
@@ -679,12 +684,16 @@ template <typename T, bool KEYS_ONLY>
 __global__ void __launch_bounds__(kProjectThreads, 4)
 project_outline_kernel(GaussiansView<T> G, ProjectParams p, const Cam* __restrict__ cams, int32_t nv,
                        int32_t ranges, ProjectOut out) {
-    if (KEYS_ONLY && *out.gate == 0u) return;
+    if (KEYS_ONLY) {
+        after_previous(cams, out.gate, out.slice);
+        if (*out.gate == 0u) return;
+    }
     const BlockWork bw = block_work<false>(nv, ranges);
     const int64_t g = bw.gblock * int64_t(kProjectThreads) + threadIdx.x;
     GaussState gs{};
     gs.vis = false;
     if (g < p.n) gs = load_gauss(G, g);
+    if (!KEYS_ONLY) after_previous(cams, out.slice);
     const uint32_t ntiles = uint32_t(p.ntx * p.nty);
     unsigned long long my_total = 0;
     bool over = false;
@@ -746,6 +755,7 @@ __device__ __forceinline__ uint32_t block_sum(uint32_t v) {
 __global__ void __launch_bounds__(kSliceThreads)
 slice_sums_kernel(const uint32_t* __restrict__ cursor, const uint32_t* __restrict__ slice,
                   int64_t n_groups, uint32_t* __restrict__ sums) {
+    after_previous(cursor, slice);
     const int64_t base = int64_t(blockIdx.x) * kSliceTile + threadIdx.x;
     uint32_t v = 0;
 #pragma unroll 4
@@ -759,6 +769,7 @@ __global__ void __launch_bounds__(kSliceThreads)
 slice_layout_kernel(uint32_t* cursor, const uint32_t* __restrict__ slice, int64_t n_groups,
                     const uint32_t* __restrict__ sums, uint32_t* __restrict__ next,
                     uint32_t* __restrict__ d_total, const uint32_t* __restrict__ redo) {
+    after_previous(cursor, slice, sums, redo);
     uint32_t before = 0;
     for (int b = threadIdx.x; b < int(blockIdx.x); b += kSliceThreads) before += sums[b];
     before = block_sum(before);
@@ -808,6 +819,7 @@ __global__ void begin_frame_kernel(CamBatch b, int32_t n_cams, Cam* __restrict__
                                    uint32_t* __restrict__ zero, int32_t n_zero,
                                    const uint32_t* __restrict__ layout, int64_t n_groups,
                                    uint32_t* __restrict__ cursor) {
+    after_previous(layout);
     if (blockIdx.x == 0) {
         if (int(threadIdx.x) < n_cams) dst[threadIdx.x] = b.cam[threadIdx.x];
         for (int i = threadIdx.x; i < n_zero; i += blockDim.x) zero[i] = 0u;
@@ -818,6 +830,7 @@ __global__ void begin_frame_kernel(CamBatch b, int32_t n_cams, Cam* __restrict__
 __global__ void begin_slot_kernel(uint32_t* __restrict__ zero, int32_t n_zero,
                                   const uint32_t* __restrict__ layout, int64_t n_groups,
                                   uint32_t* __restrict__ cursor, uint32_t* __restrict__ copy) {
+    after_previous(layout);
     if (blockIdx.x == 0)
         for (int i = threadIdx.x; i < n_zero; i += blockDim.x) zero[i] = 0u;
     begin_groups(layout, n_groups, cursor, copy);
@@ -852,9 +865,11 @@ cudaError_t launch_slice_layout(uint32_t* cursor, const uint32_t* slice, int64_t
                                 cudaStream_t s) {
     const unsigned grid = unsigned((n_groups + kSliceTile) / kSliceTile);  // of n_groups + 1 entries
     uint32_t* const sums = static_cast<uint32_t*>(tmp);
-    slice_sums_kernel<<<grid, kSliceThreads, 0, s>>>(cursor, slice, n_groups, sums);
-    slice_layout_kernel<<<grid, kSliceThreads, 0, s>>>(cursor, slice, n_groups, sums, next, d_total, redo);
-    return cudaGetLastError();
+    const cudaError_t e =
+        launch_after(slice_sums_kernel, grid, kSliceThreads, 0, s, cursor, slice, n_groups, sums);
+    if (e != cudaSuccess) return e;
+    return launch_after(slice_layout_kernel, grid, kSliceThreads, 0, s, cursor, slice, n_groups, sums,
+                        next, d_total, redo);
 }
 
 template <typename T>
@@ -901,17 +916,16 @@ static cudaError_t launch_project_direct_t(const void* const* attrs, const Proje
     if (blocks <= 0) return cudaSuccess;
     const int32_t ranges = view_ranges(blocks, nv);
     const unsigned grid = unsigned(blocks * ranges);
-    if (keys_only) {  // no colour: the SH degree does not matter
-        project_direct_kernel<T, 0, true><<<grid, block, 0, s>>>(G, p, cams, nv, ranges, out);
-        return cudaGetLastError();
-    }
+    auto go = [&](auto kernel, size_t smem) {
+        return launch_after(kernel, grid, block, smem, s, G, p, cams, nv, ranges, out);
+    };
+    if (keys_only) return go(project_direct_kernel<T, 0, true>, 0);  // no colour: any SH degree
     switch (p.sh_degree) {
-        case 0: project_direct_kernel<T, 0, false><<<grid, block, sh_smem_bytes<0>(), s>>>(G, p, cams, nv, ranges, out); break;
-        case 1: project_direct_kernel<T, 1, false><<<grid, block, sh_smem_bytes<1>(), s>>>(G, p, cams, nv, ranges, out); break;
-        case 2: project_direct_kernel<T, 2, false><<<grid, block, sh_smem_bytes<2>(), s>>>(G, p, cams, nv, ranges, out); break;
-        default: project_direct_kernel<T, 3, false><<<grid, block, sh_smem_bytes<3>(), s>>>(G, p, cams, nv, ranges, out); break;
+        case 0: return go(project_direct_kernel<T, 0, false>, sh_smem_bytes<0>());
+        case 1: return go(project_direct_kernel<T, 1, false>, sh_smem_bytes<1>());
+        case 2: return go(project_direct_kernel<T, 2, false>, sh_smem_bytes<2>());
+        default: return go(project_direct_kernel<T, 3, false>, sh_smem_bytes<3>());
     }
-    return cudaGetLastError();
 }
 
 cudaError_t launch_project_direct(int dtype, const void* const* attrs, const ProjectParams& p,
@@ -936,11 +950,8 @@ static cudaError_t launch_project_outline_t(const void* const* attrs, const Proj
     if (blocks <= 0) return cudaSuccess;
     const int32_t ranges = view_ranges(blocks, nv);
     const unsigned grid = unsigned(blocks * ranges);
-    if (keys_only)
-        project_outline_kernel<T, true><<<grid, kProjectThreads, 0, s>>>(G, p, cams, nv, ranges, out);
-    else
-        project_outline_kernel<T, false><<<grid, kProjectThreads, 0, s>>>(G, p, cams, nv, ranges, out);
-    return cudaGetLastError();
+    return launch_after(keys_only ? project_outline_kernel<T, true> : project_outline_kernel<T, false>, grid,
+                        kProjectThreads, 0, s, G, p, cams, nv, ranges, out);
 }
 
 cudaError_t launch_project_outline(int dtype, const void* const* attrs, const ProjectParams& p,
