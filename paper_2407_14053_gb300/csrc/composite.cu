@@ -334,6 +334,9 @@ composite_rays_kernel(CompositeParams p, const int4* __restrict__ work,
     }
 }
 
+// A thread per pixel, so blocks of up to 1024 threads (the largest tile): 40
+// registers a thread, and 48 bytes of shared memory a thread are exactly the
+// 48 KB that a block has without asking for more.
 __global__ void composite_full_kernel(CompositeParams p, const uint2* __restrict__ ranges,
                                       const uint32_t* __restrict__ vals,
                                       const float4* __restrict__ rec, float* __restrict__ Mm,
@@ -1790,7 +1793,7 @@ cudaError_t launch_composite_full(const CompositeParams& p, int32_t nv, const ui
                                   const uint32_t* vals, const float4* rec, float* Mm,
                                   unsigned long long* pairs, cudaStream_t s) {
     const int nthr = p.tile_w * p.tile_h;
-    const size_t smem = size_t(nthr) * 3 * sizeof(float4) + size_t(nthr / 32) * 64 * sizeof(int);
+    const size_t smem = size_t(nthr) * 3 * sizeof(float4);
     const int64_t blocks = int64_t(nv) * p.ntiles;
     composite_full_kernel<<<unsigned(blocks), nthr, smem, s>>>(p, ranges, vals, rec, Mm, pairs);
     return cudaGetLastError();
