@@ -1335,6 +1335,41 @@ __device__ __forceinline__ void blend_run(Px2& p, const PatchBatch& S, int k) {
     }
 }
 
+// A patch again, record by record as blend() takes them, for a lane's pixels
+// (x0, y) and (x1, y), written to o (in0, in1: those inside the view); returns
+// the records blended.  blend_run multiplies every record's colour, those below
+// the threshold by an alpha of 0, which turns a colour that overflowed to
+// infinity into NaN in every pixel of the patch, and nothing else does.  So a
+// patch that ends with a NaN comes here.  (A vote a batch for infinite colours
+// cost every frame 1.7 %: 1080p 4.72 -> 4.80 ms.  Not inlined, so that it
+// takes no registers from the loop.)
+template <bool COUNT, class Index>
+__device__ __noinline__ uint32_t patch_by_records(const uint4* masks, int comp, Index index, int len,
+                                                  const float4* __restrict__ base, float x0, float x1,
+                                                  float y, bool in0, bool in1, float* o) {
+    Acc a{1.f, 0.f, 0.f, 0.f, 0u}, b = a;
+    bool open0 = in0, open1 = in1;
+    for (int i0 = 0; i0 < len && __any_sync(0xffffffffu, open0 || open1); i0 += 32) {
+        for (unsigned m = reinterpret_cast<const unsigned*>(masks + (i0 >> 5))[comp]; m; m &= m - 1u) {
+            const float4* r = base + kRecordFloat4 * int64_t(index(i0 + __ffs(m) - 1));
+            const float4 q0 = __ldg(r), q1 = __ldg(r + 1);
+            if (open0) open0 = blend_rec<true, COUNT>(a, x0, y, q0, q1);
+            if (open1) open1 = blend_rec<true, COUNT>(b, x1, y, q0, q1);
+        }
+    }
+    if (in0) {
+        o[0] = a.c0;
+        o[1] = a.c1;
+        o[2] = a.c2;
+    }
+    if (in1) {
+        o[3] = b.c0;
+        o[4] = b.c1;
+        o[5] = b.c2;
+    }
+    return a.blended + b.blended;
+}
+
 // Composites one patch for the warp (columns from col0, rows from row0 of
 // view v): the records index(0 .. len) that masks (component `comp` of a
 // batch's uint4) select, in list order, and writes its pixels.
@@ -1402,6 +1437,12 @@ __device__ __forceinline__ void composite_patch(const CompositeParams& p, int v,
     }
     __syncwarp();
     float* o = Mm + ((int64_t(v) * p.height + row) * p.width + col) * 3;
+    const float sum = ((q.r.x + q.r.y) + (q.g.x + q.g.y)) + (q.b.x + q.b.y);
+    if (__any_sync(0xffffffffu, sum != sum)) {
+        q.blended = patch_by_records<COUNT>(masks, comp, index, len, base, q.x0, q.x1, q.y, in0, in1, o);
+        if (COUNT) blended += q.blended;
+        return;
+    }
     if (in0) {
         o[0] = q.r.x;
         o[1] = q.g.x;
@@ -1546,7 +1587,7 @@ composite_views_block_kernel(CompositeParams p, const int4* __restrict__ block_i
     block_sort(keys, uint32_t(it.y), it.w, cap, sk, cnt);
     const uint32_t* idx = block_narrow(sk, it.w);
     uint32_t evals = 0, blended = 0;
-    composite_quads<COUNT, true>(p, it.x, [&](int i) { return idx[i] >> 4; }, it.w, rec, masks,
+    composite_quads<COUNT, true>(p, it.x, [idx](int i) { return idx[i] >> 4; }, it.w, rec, masks,
                                  batches[threadIdx.x >> 5], Mm, evals, blended);
     if (COUNT) count_pairs(pairs, evals, blended);
 }
