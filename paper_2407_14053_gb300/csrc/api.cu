@@ -518,16 +518,8 @@ dl_status build_cast_lists(dl_ctx* ctx, Scene& S, Display& D, TileGroups& G, Fra
     if (hint.no_lists || ne >= (int64_t(1) << 31) || ngroups >= (int64_t(1) << 31) - 1) return DL_OK;
     const size_t words = 4 * size_t(ngroups + 1);
     // memory that the tree would not need: without it the tree renders
-    auto reserve = [&](DevBuf& b, size_t bytes) {
-        const size_t had = b.bytes;
-        if (b.reserve(bytes) == cudaSuccess) return true;
-        // the buffer was given up for the larger one: other signatures' sizing
-        // counts on it
-        if (had == 0 || b.reserve(had - had / 8) != cudaSuccess)
-            for (auto& h : ctx->hints) h.second.sized = false;
-        return false;
-    };
-    const bool sizing = !hint.sized || !hint.slices_ready;
+    auto reserve = [](DevBuf& b, size_t bytes) { return b.reserve(bytes) == cudaSuccess; };
+    const bool sizing = !hint.fits(W.keys[0]) || !hint.slices_ready;
     if (!reserve(W.rec, 16 * kRecordFloat4 * size_t(ne)) || !reserve(W.gfill, words) ||
         !reserve(W.gscan_tmp, slice_tmp_bytes(ngroups)) ||
         !reserve(hint.slices[0], words) || !reserve(hint.slices[1], words) ||
@@ -1245,7 +1237,8 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
     // signature's capacities and device counters, and are dropped on the
     // device (status word, output untouched) when they exceed them.
     FrameHint& hint = ctx->hints[FrameSig{scene_id, display_id, mode, tw, th, rw, rh}];
-    const bool on_device = warp_path && hint.sized && ctx->sort_mode != DL_SORT_RADIX;
+    const bool sized = hint.fits(W.keys[0]) && ctx->sort_mode != DL_SORT_RADIX;
+    const bool on_device = warp_path && sized;
     // keys emitted by the projection, into the slices the signature's last
     // frame laid out
     const bool in_projection = emit_in_projection(ctx->key_emission);
@@ -1253,7 +1246,7 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
     // a frame that did not fit is then rendered again by the two passes).  Its
     // 93 million rays at 1080p: projection and emission 0.50 against 0.69 ms;
     // at 4K 2.19 against 2.72 + the metadata's scan, frame 19.7 against 20.3
-    const bool laid_out = on_device || (views_path && hint.sized && ctx->sort_mode != DL_SORT_RADIX);
+    const bool laid_out = on_device || (views_path && sized);
     const bool direct = laid_out && in_projection && hint.slices_ready;
     DL_CK(W.rec.reserve(16 * kRecordFloat4 * size_t(ne)), "alloc records");
     if (!direct) DL_CK(W.meta.reserve(16 * size_t(ne)), "alloc tile metadata");
@@ -1268,7 +1261,7 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
     uint32_t* d_redo = d_total32 + 1;  // a key found its slice full (direct emission)
     uint32_t* d_meta = reinterpret_cast<uint32_t*>(W.small.as<char>() + 128);
     uint32_t* d_status = d_meta + 7;
-    // the key buffer only grows, so its capacity covers every earlier sizing
+    // all of the key buffer: at least what the signature was sized for
     const uint32_t key_cap =
         laid_out ? uint32_t(std::min<size_t>(W.keys[0].bytes / 8, size_t((1u << 31) - 2))) : 0u;
     const void* attrs[5] = {S.mean.p, S.log_scale.p, S.rot.p, S.opacity.p, S.sh.p};

@@ -177,6 +177,9 @@ struct FrameHint {
     bool no_lists = false;  // DL_RAYCAST: the tile lists do not fit; walk the tree
     int cur = 0;
     DevBuf slices[2];  // n_groups + 1 slot offsets each
+    // The key buffer is every signature's: a larger one that could not be had
+    // leaves it smaller, or gone, and this signature to be sized again.
+    bool fits(const DevBuf& keys) const { return sized && 8 * size_t(key_cap) <= keys.bytes; }
 };
 using FrameSig = std::array<int32_t, 7>;
 

@@ -1,0 +1,49 @@
+"""Frames where device memory runs short: what a call cannot have costs that
+call, and no other its frame."""
+import numpy as np
+import pytest
+import torch
+
+import workloads as W
+from memory_pressure import free_bytes
+
+pytestmark = pytest.mark.gpu
+
+MB = 1 << 20
+
+
+def _covering_scene(n, views_filled, seed=1):
+    """n faint Gaussians; with views_filled each of them reaches every tile."""
+    scene = W.make_scene(W.SceneSpec(n, 0, "uniform", "f32", seed=seed))
+    if views_filled:
+        scene["mean"] *= np.float32(0.1)
+        scene["log_scale"][:] = np.float32(1.0)
+        scene["opacity_logit"][:] = np.float32(-4.0)
+    return scene
+
+
+PANEL = W.Display(960, 540, 8, 5.3, 1 / 6, view_span_deg=8.0)
+L0 = W.light_field_centre(4.0, 1.0)
+
+
+@pytest.mark.parametrize("mode", ["directl", "standard"])
+def test_a_key_buffer_that_cannot_grow_costs_no_other_frame(mode):
+    """The key buffer is given up for a larger one that cannot be had: the
+    frames of a signature sized before come out whole."""
+    from paper_2407_14053_gb300 import DirectLError, Renderer
+    r = Renderer(0)
+    did = r.set_display(PANEL)
+    small = r.load_gaussians(_covering_scene(400, False), "f32")
+    large = r.load_gaussians(_covering_scene(4000, True), "f32")  # 4000 x 8 views x 510 tiles: 16 M keys
+    want = r.render(small, did, L0, mode).clone()
+    for _ in range(2):
+        assert torch.equal(r.render(small, did, L0, mode), want)
+    with free_bytes(96 * MB):  # of at least 130 for the keys alone
+        with pytest.raises(DirectLError, match="OOM"):
+            r.render(large, did, L0, mode)
+        for _ in range(2):
+            out = torch.full_like(want, -1.0)
+            assert torch.equal(r.render(small, did, L0, mode, out), want)
+    out = r.render(large, did, L0, mode)
+    assert torch.isfinite(out).all() and out.max() > 0.05
+    r.close()
