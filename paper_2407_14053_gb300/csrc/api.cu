@@ -452,31 +452,35 @@ static dl_status enqueue_readback(dl_ctx* ctx, FrameHint& hint, int64_t frame, c
 // calls earlier.
 enum OutKind : int32_t { kOutHost = 0, kOutDevice = 1, kOutHostAsync = 2 };
 
-dl_status out_target(dl_ctx* ctx, float* out, int32_t kind, size_t bytes, cudaStream_t s,
-                     float** dst) {
+// The frame's memory is reserved before its sizing may ask for room for later
+// frames; out_target then orders it after the copy that read it.
+dl_status reserve_out(dl_ctx* ctx, int32_t kind, size_t bytes) {
     Workspace& W = ctx->ws;
-    if (kind == kOutDevice) {
-        *dst = out;
-        return DL_OK;
-    }
-    if (kind == kOutHost) {
-        DL_CK(W.out.reserve(bytes), "alloc out");
-        *dst = W.out.as<float>();
-        return DL_OK;
-    }
+    if (kind == kOutHost) DL_CK(W.out.reserve(bytes), "alloc out");
+    if (kind != kOutHostAsync) return DL_OK;
     const int k = W.aslot;
     for (int i = 0; i < 2; ++i) {
         if (!W.ev_frame[i]) DL_CK(cudaEventCreateWithFlags(&W.ev_frame[i], cudaEventDisableTiming), "event");
         if (!W.ev_copied[i]) DL_CK(cudaEventCreateWithFlags(&W.ev_copied[i], cudaEventDisableTiming), "event");
     }
-    if (W.copy_pending[k]) {
-        if (W.aout[k].bytes < bytes)  // the frame is replaced: its copy must have ended
-            DL_CK(cudaEventSynchronize(W.ev_copied[k]), "wait for an earlier copy");
-        else
-            DL_CK(cudaStreamWaitEvent(s, W.ev_copied[k], 0), "order after an earlier copy");
-    }
+    if (W.copy_pending[k] && W.aout[k].bytes < bytes)  // the frame is replaced: its copy must have ended
+        DL_CK(cudaEventSynchronize(W.ev_copied[k]), "wait for an earlier copy");
     DL_CK(W.aout[k].reserve(bytes), "alloc out");
-    *dst = W.aout[k].as<float>();
+    return DL_OK;
+}
+
+dl_status out_target(dl_ctx* ctx, float* out, int32_t kind, cudaStream_t s, float** dst) {
+    Workspace& W = ctx->ws;
+    if (kind == kOutDevice) {
+        *dst = out;
+    } else if (kind == kOutHost) {
+        *dst = W.out.as<float>();
+    } else {
+        const int k = W.aslot;
+        if (W.copy_pending[k])
+            DL_CK(cudaStreamWaitEvent(s, W.ev_copied[k], 0), "order after an earlier copy");
+        *dst = W.aout[k].as<float>();
+    }
     return DL_OK;
 }
 
@@ -605,6 +609,10 @@ dl_status render_raycast(dl_ctx* ctx, int32_t scene_id, int32_t display_id, Scen
     TileGroups* G = nullptr;
     st = get_groups(ctx, D, R, ctx->tile[DL_DIRECTL][0], ctx->tile[DL_DIRECTL][1], s, &G);
     if (st) return st;
+    const size_t out_bytes = 12 * size_t(w) * size_t(h);
+    st = reserve_out(ctx, kind, out_bytes);
+    if (st) return st;
+    DL_CK(W.raycol.reserve(12 * size_t(R.n_rays > 0 ? R.n_rays : 1)), "alloc ray colours");
     FrameHint& hint = ctx->hints[FrameSig{scene_id, display_id, DL_RAYCAST, G->tw, G->th, w, h}];
     GroupSlices sl;
     uint32_t* over = nullptr;
@@ -621,7 +629,6 @@ dl_status render_raycast(dl_ctx* ctx, int32_t scene_id, int32_t display_id, Scen
         if (st) return st;
     }
     for (int i = 1; i <= 6; ++i) DL_CK(mark(i), "event");
-    DL_CK(W.raycol.reserve(12 * size_t(R.n_rays > 0 ? R.n_rays : 1)), "alloc ray colours");
     const double pi = 3.14159265358979323846;
     const double focal = 0.5 * w / std::tan(0.5 * D.prm.fov_x_deg * pi / 180.0);
     if (lists) {
@@ -656,9 +663,8 @@ dl_status render_raycast(dl_ctx* ctx, int32_t scene_id, int32_t display_id, Scen
                          lists ? over : nullptr, s),
           "ray-order rendering");
     DL_CK(mark(7), "event");
-    const size_t out_bytes = 12 * size_t(w) * size_t(h);
     float* dst = nullptr;
-    st = out_target(ctx, out, kind, out_bytes, s, &dst);
+    st = out_target(ctx, out, kind, s, &dst);
     if (st) return st;
     DL_CK(launch_reorder(G->slot_of.as<uint32_t>(), W.raycol.as<float>(), w, h, dst, nullptr, s),
           "reorder");
@@ -1248,6 +1254,12 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
     // at 4K 2.19 against 2.72 + the metadata's scan, frame 19.7 against 20.3
     const bool laid_out = on_device || (views_path && sized);
     const bool direct = laid_out && in_projection && hint.slices_ready;
+    // everything that the frame cannot do without first
+    const size_t out_bytes = 12 * size_t(w) * size_t(h);
+    st = reserve_out(ctx, kind, out_bytes);
+    if (st) return st;
+    if (mode == DL_STANDARD)
+        DL_CK(W.Mm.reserve(12 * size_t(nv) * size_t(rw) * size_t(rh)), "alloc M_m");
     DL_CK(W.rec.reserve(16 * kRecordFloat4 * size_t(ne)), "alloc records");
     if (!direct) DL_CK(W.meta.reserve(16 * size_t(ne)), "alloc tile metadata");
     DL_CK(W.gcount.reserve(4 * size_t(ngroups + 1)), "alloc group counts");
@@ -1446,7 +1458,11 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
             int64_t want = laid + laid / 4 + 65536;
             int bc = 2048;
             while (bc < kLargeCap && bc < max_len + max_len / 4) bc <<= 1;
-            if (want < (int64_t(1) << 31) - 2 &&
+            // (the standard paradigm's frames are whole without: where the room
+            // could not be had they keep to the two passes for a while)
+            const bool ask = warp_path || hint.ask_in <= 0;
+            if (!ask) --hint.ask_in;
+            if (ask && want < (int64_t(1) << 31) - 2 &&
                 (views_path || block_smem_bytes(bc) <= max_smem_optin(ctx->device))) {
                 cudaError_t room = cudaErrorMemoryAllocation;
                 if (in_projection) {  // as many keys again in slices
@@ -1456,10 +1472,9 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
                     if (room == cudaSuccess) want = most;
                 }
                 if (room != cudaSuccess) room = W.keys[0].reserve(8 * size_t(want));
-                // (the standard paradigm's views may leave no room for the
-                // larger buffer: its frames then keep to the two passes)
                 if (warp_path) DL_CK(room, "alloc keys");
                 hint.sized = room == cudaSuccess;
+                hint.ask_in = hint.sized ? 0 : kAskAgain;
                 hint.key_cap = want;
                 hint.block_cap = bc;
                 hint.block_keys = std::min(bc, list_capacity(max_len + max_len / 4));
@@ -1469,18 +1484,11 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
     unsigned long long* pairs =
         timing && ctx->count_pairs ? W.pairs.as<unsigned long long>() : nullptr;
 
-    const size_t out_bytes = 12 * size_t(w) * size_t(h);
     float* dst = nullptr;
-    st = out_target(ctx, out, kind, out_bytes, s, &dst);
+    st = out_target(ctx, out, kind, s, &dst);
     if (st) return st;
-    float* Mm = nullptr;
-    float* raycol = nullptr;
-    if (mode == DL_STANDARD) {
-        DL_CK(W.Mm.reserve(12 * size_t(nv) * size_t(rw) * size_t(rh)), "alloc M_m");
-        Mm = W.Mm.as<float>();
-    } else {
-        raycol = W.raycol.as<float>();
-    }
+    float* const Mm = mode == DL_STANDARD ? W.Mm.as<float>() : nullptr;
+    float* const raycol = mode == DL_STANDARD ? nullptr : W.raycol.as<float>();
     int sort_bits = 0;
     // projection, scan (direct emission: the layout's two and the gated
     // re-emission), partition
@@ -1500,14 +1508,19 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
                   "emit binned");
             if ((warp_path || views_path) && hint.sized && in_projection) {
                 // the signature's first slices for keys emitted by the
-                // projection, from this frame's counts
-                for (DevBuf& b : hint.slices)
-                    DL_CK(b.reserve(4 * size_t(ngroups + 1)), "alloc slices");
-                DL_CK(launch_slice_layout(W.gcount.as<uint32_t>(), nullptr, ngroups, W.gscan_tmp.p,
-                                          hint.slices[hint.cur].as<uint32_t>(), d_total32, nullptr, s),
-                      "slice layout");
+                // projection, from this frame's counts (without memory for
+                // them its frames keep to the two passes)
                 hint.slices_ready = true;
-                launches += 2;
+                for (DevBuf& b : hint.slices)
+                    hint.slices_ready =
+                        hint.slices_ready && b.reserve(4 * size_t(ngroups + 1)) == cudaSuccess;
+                if (hint.slices_ready) {
+                    DL_CK(launch_slice_layout(W.gcount.as<uint32_t>(), nullptr, ngroups, W.gscan_tmp.p,
+                                              hint.slices[hint.cur].as<uint32_t>(), d_total32, nullptr,
+                                              s),
+                          "slice layout");
+                    launches += 2;
+                }
             }
         }
         DL_CK(mark(4), "event");

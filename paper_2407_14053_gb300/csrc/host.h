@@ -168,12 +168,16 @@ struct SideStreams {
     SideStreams& operator=(const SideStreams&) = delete;
 };
 
+// frames that do without memory that could not be had, before it is asked for again
+constexpr int32_t kAskAgain = 64;
+
 struct FrameHint {
     bool sized = false;
     int32_t block_cap = 2048;   // longest list of a later frame, a power of two
     int32_t block_keys = 2048;  // keys the block class sorts in shared memory
     int64_t key_cap = 0;
     bool slices_ready = false;
+    int32_t ask_in = 0;  // frames until memory that could not be had is asked for again
     bool no_lists = false;  // DL_RAYCAST: the tile lists do not fit; walk the tree
     int cur = 0;
     DevBuf slices[2];  // n_groups + 1 slot offsets each

@@ -47,3 +47,20 @@ def test_a_key_buffer_that_cannot_grow_costs_no_other_frame(mode):
     out = r.render(large, did, L0, mode)
     assert torch.isfinite(out).all() and out.max() > 0.05
     r.close()
+
+
+def test_a_standard_frame_asks_for_its_views_first():
+    """Room for M_m and the frame's keys (56 and 147 MB with the buffers'
+    slack), but not for the larger key buffer (239 MB) of later frames as well."""
+    from paper_2407_14053_gb300 import Renderer
+    r = Renderer(0)
+    did = r.set_display(PANEL)
+    sid = r.load_gaussians(_covering_scene(1000, True), "f32")
+    with free_bytes(250 * MB):
+        first = r.render(sid, did, L0, "standard").clone()
+        assert r.stats()["n_keys"] == 1000 * 8 * 60 * 34
+        again = r.render(sid, did, L0, "standard").clone()
+    assert torch.equal(first, again) and first.max() > 0.05
+    later = [r.render(sid, did, L0, "standard").clone() for _ in range(70)]
+    assert all(torch.equal(x, first) for x in later)
+    r.close()
