@@ -28,6 +28,15 @@ dl_status fail(dl_ctx* c, dl_status s, const char* fmt, ...) {
     return s;
 }
 
+cudaError_t reserve_needed(dl_ctx* ctx, DevBuf& b, size_t bytes) {
+    Workspace& W = ctx->ws;
+    const cudaError_t e = b.reserve(bytes);
+    if (e != cudaErrorMemoryAllocation || W.enqueuing || (!W.cast.p && !W.keys[0].p)) return e;
+    W.cast.release();
+    W.keys[0].release();
+    return b.reserve(bytes);
+}
+
 dl_status cuda_fail(dl_ctx* c, cudaError_t e, const char* what) {
     const dl_status s = (e == cudaErrorMemoryAllocation) ? DL_ERR_OOM : DL_ERR_CUDA;
     return fail(c, s, "%s: %s", what, cudaGetErrorString(e));
@@ -92,12 +101,12 @@ dl_status make_display_q(dl_ctx* ctx, const dl_display_params& p, DisplayQ* q) {
 dl_status build_rayset(dl_ctx* ctx, Display& D, RaySet& R, bool identity, cudaStream_t s) {
     const DisplayQ& q = D.q;
     const size_t n = 3 * size_t(q.w) * q.h;
-    DL_CK(R.src.reserve(4 * n), "alloc src");
+    DL_CK(reserve_needed(ctx, R.src, 4 * n), "alloc src");
     DL_CK(launch_repurpose(q, R.src.as<uint32_t>(), identity ? 1 : 0, s), "repurpose");
-    DL_CK(R.ray_of.reserve(4 * n), "alloc ray_of");
+    DL_CK(reserve_needed(ctx, R.ray_of, 4 * n), "alloc ray_of");
     DevBuf tmp;
-    DL_CK(tmp.reserve(ray_table_tmp_bytes(q)), "alloc ray-table scratch");
-    DL_CK(ctx->ws.small.reserve(256), "alloc small");
+    DL_CK(reserve_needed(ctx, tmp, ray_table_tmp_bytes(q)), "alloc ray-table scratch");
+    DL_CK(reserve_needed(ctx, ctx->ws.small, 256), "alloc small");
     uint32_t* d_n = ctx->ws.small.as<uint32_t>();
     DL_CK(launch_ray_table(q, D.V.as<uint16_t>(), R.src.as<uint32_t>(), R.ray_of.as<uint32_t>(),
                            tmp.p, d_n, s),
@@ -106,8 +115,8 @@ dl_status build_rayset(dl_ctx* ctx, Display& D, RaySet& R, bool identity, cudaSt
     DL_CK(cudaMemcpyAsync(&h_n, d_n, sizeof(uint32_t), cudaMemcpyDeviceToHost, s), "copy");
     DL_CK(cudaStreamSynchronize(s), "sync");
     R.n_rays = int64_t(h_n);
-    DL_CK(R.ray_view.reserve(4 * size_t(R.n_rays)), "alloc rays");
-    DL_CK(R.ray_pix.reserve(4 * size_t(R.n_rays)), "alloc rays");
+    DL_CK(reserve_needed(ctx, R.ray_view, 4 * size_t(R.n_rays)), "alloc rays");
+    DL_CK(reserve_needed(ctx, R.ray_pix, 4 * size_t(R.n_rays)), "alloc rays");
     DL_CK(launch_ray_attributes(q, D.V.as<uint16_t>(), tmp.p, R.ray_view.as<uint32_t>(),
                                 R.ray_pix.as<uint32_t>(), s),
           "ray attributes");
@@ -160,12 +169,12 @@ dl_status get_groups(dl_ctx* ctx, Display& D, RaySet& R, int32_t tw, int32_t th,
     const int64_t ngroups = int64_t(D.q.nv) * G->ntiles;
     const int64_t nr = R.n_rays;
     DevBuf k0, k1, v0, v1, rtmp, ranges, counts;
-    DL_CK(k0.reserve(8 * size_t(nr)), "alloc");
-    DL_CK(k1.reserve(8 * size_t(nr)), "alloc");
-    DL_CK(v0.reserve(4 * size_t(nr)), "alloc");
-    DL_CK(v1.reserve(4 * size_t(nr)), "alloc");
-    DL_CK(rtmp.reserve(radix_tmp_bytes(nr)), "alloc");
-    DL_CK(ranges.reserve(8 * size_t(ngroups)), "alloc");
+    DL_CK(reserve_needed(ctx, k0, 8 * size_t(nr)), "alloc");
+    DL_CK(reserve_needed(ctx, k1, 8 * size_t(nr)), "alloc");
+    DL_CK(reserve_needed(ctx, v0, 4 * size_t(nr)), "alloc");
+    DL_CK(reserve_needed(ctx, v1, 4 * size_t(nr)), "alloc");
+    DL_CK(reserve_needed(ctx, rtmp, radix_tmp_bytes(nr)), "alloc");
+    DL_CK(reserve_needed(ctx, ranges, 8 * size_t(ngroups)), "alloc");
     const int shift = 2 * bits_for(std::max(tw, th));  // Morton bits (powers of two)
     DL_CK(launch_ray_group_keys(R.ray_view.as<uint32_t>(), R.ray_pix.as<uint32_t>(), nr, tw, th,
                                 G->ntx, D.q.nv, shift, k0.as<unsigned long long>(),
@@ -180,7 +189,7 @@ dl_status get_groups(dl_ctx* ctx, Display& D, RaySet& R, int32_t tw, int32_t th,
     uint32_t* vs = alt ? v1.as<uint32_t>() : v0.as<uint32_t>();
     DL_CK(cudaMemsetAsync(ranges.p, 0, 8 * size_t(ngroups), s), "memset");
     DL_CK(launch_key_ranges(ks, nr, shift, ranges.as<uint2>(), ngroups, s), "group ranges");
-    DL_CK(G->grouped.reserve(8 * size_t(nr)), "alloc");
+    DL_CK(reserve_needed(ctx, G->grouped, 8 * size_t(nr)), "alloc");
     DL_CK(launch_ray_group_gather(vs, R.ray_pix.as<uint32_t>(), nr, G->grouped.as<int2>(), s),
           "group gather");
     // the work lists, made on the device from the ranges: the compositing
@@ -189,7 +198,7 @@ dl_status get_groups(dl_ctx* ctx, Display& D, RaySet& R, int32_t tw, int32_t th,
     // the DRAM reads).  The loops over the groups took the host 3 ms at 4K.
     const size_t ng1 = size_t(ngroups + 1);
     const size_t scan_bytes = scan_tmp_bytes(ngroups + 1);
-    DL_CK(counts.reserve(16 * ng1 + scan_bytes + 512), "alloc");
+    DL_CK(reserve_needed(ctx, counts, 16 * ng1 + scan_bytes + 512), "alloc");
     uint32_t* chunks = counts.as<uint32_t>();
     uint32_t *used = chunks + ng1, *chunk_at = used + ng1, *used_at = chunk_at + ng1;
     uint32_t* totals = used_at + ng1;
@@ -202,7 +211,7 @@ dl_status get_groups(dl_ctx* ctx, Display& D, RaySet& R, int32_t tw, int32_t th,
     uint32_t h_totals[2] = {0u, 0u};
     DL_CK(cudaMemcpyAsync(h_totals, totals, 8, cudaMemcpyDeviceToHost, s), "copy");
     const int64_t nsub = 3 * int64_t(D.q.w) * D.q.h;
-    DL_CK(G->slot_of.reserve(4 * size_t(nsub)), "alloc");
+    DL_CK(reserve_needed(ctx, G->slot_of, 4 * size_t(nsub)), "alloc");
     DL_CK(launch_group_slots(G->grouped.as<int2>(), nr, R.ray_of.as<uint32_t>(), nsub,
                              alt ? v0.as<uint32_t>() : v1.as<uint32_t>(), G->slot_of.as<uint32_t>(),
                              s),
@@ -210,8 +219,8 @@ dl_status get_groups(dl_ctx* ctx, Display& D, RaySet& R, int32_t tw, int32_t th,
     DL_CK(cudaStreamSynchronize(s), "sync");
     G->n_work = int64_t(h_totals[0]);
     G->n_gwork = int64_t(h_totals[1]);
-    DL_CK(G->work.reserve(16 * size_t(std::max<int64_t>(G->n_work, 1))), "alloc");
-    DL_CK(G->gwork.reserve(16 * size_t(std::max<int64_t>(G->n_gwork, 1))), "alloc");
+    DL_CK(reserve_needed(ctx, G->work, 16 * size_t(std::max<int64_t>(G->n_work, 1))), "alloc");
+    DL_CK(reserve_needed(ctx, G->gwork, 16 * size_t(std::max<int64_t>(G->n_gwork, 1))), "alloc");
     DL_CK(launch_list_fill(ranges.as<uint2>(), ngroups, G->ntiles, D.q.nv, kRaysPerBlock, chunk_at,
                            used_at, G->work.as<int4>(), G->gwork.as<int4>(), s),
           "list fill");
@@ -275,8 +284,8 @@ bool make_cams(const dl_display_params& p, const double L0[16], std::vector<Cam>
 dl_status begin_frame(dl_ctx* ctx, const std::vector<Cam>& cams, const uint32_t* layout,
                       int64_t n_groups, uint32_t* cursor, cudaStream_t s, int32_t* launches) {
     Workspace& W = ctx->ws;
-    DL_CK(W.cams.reserve(sizeof(Cam) * cams.size()), "alloc cams");
-    DL_CK(W.small.reserve(256), "alloc");
+    DL_CK(reserve_needed(ctx, W.cams, sizeof(Cam) * cams.size()), "alloc cams");
+    DL_CK(reserve_needed(ctx, W.small, 256), "alloc");
     Cam* dst = W.cams.as<Cam>();
     for (size_t v0 = 0; v0 < cams.size(); v0 += kCamBatch) {
         CamBatch b;
@@ -336,16 +345,18 @@ float elapsed(cudaEvent_t a, cudaEvent_t b) {
 
 // Per-Gaussian data and the 8-wide SAH tree of the ray-order renderer.
 dl_status build_raycast(dl_ctx* ctx, Scene& S, cudaStream_t s) {
-    DL_CK(S.rc_gauss.reserve(48 * size_t(std::max<int64_t>(S.n, 1))), "alloc ray-order data");
-    DL_CK(S.rc_gbox.reserve(32 * size_t(std::max<int64_t>(S.n, 1))), "alloc ray-order boxes");
+    const size_t n1 = size_t(std::max<int64_t>(S.n, 1));
+    DL_CK(reserve_needed(ctx, S.rc_gauss, 48 * n1), "alloc ray-order data");
+    DL_CK(reserve_needed(ctx, S.rc_gbox, 32 * n1), "alloc ray-order boxes");
     const void* attrs[5] = {S.mean.p, S.log_scale.p, S.rot.p, S.opacity.p, S.sh.p};
     DL_CK(launch_raycast_prepare(S.dtype, attrs, S.n, S.rc_gauss.as<float4>(), S.rc_gbox.as<float4>(), s),
           "ray-order preparation");
     DevBuf tmp;
-    DL_CK(tmp.reserve(raycast_build_tmp_bytes(S.n)), "alloc tree build");
+    DL_CK(reserve_needed(ctx, tmp, raycast_build_tmp_bytes(S.n)), "alloc tree build");
     int64_t n_bin = 0;
     DL_CK(raycast_build_binary(S.rc_gbox.as<float4>(), S.n, tmp.p, &n_bin, s), "SAH tree");
-    DL_CK(S.rc_nodes.reserve(sizeof(RayNode) * size_t(std::max<int64_t>(n_bin, 1))), "alloc tree");
+    DL_CK(reserve_needed(ctx, S.rc_nodes, sizeof(RayNode) * size_t(std::max<int64_t>(n_bin, 1))),
+          "alloc tree");
     int64_t n_wide = 0;
     int depth = 0;
     DL_CK(raycast_collapse(S.rc_gbox.as<float4>(), S.n, tmp.p, n_bin, S.rc_nodes.as<RayNode>(), &n_wide,
@@ -456,7 +467,7 @@ enum OutKind : int32_t { kOutHost = 0, kOutDevice = 1, kOutHostAsync = 2 };
 // frames; out_target then orders it after the copy that read it.
 dl_status reserve_out(dl_ctx* ctx, int32_t kind, size_t bytes) {
     Workspace& W = ctx->ws;
-    if (kind == kOutHost) DL_CK(W.out.reserve(bytes), "alloc out");
+    if (kind == kOutHost) DL_CK(reserve_needed(ctx, W.out, bytes), "alloc out");
     if (kind != kOutHostAsync) return DL_OK;
     const int k = W.aslot;
     for (int i = 0; i < 2; ++i) {
@@ -465,7 +476,7 @@ dl_status reserve_out(dl_ctx* ctx, int32_t kind, size_t bytes) {
     }
     if (W.copy_pending[k] && W.aout[k].bytes < bytes)  // the frame is replaced: its copy must have ended
         DL_CK(cudaEventSynchronize(W.ev_copied[k]), "wait for an earlier copy");
-    DL_CK(W.aout[k].reserve(bytes), "alloc out");
+    DL_CK(reserve_needed(ctx, W.aout[k], bytes), "alloc out");
     return DL_OK;
 }
 
@@ -531,7 +542,7 @@ dl_status build_cast_lists(dl_ctx* ctx, Scene& S, Display& D, TileGroups& G, Fra
         hint.no_lists = true;
         return DL_OK;
     }
-    DL_CK(W.small.reserve(256), "alloc");
+    DL_CK(reserve_needed(ctx, W.small, 256), "alloc");
     unsigned long long* d_total64 = W.small.as<unsigned long long>();
     uint32_t* d_total32 = reinterpret_cast<uint32_t*>(W.small.as<char>() + 64);
     uint32_t* d_redo = d_total32 + 1;
@@ -612,8 +623,10 @@ dl_status render_raycast(dl_ctx* ctx, int32_t scene_id, int32_t display_id, Scen
     const size_t out_bytes = 12 * size_t(w) * size_t(h);
     st = reserve_out(ctx, kind, out_bytes);
     if (st) return st;
-    DL_CK(W.raycol.reserve(12 * size_t(R.n_rays > 0 ? R.n_rays : 1)), "alloc ray colours");
+    DL_CK(reserve_needed(ctx, W.raycol, 12 * size_t(R.n_rays > 0 ? R.n_rays : 1)),
+          "alloc ray colours");
     FrameHint& hint = ctx->hints[FrameSig{scene_id, display_id, DL_RAYCAST, G->tw, G->th, w, h}];
+    W.enqueuing = true;
     GroupSlices sl;
     uint32_t* over = nullptr;
     int32_t launches = 0;
@@ -791,18 +804,18 @@ dl_status dl_load_gaussians(dl_ctx* ctx, const dl_gaussians_desc* d, void* strea
                   {&sc->opacity, d->opacity_logit, es * n},
                   {&sc->sh, d->sh, 3 * nc * es * n}};
     for (auto& pt : parts) {
-        DL_CK(pt.b->reserve(pt.bytes), "alloc scene");
+        DL_CK(reserve_needed(ctx, *pt.b, pt.bytes), "alloc scene");
         DL_CK(cudaMemcpyAsync(pt.b->p, pt.src, pt.bytes, kind, s), "copy scene");
     }
     if (sc->n > 1) {
         // Morton order of the means (see scene.cu)
         DevBuf tmp;
-        DL_CK(tmp.reserve(spatial_order_tmp_bytes(sc->n)), "alloc reorder scratch");
+        DL_CK(reserve_needed(ctx, tmp, spatial_order_tmp_bytes(sc->n)), "alloc reorder scratch");
         uint32_t* perm = nullptr;
         DL_CK(launch_spatial_order(sc->mean.as<float>(), sc->n, tmp.p, &perm, s), "spatial order");
         for (auto& pt : parts) {
             DevBuf sorted;
-            DL_CK(sorted.reserve(pt.bytes), "alloc scene");
+            DL_CK(reserve_needed(ctx, sorted, pt.bytes), "alloc scene");
             DL_CK(launch_gather_records(pt.b->p, sorted.p, perm, sc->n, pt.bytes / n, s), "gather");
             std::swap(pt.b->p, sorted.p);
             std::swap(pt.b->bytes, sorted.bytes);
@@ -856,7 +869,7 @@ dl_status dl_set_display(dl_ctx* ctx, const dl_display_params* params, void* str
     st = make_display_q(ctx, D->prm, &D->q);
     if (st) return st;
     const size_t n = 3 * size_t(D->q.w) * D->q.h;
-    DL_CK(D->V.reserve(2 * n), "alloc V");
+    DL_CK(reserve_needed(ctx, D->V, 2 * n), "alloc V");
     DL_CK(launch_view_map(D->q, D->V.as<uint16_t>(), s), "view map");
     st = build_rayset(ctx, *D, D->rep, D->prm.repurpose == 0, s);
     if (st) return st;
@@ -947,7 +960,7 @@ dl_status dl_get_ray_table(dl_ctx* ctx, int32_t display_id, uint32_t* ray_of, in
                   "rays export");
         } else {
             DevBuf tmp;
-            DL_CK(tmp.reserve(bytes), "alloc");
+            DL_CK(reserve_needed(ctx, tmp, bytes), "alloc");
             DL_CK(launch_rays_export(D.rep.ray_view.as<uint32_t>(), D.rep.ray_pix.as<uint32_t>(),
                                      D.rep.n_rays, tmp.as<int32_t>(), s),
                   "rays export");
@@ -1041,7 +1054,7 @@ dl_status dl_enable_stage_timing(dl_ctx* ctx, int32_t enable) {
     if (st) return st;
     if (enable < 0 || enable > 2) return fail(ctx, DL_ERR_INVALID_ARG, "stage timing mode %d", enable);
     if (enable == 1 && !ctx->ws.pairs.p) {
-        DL_CK(ctx->ws.pairs.reserve(16), "alloc counters");
+        DL_CK(reserve_needed(ctx, ctx->ws.pairs, 16), "alloc counters");
         DL_CK(cudaMemset(ctx->ws.pairs.p, 0, 16), "memset");
     }
     ctx->timing = enable != 0;
@@ -1163,6 +1176,11 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
     Scene& S = *si->second;
     Display& D = *di->second;
     Workspace& W = ctx->ws;
+    struct Enqueuing {  // until the call ends
+        bool& flag;
+        explicit Enqueuing(bool& f) : flag(f) { flag = false; }
+        ~Enqueuing() { flag = false; }
+    } enqueuing(W.enqueuing);
     // counters of earlier frames that have arrived update their signatures'
     // capacities before this frame is sized
     st = harvest_readbacks(ctx, false);
@@ -1243,31 +1261,43 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
     // signature's capacities and device counters, and are dropped on the
     // device (status word, output untouched) when they exceed them.
     FrameHint& hint = ctx->hints[FrameSig{scene_id, display_id, mode, tw, th, rw, rh}];
-    const bool sized = hint.fits(W.keys[0]) && ctx->sort_mode != DL_SORT_RADIX;
-    const bool on_device = warp_path && sized;
-    // keys emitted by the projection, into the slices the signature's last
-    // frame laid out
-    const bool in_projection = emit_in_projection(ctx->key_emission);
-    // (the standard paradigm too, though it reads its totals back every frame:
-    // a frame that did not fit is then rendered again by the two passes).  Its
-    // 93 million rays at 1080p: projection and emission 0.50 against 0.69 ms;
-    // at 4K 2.19 against 2.72 + the metadata's scan, frame 19.7 against 20.3
-    const bool laid_out = on_device || (views_path && sized);
-    const bool direct = laid_out && in_projection && hint.slices_ready;
     // everything that the frame cannot do without first
     const size_t out_bytes = 12 * size_t(w) * size_t(h);
     st = reserve_out(ctx, kind, out_bytes);
     if (st) return st;
     if (mode == DL_STANDARD)
-        DL_CK(W.Mm.reserve(12 * size_t(nv) * size_t(rw) * size_t(rh)), "alloc M_m");
-    DL_CK(W.rec.reserve(16 * kRecordFloat4 * size_t(ne)), "alloc records");
-    if (!direct) DL_CK(W.meta.reserve(16 * size_t(ne)), "alloc tile metadata");
-    DL_CK(W.gcount.reserve(4 * size_t(ngroups + 1)), "alloc group counts");
-    DL_CK(W.gstart.reserve(4 * size_t(ngroups + 1)), "alloc group starts");
-    DL_CK(W.gfill.reserve(4 * size_t(ngroups)), "alloc cursors");
-    DL_CK(W.gscan_tmp.reserve(std::max(scan_tmp_bytes(ngroups + 1), slice_tmp_bytes(ngroups))),
+        DL_CK(reserve_needed(ctx, W.Mm, 12 * size_t(nv) * size_t(rw) * size_t(rh)), "alloc M_m");
+    DL_CK(reserve_needed(ctx, W.rec, 16 * kRecordFloat4 * size_t(ne)), "alloc records");
+    DL_CK(reserve_needed(ctx, W.gcount, 4 * size_t(ngroups + 1)), "alloc group counts");
+    DL_CK(reserve_needed(ctx, W.gstart, 4 * size_t(ngroups + 1)), "alloc group starts");
+    DL_CK(reserve_needed(ctx, W.gfill, 4 * size_t(ngroups)), "alloc cursors");
+    DL_CK(reserve_needed(ctx, W.gscan_tmp,
+                         std::max(scan_tmp_bytes(ngroups + 1), slice_tmp_bytes(ngroups))),
           "alloc scan");
-    DL_CK(W.small.reserve(256), "alloc");
+    DL_CK(reserve_needed(ctx, W.small, 256), "alloc");
+    const int64_t n_work = mode == DL_STANDARD ? ngroups : G->n_gwork;
+    const size_t nw1 = size_t(std::max<int64_t>(n_work, 1));
+    DL_CK(reserve_needed(ctx, W.lists, 32 * nw1 + 16), "alloc lists");
+    if (mode != DL_STANDARD)
+        DL_CK(reserve_needed(ctx, W.raycol, 12 * size_t(R->n_rays > 0 ? R->n_rays : 1)),
+              "alloc ray colours");
+    if (warp_path) DL_CK(reserve_needed(ctx, W.fdesc, sizeof(FrameDesc)), "alloc frame table");
+    // keys emitted by the projection, into the slices the signature's last
+    // frame laid out (the standard paradigm too, though it reads its totals
+    // back every frame: a frame that did not fit is then rendered again by the
+    // two passes).  Its 93 million rays at 1080p: projection and emission 0.50
+    // against 0.69 ms; at 4K 2.19 against 2.72 + the metadata's scan, frame 19.7
+    // against 20.3
+    const bool in_projection = emit_in_projection(ctx->key_emission);
+    auto sized_now = [&]() { return hint.fits(W.keys[0]) && ctx->sort_mode != DL_SORT_RADIX; };
+    if (!((warp_path || views_path) && sized_now() && in_projection && hint.slices_ready))
+        DL_CK(reserve_needed(ctx, W.meta, 16 * size_t(ne)), "alloc tile metadata");
+    // (the reservations above may have taken the key buffer's memory)
+    const bool sized = sized_now();
+    const bool on_device = warp_path && sized;
+    const bool laid_out = on_device || (views_path && sized);
+    const bool direct = laid_out && in_projection && hint.slices_ready;
+    W.enqueuing = laid_out;
     unsigned long long* d_total64 = W.small.as<unsigned long long>();
     uint32_t* d_total32 = reinterpret_cast<uint32_t*>(W.small.as<char>() + 64);
     uint32_t* d_redo = d_total32 + 1;  // a key found its slice full (direct emission)
@@ -1278,17 +1308,12 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
         laid_out ? uint32_t(std::min<size_t>(W.keys[0].bytes / 8, size_t((1u << 31) - 2))) : 0u;
     const void* attrs[5] = {S.mean.p, S.log_scale.p, S.rot.p, S.opacity.p, S.sh.p};
     const int4* gwork = mode == DL_STANDARD ? nullptr : G->gwork.as<int4>();
-    const int64_t n_work = mode == DL_STANDARD ? ngroups : G->n_gwork;
-    const size_t nw1 = size_t(std::max<int64_t>(n_work, 1));
-    DL_CK(W.lists.reserve(32 * nw1 + 16), "alloc lists");
     // warp path: items, then block items; otherwise the two class lists
     int4* items = W.lists.as<int4>();
     int4* block_items = items + nw1;
     int32_t* small_list = W.lists.as<int32_t>();
     int32_t* large_list = small_list + nw1;
     uint32_t* cursor = W.gfill.as<uint32_t>();
-    if (mode != DL_STANDARD)
-        DL_CK(W.raycol.reserve(12 * size_t(R->n_rays > 0 ? R->n_rays : 1)), "alloc ray colours");
     CompositeParams cp{};
     cp.n = S.n;
     cp.width = rw;
@@ -1303,7 +1328,6 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
     // one frame through the frame-batched persistent kernels
     SingleFrame single;
     if (warp_path) {
-        DL_CK(W.fdesc.reserve(sizeof(FrameDesc)), "alloc frame table");
         FrameDesc& fd = single.fd;
         fd.cp = cp;
         fd.grouped = G->grouped.as<int2>();
@@ -1493,7 +1517,18 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
     // projection, scan (direct emission: the layout's two and the gated
     // re-emission), partition
     launches += 1 + 3 + (n_work > 0 ? 1 : 0);
-    DL_CK(W.keys[0].reserve(8 * size_t(nk > 0 ? nk : 1)), "alloc keys");
+    const size_t nk1 = size_t(nk > 0 ? nk : 1);
+    if (!binned) {
+        DL_CK(reserve_needed(ctx, W.count, 4 * size_t(ne)), "alloc counts");
+        DL_CK(reserve_needed(ctx, W.offset, 4 * size_t(ne)), "alloc offsets");
+        DL_CK(reserve_needed(ctx, W.scan_tmp, scan_tmp_bytes(ne)), "alloc scan");
+        DL_CK(reserve_needed(ctx, W.keys[1], 8 * nk1), "alloc keys");
+        for (DevBuf& b : W.vals) DL_CK(reserve_needed(ctx, b, 4 * nk1), "alloc vals");
+        DL_CK(reserve_needed(ctx, W.radix_tmp, radix_tmp_bytes(nk)), "alloc radix");
+        DL_CK(reserve_needed(ctx, W.ranges, 8 * size_t(ngroups)), "alloc ranges");
+    }
+    DL_CK(reserve_needed(ctx, W.keys[0], 8 * nk1), "alloc keys");
+    W.enqueuing = true;
     if (binned) {
         // ---- binned keys, sorted per tile in shared memory while compositing ----
         DL_CK(mark(3), "event");
@@ -1586,13 +1621,6 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
                     (n_large > 0 ? 1 : 0);
     } else {
         // ---- global tile keys and a stable LSD radix sort ----
-        DL_CK(W.count.reserve(4 * size_t(ne)), "alloc counts");
-        DL_CK(W.offset.reserve(4 * size_t(ne)), "alloc offsets");
-        DL_CK(W.scan_tmp.reserve(scan_tmp_bytes(ne)), "alloc scan");
-        DL_CK(W.keys[1].reserve(8 * size_t(nk > 0 ? nk : 1)), "alloc keys");
-        for (int i = 0; i < 2; ++i) DL_CK(W.vals[i].reserve(4 * size_t(nk > 0 ? nk : 1)), "alloc vals");
-        DL_CK(W.radix_tmp.reserve(radix_tmp_bytes(nk)), "alloc radix");
-        DL_CK(W.ranges.reserve(8 * size_t(ngroups)), "alloc ranges");
         DL_CK(mark(3), "event");
         DL_CK(launch_meta_counts(W.meta.as<uint4>(), ne, W.count.as<uint32_t>(), s), "counts");
         DL_CK(launch_exclusive_scan(W.count.as<uint32_t>(), W.offset.as<uint32_t>(), ne, nullptr,

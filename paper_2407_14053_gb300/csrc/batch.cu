@@ -317,7 +317,7 @@ dl_status dl_batch_create(dl_ctx* ctx, int32_t n_slots, const dl_slot_plan* plan
         int32_t tw = 0, th = 0;
         st = resolve_frame(ctx, pl.scene_id, pl.display_id, pl.tile_w, pl.tile_h, &S, &D, &tw, &th);
         if (st) break;
-        if (tmp_out.reserve(12 * size_t(D->q.w) * D->q.h) != cudaSuccess) {
+        if (reserve_needed(ctx, tmp_out, 12 * size_t(D->q.w) * D->q.h) != cudaSuccess) {
             st = fail(ctx, DL_ERR_OOM, "sizing frame output");
             break;
         }
@@ -381,14 +381,14 @@ dl_status dl_batch_create(dl_ctx* ctx, int32_t n_slots, const dl_slot_plan* plan
     b->o_prefix = take(8 * 3 * size_t(n_slots + 1));
     b->globals_bytes = 4 * (8 + size_t(n_slots));
     b->o_globals = take(b->globals_bytes);
-    DL_CK(b->arena.reserve(off), "alloc batch arena");
+    DL_CK(reserve_needed(ctx, b->arena, off), "alloc batch arena");
     const int n_side = std::max(2, std::min<int>(n_slots, kMaxSide));
     DL_CK(b->side.create(n_side), "streams");
     b->scan_stride = align_up(std::max<size_t>(scan_bytes, 256), 256);
-    DL_CK(b->scan_tmp.reserve(b->scan_stride * size_t(n_side)), "alloc scan scratch");
+    DL_CK(reserve_needed(ctx, b->scan_tmp, b->scan_stride * size_t(n_side)), "alloc scan scratch");
     b->cams_offset = align_up(sizeof(FrameDesc) * size_t(n_slots), 256);
     b->stage_bytes = b->cams_offset + sizeof(Cam) * size_t(b->total_views);
-    DL_CK(b->stage_d.reserve(b->stage_bytes), "alloc staging");
+    DL_CK(reserve_needed(ctx, b->stage_d, b->stage_bytes), "alloc staging");
     void* h = nullptr;
     DL_CK(cudaHostAlloc(&h, b->stage_bytes, cudaHostAllocDefault), "pinned staging");
     b->stage_h = static_cast<unsigned char*>(h);
@@ -584,7 +584,7 @@ dl_status dl_autotune_tile(dl_ctx* ctx, int32_t scene_id, int32_t display_id,
     const Display& D = *di->second;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     DevBuf out;
-    DL_CK(out.reserve(12 * size_t(D.q.w) * D.q.h), "alloc");
+    DL_CK(reserve_needed(ctx, out, 12 * size_t(D.q.w) * D.q.h), "alloc");
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     DL_CK(cudaEventCreate(&e0), "event");
     if (cudaEventCreate(&e1) != cudaSuccess) {

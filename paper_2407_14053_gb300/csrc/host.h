@@ -210,6 +210,7 @@ struct Workspace {
     int64_t last_async = -1;   // frame number of the last frame read back asynchronously
     int64_t dropped = 0;       // frames dropped on the device (capacity exceeded)
     size_t last_bytes = 0;
+    bool enqueuing = false;  // the frame being enqueued counts on keys[0] and cast
     std::vector<StageEvents*> ev_free;
     std::vector<PendingFrame> pending;
     // frames copied to the host on the caller's copy stream
@@ -274,6 +275,12 @@ namespace dl {
 
 dl_status fail(dl_ctx* c, dl_status s, const char* fmt, ...);
 dl_status cuda_fail(dl_ctx* c, cudaError_t e, const char* what);
+// Memory that a call cannot do without.  When the device has none left, what
+// frames keep for later ones is given back first: the ray-order renderer's
+// intersection lists (2 GB) and the key buffer (more than a frame's keys; the
+// signatures that counted on it are sized again), unless the frame being
+// enqueued counts on them.
+cudaError_t reserve_needed(dl_ctx* ctx, DevBuf& b, size_t bytes);
 dl_status check_ctx(dl_ctx* ctx);
 int bits_for(int64_t n);
 size_t max_smem_optin(int device);

@@ -64,3 +64,27 @@ def test_a_standard_frame_asks_for_its_views_first():
     later = [r.render(sid, did, L0, "standard").clone() for _ in range(70)]
     assert all(torch.equal(x, first) for x in later)
     r.close()
+
+
+def test_what_is_kept_for_later_frames_is_given_back():
+    """The ray-order renderer's intersection lists (900 MB here) do not keep a
+    frame or a scene from the memory that it cannot do without, and are there
+    again when the next ray-order frame wants them."""
+    from paper_2407_14053_gb300 import Renderer
+    r = Renderer(0)
+    did = r.set_display(PANEL)
+    sid = r.load_gaussians(_covering_scene(1000, True), "f32")
+    rays = [r.render(sid, did, L0, "raycast").clone() for _ in range(2)]
+    with free_bytes(64 * MB):
+        standard = r.render(sid, did, L0, "standard").clone()  # 203 MB
+    with free_bytes(64 * MB):
+        directl = r.render(sid, did, L0, "directl").clone()
+    rays.append(r.render(sid, did, L0, "raycast").clone())
+    with free_bytes(64 * MB):
+        other = r.load_gaussians(_covering_scene(600_000, False), "f32")  # 150 MB with its copies
+    rays.append(r.render(sid, did, L0, "raycast").clone())
+    assert all(torch.equal(x, rays[0]) for x in rays) and rays[0].max() > 0.05
+    assert torch.equal(r.render(sid, did, L0, "standard"), standard)
+    assert torch.equal(r.render(sid, did, L0, "directl"), directl)
+    r.free_scene(other)
+    r.close()
