@@ -530,7 +530,18 @@ dl_status build_cast_lists(dl_ctx* ctx, Scene& S, Display& D, TileGroups& G, Fra
     const int32_t nv = D.q.nv;
     const ProjectParams pp = make_project_params(S, D, G.tw, G.th);
     const int64_t ne = int64_t(nv) * S.n, ngroups = int64_t(nv) * G.ntiles;
-    if (hint.no_lists || ne >= (int64_t(1) << 31) || ngroups >= (int64_t(1) << 31) - 1) return DL_OK;
+    if (ne >= (int64_t(1) << 31) || ngroups >= (int64_t(1) << 31) - 1) return DL_OK;
+    // lists that could not be held (this pose's keys, or memory) are tried
+    // again after some frames, and at once with fewer entries a ray
+    if (hint.ask_in > 0 && ctx->heap_cap >= hint.ask_heap) {
+        --hint.ask_in;
+        return DL_OK;
+    }
+    auto without = [&]() {
+        hint.ask_in = kAskAgain;
+        hint.ask_heap = ctx->heap_cap;
+        return DL_OK;
+    };
     const size_t words = 4 * size_t(ngroups + 1);
     // memory that the tree would not need: without it the tree renders
     auto reserve = [](DevBuf& b, size_t bytes) { return b.reserve(bytes) == cudaSuccess; };
@@ -538,10 +549,8 @@ dl_status build_cast_lists(dl_ctx* ctx, Scene& S, Display& D, TileGroups& G, Fra
     if (!reserve(W.rec, 16 * kRecordFloat4 * size_t(ne)) || !reserve(W.gfill, words) ||
         !reserve(W.gscan_tmp, slice_tmp_bytes(ngroups)) ||
         !reserve(hint.slices[0], words) || !reserve(hint.slices[1], words) ||
-        !reserve(W.cast, cast_tmp_bytes(chunk, ctx->heap_cap))) {
-        hint.no_lists = true;
-        return DL_OK;
-    }
+        !reserve(W.cast, cast_tmp_bytes(chunk, ctx->heap_cap)))
+        return without();
     DL_CK(reserve_needed(ctx, W.small, 256), "alloc");
     unsigned long long* d_total64 = W.small.as<unsigned long long>();
     uint32_t* d_total32 = reinterpret_cast<uint32_t*>(W.small.as<char>() + 64);
@@ -571,13 +580,11 @@ dl_status build_cast_lists(dl_ctx* ctx, Scene& S, Display& D, TileGroups& G, Fra
         const unsigned long long nk = W.h_total[0];
         const int64_t laid = nk < (1ull << 31) ? int64_t(nk + nk / 8) + 16 * ngroups : int64_t(1) << 31;
         const int64_t want = laid + laid / 4 + 65536;
-        if (want >= (int64_t(1) << 31) - 2 || !reserve(W.keys[0], 8 * size_t(want))) {
-            hint.no_lists = true;
-            return DL_OK;
-        }
+        if (want >= (int64_t(1) << 31) - 2 || !reserve(W.keys[0], 8 * size_t(want))) return without();
         hint.sized = true;
         hint.slices_ready = true;
         hint.key_cap = want;
+        hint.ask_in = 0;
         po.keys = W.keys[0].as<unsigned long long>();
         po.key_cap = uint32_t(std::min<size_t>(W.keys[0].bytes / 8, size_t((1u << 31) - 2)));
     }

@@ -177,8 +177,8 @@ struct FrameHint {
     int32_t block_keys = 2048;  // keys the block class sorts in shared memory
     int64_t key_cap = 0;
     bool slices_ready = false;
-    int32_t ask_in = 0;  // frames until memory that could not be had is asked for again
-    bool no_lists = false;  // DL_RAYCAST: the tile lists do not fit; walk the tree
+    int32_t ask_in = 0;    // frames until memory that could not be had is asked for again
+    int32_t ask_heap = 0;  // DL_RAYCAST: the c_h it could not be had with
     int cur = 0;
     DevBuf slices[2];  // n_groups + 1 slot offsets each
     // The key buffer is every signature's: a larger one that could not be had

@@ -88,3 +88,33 @@ def test_what_is_kept_for_later_frames_is_given_back():
     assert torch.equal(r.render(sid, did, L0, "directl"), directl)
     r.free_scene(other)
     r.close()
+
+
+def _lists(r):  # a ray-order frame from tile lists is nine launches, a tree walk three
+    return r.stats()["n_launches"] > 5
+
+
+def test_ray_order_lists_are_asked_for_again():
+    """Without memory for its lists (900 MB) a ray-order frame walks the tree;
+    with less to ask for, or the memory free again, it has lists again."""
+    from paper_2407_14053_gb300 import Renderer
+    r = Renderer(0)
+    warm = r.set_display(W.WORKLOADS["tiny"].display)
+    did = r.set_display(PANEL)
+    sid = r.load_gaussians(_covering_scene(1000, True), "f32")
+    r.render(sid, warm, L0, "raycast")
+    with free_bytes(400 * MB):
+        walked = r.render(sid, did, L0, "raycast").clone()
+        assert not _lists(r)
+        assert torch.equal(r.render(sid, did, L0, "raycast"), walked) and not _lists(r)
+        r.set_heap_capacity(16)  # 112 MB
+        r.render(sid, did, L0, "raycast")
+        assert _lists(r)
+        r.set_heap_capacity(128)
+        r.render(sid, did, L0, "raycast")
+        assert not _lists(r)
+    for _ in range(65):
+        got = r.render(sid, did, L0, "raycast")
+    assert _lists(r)
+    assert (got - walked).abs().max() < 1e-5  # the same hits, blended in another order of sums
+    r.close()
