@@ -514,6 +514,13 @@ dl_status out_finish(dl_ctx* ctx, float* out, int32_t kind, const float* dst, si
     return DL_OK;
 }
 
+// Rays that a DL_RAYCAST frame takes at a time: at most 2 GB of lists, evenly.
+int64_t cast_chunk(int64_t n_rays, int32_t heap_cap) {
+    const int64_t most = std::max<int64_t>((int64_t(1) << 31) / (8 * heap_cap), 1);
+    const int64_t chunks = (n_rays + most - 1) / most;
+    return chunks > 0 ? (n_rays + chunks - 1) / chunks : 1;
+}
+
 // The tile lists of a DL_RAYCAST frame: per (view, Gaussian) the outline of its
 // alpha >= 1/255 ellipsoid, and a key in every tile that it reaches, emitted
 // into slices laid out from the signature's previous frame (and again, on the
@@ -638,10 +645,8 @@ dl_status render_raycast(dl_ctx* ctx, int32_t scene_id, int32_t display_id, Scen
     uint32_t* over = nullptr;
     int32_t launches = 0;
     bool lists = false;
-    // rays a chunk: 2 GB of lists, evenly
-    const int64_t most = std::max<int64_t>((int64_t(1) << 31) / (8 * ctx->heap_cap), 1);
-    const int64_t chunks = (R.n_rays + most - 1) / most;
-    const int64_t chunk = chunks > 0 ? (R.n_rays + chunks - 1) / chunks : 1;
+    const int64_t chunk = cast_chunk(R.n_rays, ctx->heap_cap);
+    const int64_t chunks = (R.n_rays + chunk - 1) / chunk;
     st = build_cast_lists(ctx, S, D, *G, hint, cams, chunk, s, &sl, &over, &launches, &lists);
     if (st) return st;
     if (!lists) {
@@ -1145,6 +1150,10 @@ dl_status dl_query_footprint(dl_ctx* ctx, int32_t scene_id, int32_t display_id, 
     const size_t keys = 2 * ne;
     b += 2 * keys * 12 + radix_tmp_bytes(int64_t(keys));
     if (mode == DL_STANDARD || mode == DL_STANDARD_SR) b += size_t(D.q.nv) * D.q.w * D.q.h * 12;
+    if (mode == DL_RAYCAST) {  // intersection lists, with a buffer's slack
+        const size_t lists = cast_tmp_bytes(cast_chunk(D.rep.n_rays, ctx->heap_cap), ctx->heap_cap);
+        b += lists + lists / 8;
+    }
     *bytes = std::max(b, ctx->ws.last_bytes);
     return DL_OK;
 }

@@ -118,3 +118,15 @@ def test_ray_order_lists_are_asked_for_again():
     assert _lists(r)
     assert (got - walked).abs().max() < 1e-5  # the same hits, blended in another order of sums
     r.close()
+
+
+@pytest.mark.parametrize("heap", [16, 128])
+def test_footprint_estimate_counts_the_intersection_lists(heap):
+    from paper_2407_14053_gb300 import Renderer
+    r = Renderer(0)
+    did = r.set_display(PANEL)
+    sid = r.load_gaussians(_covering_scene(20_000, False), "f32")
+    r.set_heap_capacity(heap)
+    lists = 8 * heap * r.display_info(did)[0]
+    assert r.footprint(sid, did, "raycast") > lists > r.footprint(sid, did, "directl")
+    r.close()
