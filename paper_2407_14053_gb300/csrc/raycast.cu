@@ -755,10 +755,18 @@ __global__ void __launch_bounds__(kCastWarps * 32, 5) rc_cast_kernel(CastParams 
             const uint32_t pixel = uint32_t(P.grouped[active ? rid : wi.z - 1].x);
             const Ray ray = make_ray(cam, pixel, P.focal, P.half_w, P.half_h);
             const int col = int(pixel & 0xFFFFu), row = int(pixel >> 16);
-            const float ox = 0.5f * float(__reduce_min_sync(0xffffffffu, col) +
-                                          __reduce_max_sync(0xffffffffu, col));
-            const float oy = 0.5f * float(__reduce_min_sync(0xffffffffu, row) +
-                                          __reduce_max_sync(0xffffffffu, row));
+            const int c0x = __reduce_min_sync(0xffffffffu, col), c1x = __reduce_max_sync(0xffffffffu, col);
+            const int r0y = __reduce_min_sync(0xffffffffu, row), r1y = __reduce_max_sync(0xffffffffu, row);
+            const float ox = 0.5f * float(c0x + c1x), oy = 0.5f * float(r0y + r1y);
+            // 1 + a margin for the rounding of the test below: with the rays'
+            // box of diagonal d, a ray inside an outline is at most sqrt(e) + d
+            // pixels (and the box's centre at most that) from the outline's
+            // centre, e the largest of E, so the terms are at most that squared
+            // over E's floor 0.5 + 2e-5 e, i.e. below 2 d^2 + 5e4.  Six roundings
+            // of 2^-24 of that, at least the 0.02 of a 32 x 32 tile (a search of
+            // 20 million outlines against 64 bits found 1.25 at most).
+            const float dw = float(c1x - c0x), dh = float(r1y - r0y);
+            const float inside = 1.f + fmaxf(0.02f, fmaf(dw * dw + dh * dh, 7.2e-7f, 0.018f));
             // lanes past the group's rays add nothing (their rays are not open)
             RayHits<CastList, true> hits;
             hits.list = {P.hits + (rid - P.ray0), P.chunk + kCastSpill};
@@ -802,10 +810,7 @@ __global__ void __launch_bounds__(kCastWarps * 32, 5) rc_cast_kernel(CastParams 
                     float A = 0.f, B = 0.f, C = 0.f, D = 0.f, E = 0.f, F = -1e30f;
                     if (lane < n) {
                         // 1 + the outline's quadratic, expanded about (ox, oy),
-                        // and a margin of 0.02 for its rounding: a ray inside is
-                        // at most sqrt(e) + 45 pixels from the centre, e the
-                        // largest of E, and the terms at most that squared over
-                        // E's floor 0.5 + 2e-5 e, i.e. below 5e4
+                        // and the margin
                         const float4 q0 = W.c.rec[slot][0][lane];
                         const float du = q0.x - (ox - P.half_w), dv = q0.y - (oy - P.half_h);
                         A = q0.z;
@@ -813,7 +818,7 @@ __global__ void __launch_bounds__(kCastWarps * 32, 5) rc_cast_kernel(CastParams 
                         C = W.c.rec[slot][1][lane].x;
                         D = -fmaf(2.f * A, du, B * dv);
                         E = -fmaf(2.f * C, dv, B * du);
-                        F = fmaf(du, fmaf(A, du, B * dv), C * dv * dv) + 1.02f;
+                        F = fmaf(du, fmaf(A, du, B * dv), C * dv * dv) + inside;
                     }
                     const float2 A2 = make_float2(A, A), B2 = make_float2(B, B), C2 = make_float2(C, C);
                     const float2 D2 = make_float2(D, D), E2 = make_float2(E, E), F2 = make_float2(F, F);
