@@ -102,7 +102,7 @@ dl_status build_rayset(dl_ctx* ctx, Display& D, RaySet& R, bool identity, cudaSt
     const DisplayQ& q = D.q;
     const size_t n = 3 * size_t(q.w) * q.h;
     DL_CK(reserve_needed(ctx, R.src, 4 * n), "alloc src");
-    DL_CK(launch_repurpose(q, R.src.as<uint32_t>(), identity ? 1 : 0, s), "repurpose");
+    DL_CK(launch_repurpose(q, D.V.as<uint16_t>(), R.src.as<uint32_t>(), identity ? 1 : 0, s), "repurpose");
     DL_CK(reserve_needed(ctx, R.ray_of, 4 * n), "alloc ray_of");
     DevBuf tmp;
     DL_CK(reserve_needed(ctx, tmp, ray_table_tmp_bytes(q)), "alloc ray-table scratch");

@@ -2,6 +2,7 @@
 // Eqs. (1)-(3)), subpixel repurposing (Sec. 5, Alg. 2) and the R-first ray
 // table (Sec. 5, last part).  Integer arithmetic throughout, so the tables
 // are exact.
+#include <algorithm>
 #include <mutex>
 
 #include "../../include/directl.h"
@@ -12,12 +13,12 @@ namespace {
 
 constexpr int64_t kQ32 = int64_t(1) << 32;
 
-__device__ __forceinline__ int64_t floor_div(int64_t a, int64_t b) {
+__host__ __device__ __forceinline__ int64_t floor_div(int64_t a, int64_t b) {
     int64_t q = a / b;
     return (a % b != 0 && ((a < 0) != (b < 0))) ? q - 1 : q;
 }
 // d_offset (Eq. (1)) of subpixel column s in row x, Q32.
-__device__ __forceinline__ int64_t d_offset(const DisplayQ& q, int64_t x, int64_t s) {
+__host__ __device__ __forceinline__ int64_t d_offset(const DisplayQ& q, int64_t x, int64_t s) {
     return s * kQ32 + x * q.t3q - q.kq;
 }
 
@@ -233,6 +234,113 @@ repurpose_kernel(DisplayQ q, uint32_t* src) {
             __syncwarp();  // the group's lanes read what its first lane wrote
         }
     }
+}
+
+// Alg. 2, a warp per area, which takes the area's chains in turn and searches V
+// 32 candidates at a time.  It does not depend on how many views an area shows
+// nor on how many units a window holds, and is the better one where the
+// kernel above has few groups of lanes to run or many units to look at:
+//  - a pitch below a subpixel.  Panel set-up at 1080p with 45 views and an
+//    irregular slant: pitch 0.31 6.2 ms (50.8 with the kernel above), 0.52 5.2
+//    (14.6), 0.71 6.9 (12.0), 0.96 9.3 (10.2); 480 x 270 at 0.01 1.8 (662);
+//  - a pitch below 3.5 subpixels that, with the slant, repeats after a few
+//    subpixels, so that few of the views are shown.  Slant 1/6: pitch 1.05 45 ms
+//    (81), 1.5 26 (101), 2 21 (45), 3 16.0 (16.3); 200 views, 3 174 (226); slant
+//    1/3, 3 16.0 (20.7).  From 3.5 on the kernel above wins (4: 8.2 against
+//    18.6, slant 1/3 13.3 against 18.5), as it does where most views are shown
+//    (1.37: 7.2 against 13.9, 3.17: 4.3 against 19.2).
+__global__ void __launch_bounds__(128)
+repurpose_area_kernel(DisplayQ q, const uint16_t* __restrict__ V, uint32_t* src) {
+    const int lane = threadIdx.x & 31;
+    const int64_t warp = (blockIdx.x * int64_t(blockDim.x) + threadIdx.x) >> 5;
+    if (warp >= q.n_areas) return;
+    const int64_t a = q.area_min + warp;
+    const int64_t S = 3 * int64_t(q.w);
+    const int64_t most_u = (int64_t(1) << 53) / q.lq + 2;  // past every panel's units
+    // the area covers d in [lo_d, hi_d)
+    const int64_t lo_d = max(a * q.pw, -most_u) * q.lq, hi_d = min((a + 1) * q.pw, most_u) * q.lq;
+    for (int64_t x = 0; x < q.h; ++x) {
+        const int64_t base = x * q.t3q - q.kq;
+        const int64_t s_lo = max(ceil_q32(lo_d - base), 0), s_hi = min(int64_t(ceil_q32(hi_d - base)), S);
+        for (int64_t s = s_lo; s < s_hi; ++s) {
+            int64_t ci = x * S + s;
+            uint32_t cur = 0;
+            if (lane == 0) cur = src[ci];
+            cur = __shfl_sync(0xffffffffu, cur, 0);
+            if (cur != kEmpty) continue;
+            const uint16_t vi = V[ci];
+            uint32_t B0 = kEmpty, B1 = kEmpty, B2 = kEmpty;  // B_rgb(v_i, .)
+            int64_t cx = x, cy = s / 3;
+            int ck = int(s % 3);
+            while (true) {
+                const uint32_t Bk = ck == 0 ? B0 : (ck == 1 ? B1 : B2);
+                const bool idle = Bk != kEmpty;
+                const uint32_t own = pack_px(cx, cy);
+                if (lane == 0) src[ci] = idle ? Bk : own;  // Eq. (13) / (11)
+                // Eq. (12); used channels are cleared
+                B0 = ck == 0 ? kEmpty : (idle ? B0 : own);
+                B1 = ck == 1 ? kEmpty : (idle ? B1 : own);
+                B2 = ck == 2 ? kEmpty : (idle ? B2 : own);
+                // Eq. (14): rows [x + 2, x + win_dx], columns from y outward
+                const int64_t r0 = min(cx + 2, int64_t(q.h) - 1), r1 = min(cx + q.win_dx, int64_t(q.h) - 1);
+                const int64_t step = q.slant_neg ? 1 : -1;
+                const int64_t last = q.slant_neg ? min(cy + q.win_dy, int64_t(q.w) - 1)
+                                                 : max(cy - q.win_dy, int64_t(0));
+                const int64_t row = 3 * ((last - cy) * step + 1);  // candidates a row
+                const int64_t ncand = r1 >= r0 ? (r1 - r0 + 1) * row : 0;
+                int64_t found = -1;
+                for (int64_t b = 0; b < ncand; b += 32) {
+                    const int64_t j = b + lane;
+                    bool match = false;
+                    if (j < ncand) {
+                        const int64_t r = j / row, rem = j - r * row;
+                        const int ch = int(rem % 3);
+                        match = (ch == 0 ? B0 : (ch == 1 ? B1 : B2)) != kEmpty &&
+                                V[(r0 + r) * S + 3 * (cy + step * (rem / 3)) + ch] == vi;
+                    }
+                    const unsigned hit = __ballot_sync(0xffffffffu, match);
+                    if (hit) {
+                        found = b + (__ffs(hit) - 1);
+                        break;
+                    }
+                }
+                if (found < 0) break;  // no position left for view v_i
+                const int64_t r = found / row, rem = found - r * row;
+                cx = r0 + r;
+                cy += step * (rem / 3);
+                ck = int(rem % 3);
+                ci = cx * S + 3 * cy + ck;
+                // while condition of Alg. 2: inside the area and still empty
+                const int64_t d = d_offset(q, cx, 3 * cy + ck);
+                uint32_t next = 0;
+                if (lane == 0) next = src[ci];
+                next = __shfl_sync(0xffffffffu, next, 0);
+                if (d < lo_d || d >= hi_d || next != kEmpty) break;
+            }
+        }
+    }
+}
+
+// Whether x_offset takes few values (so few of the views are shown), by 64 runs
+// of 64 subpixels spread over the panel: fewer than half of four bins a view
+// (finer than the views, as values that lie on the border of two views show
+// both).
+bool few_offsets(const DisplayQ& q) {
+    constexpr int kRuns = 64, kRun = 64;
+    const int64_t S = 3 * int64_t(q.w), bins = std::min(4 * q.nv, kRuns * kRun / 4);
+    bool seen[kRuns * kRun / 4] = {};
+    int64_t filled = 0;
+    for (int i = 0; i < kRuns; ++i) {
+        const int64_t x = int64_t(q.h) * i / kRuns, s0 = (S * i / kRuns) * 7;
+        for (int j = 0; j < kRun; ++j) {
+            const int64_t d = d_offset(q, x, (s0 + j) % S);
+            const int64_t xo = d - floor_div(d, q.lq) * q.lq;
+            bool& f = seen[bins * xo / q.lq];
+            filled += f ? 0 : 1;
+            f = true;
+        }
+    }
+    return 2 * filled < bins;
 }
 
 __global__ void identity_src_kernel(int32_t w, int32_t h, uint32_t* __restrict__ src) {
@@ -455,13 +563,18 @@ cudaError_t launch_view_map(const DisplayQ& q, uint16_t* V, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_repurpose(const DisplayQ& q, uint32_t* src, int identity, cudaStream_t s) {
+cudaError_t launch_repurpose(const DisplayQ& q, const uint16_t* V, uint32_t* src, int identity,
+                             cudaStream_t s) {
     if (identity) {
         identity_src_kernel<<<grid_for(3 * int64_t(q.w) * q.h, 256), 256, 0, s>>>(q.w, q.h, src);
         return cudaGetLastError();
     }
     cudaError_t e = cudaMemsetAsync(src, 0xFF, sizeof(uint32_t) * 3 * size_t(q.w) * q.h, s);
     if (e != cudaSuccess) return e;
+    if (q.lq < kQ32 || (2 * q.lq < 7 * kQ32 && few_offsets(q))) {
+        repurpose_area_kernel<<<(q.n_areas + 3) / 4, 128, 0, s>>>(q, V, src);
+        return cudaGetLastError();
+    }
     // a warp a block: the warps' lengths differ with the areas on the panel
     const int64_t blocks = (int64_t(q.n_areas) * q.nv * kChainLanes + 31) / 32;
     repurpose_kernel<<<unsigned(blocks < 0x7FFFFFFF ? blocks : 0x7FFFFFFF), 32, 0, s>>>(q, src);

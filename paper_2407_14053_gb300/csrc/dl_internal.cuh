@@ -166,7 +166,9 @@ cudaError_t launch_gather_records(const void* src, void* dst, const uint32_t* pe
 
 // ---- a1..a3: display tables (display.cu) --------------------------------
 cudaError_t launch_view_map(const DisplayQ& q, uint16_t* V, cudaStream_t s);
-cudaError_t launch_repurpose(const DisplayQ& q, uint32_t* src, int identity, cudaStream_t s);
+// (V: the view map of launch_view_map)
+cudaError_t launch_repurpose(const DisplayQ& q, const uint16_t* V, uint32_t* src, int identity,
+                             cudaStream_t s);
 // Ray table: fills ray_of (3wh) and *d_n_rays (device); rays are numbered in
 // order of first use by R, then G, then B subpixels.  Scratch comes from
 // `tmp` (>= ray_table_tmp_bytes(q)); launch_ray_attributes then reads the
