@@ -437,9 +437,19 @@ dl_status harvest_readbacks(dl_ctx* ctx, bool wait) {
     return DL_OK;
 }
 
+// Whether the caller is capturing `s` into a graph: nothing may be waited for
+// or queried then, and what is enqueued has not run when the call returns.
+static bool capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) cudaGetLastError();
+    return st != cudaStreamCaptureStatusNone;
+}
+
 // Copies a frame's counter block to the next pinned slot of the ring (a slot
-// still in use is waited for and read first).
+// still in use is waited for and read first).  A captured frame's counters are
+// not read: its copy runs with every replay.
 static dl_status enqueue_readback(dl_ctx* ctx, FrameHint& hint, int64_t frame, cudaStream_t s) {
+    if (capturing(s)) return DL_OK;
     Workspace& W = ctx->ws;
     Readback& r = W.rb[W.rb_next];
     if (r.busy) {
@@ -553,6 +563,7 @@ dl_status build_cast_lists(dl_ctx* ctx, Scene& S, Display& D, TileGroups& G, Fra
     // memory that the tree would not need: without it the tree renders
     auto reserve = [](DevBuf& b, size_t bytes) { return b.reserve(bytes) == cudaSuccess; };
     const bool sizing = !hint.fits(W.keys[0]) || !hint.slices_ready;
+    if (sizing && capturing(s)) return DL_OK;  // sizing waits for the frame's counts
     if (!reserve(W.rec, 16 * kRecordFloat4 * size_t(ne)) || !reserve(W.gfill, words) ||
         !reserve(W.gscan_tmp, slice_tmp_bytes(ngroups)) ||
         !reserve(hint.slices[0], words) || !reserve(hint.slices[1], words) ||
@@ -1199,7 +1210,7 @@ dl_status render_frame(dl_ctx* ctx, int32_t scene_id, int32_t display_id, const 
     } enqueuing(W.enqueuing);
     // counters of earlier frames that have arrived update their signatures'
     // capacities before this frame is sized
-    st = harvest_readbacks(ctx, false);
+    if (!capturing(s)) st = harvest_readbacks(ctx, false);
     if (st) return st;
     const int64_t frame = W.frame_no++;
     const bool timing = ctx->timing;
