@@ -337,7 +337,9 @@ typedef struct {
     int32_t tile_w, tile_h;
     int32_t sort_bits;       /* key bits the radix sort ordered              */
     int32_t n_launches;      /* kernels the frame launched                   */
-    int64_t lists_small;     /* tile lists composited by the small class     */
+    int64_t lists_small;     /* tile lists composited by the small class
+                                (DL_RAYCAST: the lists that the rays were cast
+                                through, 0 when they walked the tree)        */
     int64_t lists_large;     /* tile lists composited by the large class     */
     int64_t max_list;        /* longest tile list (keys)                     */
     int64_t n_visible;       /* (view, Gaussian) records the projection wrote

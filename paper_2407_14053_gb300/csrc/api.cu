@@ -386,8 +386,11 @@ static void apply_readback(dl_ctx* ctx, Readback& r) {
     const uint32_t* m = reinterpret_cast<const uint32_t*>(hb + 128);
     const uint32_t* t32 = reinterpret_cast<const uint32_t*>(hb + 64);
     const int64_t nkeys = int64_t(h[0]), vis = int64_t(h[1]), slice_end = int64_t(t32[0]);
-    const int32_t reemitted = t32[1] != 0u ? 1 : 0;
-    const int64_t lists_small = int64_t(m[0]) + int64_t(m[4]), lists_large = m[1], longest = m[2];
+    const int32_t reemitted = t32[1] != 0u && !r.sizing ? 1 : 0;
+    // (ray-order frames have lists, and none where they walked the tree, but no classes)
+    const bool cast = r.cast >= 0;
+    const int64_t lists_small = cast ? (m[8] ? 0 : r.cast) : int64_t(m[0]) + int64_t(m[4]);
+    const int64_t lists_large = m[1], longest = m[2];
     const int32_t status = int32_t(m[7]);
     if (r.hint && (status != 0 || nkeys * 100 > r.hint->key_cap * 85 ||
                    slice_end * 100 > r.hint->key_cap * 85 ||
@@ -448,7 +451,8 @@ static bool capturing(cudaStream_t s) {
 // Copies a frame's counter block to the next pinned slot of the ring (a slot
 // still in use is waited for and read first).  A captured frame's counters are
 // not read: its copy runs with every replay.
-static dl_status enqueue_readback(dl_ctx* ctx, FrameHint& hint, int64_t frame, cudaStream_t s) {
+static dl_status enqueue_readback(dl_ctx* ctx, FrameHint& hint, int64_t frame, cudaStream_t s,
+                                  int64_t cast = -1, bool sizing = false) {
     if (capturing(s)) return DL_OK;
     Workspace& W = ctx->ws;
     Readback& r = W.rb[W.rb_next];
@@ -461,6 +465,8 @@ static dl_status enqueue_readback(dl_ctx* ctx, FrameHint& hint, int64_t frame, c
     r.busy = true;
     r.frame = frame;
     r.hint = &hint;
+    r.cast = cast;
+    r.sizing = sizing;
     W.rb_next = (W.rb_next + 1) % kReadbacks;
     return DL_OK;
 }
@@ -536,11 +542,11 @@ int64_t cast_chunk(int64_t n_rays, int32_t heap_cap) {
 // into slices laid out from the signature's previous frame (and again, on the
 // device, into slices of the frame's own counts when one is outgrown).  The
 // first frame of a signature starts from empty slices and reads its key total
-// back once to size the key buffer.  *over (device) is set when the keys do
+// back once to size the key buffer (sizing).  *over (device) is set when the keys do
 // not fit after all; *ready is false, and nothing is left to use, when the
 // signature's lists cannot be held (memory, or 2^31 entries).
 dl_status build_cast_lists(dl_ctx* ctx, Scene& S, Display& D, TileGroups& G, FrameHint& hint,
-                           const std::vector<Cam>& cams, int64_t chunk, cudaStream_t s,
+                           const std::vector<Cam>& cams, int64_t chunk, bool sizing, cudaStream_t s,
                            GroupSlices* sl, uint32_t** over, int32_t* launches, bool* ready) {
     Workspace& W = ctx->ws;
     *ready = false;
@@ -562,7 +568,6 @@ dl_status build_cast_lists(dl_ctx* ctx, Scene& S, Display& D, TileGroups& G, Fra
     const size_t words = 4 * size_t(ngroups + 1);
     // memory that the tree would not need: without it the tree renders
     auto reserve = [](DevBuf& b, size_t bytes) { return b.reserve(bytes) == cudaSuccess; };
-    const bool sizing = !hint.fits(W.keys[0]) || !hint.slices_ready;
     if (sizing && capturing(s)) return DL_OK;  // sizing waits for the frame's counts
     if (!reserve(W.rec, 16 * kRecordFloat4 * size_t(ne)) || !reserve(W.gfill, words) ||
         !reserve(W.gscan_tmp, slice_tmp_bytes(ngroups)) ||
@@ -658,7 +663,8 @@ dl_status render_raycast(dl_ctx* ctx, int32_t scene_id, int32_t display_id, Scen
     bool lists = false;
     const int64_t chunk = cast_chunk(R.n_rays, ctx->heap_cap);
     const int64_t chunks = (R.n_rays + chunk - 1) / chunk;
-    st = build_cast_lists(ctx, S, D, *G, hint, cams, chunk, s, &sl, &over, &launches, &lists);
+    const bool sizing = !hint.fits(W.keys[0]) || !hint.slices_ready;
+    st = build_cast_lists(ctx, S, D, *G, hint, cams, chunk, sizing, s, &sl, &over, &launches, &lists);
     if (st) return st;
     if (!lists) {
         st = begin_frame(ctx, cams, nullptr, 0, nullptr, s, &launches);
@@ -705,7 +711,7 @@ dl_status render_raycast(dl_ctx* ctx, int32_t scene_id, int32_t display_id, Scen
     DL_CK(launch_reorder(G->slot_of.as<uint32_t>(), W.raycol.as<float>(), w, h, dst, nullptr, s),
           "reorder");
     if (lists) {
-        st = enqueue_readback(ctx, hint, frame, s);
+        st = enqueue_readback(ctx, hint, frame, s, G->n_gwork, sizing);
         if (st) return st;
     }
     DL_CK(mark(8), "event");
@@ -713,7 +719,7 @@ dl_status render_raycast(dl_ctx* ctx, int32_t scene_id, int32_t display_id, Scen
     if (st) return st;
     dl_frame_stats& fs = ctx->stats;
     fs = dl_frame_stats{};
-    W.last_async = -1;
+    W.last_async = lists ? frame : -1;  // the keys and lists arrive with the counters
     fs.n_rays = R.n_rays;
     fs.n_launches = launches + 2;
     if (E) {

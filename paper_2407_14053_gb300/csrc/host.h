@@ -198,6 +198,8 @@ struct Readback {
     bool busy = false;
     int64_t frame = -1;
     FrameHint* hint = nullptr;
+    int64_t cast = -1;    // DL_RAYCAST: tile lists that the rays were to be cast through
+    bool sizing = false;  // and whether the frame laid out its own slices
 };
 
 struct Workspace {
