@@ -298,12 +298,17 @@ enum { DL_OPT_SORT_MODE = 1, DL_OPT_EVAL_DIRECTL = 2, DL_OPT_EVAL_STANDARD = 3,
  * are blended in t order (alpha clamped to 0.99, stop before T < 1e-4) with
  * the SH colour at d.  The rays of a (view, tile) go through the list of the
  * Gaussians whose alpha >= 1/255 outline reaches it; the first such frame of a
- * (scene, display, tile shape) synchronises `stream` once in mid-frame to size
- * the lists.  A frame whose lists do not fit walks an 8-wide tree of the
+ * (scene, display, tile shape), and one after a frame that used most of their
+ * room, synchronises `stream` once in mid-frame to size the lists.  A frame
+ * whose lists do not fit, or whose lists would have to be sized while the
+ * caller captures `stream` into a graph, walks an 8-wide tree of the
  * Gaussians' alpha >= 1/255 boxes instead (binary SAH splits over the scene's
  * stored Morton order, collapsed into 8-wide nodes; Sec. 7), built on the GPU
- * on the first such frame of a scene and kept with it.  Same image either
- * way. */
+ * on the first such frame of a scene and kept with it.  The intersections are
+ * the same either way, the colours equal to FP32 rounding (the order of the SH
+ * sums).  The lists take up to 2 GB, given back when another call needs
+ * memory; where they could not be had they are asked for again 64 frames
+ * later, or with a smaller c_h. */
 /* DL_OPT_STANDARD_VIEW_SIZE: resolution at which DL_STANDARD renders each
  * view, value = (view_w << 16) | view_h, 0 = the panel's (HR).  Below panel
  * resolution (the LR / MR configurations of the paper's experiments) every

@@ -1915,7 +1915,7 @@ cudaError_t launch_views(const CompositeParams& p, const int4* items, const int4
                          int64_t n_work, const int64_t n[3], int block_cap, uint32_t* const cursor[2],
                          const unsigned long long* keys, const float4* rec, float* Mm,
                          unsigned long long* pairs, cudaStream_t s) {
-    // the longest lists first: the short ones fill the tail
+    // one after another on the one stream, the longest lists first
     if (n[2] > 0) {
         const size_t smem = views_block_smem_bytes(block_cap);
         cudaError_t e = cudaFuncSetAttribute(composite_views_block_kernel<COUNT>,

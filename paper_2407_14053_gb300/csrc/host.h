@@ -99,19 +99,6 @@ struct PendingFrame {
     int32_t reemitted = 0;
 };
 
-// Capacities a frame signature (scene, display, mode, tile, view size) runs
-// with once one of its frames has been sized on the host: the tile-key
-// buffer's capacity at that time and the long-list capacity.  Later frames
-// of the signature size their launches from device counters and these
-// capacities, with no host synchronisation; a frame that exceeds them is
-// dropped on the device (its output left untouched, its status word set),
-// and the next frame of the signature is sized on the host again, as is one
-// after a frame that used more than 85 % of either capacity or had a list that
-// its block class could not sort in shared memory.
-// With the keys emitted by the projection, the signature also keeps the
-// slices of the key buffer its next frame emits into: every group gets its
-// key count in the last frame plus an eighth and 16 (slices[cur]); a frame
-// writes the next layout into slices[cur ^ 1] and flips cur.
 // DL_OPT_KEY_EMISSION: 0 is the two-pass emission; 1 and 2 (the library's
 // choice) have the projection emit the keys.  With the views split into ranges
 // for small scenes that is the faster one at every size measured: 107 against
@@ -171,6 +158,19 @@ struct SideStreams {
 // frames that do without memory that could not be had, before it is asked for again
 constexpr int32_t kAskAgain = 64;
 
+// Capacities a frame signature (scene, display, mode, tile, view size) runs
+// with once one of its frames has been sized on the host: the tile-key
+// buffer's capacity at that time and the long-list capacity.  Later frames
+// of the signature size their launches from device counters and these
+// capacities, with no host synchronisation; a frame that exceeds them is
+// dropped on the device (its output left untouched, its status word set),
+// and the next frame of the signature is sized on the host again, as is one
+// after a frame that used more than 85 % of either capacity or had a list that
+// its block class could not sort in shared memory.
+// With the keys emitted by the projection, the signature also keeps the
+// slices of the key buffer its next frame emits into: every group gets its
+// key count in the last frame plus an eighth and 16 (slices[cur]); a frame
+// writes the next layout into slices[cur ^ 1] and flips cur.
 struct FrameHint {
     bool sized = false;
     int32_t block_cap = 2048;   // longest list of a later frame, a power of two
@@ -263,7 +263,7 @@ struct dl_ctx {
     int32_t sort_mode = DL_SORT_AUTO;
     int32_t eval_transposed[3] = {1, 0, 1};  // per mode
     int32_t warp_cap = 512;
-    int32_t key_emission = 2;  // DL_OPT_KEY_EMISSION (2: by scene size)
+    int32_t key_emission = 2;  // DL_OPT_KEY_EMISSION (2: the library's choice)
     int32_t std_view_w = 0, std_view_h = 0;  // DL_OPT_STANDARD_VIEW_SIZE (0: panel)
     int32_t heap_cap = 128;                  // DL_OPT_HEAP_CAPACITY
     bool timing = false;

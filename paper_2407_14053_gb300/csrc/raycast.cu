@@ -13,7 +13,8 @@
 // their (view, tile), which holds every Gaussian whose alpha >= 1/255 outline
 // reaches the tile (rc_cast_kernel).  When the lists of a frame do not fit
 // their memory, the rays walk the scene's tree (rc_trace_kernel).  Both test
-// with rc_alpha and keep the same list, so the image is the same.
+// with rc_alpha and keep the same list; the colours may differ by the order of
+// the SH sums (rc_blend_kernel).
 //
 // The tree (Sec. 7: a compact 8-wide bounding-volume hierarchy built with
 // the surface area heuristic): every Gaussian is bounded by the box of its
@@ -690,12 +691,14 @@ rc_trace_kernel(const float4* __restrict__ gauss, const RayNode* __restrict__ no
 // candidates through the exact rc_alpha into its list.  In depth order a ray
 // finds its hits nearly sorted, and a list ends for the warp once every ray's
 // bound lies before the next record's least depth.  The lists only say which
-// Gaussians are tested and in which order, so the image is the tree walk's bit
-// for bit.
+// Gaussians are tested and in which order, so a ray's intersections are the
+// tree walk's.  (Gaussians thinner than about 400 : 1 apart: the FP32 test then
+// also passes points that 64 bits put below 1/255, and of those the lists hold
+// what lies inside the outline.)
 //
 // Bound by the latency of the candidates' evaluation and insertion at half the
 // lanes (rays have different numbers of candidates in a batch).  1080p frame,
-// 200k Gaussians, c_h 128: 3.8 ms, of which outlines and keys 0.28, cast 2.4,
+// 200k Gaussians, c_h 128: 3.8 ms, of which outlines and keys 0.23, cast 2.4,
 // blend 1.2; the tree walk takes 10.0 ms.
 constexpr int kCastCap = 512;
 constexpr int kCastWarps = 4;
